@@ -82,7 +82,7 @@ def draw(rng):
     if kind in ("pstep", "pjvp"):
         mt, kz = rng.randint(4, 12), rng.randint(6, 24)
         good = [n for n in (16, 18, 24, 32, 36, 48, 54, 64, 72, 96)]
-        c = _pipe("", kind, "fp64" if kind == "pstep" else prec, nr=rng.randint(32, 64), mt=mt, kz=kz,
+        c = _pipe("", kind, "fp64" if kind == "pstep" else prec, nr=2 * rng.randint(16, 32), mt=mt, kz=kz,
                   ntheta=min(n for n in good if n >= 3 * mt + 1), nz=min(n for n in good if n >= 3 * kz + 1),
                   alpha=rng.choice([0.8, 1.25, 1.7]), re=round(rng.uniform(500, 3000), 1),
                   dt=rng.choice([10.0, 50.0, 100.0]), n_dir=1 if kind == "pstep" else spread(1, 64))
