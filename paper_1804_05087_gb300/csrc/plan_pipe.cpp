@@ -173,7 +173,7 @@ sp_status sp_build_pipe_plan(sp_ctx* c) {
   if (kl > kPipeKL || kl + ku + 1 > kPipeKW) return sp_fail(c, SP_EINVAL, "radial stencil band wider than supported");
   kl = kPipeKL;               // the factors are stored with the fixed widths the kernel is built for
   const int kw = kPipeKW;     // upper factor after the row interchanges
-  const size_t chunk = (size_t)nr * (kw + kl) * 8 + ((size_t)nr * 4 + 15) / 16 * 16;
+  const size_t chunk = ((size_t)nr * (kw + kl) * 8 + (size_t)nr * 4 + 15) / 16 * 16;  // bulk copies: multiples of 16 bytes
   c->pb_chunk = chunk;
   const size_t nu4 = (size_t)c->n_unique * 4;
   std::vector<unsigned char> fac(nu4 * chunk, 0);
