@@ -92,7 +92,8 @@ static void free_ctx(sp_ctx* c) {
                   c->twx_f, c->twz_f, c->ops, c->ws6, c->ws3, c->base64, c->base32, c->U0,
                   c->G0, c->tmp, c->red, c->kry, c->wsG, c->pb_fac, c->pb_uh, c->pb_dinv, c->fd_w1, c->fd_c1, c->dzU,
                   c->traj, c->nbuf, c->traj_base, c->chain, c->Tp, c->TDp, c->tq,
-                  c->Tp_f, c->TDp_f, c->tq_f, c->Cq, c->Cq_f, c->yinv_tc_mat, c->rhs_tc_mat};
+                  c->Tp_f, c->TDp_f, c->tq_f, c->Cq, c->Cq_f, c->yinv_tc_mat, c->rhs_tc_mat, c->fx_tw, c->fx_G,
+                  c->fx_gmeta, c->base_fx};
   for (void* p : ptrs)
     if (p) cudaFree(p);
   if (c->red_host) cudaFreeHost(c->red_host);
@@ -167,7 +168,6 @@ static bool alloc_workspaces(sp_ctx* c) {
   const size_t grid = (size_t)c->NY * c->nx * c->nz;
   c->red_blocks = 2 * c->sm_count;
   bool ok = cudaMalloc(&c->ws6, B * plane6) == cudaSuccess && cudaMalloc(&c->ws3, B * plane3) == cudaSuccess &&
-            cudaMalloc((void**)&c->base64, 6 * grid * 8) == cudaSuccess &&
             cudaMalloc((void**)&c->base32, 6 * grid * 4) == cudaSuccess &&
             cudaMalloc((void**)&c->base32t, 6 * grid * 4) == cudaSuccess &&
             cudaMalloc((void**)&c->U0, c->state_len * 8) == cudaSuccess &&
@@ -175,9 +175,11 @@ static bool alloc_workspaces(sp_ctx* c) {
             cudaMalloc((void**)&c->tmp, B * c->state_len * 8) == cudaSuccess &&
             cudaMalloc((void**)&c->red, (size_t)64 * c->red_blocks * 8 + 4096) == cudaSuccess &&
             cudaMallocHost((void**)&c->red_host, (size_t)64 * c->red_blocks * 8 + 4096) == cudaSuccess;
+  if (ok) ok = sp_fx_setup(c) == SP_OK;
   const size_t gplane = sp_xz_global_plane_bytes(c);
   if (ok && gplane) ok = cudaMalloc(&c->wsG, B * gplane) == cudaSuccess;
   if (ok && c->geom == 1) ok = cudaMalloc((void**)&c->dzU, c->state_len * 8) == cudaSuccess;
+  if (ok && !c->use_fx) ok = cudaMalloc((void**)&c->base64, 6 * grid * 8) == cudaSuccess;
   if (!ok) cudaGetLastError();
   return ok;
 }
@@ -585,7 +587,8 @@ extern "C" sp_status sp_step_n(sp_ctx* c, const double* U, double* G, int n, voi
 // bytes of one trajectory step's base fields in the precision of the tangent
 static size_t base_slot_bytes(const sp_ctx* c) {
   const size_t grid = (size_t)6 * c->NY * c->nx * c->nz;
-  return c->cfg.prec == SP_MIXED ? 2 * grid * 4 : grid * 8;
+  if (c->cfg.prec == SP_MIXED) return 2 * grid * 4;
+  return c->use_fx ? grid * 8 + (size_t)c->NY * 16 : grid * 8;
 }
 
 // copy the base fields of the tangent's precision to (save = true) or from trajectory slot k
@@ -601,6 +604,7 @@ static sp_status base_slot(sp_ctx* c, int k, bool save, cudaStream_t st) {
     if (e == cudaSuccess) e = cp(c->base32t, slot + grid * 4, grid * 4);
     return sp_cuda(c, e, "trajectory base fields");
   }
+  if (c->use_fx) return sp_cuda(c, cp(c->base_fx, slot, base_slot_bytes(c)), "trajectory base fields");
   return sp_cuda(c, cp(c->base64, slot, grid * 8), "trajectory base fields");
 }
 

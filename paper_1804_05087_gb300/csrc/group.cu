@@ -194,6 +194,24 @@ __global__ void __launch_bounds__(kVecThreads) k_gscale(double* __restrict__ dst
     dst[r.off + e] = f * src[r.off + e];
 }
 
+// every member's linearisation point and its G from group vectors into the members' own buffers
+struct GBase {
+  double *u0, *g0;
+};
+__global__ void __launch_bounds__(kVecThreads) k_gbase(const double* __restrict__ U, const double* __restrict__ G,
+                                                       const GBase* __restrict__ dst, const GVec* __restrict__ recs,
+                                                       const int* __restrict__ inst) {
+  const int i = inst[blockIdx.x];
+  const GVec r = recs[i];
+  const GBase d = dst[i];
+  const int b = blockIdx.x - r.first_el;
+  const size_t len = 2 * r.ncplx;
+  for (size_t e = (size_t)b * blockDim.x + threadIdx.x; e < len; e += (size_t)r.nb_el * blockDim.x) {
+    d.u0[e] = U[r.off + e];
+    d.g0[e] = G[r.off + e];
+  }
+}
+
 double now_ms() {
   return std::chrono::duration<double, std::milli>(std::chrono::steady_clock::now().time_since_epoch()).count();
 }
@@ -212,6 +230,7 @@ struct sp_group {
   GrpPlan plan;
   // vector launches
   GVec* vrecs = nullptr;
+  GBase* brecs = nullptr;   // where the members keep U0 and G0
   int* vinst = nullptr;     // block -> member, reduction launches
   int vblocks = 0;
   int* einst = nullptr;     // block -> member, elementwise launches
@@ -255,7 +274,7 @@ static void drop_graphs(sp_group* g) {
 static void free_group(sp_group* g) {
   drop_graphs(g);
   grp_plan_free(&g->plan);
-  for (void* p : {(void*)g->vrecs, (void*)g->vinst, (void*)g->einst, (void*)g->act, (void*)g->scal, (void*)g->part, (void*)g->tmpv,
+  for (void* p : {(void*)g->vrecs, (void*)g->brecs, (void*)g->vinst, (void*)g->einst, (void*)g->act, (void*)g->scal, (void*)g->part, (void*)g->tmpv,
                   (void*)g->kry})
     if (p) cudaFree(p);
   if (g->act_h) cudaFreeHost(g->act_h);
@@ -296,9 +315,8 @@ extern "C" sp_status sp_group_create(const sp_config* cfgs, int n, sp_group** ou
     c.max_batch = 1;
     sp_status s = sp_create(&c, &g->mem[i]);
     if (s != SP_OK) return bail(s, "member " + std::to_string(i) + ": " + sp_last_error(nullptr));
-    // the grouped FP64 plane stage is the generic kernel: a member's own calls use it too,
-    // so that they compute exactly what the group computes for it
-    g->mem[i]->use_xz_reg64 = 0;
+    // a member's own calls use the kernels of the grouped launches, so that they compute exactly
+    // what the group computes for it
     g->mem[i]->use_yinv_tc = 0;
     g->mem[i]->use_rhs_tc = 0;
     g->off[i] = pos;
@@ -333,7 +351,10 @@ extern "C" sp_status sp_group_create(const sp_config* cfgs, int n, sp_group** ou
   }
   g->vblocks = (int)vinst.size();
   g->eblocks = (int)einst.size();
-  if ((e = grp_upload((void**)&g->vrecs, g->vrecs_h.data(), n * sizeof(GVec))) != cudaSuccess ||
+  std::vector<GBase> brecs(n);
+  for (int i = 0; i < n; ++i) brecs[i] = {g->mem[i]->U0, g->mem[i]->G0};
+  if ((e = grp_upload((void**)&g->brecs, brecs.data(), n * sizeof(GBase))) != cudaSuccess ||
+      (e = grp_upload((void**)&g->vrecs, g->vrecs_h.data(), n * sizeof(GVec))) != cudaSuccess ||
       (e = grp_upload((void**)&g->vinst, vinst.data(), vinst.size() * sizeof(int))) != cudaSuccess ||
       (e = grp_upload((void**)&g->einst, einst.data(), einst.size() * sizeof(int))) != cudaSuccess)
     return bail(SP_ECUDA, std::string("vector tables: ") + cudaGetErrorString(e));
@@ -395,25 +416,20 @@ static sp_status group_jvp(sp_group* g, const double* du, double* Jdu, const int
   return gcuda(g, grp_launch_solve(g->plan, f32, du, Jdu, act, st), "group solve");
 }
 
-// base fields of every member (FP64 and float copies); with_g0 also stores each
-// member's U0 and G(U0) for its finite-difference action
+// base fields of every member in the tangent's precision; with_g0 also stores each member's U0
+// and G(U0) for its finite-difference action: one pass of curl, values and inverse transforms then
+// serves both the base fields and the step's product (as in sp_set_base)
 static sp_status group_base(sp_group* g, const double* U, bool with_g0, const int* act, cudaStream_t st) {
   sp_status s;
   if ((s = gcuda(g, grp_launch_yinv(g->plan, false, U, act, st), "group yinv")) != SP_OK) return s;
-  if ((s = gcuda(g, grp_launch_xz(g->plan, false, XZ_BASE, act, st), "group xz base")) != SP_OK) return s;
+  if ((s = gcuda(g, grp_launch_xz(g->plan, false, with_g0 ? XZ_STEP_BASE : XZ_BASE, act, st), "group xz base")) != SP_OK)
+    return s;
   for (sp_ctx* c : g->mem)
     if ((s = gcuda(g, launch_base_to_f32(c, st), "base f32")) != SP_OK) return s;
   if (with_g0) {
-    if ((s = group_step(g, U, g->tmpv, nullptr, st)) != SP_OK) return s;
-    for (int i = 0; i < g->n; ++i) {
-      sp_ctx* c = g->mem[i];
-      const size_t bytes = c->state_len * 8;
-      if ((s = gcuda(g, cudaMemcpyAsync(c->U0, U + g->off[i], bytes, cudaMemcpyDeviceToDevice, st), "U0")) != SP_OK)
-        return s;
-      if ((s = gcuda(g, cudaMemcpyAsync(c->G0, g->tmpv + g->off[i], bytes, cudaMemcpyDeviceToDevice, st), "G0")) !=
-          SP_OK)
-        return s;
-    }
+    if ((s = gcuda(g, grp_launch_solve(g->plan, false, U, g->tmpv, act, st), "group solve")) != SP_OK) return s;
+    k_gbase<<<g->eblocks, kVecThreads, 0, st>>>(U, g->tmpv, g->brecs, g->vrecs, g->einst);
+    if ((s = gcuda(g, cudaGetLastError(), "U0, G0")) != SP_OK) return s;
   }
   for (sp_ctx* c : g->mem) c->has_base = 1;
   return SP_OK;

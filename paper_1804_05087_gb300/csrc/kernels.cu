@@ -1619,7 +1619,7 @@ size_t sp_xz_global_plane_bytes(const sp_ctx* c) {
   const size_t RS = 6 * (size_t)(c->MZ + 1);
   const size_t per = (size_t)c->NY * c->nx * RS;  // complex values per direction
   size_t b = 0;
-  if (c->xz_gglob64) b = per * 16;
+  if (c->xz_gglob64 && !c->use_fx) b = per * 16;
   if (c->xz_gglob32 && per * 8 > b) b = per * 8;
   return b;
 }
@@ -1686,9 +1686,7 @@ cudaError_t launch_xz(const sp_ctx* c, bool fp32, int mode, const void* in6, voi
                       cudaStream_t st) {
   if (fp32 && c->use_xz_reg && sp_xz_reg_supported(c) && (mode == XZ_TANGENT || mode == XZ_ADJOINT))
     return launch_xz_reg(c, mode, in6, out3, n_dir, st);
-  if (!fp32 && c->use_xz_reg64 && sp_xz_reg64_supported(c) &&
-      (mode == XZ_TANGENT || mode == XZ_ADJOINT || mode == XZ_STEP || mode == XZ_STEP_BASE))
-    return launch_xz_reg64(c, mode, in6, out3, n_dir, st);
+  if (!fp32 && c->use_fx) return launch_xz_fx(c, mode, in6, out3, n_dir, st);
   if (fp32) {
     const C2<float>* tx = reinterpret_cast<const C2<float>*>(c->twx_f);
     const C2<float>* tz = reinterpret_cast<const C2<float>*>(c->twz_f);
@@ -1865,6 +1863,7 @@ cudaError_t launch_finish_adj(const sp_ctx* c, const double* r, double* out, int
 }
 
 cudaError_t launch_base_to_f32(const sp_ctx* c, cudaStream_t st) {
+  if (c->use_fx) return cudaSuccess;  // the plane stage writes what the tangent reads
   size_t n = (size_t)6 * c->NY * c->nx * c->nz;
   k_f64_to_f32<<<grid_for(n, 256, c->sm_count), 256, 0, st>>>(c->base64, c->base32, c->base32t, n, c->nx, c->nz);
   return cudaGetLastError();
@@ -1973,7 +1972,8 @@ void grp_kernel_free(GrpKernel* k) {
 }
 
 void grp_plan_free(GrpPlan* p) {
-  for (GrpKernel* k : {&p->yinv64, &p->yinv32, &p->xz64, &p->xz32, &p->solve64, &p->solve32}) grp_kernel_free(k);
+  for (GrpKernel* k : {&p->yinv64, &p->yinv32, &p->xz64, &p->xz32, &p->solve64, &p->solve32, &p->fx[0], &p->fx[1]})
+    grp_kernel_free(k);
   for (GrpKernel& k : p->xzr) grp_kernel_free(&k);
   p->n = 0;
 }
@@ -2042,7 +2042,7 @@ static cudaError_t grp_build_xz(GrpKernel* k, sp_ctx* const* mem, int n, const i
     }
     nblk[m] = skip && (*skip)[m] ? 0 : c->NY;
   }
-  for (auto fn : {k_xz_grp<T, XZ_STEP>, k_xz_grp<T, XZ_BASE>, k_xz_grp<T, XZ_TANGENT>}) {
+  for (auto fn : {k_xz_grp<T, XZ_STEP>, k_xz_grp<T, XZ_BASE>, k_xz_grp<T, XZ_STEP_BASE>, k_xz_grp<T, XZ_TANGENT>}) {
     cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
   }
@@ -2084,7 +2084,10 @@ cudaError_t grp_plan_build(GrpPlan* p, sp_ctx* const* mem, int n, const size_t* 
   cudaError_t e;
   if ((e = grp_build_yinv<double>(&p->yinv64, mem, n, offs, order, jsplit)) != cudaSuccess) return e;
   if ((e = grp_build_yinv<float>(&p->yinv32, mem, n, offs, order, jsplit)) != cudaSuccess) return e;
-  if ((e = grp_build_xz<double>(&p->xz64, mem, n, order)) != cudaSuccess) return e;
+  std::vector<int> fxm(n);
+  for (int m = 0; m < n; ++m) fxm[m] = mem[m]->use_fx;
+  if ((e = grp_build_xz<double>(&p->xz64, mem, n, order, &fxm)) != cudaSuccess) return e;
+  if ((e = grp_build_xz_fx(p, mem, n, order)) != cudaSuccess) return e;
   // float plane stage: the register-FFT kernel for the members whose own context uses it,
   // the generic kernel for the others (so every member computes exactly as on its own)
   std::vector<int> reg(n);
@@ -2118,12 +2121,17 @@ cudaError_t grp_launch_xz(const GrpPlan& p, bool fp32, int mode, const int* acti
                                                                        k.inst, k.first, active);
     return cudaGetLastError();
   }
+  const cudaError_t e = grp_launch_xz_fx(p, mode, active, st);
+  if (e != cudaSuccess) return e;
   const GrpKernel& k = p.xz64;
   if (k.blocks == 0) return cudaSuccess;
   const XzArgs<double>* r = static_cast<const XzArgs<double>*>(k.recs);
   switch (mode) {
     case XZ_STEP: k_xz_grp<double, XZ_STEP><<<k.blocks, kThreadsXZ, k.smem, st>>>(r, k.inst, k.first, active); break;
     case XZ_BASE: k_xz_grp<double, XZ_BASE><<<k.blocks, kThreadsXZ, k.smem, st>>>(r, k.inst, k.first, active); break;
+    case XZ_STEP_BASE:
+      k_xz_grp<double, XZ_STEP_BASE><<<k.blocks, kThreadsXZ, k.smem, st>>>(r, k.inst, k.first, active);
+      break;
     case XZ_TANGENT:
       k_xz_grp<double, XZ_TANGENT><<<k.blocks, kThreadsXZ, k.smem, st>>>(r, k.inst, k.first, active);
       break;

@@ -124,7 +124,7 @@ struct sp_ctx {
   // device workspaces
   void* ws6 = nullptr;           // [batch][6][NY][Mm] complex (double-sized)
   void* ws3 = nullptr;           // [batch][3][NY][Mm] complex (double-sized)
-  double* base64 = nullptr;      // [6][NY][nx][nz]
+  double* base64 = nullptr;      // [6][NY][nx][nz] (without use_fx)
   float* base32 = nullptr;
   float* base32t = nullptr;      // [6][NY][nz][nx]: transposed copy for the register-FFT kernel
   double* U0 = nullptr;          // linearisation point
@@ -136,7 +136,6 @@ struct sp_ctx {
   int red_blocks = 0;
   int has_base = 0;
   int use_xz_reg = 1;            // float plane stage: register FFT kernel when the size allows
-  int use_xz_reg64 = 1;          // FP64 tangent/adjoint plane stage: register FFT kernel (xz_reg64.cu)
   int use_rhs_tc = 0;             // float forward transform of the chains on the tensor cores (yinv_tc.cu)
   int use_yinv_tc = 1;           // float inverse Chebyshev transform on the tensor cores (yinv_tc.cu)
   int solve_shape_tan = 0;       // k_solve tile shape of the tangent (sp_autotune)
@@ -147,6 +146,14 @@ struct sp_ctx {
   int xz_cx64 = 1, xz_cx32 = 1;
   int xz_gglob64 = 0, xz_gglob32 = 0;  // plane buffer in global memory (grid too large for chip)
   void* wsG = nullptr;           // [batch][NY][nx * RS] complex, only when a plane does not fit
+  // fixed-point FP64 plane stage (xz_fx.cuh): grids whose sizes factor into its radices
+  int use_fx = 0;
+  int fx_n1x = 0, fx_n2x = 0, fx_n1z = 0, fx_n2z = 0;  // nx = n1x n2x, nz = n1z n2z
+  int4* fx_tw = nullptr;         // [nx + nz] twiddles
+  void* fx_G = nullptr;          // planes between the launches of a split call
+  int* fx_gmeta = nullptr;       // their exponents
+  long long* base_fx = nullptr;  // FP64 contexts: base fields as integers, then base_meta
+  int* base_meta = nullptr;      // [NY][4] exponents and bit lengths
   std::string err;
   // tracing: event pairs per stage, recorded while `trace` is on
   bool trace = false;
@@ -225,6 +232,8 @@ struct GrpPlan {
   GrpKernel yinv64, yinv32, xz64, solve64, solve32;
   GrpKernel xz32;                 // float plane stage of the members without a register-FFT kernel
   GrpKernel xzr[kGrpRegClasses];  // float plane stage of the others, per grid size class (xz_reg.cu)
+  GrpKernel fx[2];                // FP64 plane stage in fixed point, per shared-memory class (xz_fx.cu)
+  std::vector<std::pair<int, sp_ctx*>> fx_own;  // members with their own split launches
 };
 // members: n contexts; offs: offset (doubles) of each member's state in a group
 // vector; order: member indices, largest first (blocks are laid out in this order)
@@ -240,6 +249,9 @@ cudaError_t grp_launch_solve(const GrpPlan& p, bool fp32, const double* du_base,
 cudaError_t grp_build_xz_reg(GrpKernel* ks, sp_ctx* const* members, int n, const int* order,
                              const std::vector<int>& use);
 cudaError_t grp_launch_xz_reg(const GrpKernel* ks, const int* active, cudaStream_t st);
+// FP64 plane stage of the members that take the fixed-point kernels (the others: xz64)
+cudaError_t grp_build_xz_fx(GrpPlan* p, sp_ctx* const* members, int n, const int* order);
+cudaError_t grp_launch_xz_fx(const GrpPlan& p, int mode, const int* active, cudaStream_t st);
 // device copy of a host table; frees nothing on failure
 cudaError_t grp_upload(void** dst, const void* src, size_t bytes);
 void grp_kernel_free(GrpKernel* k);
@@ -267,9 +279,9 @@ cudaError_t launch_rhs_tc(const sp_ctx* c, const void* in3, const double* du, vo
                           long long sd, long long sn, cudaStream_t st);
 std::vector<float> rhs_tc_image(const double* cf, int NY, int NR);
 size_t yinv_tc_smem(int NY);
-// FP64 plane stage with register-resident FFTs (xz_reg64.cu), square grids 16..48
-bool sp_xz_reg64_supported(const sp_ctx* c);
-cudaError_t launch_xz_reg64(const sp_ctx* c, int mode, const void* in, void* out, int n_dir, cudaStream_t st);
+// fixed-point plane stage (xz_fx.cu): every FP64 mode; setup sets use_fx when the grid is covered
+sp_status sp_fx_setup(sp_ctx* c);
+cudaError_t launch_xz_fx(const sp_ctx* c, int mode, const void* in, void* out, int n_dir, cudaStream_t st);
 // batched tangent solve by O(N) chains (solve_chain.cu), two launches: k_rhs (values ->
 // right-hand sides in work, n_unique x 3 x (N-1) complex per direction), then k_chain
 // (one thread per mode, parity and direction); together the same inputs and outputs as
