@@ -91,8 +91,7 @@ static void free_ctx(sp_ctx* c) {
   void* ptrs[] = {c->Th, c->TDh, c->Cfh, c->yv, c->lam6, c->Th_f, c->TDh_f, c->Cfh_f, c->twx, c->twz, c->base32t,
                   c->twx_f, c->twz_f, c->ops, c->ws6, c->ws3, c->base64, c->base32, c->U0,
                   c->G0, c->tmp, c->red, c->kry, c->wsG, c->pb_fac, c->pb_uh, c->pb_dinv, c->fd_w1, c->fd_c1, c->dzU,
-                  c->traj, c->nbuf, c->traj_base, c->chain, c->Tp, c->TDp, c->tq,
-                  c->Tp_f, c->TDp_f, c->tq_f, c->Cq, c->Cq_f, c->yinv_tc_mat, c->rhs_tc_mat, c->fx_tw, c->fx_G,
+                  c->traj, c->nbuf, c->traj_base, c->chain, c->cheb_fx, c->wave, c->rowidx, c->cft_f, c->Cq_f, c->yinv_tc_mat, c->rhs_tc_mat, c->fx_tw, c->fx_G,
                   c->fx_gmeta, c->base_fx};
   for (void* p : ptrs)
     if (p) cudaFree(p);
@@ -285,7 +284,7 @@ static sp_status step_batch(sp_ctx* c, const double* U, double* G, int n, cudaSt
     }
     if ((s = sp_cuda(c, traced(c, SP_STAGE_STEP, st, [&] { return launch_yinv(c, false, u, c->ws6, nb, st); }), "yinv")) != SP_OK) return s;
     if ((s = sp_cuda(c, traced(c, SP_STAGE_STEP, st, [&] { return launch_xz(c, false, XZ_STEP, c->ws6, c->ws3, nb, st); }), "xz step")) != SP_OK) return s;
-    if ((s = sp_cuda(c, traced(c, SP_STAGE_STEP, st, [&] { return launch_solve(c, false, c->ws3, u, g, nb, st, c->solve_shape_step); }), "solve")) != SP_OK) return s;
+    if ((s = sp_cuda(c, traced(c, SP_STAGE_STEP, st, [&] { return launch_solve(c, false, c->ws3, u, g, c->ws6, nb, st, c->solve_shape_step); }), "solve")) != SP_OK) return s;
   }
   return SP_OK;
 }
@@ -334,7 +333,7 @@ extern "C" sp_status sp_set_base(sp_ctx* c, const double* U, void* stream) {
     if ((s = sp_cuda(c, traced(c, SP_STAGE_STEP, st, [&] { return launch_yinv(c, false, c->U0, c->ws6, 1, st); }), "yinv")) != SP_OK) return s;
     if ((s = sp_cuda(c, traced(c, SP_STAGE_STEP, st, [&] { return launch_xz(c, false, XZ_STEP_BASE, c->ws6, c->ws3, 1, st); }), "xz step+base")) != SP_OK) return s;
     if ((s = sp_cuda(c, traced(c, SP_STAGE_STEP, st, [&] { return launch_base_to_f32(c, st); }), "base f32")) != SP_OK) return s;
-    if ((s = sp_cuda(c, traced(c, SP_STAGE_STEP, st, [&] { return launch_solve(c, false, c->ws3, c->U0, c->G0, 1, st, c->solve_shape_step); }), "solve")) != SP_OK) return s;
+    if ((s = sp_cuda(c, traced(c, SP_STAGE_STEP, st, [&] { return launch_solve(c, false, c->ws3, c->U0, c->G0, c->ws6, 1, st, c->solve_shape_step); }), "solve")) != SP_OK) return s;
     c->has_base = 1;
     c->traj_n = 1;
     return SP_OK;
@@ -376,7 +375,7 @@ sp_status sp_tangent_solve(sp_ctx* c, bool f32, void* vals, size_t vals_bytes, c
     return sp_cuda(c, traced(c, SP_STAGE_SOLVE, st, [&] { return launch_chain_solve(c, du, out, work, vals, nb, st); }),
                    "chain solve");
   }
-  return sp_cuda(c, traced(c, SP_STAGE_SOLVE, st, [&] { return launch_solve(c, f32, vals, du, out, nb, st); }), "solve");
+  return sp_cuda(c, traced(c, SP_STAGE_SOLVE, st, [&] { return launch_solve(c, f32, vals, du, out, work, nb, st); }), "solve");
 }
 
 extern "C" sp_status sp_jvp(sp_ctx* c, const double* du, double* Jdu, int n_dir, void* stream) {
@@ -643,7 +642,7 @@ extern "C" sp_status sp_set_base_n(sp_ctx* c, const double* U, int n, void* stre
           (s = sp_cuda(c, traced(c, SP_STAGE_STEP, st, [&] { return launch_base_to_f32(c, st); }), "base f32")) != SP_OK)
         return s;
       if ((s = base_slot(c, k, true, st)) != SP_OK) return s;
-      if ((s = sp_cuda(c, traced(c, SP_STAGE_STEP, st, [&] { return launch_solve(c, false, c->ws3, Xk, D, 1, st, c->solve_shape_step); }), "solve")) != SP_OK) return s;
+      if ((s = sp_cuda(c, traced(c, SP_STAGE_STEP, st, [&] { return launch_solve(c, false, c->ws3, Xk, D, c->ws6, 1, st, c->solve_shape_step); }), "solve")) != SP_OK) return s;
     } else if ((s = step_batch(c, Xk, D, 1, st)) != SP_OK) {
       return s;
     }

@@ -1,0 +1,534 @@
+// Chebyshev transforms of the FP64 step and tangent in 64-bit fixed point (Sec. 3.2: Chebyshev in y).
+//
+//   k_yinv_fx: per Fourier mode, coefficients of u, v, w -> values of u, v, w and of the vorticity at
+//              the Gauss-Lobatto points (curl in spectral space), plane-major: the inputs and
+//              outputs of k_yinv (kernels.cu).
+//   k_rhs_fx : values of the product -> coefficients of the rows 0..N-2, plus u/dt: the right-hand
+//              sides of the per-mode solves (k_chain, k_solve).
+//
+// Both are sums over the constants T_n(y_j) = cos(pi j n / N). The FP64 pipe issues 2 operations per
+// SM and clock, the integer pipes 64 multiply-adds of 32-bit halves, three of which make one term of
+// a sum whose inputs share a scale. A column (one component of one mode) is scaled by its largest
+// value (59 bits) and its sum of moduli (62 bits, a bound of every result) and split as
+// x = hi 2^28 + lo; the constants are 56-bit, split the same way. hi hi and hi lo + lo hi are summed
+// in two 64-bit accumulators (both stay below 2^63 up to 129 terms, N <= 256); lo lo, below a quarter
+// of a unit, is dropped. Derivatives: n^2 a_n, scaled as a column of its own, times T_n'(y_j) / n^2.
+// Points y and -y share a table row: T_n(-y) = (-1)^n T_n(y), T_n'(-y) = -(-1)^n T_n'(y).
+#include <algorithm>
+#include <cmath>
+#include <vector>
+
+#include "fx_arith.h"
+#include "sp_internal.h"
+
+namespace {
+
+using namespace fx;
+
+constexpr int kThreadsC = 256;
+constexpr int kModes = 8;                       // modes per block
+constexpr int kColsY = 5 * kModes, kStrideY = kColsY + 1;  // u, v, w, Du, Dw of every mode (padded row)
+constexpr int kColsR = 3 * kModes, kStrideR = kColsR + 1;
+constexpr int kSumBits = 62, kMaxBits = 59;     // bits of a column's sum of moduli and of its values
+constexpr int kNotFinite = 1 << 28;             // exponent of a column with a non-finite input
+
+// x = hi 2^28 + lo, both signed
+__device__ __forceinline__ int2 halves(i64 x) {
+  const i64 hi = (x + (1 << 27)) >> 28;
+  return make_int2((int)hi, (int)(x - (hi << 28)));
+}
+__device__ __forceinline__ int4 halves2(i64 x, i64 y) {
+  const int2 a = halves(x), b = halves(y);
+  return make_int4(a.x, a.y, b.x, b.y);
+}
+
+// sum of x c: c in units of 2^-56 as halves
+struct Sum {
+  i64 m = 0, h = 0;
+  __device__ __forceinline__ void add(int xh, int xl, int2 c) {
+    m = wide(xh, c.x, m);
+    h = wide(xh, c.y, wide(xl, c.x, h));
+  }
+  __device__ __forceinline__ i64 value() const { return m + ((h + (1 << 27)) >> 28); }
+};
+struct Sum2 {  // complex columns
+  Sum x, y;
+  __device__ __forceinline__ void add(int4 v, int2 c) {
+    x.add(v.x, v.y, c);
+    y.add(v.z, v.w, c);
+  }
+};
+
+__device__ __forceinline__ unsigned top_of(double2 v) {
+  return max((unsigned)__double2hiint(v.x) & 0x7fffffffu, (unsigned)__double2hiint(v.y) & 0x7fffffffu);
+}
+// |v| rounded up, in units of 2^(e - 1037), 15 bits
+__device__ __forceinline__ int part_of(double v, int e) {
+  const unsigned h = (unsigned)__double2hiint(v) & 0x7fffffffu;
+  return (int)(((h & 0xfffffu) | 0x100000u) >> min(31, e - (int)(h >> 20) + 6)) + 1;
+}
+// exponent that scales values of at most top 2^(e - 1037), whose moduli sum to s 2^(e - 1037)
+__device__ __forceinline__ int exponent_of(u64 s, u64 top, int e) {
+  const int bs = 64 - __clzll((i64)(s | 1)), bt = 64 - __clzll((i64)(top | 1));
+  return min(kSumBits - bs, kMaxBits - bt) - (e - 1037);
+}
+// round(v f 2^sh), f a small integer
+__device__ __forceinline__ i64 from_double_times(double v, int sh, double f) {
+  const int hi = __double2hiint(v), e = (hi >> 20) & 0x7ff;
+  const double d = __hiloint2double(hi + sh * (1 << 20), __double2loint(v));
+  return e != 0 && e + sh > 1000 ? __double2ll_rn(d * f) : 0;
+}
+
+// X 2^-sh: one operation of the FP64 pipe, the scaling on the exponent field
+__device__ __forceinline__ double unscale(i64 X, int sh) {
+  const double d = (double)X;
+  if (sh > -900 && sh < 900) {
+    return X == 0 ? 0.0 : __hiloint2double(__double2hiint(d) - sh * (1 << 20), __double2loint(d));
+  }
+  return sh == kNotFinite ? nan("") : to_double(X, sh);
+}
+__device__ __forceinline__ double2 unscale(i64 x, i64 y, int sh) { return make_double2(unscale(x, sh), unscale(y, sh)); }
+
+struct YArgs {
+  const double2* in;   // [dir][3][Mm][NY]
+  double2* out;        // [dir][6][NY][Mm]
+  const int2* tab;     // [NH][NY + 1]: T_n(y_j), then [NH][NY + 1]: T_n'(y_j) / n^2, 56-bit halves
+  int Mm, MZ, MX, Kx, NY, NH, jchunk;
+  double alpha, beta;
+};
+
+// (bx, by, bz): mode tile, chunk of the half grid, direction
+__device__ __forceinline__ void yinv_fx(const YArgs& a, int bx, int by, int bz, int4* xs, int (*sh)[kModes]) {
+  const int NY = a.NY, N = NY - 1, Mm = a.Mm, m0 = bx * kModes;
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  // one warp per (component, mode): scales, halves and derivative
+  for (int row = warp; row < 3 * kModes; row += kThreadsC / 32) {
+    const int f = row / kModes, t = row - f * kModes, m = m0 + t;
+    const double2* src = a.in + (((size_t)bz * 3 + f) * Mm + m) * NY;
+    const bool on = m < Mm;
+    unsigned em = 0;
+    for (int n = lane; n < NY; n += 32) em = max(em, on ? top_of(__ldg(src + n)) : 0u);
+    const int e = (int)(__reduce_max_sync(0xffffffffu, em) >> 20);
+    u64 s0 = 0, s2 = 0, t0 = 0, t2 = 0;  // sums and largest values of a_n and of n^2 a_n
+    for (int n = lane; n < NY; n += 32) {
+      if (!on) continue;
+      const double2 v = __ldg(src + n);
+      const unsigned px = part_of(v.x, e), py = part_of(v.y, e), q = max(px, py);
+      s0 += px + py;
+      s2 += (u64)(n * n) * (px + py);
+      t0 = max(t0, (u64)q);
+      t2 = max(t2, (u64)(n * n) * q);
+    }
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+      s0 += __shfl_xor_sync(0xffffffffu, s0, o);
+      s2 += __shfl_xor_sync(0xffffffffu, s2, o);
+      t0 = max(t0, __shfl_xor_sync(0xffffffffu, t0, o));
+      t2 = max(t2, __shfl_xor_sync(0xffffffffu, t2, o));
+    }
+    const int e0 = exponent_of(s0, t0, e), ed = exponent_of(s2, t2, e);
+    const int g = f == 0 ? 3 : 4;  // derivative column of u and w
+    if (lane == 0) {
+      sh[f][t] = e == 0x7ff ? kNotFinite : e0;
+      if (f != 1) sh[g][t] = e == 0x7ff ? kNotFinite : ed;
+    }
+    for (int n = lane; n <= NY; n += 32) {  // row NY: zero
+      double2 v = make_double2(0.0, 0.0);
+      if (on && n < NY) v = __ldg(src + n);
+      xs[n * kStrideY + row] = halves2(from_double(v.x, e0), from_double(v.y, e0));
+      if (f == 1) continue;
+      const double n2 = (double)(n * n);
+      xs[n * kStrideY + g * kModes + t] =
+          n == 0 ? make_int4(0, 0, 0, 0) : halves2(from_double_times(v.x, ed, n2), from_double_times(v.y, ed, n2));
+    }
+  }
+  __syncthreads();
+  const int j_lo = by * a.jchunk, j_hi = min(a.NH, j_lo + a.jchunk);
+  const size_t NYMm = (size_t)NY * Mm;
+  double2* o = a.out + (size_t)bz * 6 * NYMm;
+  for (int it = threadIdx.x; it < kModes * (j_hi - j_lo); it += kThreadsC) {
+    const int t = it % kModes, jh = j_lo + it / kModes, m = m0 + t;
+    Sum2 E[5], O[5];
+    const int4* tr = reinterpret_cast<const int4*>(a.tab + (size_t)jh * (NY + 1));
+    const int4* td = reinterpret_cast<const int4*>(a.tab + (size_t)(a.NH + jh) * (NY + 1));
+    const int4* x = xs + t;
+    for (int n = 0; n < NY; n += 2) {
+      const int4 c = __ldg(tr + n / 2), d = __ldg(td + n / 2);
+#pragma unroll
+      for (int f = 0; f < 5; ++f) {
+        const int4 k = f < 3 ? c : d;
+        E[f].add(x[f * kModes], make_int2(k.x, k.y));
+        O[f].add(x[kStrideY + f * kModes], make_int2(k.z, k.w));
+      }
+      x += 2 * kStrideY;
+    }
+    if (m >= Mm) continue;
+    const int pos = m / a.MZ, iz = m - pos * a.MZ;
+    const double kx = a.alpha * (pos <= a.Kx ? pos : pos - a.MX), kz = a.beta * iz;
+#pragma unroll
+    for (int side = 0; side < 2; ++side) {
+      const int j = side == 0 ? jh : N - jh;
+      if (side == 1 && j == jh) break;
+      double2 v[5];
+#pragma unroll
+      for (int f = 0; f < 5; ++f) {
+        const i64 ex = E[f].x.value(), ey = E[f].y.value(), ox = O[f].x.value(), oy = O[f].y.value();
+        if (side == 0) v[f] = unscale(ex + ox, ey + oy, sh[f][t]);
+        else v[f] = f < 3 ? unscale(ex - ox, ey - oy, sh[f][t]) : unscale(ox - ex, oy - ey, sh[f][t]);
+      }
+      double2* d = o + (size_t)j * Mm + m;
+      d[0] = v[0];
+      d[NYMm] = v[1];
+      d[2 * NYMm] = v[2];
+      // Dw - i kz v, i kz u - i kx w, i kx v - Du
+      d[3 * NYMm] = make_double2(fma(kz, v[1].y, v[4].x), fma(-kz, v[1].x, v[4].y));
+      d[4 * NYMm] = make_double2(fma(kx, v[2].y, -kz * v[0].y), fma(-kx, v[2].x, kz * v[0].x));
+      d[5 * NYMm] = make_double2(-fma(kx, v[1].y, v[3].x), fma(kx, v[1].x, -v[3].y));
+    }
+  }
+}
+
+__global__ void __launch_bounds__(kThreadsC, 2) k_yinv_fx(const __grid_constant__ YArgs a) {
+  extern __shared__ __align__(16) unsigned char smem[];
+  __shared__ int sh[5][kModes];
+  yinv_fx(a, blockIdx.x, blockIdx.y, blockIdx.z, reinterpret_cast<int4*>(smem), sh);
+}
+
+// ------------------------------------------------------------------ forward
+struct RArgs {
+  const double2* in3;  // [dir][3][NY][Mm]
+  const double2* du;   // [dir][3][Mm][NY]
+  double2* W;          // (u, d, row c (N-1) + n) at u su + d sd + row sn
+  const int2* tab;
+  long long su, sd, sn;
+  int n_unique, Mm, MX, MZ, Kx, NY, NH, rchunk;
+  double inv_dt;
+};
+
+__device__ __forceinline__ void unique_mode_of(int u, int Kx, int MZ, int* pos, int* iz) {
+  const int first = (Kx + 1) * MZ;
+  if (u < first) {
+    *pos = u / MZ;
+    *iz = u - *pos * MZ;
+  } else {
+    const int v = u - first;
+    *pos = Kx + 1 + v / (MZ - 1);
+    *iz = 1 + v % (MZ - 1);
+  }
+}
+
+struct RShared {
+  unsigned em[kColsR];
+  int sum[kColsR];
+  int sh[kColsR];
+  int pos[kModes], iz[kModes];
+};
+
+// (bx, by, bz): tile of solved modes, chunk of rows, direction
+__device__ __forceinline__ void rhs_fx(const RArgs& a, int bx, int by, int bz, int4* xs, RShared& s) {
+  const int NY = a.NY, N = NY - 1, NH = a.NH, NR = N - 1, Mm = a.Mm, u0 = bx * kModes;
+  const int tid = threadIdx.x;
+  if (tid < kModes) {
+    int pos = 0, iz = 0;
+    if (u0 + tid < a.n_unique) unique_mode_of(u0 + tid, a.Kx, a.MZ, &pos, &iz);
+    s.pos[tid] = pos;
+    s.iz[tid] = iz;
+  }
+  if (tid < kColsR) {
+    s.em[tid] = 0;
+    s.sum[tid] = 0;
+  }
+  __syncthreads();
+  // lanes take the modes fastest, then the points: value (c, j) of mode t
+  const int t = tid % kModes, part = tid / kModes, nparts = kThreadsC / kModes;
+  const bool on = u0 + t < a.n_unique;
+  const double2* src = a.in3 + (size_t)bz * 3 * NY * Mm + s.pos[t] * a.MZ + s.iz[t];
+  for (int c = 0; c < 3; ++c) {
+    unsigned em = 0;
+    for (int j = part; j < NY; j += nparts) em = max(em, on ? top_of(__ldg(src + ((size_t)c * NY + j) * Mm)) : 0u);
+    em = max(em, __shfl_xor_sync(0xffffffffu, em, 8));
+    em = max(em, __shfl_xor_sync(0xffffffffu, em, 16));
+    if ((tid & 31) < kModes) atomicMax(&s.em[c * kModes + t], em);
+  }
+  __syncthreads();
+  for (int c = 0; c < 3; ++c) {
+    const int e = (int)(s.em[c * kModes + t] >> 20);
+    int sum = 0;
+    for (int j = part; j < NY; j += nparts) {
+      if (!on) continue;
+      const double2 v = __ldg(src + ((size_t)c * NY + j) * Mm);
+      sum += part_of(v.x, e) + part_of(v.y, e);
+    }
+    sum += __shfl_xor_sync(0xffffffffu, sum, 8);
+    sum += __shfl_xor_sync(0xffffffffu, sum, 16);
+    if ((tid & 31) < kModes) atomicAdd(&s.sum[c * kModes + t], sum);
+  }
+  __syncthreads();
+  if (tid < kColsR) {
+    const int e = (int)(s.em[tid] >> 20);
+    // values below 2^(e - 1022); the parts of a pair below twice that
+    s.sh[tid] = e == 0x7ff ? kNotFinite : exponent_of((u64)s.sum[tid], 0xffff, e);
+  }
+  __syncthreads();
+  // even and odd parts of the point pairs (j, N - j): f_j + f_{N-j} at j, f_j - f_{N-j} at N - j; the
+  // end points enter with half weight
+  for (int idx = part; idx < 3 * NH; idx += nparts) {
+    const int c = idx / NH, j = idx - c * NH, col = c * kModes + t;
+    const int sh = s.sh[col] == kNotFinite ? -2000 : s.sh[col];
+    i64 px = 0, py = 0, qx = 0, qy = 0;
+    if (on) {
+      const double2 p = __ldg(src + ((size_t)c * NY + j) * Mm), q = __ldg(src + ((size_t)c * NY + N - j) * Mm);
+      px = from_double(p.x, sh);
+      py = from_double(p.y, sh);
+      qx = from_double(q.x, sh);
+      qy = from_double(q.y, sh);
+    }
+    if (2 * j == N) {
+      xs[j * kStrideR + col] = halves2(px, py);
+    } else {
+      const int d = j == 0 ? 1 : 0;
+      xs[j * kStrideR + col] = halves2((px + qx) >> d, (py + qy) >> d);
+      xs[(N - j) * kStrideR + col] = halves2((px - qx) >> d, (py - qy) >> d);
+    }
+  }
+  __syncthreads();
+  const int lo = by * a.rchunk, hi = min(NR, lo + a.rchunk);
+  if (!on) return;
+  const int pos = s.pos[t], iz = s.iz[t];
+  const int mpos = pos == 0 ? 0 : a.MX - pos;
+  const double2* dsrc = a.du + (size_t)bz * 3 * Mm * NY;
+  const int ne = (NR + 1) / 2;  // even rows come first, so that a warp runs one trip count
+  for (int r = lo + part; r < hi; r += nparts) {
+    const int n = r < ne ? 2 * r : 2 * (r - ne) + 1, odd = n & 1;
+    Sum2 S[3];
+    const int4* x = xs + t + (odd ? N * kStrideR : 0);
+    const int st = odd ? -kStrideR : kStrideR, cnt = odd ? NH - 1 : NH;
+    const int2* tc = a.tab + n;
+    for (int j = 0; j < cnt; ++j) {
+      const int2 c = __ldg(tc + (size_t)j * (NY + 1));
+#pragma unroll
+      for (int f = 0; f < 3; ++f) S[f].add(x[f * kModes], c);
+      x += st;
+    }
+    const double cn = (n == 0 ? 1.0 : 2.0) / N;  // 2 / (N cbar_n)
+#pragma unroll
+    for (int f = 0; f < 3; ++f) {
+      double2 d = __ldg(dsrc + ((size_t)f * Mm + pos * a.MZ + iz) * NY + n);
+      if (iz == 0) {  // Hermitian projection
+        const double2 w = __ldg(dsrc + ((size_t)f * Mm + mpos * a.MZ) * NY + n);
+        d = make_double2(0.5 * (d.x + w.x), 0.5 * (d.y - w.y));
+      }
+      const double2 v = unscale(S[f].x.value(), S[f].y.value(), s.sh[f * kModes + t]);
+      double2 g = make_double2(fma(cn, v.x, d.x * a.inv_dt), fma(cn, v.y, d.y * a.inv_dt));
+      if (pos == 0 && iz == 0) g.y = 0.0;
+      a.W[(u0 + t) * a.su + bz * a.sd + (long long)(f * NR + n) * a.sn] = g;
+    }
+  }
+}
+
+__global__ void __launch_bounds__(kThreadsC, 3) k_rhs_fx(const __grid_constant__ RArgs a) {
+  extern __shared__ __align__(16) unsigned char smem[];
+  __shared__ RShared s;
+  // directions fastest: with one direction per 16-byte column of W, the blocks that run together
+  // fill its sectors
+  rhs_fx(a, blockIdx.y, blockIdx.z, blockIdx.x, reinterpret_cast<int4*>(smem), s);
+}
+
+// ------------------------------------------------------------------ groups
+struct GY {
+  size_t off;  // offset (doubles) of the member's state in a group vector
+  YArgs a;
+  int gx;      // mode tiles of the member's launch
+};
+struct GR {
+  size_t off;
+  RArgs a;
+  int gx;
+};
+
+__global__ void __launch_bounds__(kThreadsC, 2) k_yinv_fx_grp(const double* __restrict__ in, const GY* __restrict__ recs,
+                                                              const int* __restrict__ inst, const int* __restrict__ first,
+                                                              const int* __restrict__ active) {
+  extern __shared__ __align__(16) unsigned char smem[];
+  __shared__ int sh[5][kModes];
+  __shared__ GY r;
+  const int i = inst[blockIdx.x];
+  if (active && !active[i]) return;
+  if (threadIdx.x == 0) {
+    r = recs[i];
+    r.a.in = reinterpret_cast<const double2*>(in + r.off);
+  }
+  __syncthreads();
+  const int b = blockIdx.x - first[i];
+  yinv_fx(r.a, b % r.gx, b / r.gx, 0, reinterpret_cast<int4*>(smem), sh);
+}
+
+__global__ void __launch_bounds__(kThreadsC, 3) k_rhs_fx_grp(const double* __restrict__ du, const GR* __restrict__ recs,
+                                                             const int* __restrict__ inst, const int* __restrict__ first,
+                                                             const int* __restrict__ active) {
+  extern __shared__ __align__(16) unsigned char smem[];
+  __shared__ RShared s;
+  __shared__ GR r;
+  const int i = inst[blockIdx.x];
+  if (active && !active[i]) return;
+  if (threadIdx.x == 0) {
+    r = recs[i];
+    r.a.du = reinterpret_cast<const double2*>(du + r.off);
+  }
+  __syncthreads();
+  const int b = blockIdx.x - first[i];
+  rhs_fx(r.a, b % r.gx, b / r.gx, 0, reinterpret_cast<int4*>(smem), s);
+}
+
+size_t smem_y(const sp_ctx* c) { return (size_t)(c->NY + 1) * kStrideY * 16; }
+size_t smem_r(const sp_ctx* c) { return (size_t)c->NY * kStrideR * 16; }
+
+// parts of the outputs of a mode tile: one block per tile when the tiles fill the GPU (each part
+// scales the inputs again)
+int parts_for(int tiles, int rows, int sms) {
+  int p = 1;
+  while (tiles * p < sms && rows > p * (kThreadsC / kModes) / 2) ++p;
+  return p;
+}
+
+YArgs y_args(const sp_ctx* c, const void* in, void* out, int parts) {
+  YArgs a;
+  a.in = static_cast<const double2*>(in);
+  a.out = static_cast<double2*>(out);
+  a.tab = c->cheb_fx;
+  a.Mm = c->Mm; a.MZ = c->MZ; a.MX = c->MX; a.Kx = c->Kx; a.NY = c->NY; a.NH = c->NH;
+  a.jchunk = (c->NH + parts - 1) / parts;
+  a.alpha = c->alpha;
+  a.beta = c->beta;
+  return a;
+}
+
+RArgs r_args(const sp_ctx* c, const void* in3, const void* du, void* W, int parts) {
+  RArgs a;
+  a.in3 = static_cast<const double2*>(in3);
+  a.du = static_cast<const double2*>(du);
+  a.W = static_cast<double2*>(W);
+  a.tab = c->cheb_fx;
+  a.su = 3LL * (c->N - 1);
+  a.sd = a.su * c->n_unique;
+  a.sn = 1;
+  a.n_unique = c->n_unique;
+  a.Mm = c->Mm; a.MX = c->MX; a.MZ = c->MZ; a.Kx = c->Kx; a.NY = c->NY; a.NH = c->NH;
+  a.rchunk = (c->N - 1 + parts - 1) / parts;
+  a.inv_dt = 1.0 / c->dt;
+  return a;
+}
+
+template <class R>
+cudaError_t upload_grp(GrpKernel* k, const std::vector<R>& recs, const std::vector<int>& nblk, const int* order, size_t smem) {
+  const int n = (int)recs.size();
+  std::vector<int> inst, first(n, 0);
+  for (int q = 0; q < n; ++q) {
+    first[order[q]] = (int)inst.size();
+    inst.insert(inst.end(), nblk[order[q]], order[q]);
+  }
+  k->blocks = (int)inst.size();
+  k->smem = smem;
+  cudaError_t e;
+  if ((e = grp_upload(&k->recs, recs.data(), recs.size() * sizeof(R))) != cudaSuccess) return e;
+  if ((e = grp_upload((void**)&k->inst, inst.data(), inst.size() * sizeof(int))) != cudaSuccess) return e;
+  return grp_upload((void**)&k->first, first.data(), first.size() * sizeof(int));
+}
+
+}  // namespace
+
+std::vector<int> cheb_fx_table(int NY) {
+  const int N = NY - 1, NH = N / 2 + 1;
+  std::vector<int> t((size_t)2 * NH * (NY + 1) * 2, 0);
+  const long double pi = 3.141592653589793238462643383279502884L;
+  // sin(pi k / N), exact at the multiples of a quarter turn
+  auto sine = [&](long long k) -> long double {
+    k = ((k % (2 * N)) + 2 * N) % (2 * N);
+    if (k % N == 0) return 0.0L;
+    if (2 * k == N) return 1.0L;
+    if (2 * k == 3 * N) return -1.0L;
+    return sinl(pi * k / N);
+  };
+  for (int j = 0; j < NH; ++j)
+    for (int n = 0; n < NY; ++n)
+      for (int d = 0; d < 2; ++d) {
+        const long long k = (long long)j * n;
+        long double v;
+        if (d == 0) {
+          const long long r = k % (2 * N);
+          v = r == 0 ? 1.0L : r == N ? -1.0L : 2 * r == N || 2 * r == 3 * N ? 0.0L : cosl(pi * r / N);
+        } else {       // T_n' / n^2 = sin(n t) / (n sin t), t = pi j / N
+          v = n == 0 ? 0.0L : j == 0 ? 1.0L : sine(k) / (n * sine(j));
+        }
+        const long long q = llrintl(v * 72057594037927936.0L);  // 2^56
+        const long long hi = (q + (1 << 27)) >> 28;
+        int* o = t.data() + (((size_t)d * NH + j) * (NY + 1) + n) * 2;
+        o[0] = (int)hi;
+        o[1] = (int)(q - hi * (1LL << 28));
+      }
+  return t;
+}
+
+cudaError_t launch_yinv_fx(const sp_ctx* c, const double* in, void* out6, int n_dir, cudaStream_t st) {
+  const int tiles = (c->Mm + kModes - 1) / kModes;
+  const YArgs a = y_args(c, in, out6, parts_for(tiles * n_dir, c->NH, c->sm_count));
+  cudaError_t e = cudaFuncSetAttribute(k_yinv_fx, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_y(c));
+  if (e != cudaSuccess) return e;
+  k_yinv_fx<<<dim3(tiles, (c->NH + a.jchunk - 1) / a.jchunk, n_dir), kThreadsC, smem_y(c), st>>>(a);
+  return cudaGetLastError();
+}
+
+cudaError_t launch_rhs_fx(const sp_ctx* c, const void* in3, const double* du, void* W, int n_dir, long long su,
+                          long long sd, long long sn, cudaStream_t st) {
+  const int tiles = (c->n_unique + kModes - 1) / kModes;
+  RArgs a = r_args(c, in3, du, W, parts_for(tiles * n_dir, c->N - 1, c->sm_count));
+  if (sn) {
+    a.su = su;
+    a.sd = sd;
+    a.sn = sn;
+  }
+  cudaError_t e = cudaFuncSetAttribute(k_rhs_fx, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_r(c));
+  if (e != cudaSuccess) return e;
+  k_rhs_fx<<<dim3(n_dir, tiles, (c->N - 1 + a.rchunk - 1) / a.rchunk), kThreadsC, smem_r(c), st>>>(a);
+  return cudaGetLastError();
+}
+
+cudaError_t grp_build_cheb_fx(GrpPlan* p, sp_ctx* const* mem, int n, const size_t* offs, const int* order) {
+  int ty = 0, tr = 0;
+  for (int m = 0; m < n; ++m) {
+    ty += (mem[m]->Mm + kModes - 1) / kModes;
+    tr += (mem[m]->n_unique + kModes - 1) / kModes;
+  }
+  std::vector<GY> ry(n);
+  std::vector<GR> rr(n);
+  std::vector<int> by(n), br(n);
+  size_t sy = 0, sr = 0;
+  for (int m = 0; m < n; ++m) {
+    const sp_ctx* c = mem[m];
+    ry[m].off = rr[m].off = offs[m];
+    ry[m].a = y_args(c, nullptr, c->ws6, parts_for(ty, c->NH, c->sm_count));
+    ry[m].gx = (c->Mm + kModes - 1) / kModes;
+    by[m] = ry[m].gx * ((c->NH + ry[m].a.jchunk - 1) / ry[m].a.jchunk);
+    rr[m].a = r_args(c, c->ws3, nullptr, c->ws6, parts_for(tr, c->N - 1, c->sm_count));
+    rr[m].gx = (c->n_unique + kModes - 1) / kModes;
+    br[m] = rr[m].gx * ((c->N - 1 + rr[m].a.rchunk - 1) / rr[m].a.rchunk);
+    sy = std::max(sy, smem_y(c));
+    sr = std::max(sr, smem_r(c));
+  }
+  cudaError_t e;
+  if ((e = cudaFuncSetAttribute(k_yinv_fx_grp, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sy)) != cudaSuccess) return e;
+  if ((e = cudaFuncSetAttribute(k_rhs_fx_grp, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sr)) != cudaSuccess) return e;
+  if ((e = upload_grp(&p->yinv64, ry, by, order, sy)) != cudaSuccess) return e;
+  return upload_grp(&p->rhs64, rr, br, order, sr);
+}
+
+cudaError_t grp_launch_yinv_fx(const GrpPlan& p, const double* in, const int* active, cudaStream_t st) {
+  const GrpKernel& k = p.yinv64;
+  k_yinv_fx_grp<<<k.blocks, kThreadsC, k.smem, st>>>(in, static_cast<const GY*>(k.recs), k.inst, k.first, active);
+  return cudaGetLastError();
+}
+cudaError_t grp_launch_rhs_fx(const GrpPlan& p, const double* du, const int* active, cudaStream_t st) {
+  const GrpKernel& k = p.rhs64;
+  k_rhs_fx_grp<<<k.blocks, kThreadsC, k.smem, st>>>(du, static_cast<const GR*>(k.recs), k.inst, k.first, active);
+  return cudaGetLastError();
+}

@@ -124,132 +124,19 @@ __device__ __forceinline__ C2<float> ld_c2(const C2<float>* p) {
 // ------------------------------------------------------------ k_yinv
 struct YinvArgs {
   int Mm, MZ, MX, Kx, NY, N, NH, jchunk;
-  int q2, NQ;  // two-level split (N divisible by 4): quarter grid jq = 0..N/4
   double alpha, beta;
 };
 
-// Chebyshev tables of k_yinv (T = double or float): Th[j][n] = T_n(y_j), TDh[j][n] = T_n'(y_j)
-// on the half grid j <= N/2; for the two-level split also, on the quarter grid jq <= N/4 and
-// odd n = 2m+1, Tp[jq][n] = T_n(y_{N/2-jq}) = (-1)^m sin(pi jq n / N) and
-// TDp[jq][n] = T_n'(y_{N/2-jq}) = (-1)^m n cos(pi jq n / N) / cos(pi jq / N), and
-// tq[jq] = tan(pi jq / N) (the even-degree derivatives at y_{N/2-jq} are tq times the
-// alternating sums at y_jq)
+// Chebyshev tables of k_yinv: Th[j][n] = T_n(y_j), TDh[j][n] = T_n'(y_j) on the half grid j <= N/2
 template <typename T>
 struct YinvTabs {
   const T* Th;
   const T* TDh;
-  const T* Tp;
-  const T* TDp;
-  const T* tq;
 };
 
 // in : [dir][3][Mm][NY] complex double (the boundary state layout)
 // out: [dir][6][NY][Mm] complex T, fields u, v, w, wx, wy, wz
 // (bx, by, bz): mode tile, Gauss-Lobatto chunk, direction
-// curl and stores at the Gauss-Lobatto point j: fields u, v, w, wx, wy, wz of mode m
-template <typename T>
-__device__ __forceinline__ void yinv_store(C2<T>* o, size_t NYMm, size_t base, T kx, T kz, C2<T> u, C2<T> v,
-                                           C2<T> w, C2<T> Du, C2<T> Dw) {
-  const C2<T> ox = Dw - mul_is(v, kz);
-  const C2<T> oy = mul_is(u, kz) - mul_is(w, kx);
-  const C2<T> oz = mul_is(v, kx) - Du;
-  o[0 * NYMm + base] = u;
-  o[1 * NYMm + base] = v;
-  o[2 * NYMm + base] = w;
-  o[3 * NYMm + base] = ox;
-  o[4 * NYMm + base] = oy;
-  o[5 * NYMm + base] = oz;
-}
-
-// Two-level even/odd split: per quarter-grid point jq the sums over degrees n = 0 and
-// n = 2 (mod 4) and over odd n give the values at the four points jq, N - jq, N/2 - jq,
-// N/2 + jq (T_n(y_{N-j}) = (-1)^n T_n(y_j); T_n(y_{N/2-j}) = +-T_n(y_j) for n = 0, 2 mod 4),
-// a quarter less work than the one-level split.
-template <typename T>
-__device__ __forceinline__ void yinv_q2(const C2<T>* sc, C2<T>* o, const YinvTabs<T>& tb, const YinvArgs& a, int m0,
-                                        int by) {
-  const int TM = kTileYinv;
-  const int NY = a.NY, Mm = a.Mm, N = a.N;
-  const int j_lo = by * a.jchunk;
-  const int j_hi = min(a.NQ, j_lo + a.jchunk);
-  const int items = TM * (j_hi - j_lo);
-  const size_t NYMm = (size_t)NY * Mm;
-  for (int it = threadIdx.x; it < items; it += blockDim.x) {
-    const int t = it % TM;
-    const int jq = j_lo + it / TM;
-    const int m = m0 + t;
-    if (m >= Mm) continue;
-    const C2<T> z = mk((T)0, (T)0);
-    // [field][0 EE, 1 EO, 2 O, 3 O'] for u, v, w; the same with the derivative tables for u, w
-    C2<T> A[3][4] = {{z, z, z, z}, {z, z, z, z}, {z, z, z, z}};
-    C2<T> Dd[2][4] = {{z, z, z, z}, {z, z, z, z}};
-    const T* trow = tb.Th + (size_t)jq * NY;
-    const T* drow = tb.TDh + (size_t)jq * NY;
-    const T* prow = tb.Tp + (size_t)jq * NY;
-    const T* qrow = tb.TDp + (size_t)jq * NY;
-    for (int n = 0; n < NY; ++n) {
-      const int r = n & 3;
-      const C2<T> u = sc[(0 * NY + n) * TM + t], v = sc[(1 * NY + n) * TM + t], w = sc[(2 * NY + n) * TM + t];
-      const T tc = trow[n], td = drow[n];
-      if (r == 0) {
-        A[0][0] = A[0][0] + scl(u, tc);
-        A[1][0] = A[1][0] + scl(v, tc);
-        A[2][0] = A[2][0] + scl(w, tc);
-        Dd[0][0] = Dd[0][0] + scl(u, td);
-        Dd[1][0] = Dd[1][0] + scl(w, td);
-      } else if (r == 2) {
-        A[0][1] = A[0][1] + scl(u, tc);
-        A[1][1] = A[1][1] + scl(v, tc);
-        A[2][1] = A[2][1] + scl(w, tc);
-        Dd[0][1] = Dd[0][1] + scl(u, td);
-        Dd[1][1] = Dd[1][1] + scl(w, td);
-      } else {
-        const T tp = prow[n], tdp = qrow[n];
-        A[0][2] = A[0][2] + scl(u, tc);
-        A[1][2] = A[1][2] + scl(v, tc);
-        A[2][2] = A[2][2] + scl(w, tc);
-        A[0][3] = A[0][3] + scl(u, tp);
-        A[1][3] = A[1][3] + scl(v, tp);
-        A[2][3] = A[2][3] + scl(w, tp);
-        Dd[0][2] = Dd[0][2] + scl(u, td);
-        Dd[1][2] = Dd[1][2] + scl(w, td);
-        Dd[0][3] = Dd[0][3] + scl(u, tdp);
-        Dd[1][3] = Dd[1][3] + scl(w, tdp);
-      }
-    }
-    const int pos = m / a.MZ, iz = m - pos * a.MZ;
-    const int ix = pos <= a.Kx ? pos : pos - a.MX;
-    const T kx = (T)(a.alpha * ix), kz = (T)(a.beta * iz);
-    const T tqv = tb.tq[jq];
-    // E at jq and at N/2 - jq; derivatives: even part at N/2 - jq is tq (EO' - EE')
-    C2<T> E1[3], E2[3];
-#pragma unroll
-    for (int f = 0; f < 3; ++f) {
-      E1[f] = A[f][0] + A[f][1];
-      E2[f] = A[f][0] - A[f][1];
-    }
-    const C2<T> DE1u = Dd[0][0] + Dd[0][1], DE1w = Dd[1][0] + Dd[1][1];
-    const C2<T> DE2u = scl(Dd[0][1] - Dd[0][0], tqv), DE2w = scl(Dd[1][1] - Dd[1][0], tqv);
-    const int jl[4] = {jq, N - jq, N / 2 - jq, N / 2 + jq};
-#pragma unroll
-    for (int q = 0; q < 4; ++q) {
-      const int j = jl[q];
-      if (q == 1 && j == jq) continue;                         // jq = N/2 would coincide (never, N >= 4)
-      if (q >= 2 && 4 * jq == N) continue;                     // N/2 - jq = jq: already written
-      if (q == 3 && jq == 0) continue;                         // N/2 + 0 = N/2 - 0
-      const bool hi = (q & 1) != 0;                            // the mirrored point N - j'
-      const T sg = hi ? (T)-1 : (T)1;
-      const int s2 = q >= 2;
-      const C2<T> uu = (s2 ? E2[0] : E1[0]) + scl(A[0][s2 ? 3 : 2], sg);
-      const C2<T> vv = (s2 ? E2[1] : E1[1]) + scl(A[1][s2 ? 3 : 2], sg);
-      const C2<T> ww = (s2 ? E2[2] : E1[2]) + scl(A[2][s2 ? 3 : 2], sg);
-      const C2<T> Du = scl(s2 ? DE2u : DE1u, sg) + Dd[0][s2 ? 3 : 2];
-      const C2<T> Dw = scl(s2 ? DE2w : DE1w, sg) + Dd[1][s2 ? 3 : 2];
-      yinv_store(o, NYMm, (size_t)j * Mm + m, kx, kz, uu, vv, ww, Du, Dw);
-    }
-  }
-}
-
 template <typename T>
 __device__ __forceinline__ void yinv_body(const double2* __restrict__ in, C2<T>* __restrict__ out,
                                           const YinvTabs<T>& tb, const YinvArgs& a, int bx, int by, int bz) {
@@ -273,10 +160,6 @@ __device__ __forceinline__ void yinv_body(const double2* __restrict__ in, C2<T>*
     sc[(c * NY + n) * TM + t] = v;
   }
   __syncthreads();
-  if (sizeof(T) == 8 && a.q2) {  // FP64 only: the float kernel is bound by memory, not arithmetic
-    yinv_q2<T>(sc, out + (size_t)dir * 6 * NY * Mm, tb, a, m0, by);
-    return;
-  }
   const T* Th = tb.Th;
   const T* TDh = tb.TDh;
   const int j_lo = by * a.jchunk;
@@ -581,19 +464,21 @@ __device__ __forceinline__ void unique_to_mode(int u, int Kx, int MZ, int* pos, 
   }
 }
 
-// in3: [dir][3][NY][Mm] complex T (values of N at the Gauss-Lobatto points)
+// in3: float: [dir][3][NY][Mm] complex values of N at the Gauss-Lobatto points; double: the
+//      right-hand sides u/dt + N of k_rhs_fx, [dir][mode][3][N - 1]
 // du : [dir][3][Mm][NY] complex double; out: same layout (G = u_new - u)
 // (bx, by): tile of solved modes, direction
 // TM: solved modes per block (any block size works; every mode's arithmetic is the same)
 // LA: laminar advection in L (right-hand side + M du, complex operators)
-template <typename T, int TM, bool LA>
+template <typename T, int TM>
 __device__ __forceinline__ void solve_body(const C2<T>* __restrict__ in3, const double2* __restrict__ du,
                                            double2* __restrict__ out, const SolveArgs& a, int bx, int by) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   const int NY = a.NY, N = a.N, NH = a.NH, Mm = a.Mm, MZ = a.MZ;
   const int NR = N - 1;  // tau rows 0..N-2
-  C2<T>* svals = reinterpret_cast<C2<T>*>(smem_raw);                    // [3][NY][TM]
-  double2* sdu = reinterpret_cast<double2*>(svals + 3 * NY * TM + (3 * NY * TM) % 2);  // [3][TM][NY]
+  constexpr bool PRE = sizeof(T) == 8;  // the forward transform is done
+  C2<T>* svals = reinterpret_cast<C2<T>*>(smem_raw);                    // [3][NY][TM] (float)
+  double2* sdu = reinterpret_cast<double2*>(svals + (PRE ? 0 : 3 * NY * TM + (3 * NY * TM) % 2));  // [3][TM][NY]
   double2* sf = sdu + 3 * TM * NY;            // [3][TM][NR]
   double2* srv = sf + 3 * TM * NR;            // [TM][2][cv]
   double2* sfb = srv + TM * 2 * a.cv;         // [TM][NR]
@@ -620,16 +505,18 @@ __device__ __forceinline__ void solve_body(const C2<T>* __restrict__ in3, const 
     s_ik[threadIdx.x] = kk > 0 ? 1.0 / kk : 0.0;
   }
   __syncthreads();
-  const C2<T>* vin = in3 + (size_t)dir * 3 * NY * Mm;
   const double2* dsrc = du + (size_t)dir * 3 * Mm * NY;
   // phase A: load values and the (Hermitian-projected) input state
-  for (int idx = threadIdx.x; idx < 3 * NY * TM; idx += blockDim.x) {
-    const int t = idx % TM;
-    const int jc = idx / TM;  // c*NY + j
-    const int c = jc / NY, jj = jc - c * NY;
-    C2<T> v = mk((T)0, (T)0);
-    if (s_u[t] < a.n_unique) v = ld_c2(vin + ((size_t)c * NY + jj) * Mm + s_pos[t] * MZ + s_iz[t]);
-    svals[idx] = v;
+  if constexpr (!PRE) {
+    const C2<T>* vin = in3 + (size_t)dir * 3 * NY * Mm;
+    for (int idx = threadIdx.x; idx < 3 * NY * TM; idx += blockDim.x) {
+      const int t = idx % TM;
+      const int jc = idx / TM;  // c*NY + j
+      const int c = jc / NY, jj = jc - c * NY;
+      C2<T> v = mk((T)0, (T)0);
+      if (s_u[t] < a.n_unique) v = ld_c2(vin + ((size_t)c * NY + jj) * Mm + s_pos[t] * MZ + s_iz[t]);
+      svals[idx] = v;
+    }
   }
   for (int idx = threadIdx.x; idx < 3 * TM * NY; idx += blockDim.x) {
     const int n = idx % NY;
@@ -648,6 +535,37 @@ __device__ __forceinline__ void solve_body(const C2<T>* __restrict__ in3, const 
     sdu[(c * TM + t) * NY + n] = v;
   }
   __syncthreads();
+  // + M du on the momentum rows of the laminar-advection step: i kx (Y du)_n, and dv_n in the
+  // x-momentum rows
+  auto add_lam = [&](double2& f, int c, int t, int n) {
+    const double2* dc = sdu + (c * TM + t) * NY;
+    double2 yv;
+    if (n == 0) yv = make_double2(0.5 * dc[1].x, 0.5 * dc[1].y);
+    else if (n == 1) yv = make_double2(dc[0].x + 0.5 * dc[2].x, dc[0].y + 0.5 * dc[2].y);
+    else yv = make_double2(0.5 * (dc[n - 1].x + dc[n + 1].x), 0.5 * (dc[n - 1].y + dc[n + 1].y));
+    const double kx = s_kx[t];
+    f.x = fma(-kx, yv.y, f.x);
+    f.y = fma(kx, yv.x, f.y);
+    if (c == 0) {
+      const double2 dv = sdu[(TM + t) * NY + n];
+      f.x += dv.x;
+      f.y += dv.y;
+    }
+  };
+  if constexpr (PRE) {
+    const double2* W = reinterpret_cast<const double2*>(in3) + ((size_t)dir * a.n_unique + u0) * 3 * NR;
+    for (int idx = threadIdx.x; idx < 3 * TM * NR; idx += blockDim.x) {
+      const int t = idx / (3 * NR), rem = idx - t * 3 * NR, c = rem / NR, n = rem - c * NR;
+      double2 f = make_double2(0.0, 0.0);
+      if (s_u[t] < a.n_unique) {
+        f = __ldg(W + idx);
+        add_lam(f, c, t, n);
+        if (s_pos[t] == 0 && s_iz[t] == 0) f.y = 0.0;
+      }
+      sf[(c * TM + t) * NR + n] = f;
+    }
+    __syncthreads();
+  } else {
   // phase A2: even/odd pairs of the values, once per (component, mode, point pair):
   // s_j = f(y_j) + f(y_N-j) replaces f(y_j), d_j = f(y_j) - f(y_N-j) replaces f(y_N-j)
   // (T_n(y_N-j) = (-1)^n T_n(y_j), so even rows read s and odd rows read d)
@@ -670,45 +588,21 @@ __device__ __forceinline__ void solve_body(const C2<T>* __restrict__ in3, const 
     const int c = idx / (TM * cnt);
     C2<T> acc = mk((T)0, (T)0);
     const C2<T>* col = svals + (c * NY) * TM + t;
-    if (sizeof(T) == 8) {
-      const double* cf = a.Cfh_d + (size_t)n * NH;
-      if ((n & 1) == 0) {
-        for (int jj = 0; jj < NH - 1; ++jj) acc = acc + scl(col[jj * TM], (T)cf[jj]);
-        acc = acc + scl(col[(NH - 1) * TM], (T)cf[NH - 1]);
-      } else {
-        for (int jj = 0; jj < NH - 1; ++jj) acc = acc + scl(col[(N - jj) * TM], (T)cf[jj]);
-      }
+    const float* cf = a.Cfh_f + (size_t)n * NH;
+    if ((n & 1) == 0) {
+      for (int jj = 0; jj < NH - 1; ++jj) acc = acc + scl(col[jj * TM], (T)cf[jj]);
+      acc = acc + scl(col[(NH - 1) * TM], (T)cf[NH - 1]);
     } else {
-      const float* cf = a.Cfh_f + (size_t)n * NH;
-      if ((n & 1) == 0) {
-        for (int jj = 0; jj < NH - 1; ++jj) acc = acc + scl(col[jj * TM], (T)cf[jj]);
-        acc = acc + scl(col[(NH - 1) * TM], (T)cf[NH - 1]);
-      } else {
-        for (int jj = 0; jj < NH - 1; ++jj) acc = acc + scl(col[(N - jj) * TM], (T)cf[jj]);
-      }
+      for (int jj = 0; jj < NH - 1; ++jj) acc = acc + scl(col[(N - jj) * TM], (T)cf[jj]);
     }
     const double2 d = sdu[(c * TM + t) * NY + n];
     double2 f = make_double2((double)acc.x + d.x * a.inv_dt, (double)acc.y + d.y * a.inv_dt);
-    if constexpr (LA) {
-      // + M du on the momentum rows: i kx (Y du)_n, and dv_n in the x-momentum rows
-      const double2* dc = sdu + (c * TM + t) * NY;
-      double2 yv;
-      if (n == 0) yv = make_double2(0.5 * dc[1].x, 0.5 * dc[1].y);
-      else if (n == 1) yv = make_double2(dc[0].x + 0.5 * dc[2].x, dc[0].y + 0.5 * dc[2].y);
-      else yv = make_double2(0.5 * (dc[n - 1].x + dc[n + 1].x), 0.5 * (dc[n - 1].y + dc[n + 1].y));
-      const double kx = s_kx[t];
-      f.x = fma(-kx, yv.y, f.x);
-      f.y = fma(kx, yv.x, f.y);
-      if (c == 0) {
-        const double2 dv = sdu[(TM + t) * NY + n];
-        f.x += dv.x;
-        f.y += dv.y;
-      }
-    }
+    add_lam(f, c, t, n);
     if (s_pos[t] == 0 && s_iz[t] == 0) f.y = 0.0;
     sf[(c * TM + t) * NR + n] = f;
   }
   __syncthreads();
+  }
   // phase C: rotate to the components along / across the wavevector; f_v goes to
   // srv (per parity), f~_a = -i f_a replaces f_x in sf (same thread, same slot)
   double2* sfa = sf;  // [TM][NR]: component 0 of sf after this phase
@@ -777,68 +671,44 @@ __device__ __forceinline__ void solve_body(const C2<T>* __restrict__ in3, const 
   // column-major operator (coalesced). The mean-mode test is hoisted out of the
   // loops so that no predicated-off double FMA occupies the FP64 pipe.
   const int nv0 = N / 2 + 1;  // even unknowns
-  if constexpr (LA) {
-    // D1: v = V' g, one complex row per thread (consecutive rows: coalesced columns)
-    for (int idx = threadIdx.x; idx < TM * NY; idx += blockDim.x) {
-      const int t = idx / NY, n = idx - t * NY;
-      if (s_u[t] >= a.n_unique || (s_pos[t] == 0 && s_iz[t] == 0)) continue;
-      const double2* V = reinterpret_cast<const double2*>(a.ops + (size_t)s_u[t] * a.op_stride + a.off_vc) + n;
-      sv[t * NY + n] = cdot4(V, NY, srv + t * 2 * a.cv, NR);
-    }
-    __syncthreads();
-    // D1b: right-hand side of b, f_b + (kz/k) v on the momentum rows
-    for (int idx = threadIdx.x; idx < TM * NR; idx += blockDim.x) {
-      const int t = idx / NR, n = idx - t * NR;
-      if (s_u[t] >= a.n_unique || (s_pos[t] == 0 && s_iz[t] == 0)) continue;
-      const double s = s_kz[t] * s_ik[t];
-      const double2 v = sv[t * NY + n];
-      double2 fb = sfb[t * NR + n];
-      fb.x = fma(s, v.x, fb.x);
-      fb.y = fma(s, v.y, fb.y);
-      sfb[t * NR + n] = fb;
-    }
-    __syncthreads();
-    // D2: b = H' (f_b + (kz/k) v); the mean mode uses the real Helmholtz operators
-    for (int idx = threadIdx.x; idx < TM * NY; idx += blockDim.x) {
-      const int t = idx / NY, k = idx - t * NY;
-      if (s_u[t] >= a.n_unique) continue;
-      const double* op = a.ops + (size_t)s_u[t] * a.op_stride;
-      if (s_pos[t] == 0 && s_iz[t] == 0) {
-        const int Q = k < nv0 ? 0 : 1, row = Q == 0 ? k : k - nv0, n = 2 * row + Q;
-        const int nrow = Q == 0 ? nv0 : NY - nv0;
-        const int rb = Q == 0 ? a.rb0 : a.rb1;
-        const double* H = op + (Q == 0 ? a.off_h0 : a.off_h1) + row;
-        sb[t * NY + n] = dot4(H, nrow, sfb + t * NR + Q, 2, rb);
-        sv[t * NY + n] = dot4(H, nrow, sfw + t * NR + Q, 2, rb);
-        continue;
-      }
-      const double2* H = reinterpret_cast<const double2*>(op + a.off_hc) + k;
-      sb[t * NY + k] = cdot4(H, NY, sfb + t * NR, NR);
-    }
-    __syncthreads();
-  } else {
+  // D1: v = V' g, one complex row per thread (consecutive rows: coalesced columns)
+  for (int idx = threadIdx.x; idx < TM * NY; idx += blockDim.x) {
+    const int t = idx / NY, n = idx - t * NY;
+    if (s_u[t] >= a.n_unique || (s_pos[t] == 0 && s_iz[t] == 0)) continue;
+    const double2* V = reinterpret_cast<const double2*>(a.ops + (size_t)s_u[t] * a.op_stride + a.off_vc) + n;
+    sv[t * NY + n] = cdot4(V, NY, srv + t * 2 * a.cv, NR);
+  }
+  __syncthreads();
+  // D1b: right-hand side of b, f_b + (kz/k) v on the momentum rows
+  for (int idx = threadIdx.x; idx < TM * NR; idx += blockDim.x) {
+    const int t = idx / NR, n = idx - t * NR;
+    if (s_u[t] >= a.n_unique || (s_pos[t] == 0 && s_iz[t] == 0)) continue;
+    const double s = s_kz[t] * s_ik[t];
+    const double2 v = sv[t * NY + n];
+    double2 fb = sfb[t * NR + n];
+    fb.x = fma(s, v.x, fb.x);
+    fb.y = fma(s, v.y, fb.y);
+    sfb[t * NR + n] = fb;
+  }
+  __syncthreads();
+  // D2: b = H' (f_b + (kz/k) v); the mean mode uses the real Helmholtz operators
   for (int idx = threadIdx.x; idx < TM * NY; idx += blockDim.x) {
     const int t = idx / NY, k = idx - t * NY;
     if (s_u[t] >= a.n_unique) continue;
     const double* op = a.ops + (size_t)s_u[t] * a.op_stride;
-    const int Q = k < nv0 ? 0 : 1, row = Q == 0 ? k : k - nv0, n = 2 * row + Q;
-    const int nrow = Q == 0 ? nv0 : NY - nv0;
-    const int rb = Q == 0 ? a.rb0 : a.rb1;
-    const double* H = op + (Q == 0 ? a.off_h0 : a.off_h1) + row;
-    const double2* fbq = sfb + t * NR + Q;
     if (s_pos[t] == 0 && s_iz[t] == 0) {
-      // mean flow: u and w from the Helmholtz operator, v = 0
-      const double2* fwq = sfw + t * NR + Q;
-      sb[t * NY + n] = dot4(H, nrow, fbq, 2, rb);
-      sv[t * NY + n] = dot4(H, nrow, fwq, 2, rb);
+      const int Q = k < nv0 ? 0 : 1, row = Q == 0 ? k : k - nv0, n = 2 * row + Q;
+      const int nrow = Q == 0 ? nv0 : NY - nv0;
+      const int rb = Q == 0 ? a.rb0 : a.rb1;
+      const double* H = op + (Q == 0 ? a.off_h0 : a.off_h1) + row;
+      sb[t * NY + n] = dot4(H, nrow, sfb + t * NR + Q, 2, rb);
+      sv[t * NY + n] = dot4(H, nrow, sfw + t * NR + Q, 2, rb);
       continue;
     }
-    sb[t * NY + n] = dot4(H, nrow, fbq, 2, rb);
-    const double* V = op + (Q == 0 ? a.off_v0 : a.off_v1) + row;
-    sv[t * NY + n] = dot4(V, nrow, srv + (t * 2 + Q) * a.cv, 1, rb);
+    const double2* H = reinterpret_cast<const double2*>(op + a.off_hc) + k;
+    sb[t * NY + k] = cdot4(H, NY, sfb + t * NR, NR);
   }
   __syncthreads();
-  }
   // (D v)_n = (2/c_n) sum_{p > n, p + n odd} p v_p: one suffix sum per (mode, parity),
   // kept in sfb (free after phase D) as S_n = sum_{p >= n, p = n mod 2} p v_p
   double2* ssum = sfb;
@@ -893,13 +763,12 @@ __device__ __forceinline__ void solve_body(const C2<T>* __restrict__ in3, const 
   }
 }
 
-template <typename T, int TM, int THREADS, bool LA>
+template <typename T, int TM, int THREADS>
 __global__ void __launch_bounds__(THREADS) k_solve(const C2<T>* __restrict__ in3, const double2* __restrict__ du,
                                                    double2* __restrict__ out, SolveArgs a) {
-  // with laminar advection in L the grid runs directions fastest: blocks that run together share a
-  // mode tile, so its complex operators (133 KB per mode) are read from DRAM once and from L2 after
-  if constexpr (LA) solve_body<T, TM, LA>(in3, du, out, a, blockIdx.y, blockIdx.x);
-  else solve_body<T, TM, LA>(in3, du, out, a, blockIdx.x, blockIdx.y);
+  // the grid runs directions fastest: blocks that run together share a mode tile, so its complex
+  // operators (133 KB per mode) are read from DRAM once and from L2 after
+  solve_body<T, TM>(in3, du, out, a, blockIdx.y, blockIdx.x);
 }
 
 
@@ -1486,22 +1355,11 @@ static YinvArgs yinv_args(const sp_ctx* c) {
   YinvArgs a;
   a.Mm = c->Mm; a.MZ = c->MZ; a.MX = c->MX; a.Kx = c->Kx; a.NY = c->NY; a.N = c->N; a.NH = c->NH;
   a.alpha = c->alpha; a.beta = c->beta;
-  a.q2 = (c->N % 4 == 0 && c->Tp != nullptr) ? 1 : 0;
-  a.NQ = c->N / 4 + 1;
   a.jchunk = 1;
   return a;
 }
 
-template <typename T>
-static YinvTabs<T> yinv_tabs(const sp_ctx* c) {
-  YinvTabs<T> t;
-  if constexpr (sizeof(T) == 8) {
-    t = {c->Th, c->TDh, c->Tp, c->TDp, c->tq};
-  } else {
-    t = {c->Th_f, c->TDh_f, c->Tp_f, c->TDp_f, c->tq_f};
-  }
-  return t;
-}
+static YinvTabs<float> yinv_tabs(const sp_ctx* c) { return {c->Th_f, c->TDh_f}; }
 
 // ------------------------------------------------------------ grouped kernels
 // One launch over several independent problems: block b runs block
@@ -1550,7 +1408,7 @@ struct GSolve {
   SolveArgs a;
 };
 
-template <typename T, bool LA>
+template <typename T>
 __global__ void __launch_bounds__(kThreadsSolveGrp) k_solve_grp(const double* __restrict__ du_base,
                                                             double* __restrict__ out_base,
                                                             const GSolve* __restrict__ recs,
@@ -1562,7 +1420,7 @@ __global__ void __launch_bounds__(kThreadsSolveGrp) k_solve_grp(const double* __
   __shared__ GSolve r;
   if (threadIdx.x == 0) r = recs[i];
   __syncthreads();
-  solve_body<T, kTileSolve, LA>(reinterpret_cast<const C2<T>*>(r.in3), reinterpret_cast<const double2*>(du_base + r.off),
+  solve_body<T, kTileSolve>(reinterpret_cast<const C2<T>*>(r.in3), reinterpret_cast<const double2*>(du_base + r.off),
                 reinterpret_cast<double2*>(out_base + r.off), r.a, blockIdx.x - first[i], 0);
 }
 
@@ -1626,26 +1484,18 @@ size_t sp_xz_global_plane_bytes(const sp_ctx* c) {
 
 cudaError_t launch_yinv(const sp_ctx* c, bool fp32, const double* in, void* out6, int n_dir,
                         cudaStream_t st) {
-  if (fp32 && c->use_yinv_tc && sp_yinv_tc_supported(c)) return launch_yinv_tc(c, in, out6, n_dir, st);
+  if (!fp32) return launch_yinv_fx(c, in, out6, n_dir, st);
+  if (c->use_yinv_tc && sp_yinv_tc_supported(c)) return launch_yinv_tc(c, in, out6, n_dir, st);
   YinvArgs a = yinv_args(c);
-  if (fp32) a.q2 = 0;
-  const int nj = a.q2 ? a.NQ : c->NH;
   const int tiles = (c->Mm + kTileYinv - 1) / kTileYinv;
   int jsplit = 1;
-  while (tiles * jsplit * n_dir < c->sm_count && jsplit < nj) ++jsplit;
-  a.jchunk = (nj + jsplit - 1) / jsplit;
-  dim3 grid(tiles, (nj + a.jchunk - 1) / a.jchunk, n_dir);
-  if (fp32) {
-    size_t sm = (size_t)3 * c->NY * kTileYinv * sizeof(C2<float>);
-    cudaFuncSetAttribute(k_yinv<float>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
-    k_yinv<float><<<grid, kThreadsYinv, sm, st>>>(reinterpret_cast<const double2*>(in),
-                                                  reinterpret_cast<C2<float>*>(out6), yinv_tabs<float>(c), a);
-  } else {
-    size_t sm = (size_t)3 * c->NY * kTileYinv * sizeof(C2<double>);
-    cudaFuncSetAttribute(k_yinv<double>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
-    k_yinv<double><<<grid, kThreadsYinv, sm, st>>>(reinterpret_cast<const double2*>(in),
-                                                   reinterpret_cast<C2<double>*>(out6), yinv_tabs<double>(c), a);
-  }
+  while (tiles * jsplit * n_dir < c->sm_count && jsplit < c->NH) ++jsplit;
+  a.jchunk = (c->NH + jsplit - 1) / jsplit;
+  dim3 grid(tiles, (c->NH + a.jchunk - 1) / a.jchunk, n_dir);
+  size_t sm = (size_t)3 * c->NY * kTileYinv * sizeof(C2<float>);
+  cudaFuncSetAttribute(k_yinv<float>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+  k_yinv<float><<<grid, kThreadsYinv, sm, st>>>(reinterpret_cast<const double2*>(in),
+                                                reinterpret_cast<C2<float>*>(out6), yinv_tabs(c), a);
   return cudaGetLastError();
 }
 
@@ -1723,7 +1573,7 @@ cudaError_t launch_xz(const sp_ctx* c, bool fp32, int mode, const void* in6, voi
 
 static size_t solve_smem(const sp_ctx* c, int esize, int TM = kTileSolve) {
   const int NY = c->NY, NR = c->N - 1;
-  size_t vals = (size_t)3 * NY * TM * 2 * esize;
+  size_t vals = esize == 8 ? 0 : (size_t)3 * NY * TM * 2 * esize;  // values to transform (float)
   vals = (vals + 15) / 16 * 16;
   size_t d = (size_t)16 * (3 * TM * NY + 3 * TM * NR + TM * 2 * c->cv + 2 * TM * NR + 2 * TM * NY);
   return vals + d + 16;
@@ -1763,12 +1613,11 @@ static cudaError_t launch_solve_t(const sp_ctx* c, const SolveArgs& a, const voi
                                   int n_dir, int threads, cudaStream_t st) {
   const size_t sm = solve_smem(c, (int)sizeof(T), TM);
   if (sm + 40 * TM + 64 > (size_t)232448 || threads > MAXT) return cudaErrorInvalidConfiguration;  // does not fit
-  auto kern = c->cfg.lam_adv ? k_solve<T, TM, MAXT, true> : k_solve<T, TM, MAXT, false>;
+  auto kern = k_solve<T, TM, MAXT>;
   cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
   if (e != cudaSuccess) return e;
   const unsigned tiles = (c->n_unique + TM - 1) / TM;
-  const dim3 grid = c->cfg.lam_adv ? dim3(n_dir, tiles) : dim3(tiles, n_dir);
-  kern<<<grid, threads, sm, st>>>(reinterpret_cast<const C2<T>*>(in3), reinterpret_cast<const double2*>(du),
+  kern<<<dim3(n_dir, tiles), threads, sm, st>>>(reinterpret_cast<const C2<T>*>(in3), reinterpret_cast<const double2*>(du),
                                   reinterpret_cast<double2*>(out), a);
   return cudaGetLastError();
 }
@@ -1792,18 +1641,25 @@ static cudaError_t launch_solve_shape(const sp_ctx* c, int shape, const SolveArg
 
 int sp_solve_shapes(const sp_ctx* c, int* tm, int* threads) {
   for (int i = 0; i < kNumSolveShapes; ++i) {
-    if (tm) tm[i] = kSolveShapes[i].tm;
-    if (threads) threads[i] = shape_threads(c, i);
+    if (tm) tm[i] = c->cfg.lam_adv ? kSolveShapes[i].tm : 1;
+    if (threads) threads[i] = c->cfg.lam_adv ? shape_threads(c, i) : solve_one_threads(c, i);
   }
   return kNumSolveShapes;
 }
 
-cudaError_t launch_solve(const sp_ctx* c, bool fp32, const void* in3, const double* du, double* out,
+cudaError_t launch_solve(const sp_ctx* c, bool fp32, const void* in3, const double* du, double* out, void* work,
                          int n_dir, cudaStream_t st, int shape) {
-  const SolveArgs a = solve_args(c);
   if (shape < 0) shape = c->solve_shape_tan;
-  if (fp32) return launch_solve_shape<float>(c, shape, a, in3, du, out, n_dir, st);
-  return launch_solve_shape<double>(c, shape, a, in3, du, out, n_dir, st);
+  if (shape >= kNumSolveShapes) return cudaErrorInvalidValue;
+  if (!fp32) {
+    const cudaError_t e = launch_rhs_fx(c, in3, du, work, n_dir, 0, 0, 0, st);
+    if (e != cudaSuccess) return e;
+  }
+  const void* in = fp32 ? in3 : work;
+  if (!c->cfg.lam_adv) return launch_solve_one(c, fp32, in, du, out, n_dir, shape, st);
+  const SolveArgs a = solve_args(c);
+  if (fp32) return launch_solve_shape<float>(c, shape, a, in, du, out, n_dir, st);
+  return launch_solve_shape<double>(c, shape, a, in, du, out, n_dir, st);
 }
 
 static size_t solve_adj_smem(const sp_ctx* c) {
@@ -1972,7 +1828,7 @@ void grp_kernel_free(GrpKernel* k) {
 }
 
 void grp_plan_free(GrpPlan* p) {
-  for (GrpKernel* k : {&p->yinv64, &p->yinv32, &p->xz64, &p->xz32, &p->solve64, &p->solve32, &p->fx[0], &p->fx[1]})
+  for (GrpKernel* k : {&p->yinv64, &p->yinv32, &p->xz64, &p->xz32, &p->solve64, &p->rhs64, &p->solve32, &p->fx[0], &p->fx[1]})
     grp_kernel_free(k);
   for (GrpKernel& k : p->xzr) grp_kernel_free(&k);
   p->n = 0;
@@ -2007,11 +1863,10 @@ static cudaError_t grp_build_yinv(GrpKernel* k, sp_ctx* const* mem, int n, const
     GYinv<T>& r = recs[m];
     r.off = offs[m];
     r.out = reinterpret_cast<C2<T>*>(c->ws6);
-    r.tb = yinv_tabs<T>(c);
+    r.tb = yinv_tabs(c);
     YinvArgs& a = r.a;
     a = yinv_args(c);
-    if (sizeof(T) == 4) a.q2 = 0;
-    const int nj = a.q2 ? a.NQ : c->NH;
+    const int nj = c->NH;
     a.jchunk = (nj + jsplit - 1) / jsplit;
     r.gx = (c->Mm + kTileYinv - 1) / kTileYinv;
     nblk[m] = r.gx * ((nj + a.jchunk - 1) / a.jchunk);
@@ -2051,21 +1906,20 @@ static cudaError_t grp_build_xz(GrpKernel* k, sp_ctx* const* mem, int n, const i
 
 static cudaError_t grp_build_solve(GrpKernel* k, sp_ctx* const* mem, int n, const size_t* offs, const int* order,
                                    int esize) {
+  if (!mem[0]->cfg.lam_adv) return grp_build_solve_one(k, mem, n, offs, order, esize);
   std::vector<GSolve> recs(n);
   std::vector<int> nblk(n);
   size_t smem = 0;
   for (int m = 0; m < n; ++m) {
     const sp_ctx* c = mem[m];
     recs[m].off = offs[m];
-    recs[m].in3 = c->ws3;
+    recs[m].in3 = esize == 8 ? c->ws6 : c->ws3;  // right-hand sides of k_rhs_fx or values
     recs[m].a = solve_args(c);
     nblk[m] = (c->n_unique + kTileSolve - 1) / kTileSolve;
     smem = std::max(smem, solve_smem(c, esize));
   }
-  const bool la = mem[0]->cfg.lam_adv != 0;
-  const void* kern = esize == 8 ? (la ? (const void*)k_solve_grp<double, true> : (const void*)k_solve_grp<double, false>)
-                                : (la ? (const void*)k_solve_grp<float, true> : (const void*)k_solve_grp<float, false>);
-  cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  cudaError_t e = esize == 8 ? cudaFuncSetAttribute(k_solve_grp<double>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem)
+                             : cudaFuncSetAttribute(k_solve_grp<float>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return e;
   return grp_make(k, recs, nblk, order, n, smem);
 }
@@ -2082,7 +1936,7 @@ cudaError_t grp_plan_build(GrpPlan* p, sp_ctx* const* mem, int n, const size_t* 
   int jsplit = 1;
   while (tiles * jsplit < 2 * mem[0]->sm_count && jsplit < nh_min) ++jsplit;
   cudaError_t e;
-  if ((e = grp_build_yinv<double>(&p->yinv64, mem, n, offs, order, jsplit)) != cudaSuccess) return e;
+  if ((e = grp_build_cheb_fx(p, mem, n, offs, order)) != cudaSuccess) return e;
   if ((e = grp_build_yinv<float>(&p->yinv32, mem, n, offs, order, jsplit)) != cudaSuccess) return e;
   std::vector<int> fxm(n);
   for (int m = 0; m < n; ++m) fxm[m] = mem[m]->use_fx;
@@ -2099,14 +1953,11 @@ cudaError_t grp_plan_build(GrpPlan* p, sp_ctx* const* mem, int n, const size_t* 
 }
 
 cudaError_t grp_launch_yinv(const GrpPlan& p, bool fp32, const double* in_base, const int* active, cudaStream_t st) {
-  const GrpKernel& k = fp32 ? p.yinv32 : p.yinv64;
+  if (!fp32) return grp_launch_yinv_fx(p, in_base, active, st);
+  const GrpKernel& k = p.yinv32;
   if (k.blocks == 0) return cudaSuccess;
-  if (fp32)
-    k_yinv_grp<float><<<k.blocks, kThreadsYinv, k.smem, st>>>(in_base, static_cast<const GYinv<float>*>(k.recs),
-                                                               k.inst, k.first, active);
-  else
-    k_yinv_grp<double><<<k.blocks, kThreadsYinv, k.smem, st>>>(in_base, static_cast<const GYinv<double>*>(k.recs),
-                                                                k.inst, k.first, active);
+  k_yinv_grp<float><<<k.blocks, kThreadsYinv, k.smem, st>>>(in_base, static_cast<const GYinv<float>*>(k.recs),
+                                                             k.inst, k.first, active);
   return cudaGetLastError();
 }
 
@@ -2144,12 +1995,15 @@ cudaError_t grp_launch_solve(const GrpPlan& p, bool fp32, const double* du_base,
                              cudaStream_t st) {
   const GrpKernel& k = fp32 ? p.solve32 : p.solve64;
   if (k.blocks == 0) return cudaSuccess;
+  if (!fp32) {
+    const cudaError_t e = grp_launch_rhs_fx(p, du_base, active, st);
+    if (e != cudaSuccess) return e;
+  }
+  if (!p.lam_adv) return grp_launch_solve_one(k, fp32, du_base, out_base, active, st);
   const GSolve* r = static_cast<const GSolve*>(k.recs);
-  auto kern = p.lam_adv ? k_solve_grp<float, true> : k_solve_grp<float, false>;
-  auto kern64 = p.lam_adv ? k_solve_grp<double, true> : k_solve_grp<double, false>;
   if (fp32)
-    kern<<<k.blocks, kThreadsSolveGrp, k.smem, st>>>(du_base, out_base, r, k.inst, k.first, active);
+    k_solve_grp<float><<<k.blocks, kThreadsSolveGrp, k.smem, st>>>(du_base, out_base, r, k.inst, k.first, active);
   else
-    kern64<<<k.blocks, kThreadsSolveGrp, k.smem, st>>>(du_base, out_base, r, k.inst, k.first, active);
+    k_solve_grp<double><<<k.blocks, kThreadsSolveGrp, k.smem, st>>>(du_base, out_base, r, k.inst, k.first, active);
   return cudaGetLastError();
 }

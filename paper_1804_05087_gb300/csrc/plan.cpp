@@ -506,28 +506,15 @@ sp_status sp_build_plan(sp_ctx* c) {
       Cfh[(size_t)n * NH + j] = 2.0 / (N * cbn) * cospi_frac((long)j * n, N) / cbj;
     }
   }
-  // the second level of the even/odd split (N divisible by 4): at y_{N/2-jq}, odd degrees
-  // n = 2m+1 give T_n = (-1)^m sin(pi jq n / N) and T_n' = (-1)^m n cos(pi jq n / N) / cos(pi jq / N)
+  // the second level of the even/odd split of the float forward transform (N divisible by 4)
   const int NQ = N / 4 + 1;
   const bool q2 = N % 4 == 0 && N >= 4;
-  std::vector<double> Tp, TDp, tq, Cq;
+  std::vector<double> Cq;
   if (q2) {
     Cq.assign((size_t)n1 * NQ, 0.0);
     for (int n = 0; n < n1; n += 2) {
       const double cbn = (n == 0 || n == N) ? 2.0 : 1.0;
       for (int jq = 0; jq < NQ; ++jq) Cq[(size_t)n * NQ + jq] = 2.0 / (N * cbn) * cospi_frac((long)jq * n, N);
-    }
-    Tp.assign((size_t)NQ * n1, 0.0);
-    TDp.assign((size_t)NQ * n1, 0.0);
-    tq.assign(NQ, 0.0);
-    for (int jq = 0; jq < NQ; ++jq) {
-      const double cj = cospi_frac(jq, N), sj = cospi_frac((long)N - 2L * jq, 2L * N);
-      tq[jq] = sj / cj;
-      for (int n = 1; n < n1; n += 2) {
-        const double sg = (((n - 1) / 2) & 1) ? -1.0 : 1.0;
-        Tp[(size_t)jq * n1 + n] = sg * cospi_frac((long)N - 2L * jq * n, 2L * N);
-        TDp[(size_t)jq * n1 + n] = sg * n * cospi_frac((long)jq * n, N) / cj;
-      }
     }
   }
   // twiddles exp(-2 pi i k / n)
@@ -555,8 +542,8 @@ sp_status sp_build_plan(sp_ctx* c) {
     c->off_vc = 0;
     c->off_hc = 2 * (N - 1) * n1;
     c->op_stride = std::max(c->op_stride, 4 * (N - 1) * n1);
-    c->op_stride += c->op_stride & 1;  // 16-byte aligned complex columns
   }
+  c->op_stride += c->op_stride & 1;  // 16-byte aligned: complex columns, bulk copies of a mode's operators
   std::vector<double> ops((size_t)c->n_unique * c->op_stride, 0.0);
   ChebOps C(N);
   int nthreads = (int)std::thread::hardware_concurrency();
@@ -656,14 +643,28 @@ sp_status sp_build_plan(sp_ctx* c) {
     if (!up((void**)&c->rhs_tc_mat, imf.data(), imf.size() * 4))
       return sp_fail(c, SP_ENOMEM, "device allocation of plan tables failed");
   }
+  const std::vector<int> fx = cheb_fx_table(n1);
+  // tables of k_solve_one: wavenumbers per solved mode, row indices, the forward transform by points
+  std::vector<double> wave((size_t)4 * c->n_unique, 0.0), rowidx(n1 + 1);
+  for (int u = 0; u < c->n_unique; ++u) {
+    int pos, iz;
+    sp_unique_mode(c, u, &pos, &iz);
+    const double kx = c->alpha * (pos <= c->Kx ? pos : pos - c->MX), kz = c->beta * iz, k = std::sqrt(kx * kx + kz * kz);
+    wave[4 * u] = kx;
+    wave[4 * u + 1] = kz;
+    wave[4 * u + 2] = k > 0 ? 1.0 / k : 0.0;
+  }
+  for (int n = 0; n <= n1; ++n) rowidx[n] = n;
+  std::vector<float> cft((size_t)NH * n1);
+  for (int j = 0; j < NH; ++j)
+    for (int n = 0; n < n1; ++n) cft[(size_t)j * n1 + n] = Cfhf[(size_t)n * NH + j];
+  if (!up((void**)&c->cheb_fx, fx.data(), fx.size() * 4) || !up((void**)&c->wave, wave.data(), wave.size() * 8) ||
+      !up((void**)&c->rowidx, rowidx.data(), rowidx.size() * 8) || !up((void**)&c->cft_f, cft.data(), cft.size() * 4))
+    return sp_fail(c, SP_ENOMEM, "device allocation of plan tables failed");
   if (q2) {
-    std::vector<float> Tpf(Tp.begin(), Tp.end()), TDpf(TDp.begin(), TDp.end()), tqf(tq.begin(), tq.end()),
-        Cqf(Cq.begin(), Cq.end());
-    ok = up((void**)&c->Cq, Cq.data(), Cq.size() * 8) && up((void**)&c->Cq_f, Cqf.data(), Cqf.size() * 4) &&
-         up((void**)&c->Tp, Tp.data(), Tp.size() * 8) && up((void**)&c->TDp, TDp.data(), TDp.size() * 8) &&
-         up((void**)&c->tq, tq.data(), tq.size() * 8) && up((void**)&c->Tp_f, Tpf.data(), Tpf.size() * 4) &&
-         up((void**)&c->TDp_f, TDpf.data(), TDpf.size() * 4) && up((void**)&c->tq_f, tqf.data(), tqf.size() * 4);
-    if (!ok) return sp_fail(c, SP_ENOMEM, "device allocation of plan tables failed");
+    std::vector<float> Cqf(Cq.begin(), Cq.end());
+    if (!up((void**)&c->Cq_f, Cqf.data(), Cqf.size() * 4))
+      return sp_fail(c, SP_ENOMEM, "device allocation of plan tables failed");
   }
   return sp_build_fft_tables(c);
 }

@@ -10,8 +10,8 @@
 // the records): O(N) FP64 work, one thread per (mode, parity, direction), lanes
 // over directions so that a warp reads each record entry once (a broadcast).
 //
-//   k_rhs  : values at the Gauss-Lobatto points -> Chebyshev coefficients of rows
-//            0..N-2, plus du/dt, for the three components (threads over rows).
+//   k_rhs  : float values at the Gauss-Lobatto points -> Chebyshev coefficients of rows
+//            0..N-2, plus du/dt, for the three components (threads over rows; FP64: k_rhs_fx).
 //   k_chain: thread (mode, P, direction) solves the (v, a, p) problem of parity P
 //            (two Helmholtz sweeps and the 2 x 2 influence correction) and the
 //            Helmholtz problem of b of parity 1-P, then writes G_v on the rows of
@@ -26,10 +26,8 @@ namespace {
 
 // ------------------------------------------------------------------ k_rhs
 struct RhsArgs {
-  const double* Cfh_d;
   const float* Cfh_f;
-  const double* Cq_d;      // second-level split (N divisible by 4), null otherwise: see k_rhs
-  const float* Cq_f;
+  const float* Cq_f;       // second-level split (N divisible by 4), null otherwise: see k_rhs
   int NQ;
   double2* W;              // right-hand sides: (u, d, row c (N-1) + n) at u su + d sd + row sn
   long long su, sd, sn;    // complex strides of W: unique mode, direction, row (c (N-1) + n)
@@ -54,11 +52,6 @@ __device__ __forceinline__ void mode_of(int u, int Kx, int MZ, int* pos, int* iz
 
 template <typename T>
 __device__ __forceinline__ C2<T> ldv(const C2<T>* p) { return *p; }
-template <>
-__device__ __forceinline__ C2<double> ldv(const C2<double>* p) {
-  const double2 v = __ldg(reinterpret_cast<const double2*>(p));
-  return mk(v.x, v.y);
-}
 template <>
 __device__ __forceinline__ C2<float> ldv(const C2<float>* p) {
   const float2 v = __ldg(reinterpret_cast<const float2*>(p));
@@ -105,7 +98,7 @@ __global__ void __launch_bounds__(kRhsThreads) k_rhs(const C2<T>* __restrict__ i
   // second level for the even degrees (N divisible by 4): with s'_j = s_j / cbar_j (cbar_0 = 2),
   // T_2m(y_{N/2-j}) = (-1)^m T_2m(y_j) pairs j with N/2 - j: slot j < N/4 receives
   // s'_j + s'_{N/2-j} (degrees 0 mod 4), slot N/2 - j receives s'_j - s'_{N/2-j} (2 mod 4)
-  const bool q2 = a.Cq_d != nullptr;
+  const bool q2 = a.Cq_f != nullptr;
   const int NQ = a.NQ, NQ1 = NQ - 1;  // NQ1 = N/4
   if (q2) {
     for (int idx = threadIdx.x; idx < 3 * TM * NQ1; idx += blockDim.x) {
@@ -135,15 +128,8 @@ __global__ void __launch_bounds__(kRhsThreads) k_rhs(const C2<T>* __restrict__ i
       if (u >= a.n_unique) continue;
       const C2<T>* col = sv + (c * NY) * TM + t;
       C2<T> acc = mk((T)0, (T)0);
-      const T* cf;
-      const T* cq;
-      if constexpr (sizeof(T) == 8) {
-        cf = a.Cfh_d + (size_t)n * NH;
-        cq = a.Cq_d + (size_t)n * NQ;
-      } else {
-        cf = a.Cfh_f + (size_t)n * NH;
-        cq = a.Cq_f + (size_t)n * NQ;
-      }
+      const T* cf = a.Cfh_f + (size_t)n * NH;
+      const T* cq = a.Cq_f + (size_t)n * NQ;
       if (cls == 0) {
         for (int jj = 0; jj < NH - 1; ++jj) acc = acc + scl(col[(N - jj) * TM], cf[jj]);
       } else if (!q2) {
@@ -402,11 +388,10 @@ cudaError_t launch_chain_rhs(const sp_ctx* c, bool fp32, const void* in3, const 
   if (n_dir <= 0) return cudaSuccess;
   RhsArgs r;
   chain_strides(c, n_dir, &r.su, &r.sd, &r.sn);
-  if (fp32 && c->use_rhs_tc && sp_rhs_tc_supported(c))  // forward transform on the tensor cores
+  if (!fp32) return launch_rhs_fx(c, in3, du, work, n_dir, r.su, r.sd, r.sn, st);
+  if (c->use_rhs_tc && sp_rhs_tc_supported(c))  // forward transform on the tensor cores
     return launch_rhs_tc(c, in3, du, work, n_dir, r.su, r.sd, r.sn, st);
-  r.Cfh_d = c->Cfh;
   r.Cfh_f = c->Cfh_f;
-  r.Cq_d = c->Cq;
   r.Cq_f = c->Cq_f;
   r.NQ = c->N / 4 + 1;
   r.W = static_cast<double2*>(work);
@@ -420,15 +405,8 @@ cudaError_t launch_chain_rhs(const sp_ctx* c, bool fp32, const void* in3, const 
   r.NH = c->NH;
   r.inv_dt = 1.0 / c->dt;
   const dim3 grid((c->n_unique + kRhsTM - 1) / kRhsTM, n_dir);
-  if (fp32) {
-    const size_t sm = sizeof(C2<float>) * 3 * c->NY * kRhsTM;
-    k_rhs<float><<<grid, kRhsThreads, sm, st>>>(static_cast<const C2<float>*>(in3),
-                                                reinterpret_cast<const double2*>(du), r);
-  } else {
-    const size_t sm = sizeof(C2<double>) * 3 * c->NY * kRhsTM;
-    k_rhs<double><<<grid, kRhsThreads, sm, st>>>(static_cast<const C2<double>*>(in3),
-                                                 reinterpret_cast<const double2*>(du), r);
-  }
+  const size_t sm = sizeof(C2<float>) * 3 * c->NY * kRhsTM;
+  k_rhs<float><<<grid, kRhsThreads, sm, st>>>(static_cast<const C2<float>*>(in3), reinterpret_cast<const double2*>(du), r);
   return cudaGetLastError();
 }
 

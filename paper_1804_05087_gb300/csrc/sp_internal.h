@@ -90,12 +90,12 @@ struct sp_ctx {
 
   // device tables
   double *Th = nullptr, *TDh = nullptr, *Cfh = nullptr;
-  // two-level split of k_yinv (N divisible by 4): Tp, TDp [N/4+1][NY], tq [N/4+1] (kernels.cu)
-  double *Tp = nullptr, *TDp = nullptr, *tq = nullptr;
-  float *Tp_f = nullptr, *TDp_f = nullptr, *tq_f = nullptr;
-  // the same for the forward transform of k_rhs: Cq[n][jq] = 2 / (N cbar_n) cos(pi jq n / N), even
+  int2* cheb_fx = nullptr;       // [2][NH][NY + 1] T_n(y_j) and T_n'(y_j) / n^2 as integers (cheb_fx.cu)
+  double* wave = nullptr;        // [n_unique][4] kx, kz, 1/k (solve_one.cu)
+  double* rowidx = nullptr;      // [NY + 1] 0, 1, ...
+  float* cft_f = nullptr;        // [NH][NY] the transpose of Cfh_f
+  // two-level forward transform of the float k_rhs (N divisible by 4): Cq[n][jq] = 2 / (N cbar_n) cos(pi jq n / N), even
   // rows n <= N-2, jq <= N/4 (solve_chain.cu)
-  double* Cq = nullptr;
   float* Cq_f = nullptr;
   // tensor-core inverse transform (41 <= NY <= 72): shared-memory image of T and T' split into
   // TF32 hi and lo parts (yinv_tc.cu)
@@ -223,13 +223,14 @@ struct GrpKernel {
   int* inst = nullptr;
   int* first = nullptr;
   int blocks = 0;
+  int threads = 0;
   size_t smem = 0;
 };
 constexpr int kGrpRegClasses = 5;  // register-FFT plane kernels: grids 16, 24, 32, 48, 64
 struct GrpPlan {
   int n = 0;
   int lam_adv = 0;                // every member has laminar advection in L (else none has)
-  GrpKernel yinv64, yinv32, xz64, solve64, solve32;
+  GrpKernel yinv64, yinv32, xz64, rhs64, solve64, solve32;
   GrpKernel xz32;                 // float plane stage of the members without a register-FFT kernel
   GrpKernel xzr[kGrpRegClasses];  // float plane stage of the others, per grid size class (xz_reg.cu)
   GrpKernel fx[2];                // FP64 plane stage in fixed point, per shared-memory class (xz_fx.cu)
@@ -252,6 +253,9 @@ cudaError_t grp_launch_xz_reg(const GrpKernel* ks, const int* active, cudaStream
 // FP64 plane stage of the members that take the fixed-point kernels (the others: xz64)
 cudaError_t grp_build_xz_fx(GrpPlan* p, sp_ctx* const* members, int n, const int* order);
 cudaError_t grp_launch_xz_fx(const GrpPlan& p, int mode, const int* active, cudaStream_t st);
+cudaError_t grp_build_cheb_fx(GrpPlan* p, sp_ctx* const* members, int n, const size_t* offs, const int* order);
+cudaError_t grp_launch_yinv_fx(const GrpPlan& p, const double* in, const int* active, cudaStream_t st);
+cudaError_t grp_launch_rhs_fx(const GrpPlan& p, const double* du, const int* active, cudaStream_t st);
 // device copy of a host table; frees nothing on failure
 cudaError_t grp_upload(void** dst, const void* src, size_t bytes);
 void grp_kernel_free(GrpKernel* k);
@@ -299,9 +303,24 @@ size_t chain_scratch_bytes(const sp_ctx* c, int n_dir);
 sp_status sp_tangent_solve(sp_ctx* c, bool f32, void* vals, size_t vals_bytes, const double* du, double* out,
                            void* work, int nb, cudaStream_t st);
 // shape: index into the tile-shape table (sp_solve_shapes); -1 = the context's tangent choice
+// work (FP64): the right-hand sides, n_unique x 3 x (N-1) complex doubles per direction
 cudaError_t launch_solve(const sp_ctx* c, bool fp32, const void* in3, const double* du,
-                         double* out, int n_dir, cudaStream_t st, int shape = -1);
-// the tile shapes of k_solve (modes per block, threads per block); returns their number
+                         double* out, void* work, int n_dir, cudaStream_t st, int shape = -1);
+// FP64 Chebyshev transforms in fixed point (cheb_fx.cu): launch_yinv's inputs and outputs; the
+// right-hand sides u/dt + N at u su + dir sd + row sn (sn = 0: [dir][mode][3][N - 1])
+std::vector<int> cheb_fx_table(int NY);
+cudaError_t launch_yinv_fx(const sp_ctx* c, const double* in, void* out6, int n_dir, cudaStream_t st);
+cudaError_t launch_rhs_fx(const sp_ctx* c, const void* in3, const double* du, void* W, int n_dir, long long su,
+                          long long sd, long long sn, cudaStream_t st);
+// solve_one.cu: one mode per block (every context without laminar advection in L); FP64 reads the
+// right-hand sides [dir][mode][3][N - 1], float the values
+int solve_one_threads(const sp_ctx* c, int shape);
+cudaError_t launch_solve_one(const sp_ctx* c, bool fp32, const void* in, const double* du, double* out, int n_dir,
+                             int shape, cudaStream_t st);
+cudaError_t grp_build_solve_one(GrpKernel* k, sp_ctx* const* members, int n, const size_t* offs, const int* order, int esize);
+cudaError_t grp_launch_solve_one(const GrpKernel& k, bool fp32, const double* du, double* out, const int* active,
+                                 cudaStream_t st);
+// the tile shapes of the per-mode solve (modes per block, threads per block); returns their number
 int sp_solve_shapes(const sp_ctx* c, int* tm, int* threads);
 cudaError_t launch_base_to_f32(const sp_ctx* c, cudaStream_t st);
 // adjoint chain (sp_vjp): solve^T + Chebyshev^T, plane stage^T (launch_xz with

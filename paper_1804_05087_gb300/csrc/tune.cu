@@ -49,7 +49,7 @@ extern "C" sp_status sp_autotune(sp_ctx* c, int n_dir, sp_tune_report* rep, void
     for (int i = 0; i < ns; ++i) {
       r.tile[i] = tm[i];
       r.threads[i] = th[i];
-      cudaError_t e = launch_solve(c, fp32, c->ws3, buf, buf + (size_t)n_dir * L, nd, st, i);  // warm-up
+      cudaError_t e = launch_solve(c, fp32, c->ws3, buf, buf + (size_t)n_dir * L, c->ws6, nd, st, i);  // warm-up
       if (e == cudaErrorInvalidConfiguration) {
         cudaGetLastError();
         ms[i] = -1.0;
@@ -58,7 +58,7 @@ extern "C" sp_status sp_autotune(sp_ctx* c, int n_dir, sp_tune_report* rep, void
       if ((s = sp_cuda(c, e, "sp_autotune: solve")) != SP_OK) break;
       cudaEventRecord(e0, st);
       for (int k = 0; k < kReps && e == cudaSuccess; ++k)
-        e = launch_solve(c, fp32, c->ws3, buf, buf + (size_t)n_dir * L, nd, st, i);
+        e = launch_solve(c, fp32, c->ws3, buf, buf + (size_t)n_dir * L, c->ws6, nd, st, i);
       cudaEventRecord(e1, st);
       if ((s = sp_cuda(c, e, "sp_autotune: solve")) != SP_OK) break;
       if ((s = sp_cuda(c, cudaEventSynchronize(e1), "sp_autotune: sync")) != SP_OK) break;
