@@ -26,9 +26,11 @@ namespace {
 using namespace fx;
 
 constexpr int kThreadsC = 256;
-constexpr int kModes = 8;                       // modes per block
-constexpr int kColsY = 5 * kModes, kStrideY = kColsY + 1;  // u, v, w, Du, Dw of every mode (padded row)
-constexpr int kColsR = 3 * kModes, kStrideR = kColsR + 1;
+// modes per block: eight share the table loads best; four, when eight leave SMs without a block
+constexpr int kModes = 8, kModesFew = 4;
+// columns of a block's rows: u, v, w, Du, Dw (values: the three components) of every mode, padded
+__host__ __device__ constexpr int stride_y(int tm) { return 5 * tm + 1; }
+__host__ __device__ constexpr int stride_r(int tm) { return 3 * tm + 1; }
 constexpr int kSumBits = 62, kMaxBits = 59;     // bits of a column's sum of moduli and of its values
 constexpr int kNotFinite = 1 << 28;             // exponent of a column with a non-finite input
 
@@ -97,22 +99,36 @@ struct YArgs {
   double alpha, beta;
 };
 
-// (bx, by, bz): mode tile, chunk of the half grid, direction
-__device__ __forceinline__ void yinv_fx(const YArgs& a, int bx, int by, int bz, int4* xs, int (*sh)[kModes]) {
-  const int NY = a.NY, N = NY - 1, Mm = a.Mm, m0 = bx * kModes;
+// (bx, by, bz): mode tile, chunk of the half grid, direction. xs: [NY + 1][stride_y]
+template <int TM>
+__device__ __forceinline__ void yinv_fx(const YArgs& a, int bx, int by, int bz, int4* xs, int (*sh)[TM]) {
+  constexpr int ST = stride_y(TM), kWarps = kThreadsC / 32, RW = (3 * TM + kWarps - 1) / kWarps;
+  const int NY = a.NY, N = NY - 1, Mm = a.Mm, m0 = bx * TM;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  // one warp per (component, mode): scales, halves and derivative
-  for (int row = warp; row < 3 * kModes; row += kThreadsC / 32) {
-    const int f = row / kModes, t = row - f * kModes, m = m0 + t;
+  // one warp per (component, mode): the rows' loads first, kept in their own slots
+  unsigned em[RW];
+#pragma unroll
+  for (int r = 0; r < RW; ++r) {
+    em[r] = 0;
+    const int row = warp + r * kWarps, f = row / TM, m = m0 + row - f * TM;
+    if (row >= 3 * TM) continue;
     const double2* src = a.in + (((size_t)bz * 3 + f) * Mm + m) * NY;
-    const bool on = m < Mm;
-    unsigned em = 0;
-    for (int n = lane; n < NY; n += 32) em = max(em, on ? top_of(__ldg(src + n)) : 0u);
-    const int e = (int)(__reduce_max_sync(0xffffffffu, em) >> 20);
+    for (int n = lane; n <= NY; n += 32) {  // row NY: zero
+      double2 v = make_double2(0.0, 0.0);
+      if (m < Mm && n < NY) v = __ldg(src + n);
+      em[r] = max(em[r], top_of(v));
+      reinterpret_cast<double2*>(xs)[n * ST + row] = v;
+    }
+  }
+  // scales, halves and derivative columns
+#pragma unroll
+  for (int r = 0; r < RW; ++r) {
+    const int row = warp + r * kWarps, f = row / TM, t = row - f * TM;
+    if (row >= 3 * TM) continue;
+    const int e = (int)(__reduce_max_sync(0xffffffffu, em[r]) >> 20);
     u64 s0 = 0, s2 = 0, t0 = 0, t2 = 0;  // sums and largest values of a_n and of n^2 a_n
     for (int n = lane; n < NY; n += 32) {
-      if (!on) continue;
-      const double2 v = __ldg(src + n);
+      const double2 v = reinterpret_cast<const double2*>(xs)[n * ST + row];
       const unsigned px = part_of(v.x, e), py = part_of(v.y, e), q = max(px, py);
       s0 += px + py;
       s2 += (u64)(n * n) * (px + py);
@@ -132,66 +148,65 @@ __device__ __forceinline__ void yinv_fx(const YArgs& a, int bx, int by, int bz, 
       sh[f][t] = e == 0x7ff ? kNotFinite : e0;
       if (f != 1) sh[g][t] = e == 0x7ff ? kNotFinite : ed;
     }
-    for (int n = lane; n <= NY; n += 32) {  // row NY: zero
-      double2 v = make_double2(0.0, 0.0);
-      if (on && n < NY) v = __ldg(src + n);
-      xs[n * kStrideY + row] = halves2(from_double(v.x, e0), from_double(v.y, e0));
+    for (int n = lane; n <= NY; n += 32) {
+      int4* x = xs + n * ST;
+      const double2 v = reinterpret_cast<const double2*>(x)[row];
+      x[row] = halves2(from_double(v.x, e0), from_double(v.y, e0));
       if (f == 1) continue;
       const double n2 = (double)(n * n);
-      xs[n * kStrideY + g * kModes + t] =
-          n == 0 ? make_int4(0, 0, 0, 0) : halves2(from_double_times(v.x, ed, n2), from_double_times(v.y, ed, n2));
+      x[g * TM + t] = n == 0 ? make_int4(0, 0, 0, 0) : halves2(from_double_times(v.x, ed, n2), from_double_times(v.y, ed, n2));
     }
   }
   __syncthreads();
-  const int j_lo = by * a.jchunk, j_hi = min(a.NH, j_lo + a.jchunk);
+  // two lanes per point pair (y, -y) of a mode: one sums the even degrees, one the odd; then each
+  // forms the values of one of the two points
+  const int j_lo = by * a.jchunk, j_hi = min(a.NH, j_lo + a.jchunk), items = 2 * TM * (j_hi - j_lo);
   const size_t NYMm = (size_t)NY * Mm;
   double2* o = a.out + (size_t)bz * 6 * NYMm;
-  for (int it = threadIdx.x; it < kModes * (j_hi - j_lo); it += kThreadsC) {
-    const int t = it % kModes, jh = j_lo + it / kModes, m = m0 + t;
-    Sum2 E[5], O[5];
-    const int4* tr = reinterpret_cast<const int4*>(a.tab + (size_t)jh * (NY + 1));
-    const int4* td = reinterpret_cast<const int4*>(a.tab + (size_t)(a.NH + jh) * (NY + 1));
-    const int4* x = xs + t;
+  for (int i0 = warp * 32; i0 < items; i0 += kThreadsC) {
+    const int it = i0 + lane, t = it % TM, odd = it / TM & 1, jh = min(j_lo + it / (2 * TM), j_hi - 1), m = m0 + t;
+    Sum2 S[5];
+    const int2* tr = a.tab + (size_t)jh * (NY + 1) + odd;
+    const int2* td = tr + (size_t)a.NH * (NY + 1);
+    const int4* x = xs + odd * ST + t;
     for (int n = 0; n < NY; n += 2) {
-      const int4 c = __ldg(tr + n / 2), d = __ldg(td + n / 2);
+      const int2 c = __ldg(tr + n), d = __ldg(td + n);
 #pragma unroll
-      for (int f = 0; f < 5; ++f) {
-        const int4 k = f < 3 ? c : d;
-        E[f].add(x[f * kModes], make_int2(k.x, k.y));
-        O[f].add(x[kStrideY + f * kModes], make_int2(k.z, k.w));
-      }
-      x += 2 * kStrideY;
+      for (int f = 0; f < 5; ++f) S[f].add(x[f * TM], f < 3 ? c : d);
+      x += 2 * ST;
     }
-    if (m >= Mm) continue;
+    i64 vx[5], vy[5];
+#pragma unroll
+    for (int f = 0; f < 5; ++f) {
+      const i64 mx = S[f].x.value(), my = S[f].y.value();
+      const i64 px = __shfl_xor_sync(0xffffffffu, mx, TM), py = __shfl_xor_sync(0xffffffffu, my, TM);
+      // even lane: E + O at jh; odd lane: values E - O, derivatives O - E at N - jh
+      vx[f] = !odd ? mx + px : f < 3 ? px - mx : mx - px;
+      vy[f] = !odd ? my + py : f < 3 ? py - my : my - py;
+    }
+    const int j = odd ? N - jh : jh;
+    if (it >= items || m >= Mm || (odd && j == jh)) continue;
     const int pos = m / a.MZ, iz = m - pos * a.MZ;
     const double kx = a.alpha * (pos <= a.Kx ? pos : pos - a.MX), kz = a.beta * iz;
+    double2 v[5];
 #pragma unroll
-    for (int side = 0; side < 2; ++side) {
-      const int j = side == 0 ? jh : N - jh;
-      if (side == 1 && j == jh) break;
-      double2 v[5];
-#pragma unroll
-      for (int f = 0; f < 5; ++f) {
-        const i64 ex = E[f].x.value(), ey = E[f].y.value(), ox = O[f].x.value(), oy = O[f].y.value();
-        if (side == 0) v[f] = unscale(ex + ox, ey + oy, sh[f][t]);
-        else v[f] = f < 3 ? unscale(ex - ox, ey - oy, sh[f][t]) : unscale(ox - ex, oy - ey, sh[f][t]);
-      }
-      double2* d = o + (size_t)j * Mm + m;
-      d[0] = v[0];
-      d[NYMm] = v[1];
-      d[2 * NYMm] = v[2];
-      // Dw - i kz v, i kz u - i kx w, i kx v - Du
-      d[3 * NYMm] = make_double2(fma(kz, v[1].y, v[4].x), fma(-kz, v[1].x, v[4].y));
-      d[4 * NYMm] = make_double2(fma(kx, v[2].y, -kz * v[0].y), fma(-kx, v[2].x, kz * v[0].x));
-      d[5 * NYMm] = make_double2(-fma(kx, v[1].y, v[3].x), fma(kx, v[1].x, -v[3].y));
-    }
+    for (int f = 0; f < 5; ++f) v[f] = unscale(vx[f], vy[f], sh[f][t]);
+    double2* d = o + (size_t)j * Mm + m;
+    d[0] = v[0];
+    d[NYMm] = v[1];
+    d[2 * NYMm] = v[2];
+    // Dw - i kz v, i kz u - i kx w, i kx v - Du
+    d[3 * NYMm] = make_double2(fma(kz, v[1].y, v[4].x), fma(-kz, v[1].x, v[4].y));
+    d[4 * NYMm] = make_double2(fma(kx, v[2].y, -kz * v[0].y), fma(-kx, v[2].x, kz * v[0].x));
+    d[5 * NYMm] = make_double2(-fma(kx, v[1].y, v[3].x), fma(kx, v[1].x, -v[3].y));
   }
 }
 
-__global__ void __launch_bounds__(kThreadsC, 2) k_yinv_fx(const __grid_constant__ YArgs a) {
+template <int TM>
+__global__ void __launch_bounds__(kThreadsC, 3) k_yinv_fx(const __grid_constant__ YArgs a) {
   extern __shared__ __align__(16) unsigned char smem[];
-  __shared__ int sh[5][kModes];
-  yinv_fx(a, blockIdx.x, blockIdx.y, blockIdx.z, reinterpret_cast<int4*>(smem), sh);
+  __shared__ int sh[5][TM];
+  yinv_fx<TM>(a, blockIdx.x, blockIdx.y, blockIdx.z, reinterpret_cast<int4*>(smem), sh);
 }
 
 // ------------------------------------------------------------------ forward
@@ -217,78 +232,85 @@ __device__ __forceinline__ void unique_mode_of(int u, int Kx, int MZ, int* pos, 
   }
 }
 
+template <int TM>
 struct RShared {
-  unsigned em[kColsR];
-  int sum[kColsR];
-  int sh[kColsR];
-  int pos[kModes], iz[kModes];
+  unsigned em[3 * TM];
+  int sum[3 * TM];
+  int sh[3 * TM];
+  int pos[TM], iz[TM];
 };
 
-// (bx, by, bz): tile of solved modes, chunk of rows, direction
-__device__ __forceinline__ void rhs_fx(const RArgs& a, int bx, int by, int bz, int4* xs, RShared& s) {
-  const int NY = a.NY, N = NY - 1, NH = a.NH, NR = N - 1, Mm = a.Mm, u0 = bx * kModes;
+// (bx, by, bz): tile of solved modes, chunk of rows, direction. xs: [NY][stride_r]
+template <int TM>
+__device__ __forceinline__ void rhs_fx(const RArgs& a, int bx, int by, int bz, int4* xs, RShared<TM>& s) {
+  constexpr int ST = stride_r(TM);
+  const int NY = a.NY, N = NY - 1, NH = a.NH, NR = N - 1, Mm = a.Mm, u0 = bx * TM;
   const int tid = threadIdx.x;
-  if (tid < kModes) {
+  if (tid < TM) {
     int pos = 0, iz = 0;
     if (u0 + tid < a.n_unique) unique_mode_of(u0 + tid, a.Kx, a.MZ, &pos, &iz);
     s.pos[tid] = pos;
     s.iz[tid] = iz;
   }
-  if (tid < kColsR) {
+  if (tid < 3 * TM) {
     s.em[tid] = 0;
     s.sum[tid] = 0;
   }
   __syncthreads();
-  // lanes take the modes fastest, then the points: value (c, j) of mode t
-  const int t = tid % kModes, part = tid / kModes, nparts = kThreadsC / kModes;
+  // lanes take the modes fastest, then the points: value (c, j) of mode t into its own slot
+  const int t = tid % TM, part = tid / TM;
+  constexpr int nparts = kThreadsC / TM;
   const bool on = u0 + t < a.n_unique;
   const double2* src = a.in3 + (size_t)bz * 3 * NY * Mm + s.pos[t] * a.MZ + s.iz[t];
+  double2* raw = reinterpret_cast<double2*>(xs);
+  unsigned em[3] = {0, 0, 0};
+#pragma unroll
+  for (int c = 0; c < 3; ++c)
+    for (int j = part; j < NY; j += nparts) {
+      const double2 v = on ? __ldg(src + ((size_t)c * NY + j) * Mm) : make_double2(0.0, 0.0);
+      em[c] = max(em[c], top_of(v));
+      raw[j * ST + c * TM + t] = v;
+    }
+#pragma unroll
   for (int c = 0; c < 3; ++c) {
-    unsigned em = 0;
-    for (int j = part; j < NY; j += nparts) em = max(em, on ? top_of(__ldg(src + ((size_t)c * NY + j) * Mm)) : 0u);
-    em = max(em, __shfl_xor_sync(0xffffffffu, em, 8));
-    em = max(em, __shfl_xor_sync(0xffffffffu, em, 16));
-    if ((tid & 31) < kModes) atomicMax(&s.em[c * kModes + t], em);
+#pragma unroll
+    for (int o = TM; o < 32; o <<= 1) em[c] = max(em[c], __shfl_xor_sync(0xffffffffu, em[c], o));
+    if ((tid & 31) < TM) atomicMax(&s.em[c * TM + t], em[c]);
   }
   __syncthreads();
+#pragma unroll
   for (int c = 0; c < 3; ++c) {
-    const int e = (int)(s.em[c * kModes + t] >> 20);
+    const int e = (int)(s.em[c * TM + t] >> 20);
     int sum = 0;
     for (int j = part; j < NY; j += nparts) {
-      if (!on) continue;
-      const double2 v = __ldg(src + ((size_t)c * NY + j) * Mm);
+      const double2 v = raw[j * ST + c * TM + t];
       sum += part_of(v.x, e) + part_of(v.y, e);
     }
-    sum += __shfl_xor_sync(0xffffffffu, sum, 8);
-    sum += __shfl_xor_sync(0xffffffffu, sum, 16);
-    if ((tid & 31) < kModes) atomicAdd(&s.sum[c * kModes + t], sum);
+#pragma unroll
+    for (int o = TM; o < 32; o <<= 1) sum += __shfl_xor_sync(0xffffffffu, sum, o);
+    if ((tid & 31) < TM) atomicAdd(&s.sum[c * TM + t], sum);
   }
   __syncthreads();
-  if (tid < kColsR) {
+  if (tid < 3 * TM) {
     const int e = (int)(s.em[tid] >> 20);
     // values below 2^(e - 1022); the parts of a pair below twice that
     s.sh[tid] = e == 0x7ff ? kNotFinite : exponent_of((u64)s.sum[tid], 0xffff, e);
   }
   __syncthreads();
-  // even and odd parts of the point pairs (j, N - j): f_j + f_{N-j} at j, f_j - f_{N-j} at N - j; the
-  // end points enter with half weight
+  // even and odd parts of the point pairs (j, N - j), in place: f_j + f_{N-j} at j, f_j - f_{N-j} at
+  // N - j; the end points enter with half weight
   for (int idx = part; idx < 3 * NH; idx += nparts) {
-    const int c = idx / NH, j = idx - c * NH, col = c * kModes + t;
+    const int c = idx / NH, j = idx - c * NH, col = c * TM + t;
     const int sh = s.sh[col] == kNotFinite ? -2000 : s.sh[col];
-    i64 px = 0, py = 0, qx = 0, qy = 0;
-    if (on) {
-      const double2 p = __ldg(src + ((size_t)c * NY + j) * Mm), q = __ldg(src + ((size_t)c * NY + N - j) * Mm);
-      px = from_double(p.x, sh);
-      py = from_double(p.y, sh);
-      qx = from_double(q.x, sh);
-      qy = from_double(q.y, sh);
-    }
+    const double2 p = raw[j * ST + col], q = raw[(N - j) * ST + col];
+    const i64 px = from_double(p.x, sh), py = from_double(p.y, sh);
     if (2 * j == N) {
-      xs[j * kStrideR + col] = halves2(px, py);
+      xs[j * ST + col] = halves2(px, py);
     } else {
+      const i64 qx = from_double(q.x, sh), qy = from_double(q.y, sh);
       const int d = j == 0 ? 1 : 0;
-      xs[j * kStrideR + col] = halves2((px + qx) >> d, (py + qy) >> d);
-      xs[(N - j) * kStrideR + col] = halves2((px - qx) >> d, (py - qy) >> d);
+      xs[j * ST + col] = halves2((px + qx) >> d, (py + qy) >> d);
+      xs[(N - j) * ST + col] = halves2((px - qx) >> d, (py - qy) >> d);
     }
   }
   __syncthreads();
@@ -301,13 +323,13 @@ __device__ __forceinline__ void rhs_fx(const RArgs& a, int bx, int by, int bz, i
   for (int r = lo + part; r < hi; r += nparts) {
     const int n = r < ne ? 2 * r : 2 * (r - ne) + 1, odd = n & 1;
     Sum2 S[3];
-    const int4* x = xs + t + (odd ? N * kStrideR : 0);
-    const int st = odd ? -kStrideR : kStrideR, cnt = odd ? NH - 1 : NH;
+    const int4* x = xs + t + (odd ? N * ST : 0);
+    const int st = odd ? -ST : ST, cnt = odd ? NH - 1 : NH;
     const int2* tc = a.tab + n;
     for (int j = 0; j < cnt; ++j) {
       const int2 c = __ldg(tc + (size_t)j * (NY + 1));
 #pragma unroll
-      for (int f = 0; f < 3; ++f) S[f].add(x[f * kModes], c);
+      for (int f = 0; f < 3; ++f) S[f].add(x[f * TM], c);
       x += st;
     }
     const double cn = (n == 0 ? 1.0 : 2.0) / N;  // 2 / (N cbar_n)
@@ -318,7 +340,7 @@ __device__ __forceinline__ void rhs_fx(const RArgs& a, int bx, int by, int bz, i
         const double2 w = __ldg(dsrc + ((size_t)f * Mm + mpos * a.MZ) * NY + n);
         d = make_double2(0.5 * (d.x + w.x), 0.5 * (d.y - w.y));
       }
-      const double2 v = unscale(S[f].x.value(), S[f].y.value(), s.sh[f * kModes + t]);
+      const double2 v = unscale(S[f].x.value(), S[f].y.value(), s.sh[f * TM + t]);
       double2 g = make_double2(fma(cn, v.x, d.x * a.inv_dt), fma(cn, v.y, d.y * a.inv_dt));
       if (pos == 0 && iz == 0) g.y = 0.0;
       a.W[(u0 + t) * a.su + bz * a.sd + (long long)(f * NR + n) * a.sn] = g;
@@ -326,12 +348,13 @@ __device__ __forceinline__ void rhs_fx(const RArgs& a, int bx, int by, int bz, i
   }
 }
 
+template <int TM>
 __global__ void __launch_bounds__(kThreadsC, 3) k_rhs_fx(const __grid_constant__ RArgs a) {
   extern __shared__ __align__(16) unsigned char smem[];
-  __shared__ RShared s;
+  __shared__ RShared<TM> s;
   // directions fastest: with one direction per 16-byte column of W, the blocks that run together
   // fill its sectors
-  rhs_fx(a, blockIdx.y, blockIdx.z, blockIdx.x, reinterpret_cast<int4*>(smem), s);
+  rhs_fx<TM>(a, blockIdx.y, blockIdx.z, blockIdx.x, reinterpret_cast<int4*>(smem), s);
 }
 
 // ------------------------------------------------------------------ groups
@@ -346,7 +369,7 @@ struct GR {
   int gx;
 };
 
-__global__ void __launch_bounds__(kThreadsC, 2) k_yinv_fx_grp(const double* __restrict__ in, const GY* __restrict__ recs,
+__global__ void __launch_bounds__(kThreadsC, 3) k_yinv_fx_grp(const double* __restrict__ in, const GY* __restrict__ recs,
                                                               const int* __restrict__ inst, const int* __restrict__ first,
                                                               const int* __restrict__ active) {
   extern __shared__ __align__(16) unsigned char smem[];
@@ -360,14 +383,14 @@ __global__ void __launch_bounds__(kThreadsC, 2) k_yinv_fx_grp(const double* __re
   }
   __syncthreads();
   const int b = blockIdx.x - first[i];
-  yinv_fx(r.a, b % r.gx, b / r.gx, 0, reinterpret_cast<int4*>(smem), sh);
+  yinv_fx<kModes>(r.a, b % r.gx, b / r.gx, 0, reinterpret_cast<int4*>(smem), sh);
 }
 
 __global__ void __launch_bounds__(kThreadsC, 3) k_rhs_fx_grp(const double* __restrict__ du, const GR* __restrict__ recs,
                                                              const int* __restrict__ inst, const int* __restrict__ first,
                                                              const int* __restrict__ active) {
   extern __shared__ __align__(16) unsigned char smem[];
-  __shared__ RShared s;
+  __shared__ RShared<kModes> s;
   __shared__ GR r;
   const int i = inst[blockIdx.x];
   if (active && !active[i]) return;
@@ -377,11 +400,11 @@ __global__ void __launch_bounds__(kThreadsC, 3) k_rhs_fx_grp(const double* __res
   }
   __syncthreads();
   const int b = blockIdx.x - first[i];
-  rhs_fx(r.a, b % r.gx, b / r.gx, 0, reinterpret_cast<int4*>(smem), s);
+  rhs_fx<kModes>(r.a, b % r.gx, b / r.gx, 0, reinterpret_cast<int4*>(smem), s);
 }
 
-size_t smem_y(const sp_ctx* c) { return (size_t)(c->NY + 1) * kStrideY * 16; }
-size_t smem_r(const sp_ctx* c) { return (size_t)c->NY * kStrideR * 16; }
+size_t smem_y(const sp_ctx* c, int tm) { return (size_t)(c->NY + 1) * stride_y(tm) * 16; }
+size_t smem_r(const sp_ctx* c, int tm) { return (size_t)c->NY * stride_r(tm) * 16; }
 
 // parts of the outputs of a mode tile: one block per tile when the tiles fill the GPU (each part
 // scales the inputs again)
@@ -469,28 +492,44 @@ std::vector<int> cheb_fx_table(int NY) {
   return t;
 }
 
-cudaError_t launch_yinv_fx(const sp_ctx* c, const double* in, void* out6, int n_dir, cudaStream_t st) {
-  const int tiles = (c->Mm + kModes - 1) / kModes;
+template <int TM>
+static cudaError_t launch_y(const sp_ctx* c, const double* in, void* out6, int n_dir, cudaStream_t st) {
+  const int tiles = (c->Mm + TM - 1) / TM;
   const YArgs a = y_args(c, in, out6, parts_for(tiles * n_dir, c->NH, c->sm_count));
-  cudaError_t e = cudaFuncSetAttribute(k_yinv_fx, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_y(c));
+  const size_t sm = smem_y(c, TM);
+  const cudaError_t e = cudaFuncSetAttribute(k_yinv_fx<TM>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
   if (e != cudaSuccess) return e;
-  k_yinv_fx<<<dim3(tiles, (c->NH + a.jchunk - 1) / a.jchunk, n_dir), kThreadsC, smem_y(c), st>>>(a);
+  k_yinv_fx<TM><<<dim3(tiles, (c->NH + a.jchunk - 1) / a.jchunk, n_dir), kThreadsC, sm, st>>>(a);
   return cudaGetLastError();
 }
 
-cudaError_t launch_rhs_fx(const sp_ctx* c, const void* in3, const double* du, void* W, int n_dir, long long su,
-                          long long sd, long long sn, cudaStream_t st) {
-  const int tiles = (c->n_unique + kModes - 1) / kModes;
+template <int TM>
+static cudaError_t launch_r(const sp_ctx* c, const void* in3, const double* du, void* W, int n_dir, long long su,
+                            long long sd, long long sn, cudaStream_t st) {
+  const int tiles = (c->n_unique + TM - 1) / TM;
   RArgs a = r_args(c, in3, du, W, parts_for(tiles * n_dir, c->N - 1, c->sm_count));
   if (sn) {
     a.su = su;
     a.sd = sd;
     a.sn = sn;
   }
-  cudaError_t e = cudaFuncSetAttribute(k_rhs_fx, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_r(c));
+  const size_t sm = smem_r(c, TM);
+  const cudaError_t e = cudaFuncSetAttribute(k_rhs_fx<TM>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
   if (e != cudaSuccess) return e;
-  k_rhs_fx<<<dim3(n_dir, tiles, (c->N - 1 + a.rchunk - 1) / a.rchunk), kThreadsC, smem_r(c), st>>>(a);
+  k_rhs_fx<TM><<<dim3(n_dir, tiles, (c->N - 1 + a.rchunk - 1) / a.rchunk), kThreadsC, sm, st>>>(a);
   return cudaGetLastError();
+}
+
+cudaError_t launch_yinv_fx(const sp_ctx* c, const double* in, void* out6, int n_dir, cudaStream_t st) {
+  if ((c->Mm + kModes - 1) / kModes * n_dir >= c->sm_count) return launch_y<kModes>(c, in, out6, n_dir, st);
+  return launch_y<kModesFew>(c, in, out6, n_dir, st);
+}
+
+cudaError_t launch_rhs_fx(const sp_ctx* c, const void* in3, const double* du, void* W, int n_dir, long long su,
+                          long long sd, long long sn, cudaStream_t st) {
+  if ((c->n_unique + kModes - 1) / kModes * n_dir >= c->sm_count)
+    return launch_r<kModes>(c, in3, du, W, n_dir, su, sd, sn, st);
+  return launch_r<kModesFew>(c, in3, du, W, n_dir, su, sd, sn, st);
 }
 
 cudaError_t grp_build_cheb_fx(GrpPlan* p, sp_ctx* const* mem, int n, const size_t* offs, const int* order) {
@@ -512,8 +551,8 @@ cudaError_t grp_build_cheb_fx(GrpPlan* p, sp_ctx* const* mem, int n, const size_
     rr[m].a = r_args(c, c->ws3, nullptr, c->ws6, parts_for(tr, c->N - 1, c->sm_count));
     rr[m].gx = (c->n_unique + kModes - 1) / kModes;
     br[m] = rr[m].gx * ((c->N - 1 + rr[m].a.rchunk - 1) / rr[m].a.rchunk);
-    sy = std::max(sy, smem_y(c));
-    sr = std::max(sr, smem_r(c));
+    sy = std::max(sy, smem_y(c, kModes));
+    sr = std::max(sr, smem_r(c, kModes));
   }
   cudaError_t e;
   if ((e = cudaFuncSetAttribute(k_yinv_fx_grp, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sy)) != cudaSuccess) return e;

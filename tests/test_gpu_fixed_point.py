@@ -58,3 +58,19 @@ def test_non_finite_input(value):
     ctx.sp_set_base(u)
     ctx.sp_jvp(d, G)
     assert not bool(torch.isfinite(torch.view_as_real(G)).all())
+
+
+# Chebyshev degrees: the smallest, warps' edges, odd halves of N, the largest; one direction and
+# passes of the batched solve's layouts (5: modes fastest, 17: directions fastest)
+@pytest.mark.parametrize("ny", [5, 7, 31, 33, 35, 63, 65, 95, 127, 129])
+@pytest.mark.parametrize("n_dir", [1, 5, 17])
+def test_chebyshev_degrees(ny, n_dir):
+    ctx, orc = make(6, ny, 4, max_batch=1 if n_dir == 1 else 32)
+    u = seeded(orc, 930, 0.1)
+    ctx.sp_set_base(dev(u))
+    base = orc.base(u)
+    ds = np.stack([seeded(orc, 931 + i, 1.0) for i in range(n_dir)])
+    J = ctx.zeros(n_dir)
+    ctx.sp_jvp(dev(ds), J)
+    for i in (0, n_dir - 1):
+        assert rel(host(J)[i], orc.jvp(base, ds[i])) < 1e-12
