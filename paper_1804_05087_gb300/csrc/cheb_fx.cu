@@ -91,19 +91,24 @@ __device__ __forceinline__ double unscale(i64 X, int sh) {
 }
 __device__ __forceinline__ double2 unscale(i64 x, i64 y, int sh) { return make_double2(unscale(x, sh), unscale(y, sh)); }
 
+// Tables of constants, 56-bit halves, each row padded to PH entries (even, zeros) so that two come
+// with one load: values [NH][2][PH] (degrees 2 q + parity at q), derivatives [NH][2][PH], forward
+// [NY][PH] (point j of row n at j). PH covers NH = N / 2 + 1 entries.
+__host__ __device__ constexpr int tab_ph(int NY) { return (NY / 2 + 2) & ~1; }
+
 struct YArgs {
   const double2* in;   // [dir][3][Mm][NY]
   double2* out;        // [dir][6][NY][Mm]
-  const int2* tab;     // [NH][NY + 1]: T_n(y_j), then [NH][NY + 1]: T_n'(y_j) / n^2, 56-bit halves
+  const int2* tab;     // T_n(y_j), T_n'(y_j) / n^2 (ChebTab)
   int Mm, MZ, MX, Kx, NY, NH, jchunk;
   double alpha, beta;
 };
 
-// (bx, by, bz): mode tile, chunk of the half grid, direction. xs: [NY + 1][stride_y]
+// (bx, by, bz): mode tile, chunk of the half grid, direction. xs: [2 PH][stride_y]
 template <int TM>
 __device__ __forceinline__ void yinv_fx(const YArgs& a, int bx, int by, int bz, int4* xs, int (*sh)[TM]) {
   constexpr int ST = stride_y(TM), kWarps = kThreadsC / 32, RW = (3 * TM + kWarps - 1) / kWarps;
-  const int NY = a.NY, N = NY - 1, Mm = a.Mm, m0 = bx * TM;
+  const int NY = a.NY, N = NY - 1, Mm = a.Mm, m0 = bx * TM, PH = tab_ph(NY), rows = 2 * PH;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   // one warp per (component, mode): the rows' loads first, kept in their own slots
   unsigned em[RW];
@@ -113,7 +118,7 @@ __device__ __forceinline__ void yinv_fx(const YArgs& a, int bx, int by, int bz, 
     const int row = warp + r * kWarps, f = row / TM, m = m0 + row - f * TM;
     if (row >= 3 * TM) continue;
     const double2* src = a.in + (((size_t)bz * 3 + f) * Mm + m) * NY;
-    for (int n = lane; n <= NY; n += 32) {  // row NY: zero
+    for (int n = lane; n < rows; n += 32) {  // zeros past the last degree
       double2 v = make_double2(0.0, 0.0);
       if (m < Mm && n < NY) v = __ldg(src + n);
       em[r] = max(em[r], top_of(v));
@@ -148,7 +153,7 @@ __device__ __forceinline__ void yinv_fx(const YArgs& a, int bx, int by, int bz, 
       sh[f][t] = e == 0x7ff ? kNotFinite : e0;
       if (f != 1) sh[g][t] = e == 0x7ff ? kNotFinite : ed;
     }
-    for (int n = lane; n <= NY; n += 32) {
+    for (int n = lane; n < rows; n += 32) {
       int4* x = xs + n * ST;
       const double2 v = reinterpret_cast<const double2*>(x)[row];
       x[row] = halves2(from_double(v.x, e0), from_double(v.y, e0));
@@ -166,14 +171,18 @@ __device__ __forceinline__ void yinv_fx(const YArgs& a, int bx, int by, int bz, 
   for (int i0 = warp * 32; i0 < items; i0 += kThreadsC) {
     const int it = i0 + lane, t = it % TM, odd = it / TM & 1, jh = min(j_lo + it / (2 * TM), j_hi - 1), m = m0 + t;
     Sum2 S[5];
-    const int2* tr = a.tab + (size_t)jh * (NY + 1) + odd;
-    const int2* td = tr + (size_t)a.NH * (NY + 1);
+    const int4* tr = reinterpret_cast<const int4*>(a.tab + (size_t)(2 * jh + odd) * PH);
+    const int4* td = tr + (size_t)a.NH * PH;  // 2 NH rows of PH / 2 loads
     const int4* x = xs + odd * ST + t;
-    for (int n = 0; n < NY; n += 2) {
-      const int2 c = __ldg(tr + n), d = __ldg(td + n);
+    for (int q = 0; q < PH / 2; ++q) {
+      const int4 c = __ldg(tr + q), d = __ldg(td + q);
 #pragma unroll
-      for (int f = 0; f < 5; ++f) S[f].add(x[f * TM], f < 3 ? c : d);
-      x += 2 * ST;
+      for (int f = 0; f < 5; ++f) {
+        const int4 k = f < 3 ? c : d;
+        S[f].add(x[f * TM], make_int2(k.x, k.y));
+        S[f].add(x[2 * ST + f * TM], make_int2(k.z, k.w));
+      }
+      x += 4 * ST;
     }
     i64 vx[5], vy[5];
 #pragma unroll
@@ -240,11 +249,12 @@ struct RShared {
   int pos[TM], iz[TM];
 };
 
-// (bx, by, bz): tile of solved modes, chunk of rows, direction. xs: [NY][stride_r]
+// (bx, by, bz): tile of solved modes, chunk of rows, direction. xs: [2 PH][stride_r]: the values, then
+// the even parts of the point pairs (rows j < PH) and the odd parts (rows PH + j)
 template <int TM>
 __device__ __forceinline__ void rhs_fx(const RArgs& a, int bx, int by, int bz, int4* xs, RShared<TM>& s) {
   constexpr int ST = stride_r(TM);
-  const int NY = a.NY, N = NY - 1, NH = a.NH, NR = N - 1, Mm = a.Mm, u0 = bx * TM;
+  const int NY = a.NY, N = NY - 1, NH = a.NH, NR = N - 1, Mm = a.Mm, u0 = bx * TM, PH = tab_ph(NY);
   const int tid = threadIdx.x;
   if (tid < TM) {
     int pos = 0, iz = 0;
@@ -263,13 +273,15 @@ __device__ __forceinline__ void rhs_fx(const RArgs& a, int bx, int by, int bz, i
   const bool on = u0 + t < a.n_unique;
   const double2* src = a.in3 + (size_t)bz * 3 * NY * Mm + s.pos[t] * a.MZ + s.iz[t];
   double2* raw = reinterpret_cast<double2*>(xs);
+  // the two points of a pair: slots j and PH + j
+  auto slot = [&](int j) { return j < NH ? j : PH + N - j; };
   unsigned em[3] = {0, 0, 0};
 #pragma unroll
   for (int c = 0; c < 3; ++c)
     for (int j = part; j < NY; j += nparts) {
       const double2 v = on ? __ldg(src + ((size_t)c * NY + j) * Mm) : make_double2(0.0, 0.0);
       em[c] = max(em[c], top_of(v));
-      raw[j * ST + c * TM + t] = v;
+      raw[slot(j) * ST + c * TM + t] = v;
     }
 #pragma unroll
   for (int c = 0; c < 3; ++c) {
@@ -283,7 +295,7 @@ __device__ __forceinline__ void rhs_fx(const RArgs& a, int bx, int by, int bz, i
     const int e = (int)(s.em[c * TM + t] >> 20);
     int sum = 0;
     for (int j = part; j < NY; j += nparts) {
-      const double2 v = raw[j * ST + c * TM + t];
+      const double2 v = raw[slot(j) * ST + c * TM + t];
       sum += part_of(v.x, e) + part_of(v.y, e);
     }
 #pragma unroll
@@ -297,20 +309,27 @@ __device__ __forceinline__ void rhs_fx(const RArgs& a, int bx, int by, int bz, i
     s.sh[tid] = e == 0x7ff ? kNotFinite : exponent_of((u64)s.sum[tid], 0xffff, e);
   }
   __syncthreads();
-  // even and odd parts of the point pairs (j, N - j), in place: f_j + f_{N-j} at j, f_j - f_{N-j} at
-  // N - j; the end points enter with half weight
-  for (int idx = part; idx < 3 * NH; idx += nparts) {
-    const int c = idx / NH, j = idx - c * NH, col = c * TM + t;
+  // even and odd parts of the point pairs (j, N - j), in place; the end points enter with half weight
+  for (int idx = part; idx < 3 * PH; idx += nparts) {
+    const int c = idx / PH, j = idx - c * PH, col = c * TM + t;
+    int4* x = xs + j * ST + col;
+    int4* y = x + PH * ST;
+    if (j >= NH) {
+      *x = *y = make_int4(0, 0, 0, 0);
+      continue;
+    }
     const int sh = s.sh[col] == kNotFinite ? -2000 : s.sh[col];
-    const double2 p = raw[j * ST + col], q = raw[(N - j) * ST + col];
+    const double2 p = *reinterpret_cast<const double2*>(x);
     const i64 px = from_double(p.x, sh), py = from_double(p.y, sh);
     if (2 * j == N) {
-      xs[j * ST + col] = halves2(px, py);
+      *x = halves2(px, py);
+      *y = make_int4(0, 0, 0, 0);
     } else {
+      const double2 q = *reinterpret_cast<const double2*>(y);
       const i64 qx = from_double(q.x, sh), qy = from_double(q.y, sh);
       const int d = j == 0 ? 1 : 0;
-      xs[j * ST + col] = halves2((px + qx) >> d, (py + qy) >> d);
-      xs[(N - j) * ST + col] = halves2((px - qx) >> d, (py - qy) >> d);
+      *x = halves2((px + qx) >> d, (py + qy) >> d);
+      *y = halves2((px - qx) >> d, (py - qy) >> d);
     }
   }
   __syncthreads();
@@ -323,14 +342,16 @@ __device__ __forceinline__ void rhs_fx(const RArgs& a, int bx, int by, int bz, i
   for (int r = lo + part; r < hi; r += nparts) {
     const int n = r < ne ? 2 * r : 2 * (r - ne) + 1, odd = n & 1;
     Sum2 S[3];
-    const int4* x = xs + t + (odd ? N * ST : 0);
-    const int st = odd ? -ST : ST, cnt = odd ? NH - 1 : NH;
-    const int2* tc = a.tab + n;
-    for (int j = 0; j < cnt; ++j) {
-      const int2 c = __ldg(tc + (size_t)j * (NY + 1));
+    const int4* x = xs + t + odd * PH * ST;
+    const int4* tc = reinterpret_cast<const int4*>(a.tab + (size_t)n * PH);
+    for (int q = 0; q < PH / 2; ++q) {
+      const int4 c = __ldg(tc + q);
 #pragma unroll
-      for (int f = 0; f < 3; ++f) S[f].add(x[f * TM], c);
-      x += st;
+      for (int f = 0; f < 3; ++f) {
+        S[f].add(x[f * TM], make_int2(c.x, c.y));
+        S[f].add(x[ST + f * TM], make_int2(c.z, c.w));
+      }
+      x += 2 * ST;
     }
     const double cn = (n == 0 ? 1.0 : 2.0) / N;  // 2 / (N cbar_n)
 #pragma unroll
@@ -403,8 +424,8 @@ __global__ void __launch_bounds__(kThreadsC, 3) k_rhs_fx_grp(const double* __res
   rhs_fx<kModes>(r.a, b % r.gx, b / r.gx, 0, reinterpret_cast<int4*>(smem), s);
 }
 
-size_t smem_y(const sp_ctx* c, int tm) { return (size_t)(c->NY + 1) * stride_y(tm) * 16; }
-size_t smem_r(const sp_ctx* c, int tm) { return (size_t)c->NY * stride_r(tm) * 16; }
+size_t smem_y(const sp_ctx* c, int tm) { return (size_t)2 * tab_ph(c->NY) * stride_y(tm) * 16; }
+size_t smem_r(const sp_ctx* c, int tm) { return (size_t)2 * tab_ph(c->NY) * stride_r(tm) * 16; }
 
 // parts of the outputs of a mode tile: one block per tile when the tiles fill the GPU (each part
 // scales the inputs again)
@@ -431,7 +452,7 @@ RArgs r_args(const sp_ctx* c, const void* in3, const void* du, void* W, int part
   a.in3 = static_cast<const double2*>(in3);
   a.du = static_cast<const double2*>(du);
   a.W = static_cast<double2*>(W);
-  a.tab = c->cheb_fx;
+  a.tab = c->cheb_fx + (size_t)4 * c->NH * tab_ph(c->NY);
   a.su = 3LL * (c->N - 1);
   a.sd = a.su * c->n_unique;
   a.sn = 1;
@@ -461,34 +482,30 @@ cudaError_t upload_grp(GrpKernel* k, const std::vector<R>& recs, const std::vect
 }  // namespace
 
 std::vector<int> cheb_fx_table(int NY) {
-  const int N = NY - 1, NH = N / 2 + 1;
-  std::vector<int> t((size_t)2 * NH * (NY + 1) * 2, 0);
-  const long double pi = 3.141592653589793238462643383279502884L;
-  // sin(pi k / N), exact at the multiples of a quarter turn
-  auto sine = [&](long long k) -> long double {
-    k = ((k % (2 * N)) + 2 * N) % (2 * N);
-    if (k % N == 0) return 0.0L;
-    if (2 * k == N) return 1.0L;
-    if (2 * k == 3 * N) return -1.0L;
-    return sinl(pi * k / N);
+  const int N = NY - 1, NH = N / 2 + 1, PH = tab_ph(NY);
+  std::vector<int> t(((size_t)4 * NH + NY) * PH * 2, 0);
+  // cos(pi k / N) for k = 0 .. 2N - 1, exact at the multiples of a quarter turn
+  std::vector<long double> cs(2 * N);
+  for (int k = 0; k < 2 * N; ++k)
+    cs[k] = k == 0 ? 1.0L : k == N ? -1.0L : 2 * k == N || 2 * k == 3 * N ? 0.0L
+                                           : cosl(3.141592653589793238462643383279502884L * k / N);
+  auto cosine = [&](long long k) { return cs[(k % (2 * N) + 2 * N) % (2 * N)]; };
+  // sin(pi k / N) = cos(pi (2k - N) / 2N): from the table where N is even
+  auto sine = [&](long long k) { return cosine(k - N / 2); };
+  auto put = [&](size_t at, long double v) {
+    const long long q = llrintl(v * 72057594037927936.0L);  // 2^56
+    const long long hi = (q + (1 << 27)) >> 28;
+    t[2 * at] = (int)hi;
+    t[2 * at + 1] = (int)(q - hi * (1LL << 28));
   };
   for (int j = 0; j < NH; ++j)
-    for (int n = 0; n < NY; ++n)
-      for (int d = 0; d < 2; ++d) {
-        const long long k = (long long)j * n;
-        long double v;
-        if (d == 0) {
-          const long long r = k % (2 * N);
-          v = r == 0 ? 1.0L : r == N ? -1.0L : 2 * r == N || 2 * r == 3 * N ? 0.0L : cosl(pi * r / N);
-        } else {       // T_n' / n^2 = sin(n t) / (n sin t), t = pi j / N
-          v = n == 0 ? 0.0L : j == 0 ? 1.0L : sine(k) / (n * sine(j));
-        }
-        const long long q = llrintl(v * 72057594037927936.0L);  // 2^56
-        const long long hi = (q + (1 << 27)) >> 28;
-        int* o = t.data() + (((size_t)d * NH + j) * (NY + 1) + n) * 2;
-        o[0] = (int)hi;
-        o[1] = (int)(q - hi * (1LL << 28));
-      }
+    for (int n = 0; n < NY; ++n) {
+      const size_t at = (size_t)(2 * j + (n & 1)) * PH + n / 2;
+      put(at, cosine((long long)j * n));
+      // T_n' / n^2 = sin(n s) / (n sin s), s = pi j / N
+      put((size_t)2 * NH * PH + at, n == 0 ? 0.0L : j == 0 ? 1.0L : sine((long long)j * n) / (n * sine(j)));
+      put((size_t)4 * NH * PH + (size_t)n * PH + j, cosine((long long)j * n));
+    }
   return t;
 }
 

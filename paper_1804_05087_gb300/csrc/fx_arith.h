@@ -24,7 +24,16 @@ __host__ __device__ __forceinline__ cx operator-(cx a, cx b) { return {a.x - b.x
 // v = hi 2^32 + lo with both halves signed
 __host__ __device__ __forceinline__ int half_hi(i64 v) { return (int)((v + 0x80000000ll) >> 32); }
 __host__ __device__ __forceinline__ int half_lo(i64 v) { return (int)v; }
-__host__ __device__ __forceinline__ i64 wide(int a, int b, i64 c) { return (i64)a * b + c; }
+// a b + c in one multiply-add (left to itself the compiler may split it into a product and two adds)
+__host__ __device__ __forceinline__ i64 wide(int a, int b, i64 c) {
+#ifdef __CUDA_ARCH__
+  i64 r;
+  asm("mad.wide.s32 %0, %1, %2, %3;" : "=l"(r) : "r"(a), "r"(b), "l"(c));
+  return r;
+#else
+  return (i64)a * b + c;
+#endif
+}
 
 __host__ __device__ constexpr int const_hi(i64 c) { return (int)((c + 0x80000000ll) >> 32); }
 __host__ __device__ constexpr int const_lo(i64 c) { return (int)(unsigned)(c & 0xffffffffll); }

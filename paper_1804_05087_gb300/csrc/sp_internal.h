@@ -90,7 +90,7 @@ struct sp_ctx {
 
   // device tables
   double *Th = nullptr, *TDh = nullptr, *Cfh = nullptr;
-  int2* cheb_fx = nullptr;       // [2][NH][NY + 1] T_n(y_j) and T_n'(y_j) / n^2 as integers (cheb_fx.cu)
+  int2* cheb_fx = nullptr;       // T_n(y_j) and T_n'(y_j) / n^2 as integers (cheb_fx.cu)
   double* wave = nullptr;        // [n_unique][4] kx, kz, 1/k (solve_one.cu)
   double* rowidx = nullptr;      // [NY + 1] 0, 1, ...
   float* cft_f = nullptr;        // [NH][NY] the transpose of Cfh_f
