@@ -346,16 +346,18 @@ extern "C" sp_status sp_set_base(sp_ctx* c, const double* U, void* stream) {
   return SP_OK;
 }
 
-// pipe: the speed slot of a tangent holds the phase condition <d/dz U, du>
+// pipe: the speed slot of a tangent holds the phase condition <d/dz U, du>; all directions of a pass
+// in two launches (partial sums of every direction fit the reduction scratch)
 static sp_status pipe_phase(sp_ctx* c, const double* du, double* out, int n_dir, cudaStream_t st) {
-  const int nb = (int)std::max<size_t>(1, std::min<size_t>(c->red_blocks, (c->cplx_per_state + 1023) / 1024));
-  for (int d = 0; d < n_dir; ++d) {
-    double* slot = out + (size_t)d * c->state_len + 2 * c->field_cplx;
-    sp_status s = sp_cuda(c, cudaMemsetAsync(slot, 0, 16, st), "phase clear");
+  const int cap = 64 * c->red_blocks;  // partial sums that the scratch holds
+  for (int d0 = 0; d0 < n_dir; d0 += cap) {
+    const int nd = std::min(cap, n_dir - d0);
+    const int blocks = (int)std::min<size_t>(c->red_blocks, (c->cplx_per_state + 1023) / 1024);
+    const int nb = std::max(1, std::min(blocks, cap / nd));
+    const sp_status s = sp_cuda(c, launch_pipe_phase(c, du + (size_t)d0 * c->state_len, out + (size_t)d0 * c->state_len,
+                                                     c->red, nb, nd, st),
+                                "phase");
     if (s != SP_OK) return s;
-    if ((s = sp_cuda(c, launch_dev_dots(c, c->dzU, 1, du + (size_t)d * c->state_len, c->red, nb, slot, nullptr, st),
-                     "phase")) != SP_OK)
-      return s;
   }
   return SP_OK;
 }

@@ -20,7 +20,7 @@ constexpr int kTileP = 8;        // modes per k_pvals block
 constexpr int kThreadsP = 256;
 
 struct PArgs {
-  const double* r;      // [NR]
+  const double* r;      // [NR], then the reciprocals [NR] (a division takes the FP64 pipe tenfold)
   const double* w1;     // [2][NR][9]
   const int* c1;        // [2][NR][9]
   const unsigned char* pb_fac;  // banded factors of the per-mode radial problems (plan_pipe.cpp)
@@ -28,7 +28,7 @@ struct PArgs {
   const double* pb_uh;  // [n_unique][3][NR]
   const double* pb_dinv;
   size_t sstride;       // complex values per state (field + speed)
-  int Mm, MX, MZ, Kx, NR, n_unique;
+  int Mm, MX, MZ, Kx, NR, n_unique, sms;
   double alpha, sym, inv_dt;
 };
 
@@ -57,7 +57,7 @@ __global__ void __launch_bounds__(kThreadsP) k_pvals(const double2* __restrict__
     const int pos = m / a.MZ, iz = m - pos * a.MZ;
     const int kzi = pos <= a.Kx ? pos : pos - a.MX;
     const double k = a.alpha * kzi, mm = a.sym * iz;
-    const double rj = a.r[j], ir = 1.0 / rj;
+    const double ir = __ldg(a.r + NR + j);
     const double2* ur = su + (0 * TM + t) * NR;
     const double2* ut = su + (1 * TM + t) * NR;
     const double2* uz = su + (2 * TM + t) * NR;
@@ -226,77 +226,74 @@ __device__ __forceinline__ bool mbar_wait_bounded(uint32_t bar, uint32_t phase) 
 // and a warp's 8-byte accesses take the minimum two wavefronts.
 __host__ __device__ __forceinline__ int psolve_nrp(int NR) { return NR + ((9 - (NR & 7)) & 7); }
 
-// threads per block: at least two warps for the parallel phases, one per serial solve
-__host__ __device__ constexpr int psolve_threads(int TM, int ND) {
-  return 6 * TM * ND <= 64 ? 64 : (6 * TM * ND + 31) / 32 * 32;
+// Warps of a block. ND = 16: the velocity chains of 16 directions fill three warps, the pressure
+// chains the fourth, so every scheduler's FP64 unit has one full warp of chains; ND = 1: two, for
+// the parallel phases (one of them runs the chains).
+__host__ __device__ constexpr int psolve_warps(int ND) { return ND >= 8 ? 4 : 2; }
+__host__ __device__ constexpr int psolve_threads(int ND) { return 32 * psolve_warps(ND); }
+
+__host__ __device__ __forceinline__ size_t psolve_smem(int ND, int NR, size_t chunk) {
+  return 3 * chunk + (size_t)ND * 4 * psolve_nrp(NR) * 16;
 }
 
-__host__ __device__ __forceinline__ size_t psolve_smem(int TM, int ND, int NR, size_t chunk) {
-  return (size_t)TM * 4 * chunk + (size_t)TM * ND * 4 * psolve_nrp(NR) * 16 + (size_t)2 * NR * 9 * (8 + 4);
+// one bulk copy of a matrix's factors
+__device__ __forceinline__ void copy_factor(unsigned char* dst, const unsigned char* src, uint32_t bytes, uint32_t bar) {
+  asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(smem_addr(dst)),
+               "l"(src), "r"(bytes), "r"(bar)
+               : "memory");
+}
+__device__ __forceinline__ void expect_bytes(uint32_t bar, uint32_t bytes) {
+  asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(bar), "r"(bytes) : "memory");
 }
 
 // in3: [dir][3][NR][Mm] values of N (T); u: the states (step: the state itself, tangent: the
-// directions); U0: the base state (tangent only); out: states. One block: TM modes of ND directions.
-// Per mode the Stokes problem is solved by banded solves (plan_pipe.cpp): the pressure p_f (Poisson,
+// directions); U0: the base state (tangent only); out: states. One block: one mode of ND directions.
+// The Stokes problem of the mode is solved by banded solves (plan_pipe.cpp): the pressure p_f (Poisson,
 // wall value zero), the three velocity components driven by f - grad p_f, and the influence
 // coefficient a of the precomputed u_h from the wall continuity row. The stencil work (div_h f,
 // grad p) runs over all threads, row by row in parallel; only the banded substitutions are serial,
-// one thread per (mode, direction, component, real/imaginary part). The TM modes' factors (4
-// matrices each) come into shared memory by bulk TMA copies while the right-hand sides are formed;
-// their wait has an iteration limit, past which the block writes NaN into its outputs.
-template <typename T, bool TANGENT, int TM, int ND, int NRT>
-__global__ void __launch_bounds__(psolve_threads(TM, ND)) k_psolve(const C2<T>* __restrict__ in3,
-                                                                   const double2* __restrict__ u,
-                                                                   const double2* __restrict__ U0,
-                                                                   double2* __restrict__ out, PArgs a, int n_dir) {
+// one thread per (direction, component, real/imaginary part), packed into as few warps as they fill:
+// a scheduler's FP64 unit takes 64 cycles per instruction whatever the lanes, and a row costs about
+// 20 of them. The factors come into shared memory by bulk TMA copies, u+ and u- beside the pressure's,
+// u~z in the pressure's place once that is solved: three matrices instead of four, so that all modes of a
+// single direction run at once (613 modes at Nr = 64; with two modes per block the last three blocks ran
+// a second wave, 280 us). Every wait has an iteration limit, past which the block writes NaN.
+template <typename T, bool TANGENT, int ND, int NRT>
+__global__ void __launch_bounds__(psolve_threads(ND)) k_psolve(const C2<T>* __restrict__ in3,
+                                                               const double2* __restrict__ u,
+                                                               const double2* __restrict__ U0,
+                                                               double2* __restrict__ out, PArgs a, int n_dir) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   const int NR = NRT > 0 ? NRT : a.NR, Mm = a.Mm, NRP = psolve_nrp(NR), n3 = 3 * NRP;
   const size_t chunk = a.pb_chunk;
-  unsigned char* sfac = smem_raw;                                             // [TM][4][chunk]
-  double2* sf = reinterpret_cast<double2*>(smem_raw + (size_t)TM * 4 * chunk);  // [TM ND][3][NRP]
-  double2* sp = sf + TM * ND * n3;                                            // [TM ND][NRP] pressure
-  double* sw = reinterpret_cast<double*>(sp + TM * ND * NRP);                 // [2][NR][9] D1 weights
-  int* sc = reinterpret_cast<int*>(sw + 2 * NR * 9);                          // [2][NR][9] their columns
-  __shared__ int s_pos[TM], s_iz[TM], s_u[TM];
-  __shared__ double s_alpha[TM * ND][2];
+  unsigned char* sfac = smem_raw;                                         // [3][chunk]: p then u~z, u+, u-
+  double2* sf = reinterpret_cast<double2*>(smem_raw + 3 * chunk);         // [ND][3][NRP]
+  double2* sp = sf + ND * n3;                                             // [ND][NRP] pressure
+  __shared__ double s_alpha[ND][2];
   __shared__ __align__(8) uint64_t s_bar;
-  const int u0 = blockIdx.x * TM, d0 = blockIdx.y * ND;
+  const int mode = blockIdx.x, d0 = blockIdx.y * ND, nd = min(ND, n_dir - d0);
+  const int tid = threadIdx.x, nt = blockDim.x;
   const uint32_t bar = smem_addr(&s_bar);
-  if (threadIdx.x < TM) {
-    const int uu = u0 + threadIdx.x;
-    int pos = 0, iz = 0;
-    if (uu < a.n_unique) unique_mode_d(uu, a.Kx, a.MZ, &pos, &iz);
-    s_pos[threadIdx.x] = pos;
-    s_iz[threadIdx.x] = iz;
-    s_u[threadIdx.x] = uu;
-  }
-  if (threadIdx.x == 0) {
+  int pos, iz;
+  unique_mode_d(mode, a.Kx, a.MZ, &pos, &iz);
+  const bool mean = pos == 0 && iz == 0;
+  const int kzi = pos <= a.Kx ? pos : pos - a.MX;
+  const double k = a.alpha * kzi, mm = a.sym * iz;
+  const int pz = ((int)mm) & 1, pe = pz ^ 1;  // parity of u_z and p, of u_r and u_theta
+  const double* wz = a.w1 + (size_t)pz * NR * 9;
+  const double* we = a.w1 + (size_t)pe * NR * 9;
+  const int* cz = a.c1 + (size_t)pz * NR * 9;
+  const int* ce = a.c1 + (size_t)pe * NR * 9;
+  const unsigned char* fac = a.pb_fac + (size_t)mode * 4 * chunk;
+  if (tid == 0) {
     asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(bar));
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
-  }
-  __syncthreads();
-  const int nvalid = min(TM, a.n_unique - u0);
-  if (threadIdx.x == 0) {
-    // the factors of the block's modes: one bulk copy per (mode, matrix), contiguous in global memory
-    const uint32_t bytes = (uint32_t)(nvalid * 4 * chunk);
-    asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(bar), "r"(bytes) : "memory");
-    for (int q = 0; q < nvalid * 4; ++q)
-      asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(
-                       smem_addr(sfac + (size_t)q * chunk)),
-                   "l"(a.pb_fac + ((size_t)u0 * 4 + q) * chunk), "r"((uint32_t)chunk), "r"(bar)
-                   : "memory");
-  }
-  for (int i = threadIdx.x; i < 2 * NR * 9; i += blockDim.x) {
-    sw[i] = __ldg(a.w1 + i);
-    sc[i] = __ldg(a.c1 + i);
+    expect_bytes(bar, (uint32_t)(3 * chunk));
+    for (int q = 0; q < 3; ++q) copy_factor(sfac + q * chunk, fac + q * chunk, (uint32_t)chunk, bar);
   }
   // f = u/dt + N + speed terms, rotated to (f+, f-, f~z) = (f_r + i f_theta, f_r - i f_theta, -i f_z)
-  for (int idx = threadIdx.x; idx < TM * ND * NR; idx += blockDim.x) {
-    const int tm = idx / NR, j = idx - tm * NR, t = tm / ND, dir = d0 + tm - t * ND;
-    if (s_u[t] >= a.n_unique || dir >= n_dir) continue;
-    const int pos = s_pos[t], iz = s_iz[t];
-    const int kzi = pos <= a.Kx ? pos : pos - a.MX;
-    const double k = a.alpha * kzi;
+  for (int idx = tid; idx < nd * NR; idx += nt) {
+    const int d = idx / NR, j = idx - d * NR, dir = d0 + d;
     const double2* us = u + (size_t)dir * a.sstride;
     const C2<T>* vin = in3 + (size_t)dir * 3 * NR * Mm;
     // speed terms: step c du/dz; tangent c0 du/dz + dc dU0/dz
@@ -314,69 +311,65 @@ __global__ void __launch_bounds__(psolve_threads(TM, ND)) k_psolve(const C2<T>* 
         f[c].x -= dc * k * w.y;
         f[c].y += dc * k * w.x;
       }
-      if (pos == 0 && iz == 0) f[c].y = 0.0;
+      if (mean) f[c].y = 0.0;
     }
-    double2* d = sf + tm * n3;
-    if (pos == 0 && iz == 0) {  // the mean mode keeps (f_r, f_theta, f_z)
-      d[j] = f[0];
-      d[NRP + j] = f[1];
-      d[2 * NRP + j] = f[2];
+    double2* d3 = sf + d * n3;
+    if (mean) {  // the mean mode keeps (f_r, f_theta, f_z)
+      d3[j] = f[0];
+      d3[NRP + j] = f[1];
+      d3[2 * NRP + j] = f[2];
     } else {
-      d[j] = make_double2(f[0].x - f[1].y, f[0].y + f[1].x);
-      d[NRP + j] = make_double2(f[0].x + f[1].y, f[0].y - f[1].x);
-      d[2 * NRP + j] = make_double2(f[2].y, -f[2].x);
+      d3[j] = make_double2(f[0].x - f[1].y, f[0].y + f[1].x);
+      d3[NRP + j] = make_double2(f[0].x + f[1].y, f[0].y - f[1].x);
+      d3[2 * NRP + j] = make_double2(f[2].y, -f[2].x);
     }
+  }
+  __syncthreads();
+  // pressure right-hand side: div_h f on the inner rows, wall value 0 (all rows in parallel)
+  for (int idx = tid; idx < nd * NR; idx += nt) {
+    const int d = idx / NR, i = idx - d * NR;
+    double2 g = make_double2(0.0, 0.0);
+    if (!mean && i > 0) {
+      const double2* fp = sf + d * n3;
+      const double2* fm = fp + NRP;
+      const double2* fz = fp + 2 * NRP;
+      double2 acc = make_double2(0.0, 0.0);
+#pragma unroll
+      for (int q = 0; q < 9; ++q) {
+        const int col = __ldg(ce + i * 9 + q);
+        const double w = __ldg(we + i * 9 + q);
+        acc.x = fma(w, fp[col].x + fm[col].x, acc.x);
+        acc.y = fma(w, fp[col].y + fm[col].y, acc.y);
+      }
+      const double ir = __ldg(a.r + NR + i);
+      g.x = 0.5 * acc.x + 0.5 * ir * ((1.0 + mm) * fp[i].x + (1.0 - mm) * fm[i].x) - k * fz[i].x;
+      g.y = 0.5 * acc.y + 0.5 * ir * ((1.0 + mm) * fp[i].y + (1.0 - mm) * fm[i].y) - k * fz[i].y;
+    }
+    sp[d * NRP + i] = g;
   }
   bool ok = mbar_wait_bounded(bar, 0);
   if (!ok) (void)mbar_wait_bounded(bar, 0);  // copies still in flight: a second limit before going on
   ok = __syncthreads_and(ok) != 0;            // the same decision in every thread of the block
   if (ok) {
-    // pressure right-hand side: div_h f on the inner rows, wall value 0 (all rows in parallel)
-    for (int idx = threadIdx.x; idx < TM * ND * NR; idx += blockDim.x) {
-      const int tm = idx / NR, i = idx - tm * NR, t = tm / ND, dir = d0 + tm - t * ND;
-      const int pos = s_pos[t], iz = s_iz[t];
-      double2 g = make_double2(0.0, 0.0);
-      if (s_u[t] < a.n_unique && dir < n_dir && !(pos == 0 && iz == 0) && i > 0) {
-        const int kzi = pos <= a.Kx ? pos : pos - a.MX;
-        const double k = a.alpha * kzi, mm = a.sym * iz;
-        const int pe = (((int)mm) + 1) & 1;
-        const double2* fp = sf + tm * n3;
-        const double2* fm = fp + NRP;
-        const double2* fz = fp + 2 * NRP;
-        double2 acc = make_double2(0.0, 0.0);
-#pragma unroll
-        for (int q = 0; q < 9; ++q) {
-          const int col = sc[(pe * NR + i) * 9 + q];
-          const double w = sw[(pe * NR + i) * 9 + q];
-          acc.x = fma(w, fp[col].x + fm[col].x, acc.x);
-          acc.y = fma(w, fp[col].y + fm[col].y, acc.y);
-        }
-        const double ir = 1.0 / __ldg(a.r + i);
-        g.x = 0.5 * acc.x + 0.5 * ir * ((1.0 + mm) * fp[i].x + (1.0 - mm) * fm[i].x) - k * fz[i].x;
-        g.y = 0.5 * acc.y + 0.5 * ir * ((1.0 + mm) * fp[i].y + (1.0 - mm) * fm[i].y) - k * fz[i].y;
-      }
-      sp[tm * NRP + i] = g;
-    }
+    // The warp of the chains: one direction fills six lanes of one warp; blocks of one SM alternate
+    // between their warps, so that the schedulers share the chains.
+    constexpr int W = psolve_warps(ND);
+    const int pt = ND >= 8 ? tid - 32 * (W - 1) : tid - 32 * ((blockIdx.x / (2 * a.sms)) & 1);
+    const int vt = ND >= 8 ? tid : pt;
+    // pressure solve: one task per (direction, part)
+    if (pt >= 0 && pt < 2 * nd && !mean)
+      band_solve_d<NRT>(reinterpret_cast<double*>(sp + (pt >> 1) * NRP) + (pt & 1), sfac, NR);
     __syncthreads();
-    // serial tasks go round-robin over the warps (task = lane * warps + warp), so that every warp
-    // of the block, on its own scheduler, runs some of the chains
-    constexpr int kWarps = psolve_threads(TM, ND) / 32;
-    const int task = (threadIdx.x & 31) * kWarps + (threadIdx.x >> 5);
-    // pressure solve: one task per (mode, direction, part)
-    if (task < 2 * TM * ND) {
-      const int tm = task >> 1, part = task & 1, t = tm / ND, dir = d0 + tm - t * ND;
-      if (s_u[t] < a.n_unique && dir < n_dir && !(s_pos[t] == 0 && s_iz[t] == 0))
-        band_solve_d<NRT>(reinterpret_cast<double*>(sp + tm * NRP) + part, sfac + (size_t)t * 4 * chunk, NR);
+    if (tid == 0 && !mean) {  // u~z takes the place of the pressure's factors
+      asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+      expect_bytes(bar, (uint32_t)chunk);
+      copy_factor(sfac, fac + 3 * chunk, (uint32_t)chunk, bar);
     }
-    __syncthreads();
     // velocity right-hand sides f - grad p on the inner rows, no slip at the wall (parallel)
-    for (int idx = threadIdx.x; idx < TM * ND * 3 * NR; idx += blockDim.x) {
-      const int tm = idx / (3 * NR), rem = idx - tm * 3 * NR, comp = rem / NR, i = rem - comp * NR;
-      const int t = tm / ND, dir = d0 + tm - t * ND;
-      if (s_u[t] >= a.n_unique || dir >= n_dir) continue;
-      const int pos = s_pos[t], iz = s_iz[t];
-      double2& x = sf[tm * n3 + comp * NRP + i];
-      if (pos == 0 && iz == 0) {  // mean flow: u_r = 0, wall rows zero
+    for (int idx = tid; idx < nd * 3 * NR; idx += nt) {
+      const int d = idx / (3 * NR), rem = idx - d * 3 * NR, comp = rem / NR, i = rem - comp * NR;
+      double2& x = sf[d * n3 + comp * NRP + i];
+      if (mean) {  // mean flow: u_r = 0, wall rows zero
         if (comp == 0 || i == 0) x = make_double2(0.0, 0.0);
         continue;
       }
@@ -384,90 +377,81 @@ __global__ void __launch_bounds__(psolve_threads(TM, ND)) k_psolve(const C2<T>* 
         x = make_double2(0.0, 0.0);
         continue;
       }
-      const int kzi = pos <= a.Kx ? pos : pos - a.MX;
-      const double k = a.alpha * kzi, mm = a.sym * iz;
-      const double2* p = sp + tm * NRP;
+      const double2* p = sp + d * NRP;
       double2 gp;
       if (comp == 2) {
         gp = make_double2(k * p[i].x, k * p[i].y);
       } else {
-        const int pz = ((int)mm) & 1;
         double2 d1 = make_double2(0.0, 0.0);
 #pragma unroll
         for (int q = 0; q < 9; ++q) {
-          const int col = sc[(pz * NR + i) * 9 + q];
-          const double w = sw[(pz * NR + i) * 9 + q];
+          const int col = __ldg(cz + i * 9 + q);
+          const double w = __ldg(wz + i * 9 + q);
           d1.x = fma(w, p[col].x, d1.x);
           d1.y = fma(w, p[col].y, d1.y);
         }
-        const double mr = mm / __ldg(a.r + i);
+        const double mr = mm * __ldg(a.r + NR + i);
         gp = comp == 0 ? make_double2(d1.x - mr * p[i].x, d1.y - mr * p[i].y)
                        : make_double2(d1.x + mr * p[i].x, d1.y + mr * p[i].y);
       }
       x.x -= gp.x;
       x.y -= gp.y;
     }
-    __syncthreads();
-    // velocity solves: one task per (mode, direction, component, part)
-    if (task < 6 * TM * ND) {
-      const int tm = task / 6, rem = task - 6 * tm, comp = rem >> 1, part = rem & 1;
-      const int t = tm / ND, dir = d0 + tm - t * ND;
-      const bool mean = s_pos[t] == 0 && s_iz[t] == 0;
-      if (s_u[t] < a.n_unique && dir < n_dir && !(mean && comp == 0)) {
-        const int slot = mean ? comp : comp + 1;
-        band_solve_d<NRT>(reinterpret_cast<double*>(sf + tm * n3 + comp * NRP) + part,
-                          sfac + ((size_t)t * 4 + slot) * chunk, NR);
-      }
+    if (!mean) {
+      ok = mbar_wait_bounded(bar, 1);
+      if (!ok) (void)mbar_wait_bounded(bar, 1);
+    }
+    ok = __syncthreads_and(ok) != 0;
+    // velocity solves: one task per (direction, component, part)
+    if (ok && vt >= 0 && vt < 6 * nd) {
+      const int d = vt / 6, rem = vt - 6 * d, comp = rem >> 1, part = rem & 1;
+      // buffers: u~z 0, u+ 1, u- 2; mean mode: u_theta 1, u_z 2
+      const int buf = mean ? comp : (comp == 2 ? 0 : comp + 1);
+      if (!(mean && comp == 0))
+        band_solve_d<NRT>(reinterpret_cast<double*>(sf + d * n3 + comp * NRP) + part, sfac + buf * chunk, NR);
     }
     __syncthreads();
     // influence coefficient from the wall continuity row: 0.5 D1 (u+ + u-) at r = 1 vanishes
-    if (threadIdx.x < 2 * TM * ND) {
-      const int tm = threadIdx.x >> 1, part = threadIdx.x & 1, t = tm / ND;
-      const int uu = s_u[t], pos = s_pos[t], iz = s_iz[t];
+    if (tid < 2 * nd) {
+      const int d = tid >> 1, part = tid & 1;
       double al = 0.0;
-      if (uu < a.n_unique && !(pos == 0 && iz == 0)) {
-        const int pe = (((int)(a.sym * iz)) + 1) & 1;
-        const double* up = reinterpret_cast<const double*>(sf + tm * n3) + part;
+      if (!mean) {
+        const double* up = reinterpret_cast<const double*>(sf + d * n3) + part;
         const double* um = up + 2 * NRP;
         double s = 0.0;
 #pragma unroll
         for (int q = 0; q < 9; ++q) {
-          const int col = sc[pe * NR * 9 + q];
-          s += sw[pe * NR * 9 + q] * (up[2 * col] + um[2 * col]);
+          const int col = __ldg(ce + q);
+          s += __ldg(we + q) * (up[2 * col] + um[2 * col]);
         }
-        al = -0.5 * s * __ldg(a.pb_dinv + uu);
+        al = -0.5 * s * __ldg(a.pb_dinv + mode);
       }
-      s_alpha[tm][part] = al;
-    }
-    __syncthreads();
-    for (int idx = threadIdx.x; idx < TM * ND * 3 * NR; idx += blockDim.x) {
-      const int tm = idx / (3 * NR), rem = idx - tm * 3 * NR, comp = rem / NR, j = rem - comp * NR;
-      const int t = tm / ND, uu = s_u[t];
-      if (uu >= a.n_unique || (s_pos[t] == 0 && s_iz[t] == 0)) continue;
-      const double h = __ldg(a.pb_uh + (size_t)uu * 3 * NR + rem);
-      double2& x = sf[tm * n3 + comp * NRP + j];
-      x.x += s_alpha[tm][0] * h;
-      x.y += s_alpha[tm][1] * h;
+      s_alpha[d][part] = al;
     }
     __syncthreads();
   }
   const double nan = __longlong_as_double(0x7ff8000000000000LL);
-  for (int idx = threadIdx.x; idx < TM * ND * NR; idx += blockDim.x) {
-    const int tm = idx / NR, j = idx - tm * NR, t = tm / ND, dir = d0 + tm - t * ND;
-    if (s_u[t] >= a.n_unique || dir >= n_dir) continue;
-    const int pos = s_pos[t], iz = s_iz[t];
+  for (int idx = tid; idx < nd * NR; idx += nt) {
+    const int d = idx / NR, j = idx - d * NR, dir = d0 + d;
     const double2* us = u + (size_t)dir * a.sstride;
     double2* dst = out + (size_t)dir * a.sstride;
-    const double2* x = sf + tm * n3;
+    const double2* x = sf + d * n3;
     double2 vr, vt, vz;
     if (!ok) {
       vr = vt = vz = make_double2(nan, nan);
-    } else if (pos == 0 && iz == 0) {
+    } else if (mean) {
       vr = make_double2(0.0, 0.0);
       vt = make_double2(x[NRP + j].x, 0.0);
       vz = make_double2(x[2 * NRP + j].x, 0.0);
     } else {
-      const double2 up = x[j], um = x[NRP + j], uzt = x[2 * NRP + j];
+      const double* h = a.pb_uh + (size_t)mode * 3 * NR + j;
+      const double ax = s_alpha[d][0], ay = s_alpha[d][1];
+      auto with = [&](int comp) {
+        const double w = __ldg(h + comp * NR);
+        const double2 v = x[comp * NRP + j];
+        return make_double2(v.x + ax * w, v.y + ay * w);
+      };
+      const double2 up = with(0), um = with(1), uzt = with(2);
       vr = make_double2(0.5 * (up.x + um.x), 0.5 * (up.y + um.y));
       vt = make_double2(0.5 * (up.y - um.y), -0.5 * (up.x - um.x));  // (u+ - u-)/(2i)
       vz = make_double2(-uzt.y, uzt.x);                                // i u~z
@@ -475,17 +459,16 @@ __global__ void __launch_bounds__(psolve_threads(TM, ND)) k_psolve(const C2<T>* 
     const double2 res[3] = {vr, vt, vz};
 #pragma unroll
     for (int c = 0; c < 3; ++c) {
-      const double2 d = sym_load(us, c, pos, iz, j, a);
-      double2 g = make_double2(res[c].x - d.x, res[c].y - d.y);
-      if (pos == 0 && iz == 0) g.y = 0.0;
+      const double2 d2 = sym_load(us, c, pos, iz, j, a);
+      double2 g = make_double2(res[c].x - d2.x, res[c].y - d2.y);
+      if (mean) g.y = 0.0;
       dst[((size_t)c * Mm + pos * a.MZ + iz) * NR + j] = g;
       if (iz == 0 && pos != 0) dst[((size_t)c * Mm + (a.MX - pos) * a.MZ) * NR + j] = make_double2(g.x, -g.y);
     }
   }
   // the speed slot of a step is zero (no equation of its own); the tangent's
   // phase condition is written afterwards
-  if (blockIdx.x == 0 && threadIdx.x < ND && d0 + (int)threadIdx.x < n_dir)
-    out[(size_t)(d0 + threadIdx.x) * a.sstride + a.sstride - 1] = make_double2(0.0, 0.0);
+  if (blockIdx.x == 0 && tid < nd) out[(size_t)(d0 + tid) * a.sstride + a.sstride - 1] = make_double2(0.0, 0.0);
 }
 
 // dzU = i k P(U) (P: Hermitian projection), speed slot zero
@@ -502,6 +485,38 @@ __global__ void k_pipe_dz(const double2* U, double2* dzU, PArgs a) {
     dzU[e] = make_double2(-k * v.y, k * v.x);
   }
   if (blockIdx.x == 0 && threadIdx.x == 0) dzU[n] = make_double2(0.0, 0.0);
+}
+
+// partial sums of <dzU, du> (the speed slots included, weights w(m')), grid (nb, directions)
+__global__ void __launch_bounds__(256) k_phase_partials(const double2* __restrict__ dz, const double2* __restrict__ du,
+                                                        double* __restrict__ partials, PArgs a) {
+  const double2* d = du + (size_t)blockIdx.y * a.sstride;
+  double acc = 0.0;
+  for (unsigned e = blockIdx.x * 256 + threadIdx.x; e < a.sstride; e += gridDim.x * 256) {
+    const unsigned iz = (e / (unsigned)a.NR) % (unsigned)a.MZ;
+    const double2 p = __ldg(dz + e), q = __ldg(d + e);
+    const double t = fma(p.x, q.x, p.y * q.y);
+    acc += iz == 0 ? t : 2.0 * t;
+  }
+  __shared__ double red[8];
+  for (int o = 16; o > 0; o >>= 1) acc += __shfl_down_sync(0xffffffffu, acc, o);
+  if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = acc;
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    for (int w = 1; w < 8; ++w) acc += red[w];
+    partials[(size_t)blockIdx.y * gridDim.x + blockIdx.x] = acc;
+  }
+}
+
+// one warp per direction
+__global__ void __launch_bounds__(128) k_phase_sum(const double* __restrict__ partials, int nb, double2* __restrict__ out,
+                                                   size_t sstride, int n_dir) {
+  const int d = blockIdx.x * 4 + (threadIdx.x >> 5), lane = threadIdx.x & 31;
+  if (d >= n_dir) return;
+  double acc = 0.0;
+  for (int b = lane; b < nb; b += 32) acc += partials[(size_t)d * nb + b];
+  for (int o = 16; o > 0; o >>= 1) acc += __shfl_down_sync(0xffffffffu, acc, o);
+  if (lane == 0) out[(size_t)(d + 1) * sstride - 1] = make_double2(acc, 0.0);
 }
 
 // seeded pipe state: A = streak part, B = poloidal part (both unscaled)
@@ -572,7 +587,7 @@ PArgs pargs(const sp_ctx* c) {
   a.pb_uh = c->pb_uh;
   a.pb_dinv = c->pb_dinv;
   a.sstride = c->cplx_per_state;
-  a.Mm = c->Mm; a.MX = c->MX; a.MZ = c->MZ; a.Kx = c->Kx; a.NR = c->NY; a.n_unique = c->n_unique;
+  a.Mm = c->Mm; a.MX = c->MX; a.MZ = c->MZ; a.Kx = c->Kx; a.NR = c->NY; a.n_unique = c->n_unique; a.sms = c->sm_count;
   a.alpha = c->alpha; a.sym = c->beta; a.inv_dt = 1.0 / c->dt;
   return a;
 }
@@ -595,34 +610,41 @@ cudaError_t launch_pvals(const sp_ctx* c, bool fp32, const double* in, void* out
   return cudaGetLastError();
 }
 
-template <typename T, bool TG, int TM, int ND, int NRT>
-static cudaError_t psolve_t(const sp_ctx* c, const PArgs& a, const void* in3, const double2* uu, const double2* U0,
-                            double2* o, int n_dir, cudaStream_t st) {
-  const size_t sm = psolve_smem(TM, ND, c->NY, c->pb_chunk);
-  auto kern = k_psolve<T, TG, TM, ND, NRT>;
-  cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
-  if (e != cudaSuccess) return e;
-  dim3 grid((c->n_unique + TM - 1) / TM, (n_dir + ND - 1) / ND);
-  kern<<<grid, psolve_threads(TM, ND), sm, st>>>(reinterpret_cast<const C2<T>*>(in3), uu, U0, o, a, n_dir);
+cudaError_t launch_pipe_phase(const sp_ctx* c, const double* du, double* out, double* partials, int nb, int n_dir,
+                              cudaStream_t st) {
+  const PArgs a = pargs(c);
+  k_phase_partials<<<dim3(nb, n_dir), 256, 0, st>>>(reinterpret_cast<const double2*>(c->dzU),
+                                                    reinterpret_cast<const double2*>(du), partials, a);
+  k_phase_sum<<<(n_dir + 3) / 4, 128, 0, st>>>(partials, nb, reinterpret_cast<double2*>(out), a.sstride, n_dir);
   return cudaGetLastError();
 }
 
-// The radial size of the pipe workload (Nr = 64) has register-resident solves; other sizes use
-// the shared-memory solve. The widest block whose staged factors and vectors fit is taken.
+template <typename T, bool TG, int ND, int NRT>
+static cudaError_t psolve_t(const sp_ctx* c, const PArgs& a, const void* in3, const double2* uu, const double2* U0,
+                            double2* o, int n_dir, cudaStream_t st) {
+  const size_t sm = psolve_smem(ND, c->NY, c->pb_chunk);
+  auto kern = k_psolve<T, TG, ND, NRT>;
+  cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+  if (e != cudaSuccess) return e;
+  kern<<<dim3(c->n_unique, (n_dir + ND - 1) / ND), psolve_threads(ND), sm, st>>>(reinterpret_cast<const C2<T>*>(in3), uu, U0, o,
+                                                                                a, n_dir);
+  return cudaGetLastError();
+}
+
+// directions per block: sixteen (full warps of chains) where two such blocks share an SM, else eight where
+// they fit, else one
 template <typename T, bool TG>
-static cudaError_t psolve_tm(const sp_ctx* c, const PArgs& a, const void* in3, const double2* uu, const double2* U0,
+static cudaError_t psolve_nd(const sp_ctx* c, const PArgs& a, const void* in3, const double2* uu, const double2* U0,
                              double2* o, int n_dir, cudaStream_t st) {
   constexpr size_t kMax = 225 * 1024;
-  auto fits = [&](int tm, int nd) { return psolve_smem(tm, nd, c->NY, c->pb_chunk) <= kMax; };
-  const bool wide = n_dir >= 8 && fits(2, 8);
-  if (c->NY == 64) {
-    return wide ? psolve_t<T, TG, 2, 8, 64>(c, a, in3, uu, U0, o, n_dir, st)
-                : psolve_t<T, TG, 2, 1, 64>(c, a, in3, uu, U0, o, n_dir, st);
-  }
-  if (wide) return psolve_t<T, TG, 2, 8, 0>(c, a, in3, uu, U0, o, n_dir, st);
-  if (fits(2, 1)) return psolve_t<T, TG, 2, 1, 0>(c, a, in3, uu, U0, o, n_dir, st);
-  if (fits(1, 1)) return psolve_t<T, TG, 1, 1, 0>(c, a, in3, uu, U0, o, n_dir, st);
-  return cudaErrorInvalidValue;
+  // the grids that a block with one mode's four matrices holds (radial counts up to 235)
+  if (4 * c->pb_chunk + (size_t)4 * psolve_nrp(c->NY) * 16 + (size_t)2 * c->NY * 9 * 12 > kMax) return cudaErrorInvalidValue;
+  const bool r64 = c->NY == 64;
+  if (n_dir >= 12 && psolve_smem(16, c->NY, c->pb_chunk) <= kMax / 2)
+    return r64 ? psolve_t<T, TG, 16, 64>(c, a, in3, uu, U0, o, n_dir, st) : psolve_t<T, TG, 16, 0>(c, a, in3, uu, U0, o, n_dir, st);
+  if (n_dir >= 4 && psolve_smem(8, c->NY, c->pb_chunk) <= kMax)
+    return r64 ? psolve_t<T, TG, 8, 64>(c, a, in3, uu, U0, o, n_dir, st) : psolve_t<T, TG, 8, 0>(c, a, in3, uu, U0, o, n_dir, st);
+  return r64 ? psolve_t<T, TG, 1, 64>(c, a, in3, uu, U0, o, n_dir, st) : psolve_t<T, TG, 1, 0>(c, a, in3, uu, U0, o, n_dir, st);
 }
 
 cudaError_t launch_psolve(const sp_ctx* c, bool fp32, bool tangent, const void* in3, const double* u, double* out,
@@ -631,10 +653,10 @@ cudaError_t launch_psolve(const sp_ctx* c, bool fp32, bool tangent, const void* 
   const double2* uu = reinterpret_cast<const double2*>(u);
   const double2* U0 = reinterpret_cast<const double2*>(c->U0);
   double2* o = reinterpret_cast<double2*>(out);
-  if (fp32) return tangent ? psolve_tm<float, true>(c, a, in3, uu, U0, o, n_dir, st)
-                           : psolve_tm<float, false>(c, a, in3, uu, U0, o, n_dir, st);
-  return tangent ? psolve_tm<double, true>(c, a, in3, uu, U0, o, n_dir, st)
-                 : psolve_tm<double, false>(c, a, in3, uu, U0, o, n_dir, st);
+  if (fp32) return tangent ? psolve_nd<float, true>(c, a, in3, uu, U0, o, n_dir, st)
+                           : psolve_nd<float, false>(c, a, in3, uu, U0, o, n_dir, st);
+  return tangent ? psolve_nd<double, true>(c, a, in3, uu, U0, o, n_dir, st)
+                 : psolve_nd<double, false>(c, a, in3, uu, U0, o, n_dir, st);
 }
 
 cudaError_t launch_pipe_dz(const sp_ctx* c, const double* U, double* dzU, cudaStream_t st) {

@@ -272,13 +272,16 @@ sp_status sp_build_pipe_plan(sp_ctx* c) {
     lam6[(size_t)j * 6 + 2] = 1.0 - r[j] * r[j];
     lam6[(size_t)j * 6 + 4] = 2.0 * r[j];
   }
+  // the radial points, then their reciprocals
+  std::vector<double> rr(r);
+  for (int j = 0; j < nr; ++j) rr.push_back(1.0 / r[j]);
   auto up = [&](void** dst, const void* src, size_t bytes) -> bool {
     if (cudaMalloc(dst, bytes) != cudaSuccess) return false;
     return cudaMemcpy(*dst, src, bytes, cudaMemcpyHostToDevice) == cudaSuccess;
   };
   const bool ok = up((void**)&c->pb_fac, fac.data(), fac.size()) &&
                   up((void**)&c->pb_uh, uh_all.data(), uh_all.size() * 8) &&
-                  up((void**)&c->pb_dinv, dinv_all.data(), dinv_all.size() * 8) && up((void**)&c->yv, r.data(), r.size() * 8) &&
+                  up((void**)&c->pb_dinv, dinv_all.data(), dinv_all.size() * 8) && up((void**)&c->yv, rr.data(), rr.size() * 8) &&
                   up((void**)&c->lam6, lam6.data(), lam6.size() * 8) &&
                   up((void**)&c->fd_w1, w1.data(), w1.size() * 8) && up((void**)&c->fd_c1, c1.data(), c1.size() * 4);
   if (!ok) return sp_fail(c, SP_ENOMEM, "device allocation of the pipe plan failed");

@@ -206,6 +206,9 @@ void sp_unique_mode(const sp_ctx* c, int u, int* pos, int* iz);
 cudaError_t launch_pvals(const sp_ctx* c, bool fp32, const double* in, void* out6, int n_dir, cudaStream_t st);
 cudaError_t launch_psolve(const sp_ctx* c, bool fp32, bool tangent, const void* in3, const double* u,
                           double* out, int n_dir, cudaStream_t st);
+// speed slots of out: <dzU, du> of n_dir directions; partials: n_dir x nb doubles
+cudaError_t launch_pipe_phase(const sp_ctx* c, const double* du, double* out, double* partials, int nb, int n_dir,
+                              cudaStream_t st);
 cudaError_t launch_pipe_dz(const sp_ctx* c, const double* U, double* dzU, cudaStream_t st);
 cudaError_t launch_pipe_seed(const sp_ctx* c, const double* streak, const double* pol, int npoly, double* A,
                              double* B, cudaStream_t st);
