@@ -232,7 +232,8 @@ __device__ __forceinline__ i64 shift_down(i64 v, int k) { return (v + ((1ll << k
 struct Div {
   unsigned d, m;
 };
-__host__ __device__ __forceinline__ Div div_of(unsigned d) { return {d, 0xffffffffu / d + 1}; }  // d >= 2
-__device__ __forceinline__ int quot(int n, Div v) { return (int)__umulhi((unsigned)n, v.m); }
+__host__ __device__ __forceinline__ Div div_of(unsigned d) { return {d, 0xffffffffu / d + 1}; }
+__device__ __forceinline__ int quot(int n, Div v) { return (int)__umulhi((unsigned)n, v.m); }  // d >= 2
+__device__ __forceinline__ int quot1(int n, Div v) { return v.d == 1 ? n : quot(n, v); }
 
 }  // namespace fx

@@ -22,6 +22,7 @@
 #include <cstdio>
 
 #include "dev_util.h"
+#include "fx_arith.h"
 #include "sp_internal.h"
 
 namespace {
@@ -42,69 +43,73 @@ constexpr int kTileSolve = 4;   // modes per k_solve block
 // input through `load(b, e)` (element e of transform b), the last stage hands
 // its outputs to `store(b, e, v)`; the stages in between ping-pong between s0
 // and s1 (layout [element][batch]). Ends with __syncthreads().
-template <typename T, class LoadF, class StoreF>
-__device__ void fft_batch(const FftPlan& pl, int nb, const C2<T>* __restrict__ tw, T sgn,
-                          C2<T>* s0, C2<T>* s1, LoadF load, StoreF store) {
-  const int n = pl.n;
+// One stage of radix P on nb transforms: butterfly bf = t0 Rp + bp of transform b.
+template <typename T, int P, class LoadF, class StoreF>
+__device__ __forceinline__ void fft_stage(int n, int L, int Rp, fx::Div dRp, int nb, fx::Div dnb, bool first, bool last,
+                                          const C2<T>* __restrict__ tw, T sgn, const C2<T>* src, C2<T>* dst, LoadF& load,
+                                          StoreF& store) {
   const T h3 = (T)0.86602540378443864676;  // sqrt(3)/2
+  const int R = Rp * P, nbf = n / P;
+  for (int idx = threadIdx.x; idx < nb * nbf; idx += blockDim.x) {
+    const int bf = fx::quot1(idx, dnb), b = idx - bf * nb;
+    const int t0 = fx::quot1(bf, dRp), bp = bf - t0 * Rp;
+    C2<T> x[P];
+#pragma unroll
+    for (int c = 0; c < P; ++c) {
+      const int e = t0 * R + bp + Rp * c;
+      x[c] = first ? load(b, e) : src[e * nb + b];
+    }
+    if (t0 != 0) {
+#pragma unroll
+      for (int c = 1; c < P; ++c) {
+        C2<T> w = tw[c * t0 * Rp];  // c t0 Rp < P L Rp = n
+        if (sgn > (T)0) w.y = -w.y;
+        x[c] = x[c] * w;
+      }
+    }
+    C2<T> y[P];
+    if constexpr (P == 2) {
+      y[0] = x[0] + x[1];
+      y[1] = x[0] - x[1];
+    } else if constexpr (P == 3) {
+      C2<T> t1 = x[1] + x[2];
+      C2<T> t2 = mul_is(x[1] - x[2], sgn * h3);
+      C2<T> m = x[0] - scl(t1, (T)0.5);
+      y[0] = x[0] + t1;
+      y[1] = m + t2;
+      y[2] = m - t2;
+    } else {
+      C2<T> a = x[0] + x[2], bb = x[0] - x[2];
+      C2<T> c = x[1] + x[3], d = mul_is(x[1] - x[3], sgn);
+      y[0] = a + c;
+      y[2] = a - c;
+      y[1] = bb + d;
+      y[3] = bb - d;
+    }
+#pragma unroll
+    for (int d = 0; d < P; ++d) {
+      const int e = (t0 + L * d) * Rp + bp;
+      if (last) store(b, e, y[d]);
+      else dst[e * nb + b] = y[d];
+    }
+  }
+}
+
+template <typename T, class LoadF, class StoreF>
+__device__ __forceinline__ void fft_batch(const FftPlan& pl, int nb, const C2<T>* __restrict__ tw, T sgn, C2<T>* s0,
+                                          C2<T>* s1, LoadF load, StoreF store) {
+  const int n = pl.n;
+  const fx::Div dnb = fx::div_of(nb);
   int L = 1;
   for (int s = 0; s < pl.nst; ++s) {
-    const int p = pl.radix[s];
-    const int R = n / L, Rp = R / p;
-    const int nbf = n / p;
+    const int p = pl.radix[s], Rp = pl.rp[s];
+    const fx::Div dRp = {(unsigned)Rp, pl.mrp[s]};
     const C2<T>* src = (s & 1) ? s0 : s1;
     C2<T>* dst = (s & 1) ? s1 : s0;
     const bool first = (s == 0), last = (s == pl.nst - 1);
-    for (int idx = threadIdx.x; idx < nb * nbf; idx += blockDim.x) {
-      const int b = idx % nb;
-      const int bf = idx / nb;
-      const int t0 = bf / Rp, bp = bf - t0 * Rp;
-      C2<T> x[4];
-#pragma unroll
-      for (int c = 0; c < 4; ++c) {
-        if (c < p) {
-          const int e = t0 * R + bp + Rp * c;
-          x[c] = first ? load(b, e) : src[e * nb + b];
-        }
-      }
-      if (t0 != 0) {
-#pragma unroll
-        for (int c = 1; c < 4; ++c) {
-          if (c < p) {
-            C2<T> w = tw[(c * t0 * Rp) % n];
-            if (sgn > (T)0) w.y = -w.y;
-            x[c] = x[c] * w;
-          }
-        }
-      }
-      C2<T> y[4];
-      if (p == 2) {
-        y[0] = x[0] + x[1];
-        y[1] = x[0] - x[1];
-      } else if (p == 3) {
-        C2<T> t1 = x[1] + x[2];
-        C2<T> t2 = mul_is(x[1] - x[2], sgn * h3);
-        C2<T> m = x[0] - scl(t1, (T)0.5);
-        y[0] = x[0] + t1;
-        y[1] = m + t2;
-        y[2] = m - t2;
-      } else {
-        C2<T> a = x[0] + x[2], bb = x[0] - x[2];
-        C2<T> c = x[1] + x[3], d = mul_is(x[1] - x[3], sgn);
-        y[0] = a + c;
-        y[2] = a - c;
-        y[1] = bb + d;
-        y[3] = bb - d;
-      }
-#pragma unroll
-      for (int d = 0; d < 4; ++d) {
-        if (d < p) {
-          const int e = (t0 + L * d) * Rp + bp;
-          if (last) store(b, e, y[d]);
-          else dst[e * nb + b] = y[d];
-        }
-      }
-    }
+    if (p == 4) fft_stage<T, 4>(n, L, Rp, dRp, nb, dnb, first, last, tw, sgn, src, dst, load, store);
+    else if (p == 3) fft_stage<T, 3>(n, L, Rp, dRp, nb, dnb, first, last, tw, sgn, src, dst, load, store);
+    else fft_stage<T, 2>(n, L, Rp, dRp, nb, dnb, first, last, tw, sgn, src, dst, load, store);
     __syncthreads();
     L *= p;
   }
@@ -240,6 +245,7 @@ struct XzArgs {
   int nx, nz, NY, Mm, MX, MZ, Kx, Kz;
   int rp, cx;         // row pairs per z chunk, columns per x chunk
   int FS, RS;         // field and row strides of the plane buffer G
+  fx::Div dMZ, dnz;   // divisions by MZ and nz
   C2<T>* Gg;          // if non-null, the plane buffers live here, [dir][NY][nx * RS] (large grids)
 };
 
@@ -279,7 +285,7 @@ __device__ __forceinline__ void xz_body(const XzArgs<T>& a, int bx, int by) {
       const int nb = min(a.cx, ncol - c0);
       auto load = [&](int b, int e) -> C2<T> {
         const int col = c0 + b;
-        const int f = col / MZ, iz = col - f * MZ;
+        const int f = fx::quot1(col, a.dMZ), iz = col - f * MZ;
         int pos;
         if (e <= Kx) pos = e;
         else if (e >= nx - Kx) pos = e - nx + a.MX;
@@ -290,7 +296,7 @@ __device__ __forceinline__ void xz_body(const XzArgs<T>& a, int bx, int by) {
       };
       auto store = [&](int b, int e, C2<T> v) {
         const int col = c0 + b;
-        const int f = col / MZ, iz = col - f * MZ;
+        const int f = fx::quot1(col, a.dMZ), iz = col - f * MZ;
         G[e * RS + f * FS + iz] = v;
       };
       fft_batch<T>(a.px, nb, stwx, (T)1, S, S + (size_t)a.cx * nx, load, store);
@@ -334,7 +340,7 @@ __device__ __forceinline__ void xz_body(const XzArgs<T>& a, int bx, int by) {
     {
       const int nbi = NIN * nq, nbo = NOUT * nq;
       for (int it = threadIdx.x; it < nq * nz; it += blockDim.x) {
-        const int qq = it / nz, k = it - qq * nz;
+        const int qq = fx::quot1(it, a.dnz), k = it - qq * nz;
         const int x0 = 2 * (q0 + qq);
         C2<T> fv[NIN];
 #pragma unroll
@@ -390,12 +396,13 @@ __device__ __forceinline__ void xz_body(const XzArgs<T>& a, int bx, int by) {
     }
     if (MODE != XZ_BASE) {
       const int nb = NOUT * nq;
+      const fx::Div dnb = fx::div_of(nb);
       auto load = [&](int b, int e) -> C2<T> { return R[e * nb + b]; };
       auto store = [&](int b, int e, C2<T> v) { Q[e * nb + b] = v; };
       fft_batch<T>(a.pz, nb, stwz, (T)-1, P0, P1, load, store);
       // separate the two real rows: A(k) = (X(k) + conj X(-k))/2, B(k) = (X(k) - conj X(-k))/(2i)
       for (int it = threadIdx.x; it < nb * MZ; it += blockDim.x) {
-        const int iz = it / nb, b = it - iz * nb;
+        const int iz = fx::quot1(it, dnb), b = it - iz * nb;
         const int qq = b / NOUT, cc = b - qq * NOUT;
         const int x0 = 2 * (q0 + qq);
         const C2<T> X = Q[iz * nb + b];
@@ -418,7 +425,7 @@ __device__ __forceinline__ void xz_body(const XzArgs<T>& a, int bx, int by) {
       const int nb = min(a.cx, ncol - c0);
       auto load = [&](int b, int e) -> C2<T> {
         const int col = c0 + b;
-        const int cc = col / MZ, iz = col - cc * MZ;
+        const int cc = fx::quot1(col, a.dMZ), iz = col - cc * MZ;
         return G[e * RS + cc * FS + iz];
       };
       auto store = [&](int b, int e, C2<T> v) {
@@ -427,7 +434,7 @@ __device__ __forceinline__ void xz_body(const XzArgs<T>& a, int bx, int by) {
         else if (e >= nx - Kx) pos = e - nx + a.MX;
         else return;
         const int col = c0 + b;
-        const int cc = col / MZ, iz = col - cc * MZ;
+        const int cc = fx::quot1(col, a.dMZ), iz = col - cc * MZ;
         const T sc = MODE == XZ_ADJOINT ? (iz == 0 ? (T)1 : (T)2) : inv_nxnz;
         out[(size_t)cc * planeMm + pos * MZ + iz] = scl(v, sc);
       };
@@ -1516,6 +1523,8 @@ static XzArgs<T> make_xz_args(const sp_ctx* c, const void* in6, void* out3, T* b
   a.rp = rp; a.cx = cx;
   a.FS = c->MZ + 1;
   a.RS = 6 * a.FS;
+  a.dMZ = fx::div_of(c->MZ);
+  a.dnz = fx::div_of(c->nz);
   const bool glob = sizeof(T) == 8 ? c->xz_gglob64 : c->xz_gglob32;
   a.Gg = glob ? reinterpret_cast<C2<T>*>(c->wsG) : nullptr;
   return a;

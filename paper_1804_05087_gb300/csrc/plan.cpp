@@ -66,6 +66,11 @@ bool make_fft_plan(int n, FftPlan* p) {
   while (m % 4 == 0) { p->radix[p->nst++] = 4; m /= 4; }
   while (m % 3 == 0) { p->radix[p->nst++] = 3; m /= 3; }
   while (m % 2 == 0) { p->radix[p->nst++] = 2; m /= 2; }
+  for (int s = 0, r = n; s < p->nst; ++s) {
+    r /= p->radix[s];
+    p->rp[s] = r;
+    p->mrp[s] = 0xffffffffu / r + 1;
+  }
   return m == 1 && p->nst <= 12;
 }
 

@@ -46,6 +46,8 @@ struct FftPlan {
   int n;
   int nst;
   int radix[12];
+  int rp[12];        // n / (product of the radices up to and with this one)
+  unsigned mrp[12];  // its reciprocal (fx_arith.h, Div)
 };
 
 // contexts whose batches reach this many directions solve the tangent's per-mode
