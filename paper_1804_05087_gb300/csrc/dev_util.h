@@ -58,3 +58,26 @@ __device__ __forceinline__ double2 cdot4(const double2* __restrict__ w, int ws, 
   }
   return make_double2((s0.x + s1.x) + (s2.x + s3.x), (s0.y + s1.y) + (s2.y + s3.y));
 }
+
+// inclusive suffix sum over rows i < cnt of x(i), one warp, chunks of 32 from the top: put(i, sum)
+template <class X, class Put>
+__device__ __forceinline__ void suffix_scan(int cnt, X x, Put put) {
+  const int lane = threadIdx.x & 31;
+  double2 carry = make_double2(0.0, 0.0);
+  for (int c0 = ((cnt - 1) >> 5) << 5; c0 >= 0; c0 -= 32) {
+    const int i = c0 + lane;
+    double2 s = i < cnt ? x(i) : make_double2(0.0, 0.0);
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const double yx = __shfl_down_sync(0xffffffffu, s.x, o), yy = __shfl_down_sync(0xffffffffu, s.y, o);
+      if (lane + o < 32) {
+        s.x += yx;
+        s.y += yy;
+      }
+    }
+    s.x += carry.x;
+    s.y += carry.y;
+    if (i < cnt) put(i, s);
+    carry = make_double2(__shfl_sync(0xffffffffu, s.x, 0), __shfl_sync(0xffffffffu, s.y, 0));
+  }
+}

@@ -456,6 +456,7 @@ struct SolveArgs {
   int n_unique, Mm, MX, MZ, Kx, NY, N, NH;
   int cv, rb0, rb1, off_v0, off_v1, off_h0, off_h1, op_stride;
   int off_vc, off_hc;  // complex operators of the laminar-advection variant
+  const double* row;   // row indices as doubles
   double alpha, beta, inv_dt;
 };
 
@@ -633,44 +634,27 @@ __device__ __forceinline__ void solve_body(const C2<T>* __restrict__ in3, const 
   }
   __syncthreads();
   // phase C2: reduced right-hand side g_n = f_v,n - (2 / (c_n k)) sum_{m > n, m + n odd,
-  // m <= N-2} m f~_a,m for each parity P. With x_n = (n+1) f~_a,n+1 the sum is the inclusive
-  // suffix sum of x over the rows of parity P: one warp per (mode, parity), a shuffle scan over
-  // chunks of 32 rows from the top, carrying the total of the chunks above.
-  {
-    const int lane = threadIdx.x & 31, nwarps = blockDim.x >> 5;
-    for (int pair = threadIdx.x >> 5; pair < 2 * TM; pair += nwarps) {
-      const int t = pair >> 1, P = pair & 1;
-      if (s_u[t] >= a.n_unique || (s_pos[t] == 0 && s_iz[t] == 0)) continue;  // whole warp
-      const double ik = s_ik[t];
-      double2* g = srv + (t * 2 + P) * a.cv;
-      const int cnt = P == 0 ? a.rb0 : a.rb1;  // rows n = 2i + P <= N-2
-      double2 carry = make_double2(0.0, 0.0);
-      for (int c0 = ((cnt - 1) >> 5) << 5; c0 >= 0; c0 -= 32) {
-        const int i = c0 + lane, n = 2 * i + P;
-        double2 x = make_double2(0.0, 0.0);
-        if (i < cnt && n + 1 <= N - 2) {
-          const double2 fa = sfa[t * NR + n + 1];
-          x = make_double2((double)(n + 1) * fa.x, (double)(n + 1) * fa.y);
-        }
-#pragma unroll
-        for (int o = 1; o < 32; o <<= 1) {
-          const double yx = __shfl_down_sync(0xffffffffu, x.x, o);
-          const double yy = __shfl_down_sync(0xffffffffu, x.y, o);
-          if (lane + o < 32) {
-            x.x += yx;
-            x.y += yy;
-          }
-        }
-        x.x += carry.x;
-        x.y += carry.y;
-        if (i < cnt) {
-          const double f = (n == 0 ? 1.0 : 2.0) * ik;
+  // m <= N-2} m f~_a,m for each parity P: with x_n = (n+1) f~_a,n+1 an inclusive suffix sum over the
+  // rows of parity P, one warp per (mode, parity)
+  for (int pair = threadIdx.x >> 5; pair < 2 * TM; pair += blockDim.x >> 5) {
+    const int t = pair >> 1, P = pair & 1;
+    if (s_u[t] >= a.n_unique || (s_pos[t] == 0 && s_iz[t] == 0)) continue;  // whole warp
+    const double ik = s_ik[t];
+    double2* g = srv + (t * 2 + P) * a.cv;
+    suffix_scan(
+        P == 0 ? a.rb0 : a.rb1,  // rows n = 2i + P <= N-2
+        [&](int i) -> double2 {
+          const int m = 2 * i + P + 1;
+          if (m > N - 2) return make_double2(0.0, 0.0);
+          const double w = __ldg(a.row + m);
+          const double2 fa = sfa[t * NR + m];
+          return make_double2(w * fa.x, w * fa.y);
+        },
+        [&](int i, double2 x) {
+          const double f = (2 * i + P == 0 ? 1.0 : 2.0) * ik;
           const double2 v = g[i];
           g[i] = make_double2(v.x - f * x.x, v.y - f * x.y);
-        }
-        carry = make_double2(__shfl_sync(0xffffffffu, x.x, 0), __shfl_sync(0xffffffffu, x.y, 0));
-      }
-    }
+        });
   }
   __syncthreads();
   // phase D: apply the per-mode operators (FP64). Threads take the even unknowns of a
@@ -719,16 +703,17 @@ __device__ __forceinline__ void solve_body(const C2<T>* __restrict__ in3, const 
   // (D v)_n = (2/c_n) sum_{p > n, p + n odd} p v_p: one suffix sum per (mode, parity),
   // kept in sfb (free after phase D) as S_n = sum_{p >= n, p = n mod 2} p v_p
   double2* ssum = sfb;
-  if (threadIdx.x < 2 * TM) {
-    const int t = threadIdx.x >> 1, par = threadIdx.x & 1;
-    double2 acc = make_double2(0.0, 0.0);
-    const int top = ((NY - 1 - par) & 1) ? NY - 2 : NY - 1;  // largest index of this parity
-    for (int p = top; p >= 0; p -= 2) {
-      const double2 vp = sv[t * NY + p];
-      acc.x += p * vp.x;
-      acc.y += p * vp.y;
-      ssum[t * NY + p] = acc;
-    }
+  for (int pair = threadIdx.x >> 5; pair < 2 * TM; pair += blockDim.x >> 5) {
+    const int t = pair >> 1, P = pair & 1;
+    suffix_scan(
+        P == 0 ? nv0 : NY - nv0,
+        [&](int i) -> double2 {
+          const int p = 2 * i + P;
+          const double w = __ldg(a.row + p);
+          const double2 vp = sv[t * NY + p];
+          return make_double2(w * vp.x, w * vp.y);
+        },
+        [&](int i, double2 x) { ssum[t * NY + 2 * i + P] = x; });
   }
   __syncthreads();
   // phase E: a = (i/k) D v, back-rotation, G = u_new - u, Hermitian output
@@ -1599,22 +1584,25 @@ static SolveArgs solve_args(const sp_ctx* c) {
   a.off_v0 = c->off_v0; a.off_v1 = c->off_v1; a.off_h0 = c->off_h0; a.off_h1 = c->off_h1;
   a.op_stride = c->op_stride;
   a.off_vc = c->off_vc; a.off_hc = c->off_hc;
+  a.row = c->rowidx;
   a.alpha = c->alpha; a.beta = c->beta; a.inv_dt = 1.0 / c->dt;
   return a;
 }
 
-// tile shapes of k_solve: (modes per block, threads per block); the autotuner picks one.
-// threads = 0: one thread per solved row, TM * NY rounded up to a whole warp.
+// tile shapes of k_solve: (modes per block, threads per block); the autotuner picks one. Shape 0, the
+// default, has a thread per solved row (threads = 0: TM * NY rounded up to a whole warp, at most
+// 1024): with 128 threads for 4 modes of 35 rows the second round held 12 of 140 rows, and an FP64
+// instruction costs a scheduler 64 cycles whatever the lanes.
 struct SolveShape {
   int tm, threads;
 };
-constexpr SolveShape kSolveShapes[SP_TUNE_MAX] = {{4, 128}, {2, 64}, {8, 256}, {4, 192},
-                                                  {16, 512}, {2, 0}, {4, 0}, {8, 0}};
+constexpr SolveShape kSolveShapes[SP_TUNE_MAX] = {{4, 0}, {2, 64}, {8, 256}, {4, 192},
+                                                  {16, 512}, {2, 0}, {4, 128}, {8, 0}};
 constexpr int kNumSolveShapes = 8;
 
 static int shape_threads(const sp_ctx* c, int shape) {
   const SolveShape sh = kSolveShapes[shape];
-  return sh.threads > 0 ? sh.threads : (sh.tm * c->NY + 31) / 32 * 32;
+  return sh.threads > 0 ? sh.threads : std::min((sh.tm * c->NY + 31) / 32 * 32, 1024);
 }
 
 template <typename T, int TM, int MAXT>
@@ -1636,13 +1624,15 @@ static cudaError_t launch_solve_shape(const sp_ctx* c, int shape, const SolveArg
                                       const double* du, double* out, int n_dir, cudaStream_t st) {
   const int th = shape_threads(c, shape);
   switch (shape) {
-    case 0: return launch_solve_t<T, 4, 128>(c, a, in3, du, out, n_dir, th, st);
+    case 0:
+    case 6:
+      if (th <= 320) return launch_solve_t<T, 4, 320>(c, a, in3, du, out, n_dir, th, st);
+      return launch_solve_t<T, 4, 1024>(c, a, in3, du, out, n_dir, th, st);
     case 1: return launch_solve_t<T, 2, 64>(c, a, in3, du, out, n_dir, th, st);
     case 2: return launch_solve_t<T, 8, 256>(c, a, in3, du, out, n_dir, th, st);
     case 3: return launch_solve_t<T, 4, 192>(c, a, in3, du, out, n_dir, th, st);
     case 4: return launch_solve_t<T, 16, 512>(c, a, in3, du, out, n_dir, th, st);
     case 5: return launch_solve_t<T, 2, 1024>(c, a, in3, du, out, n_dir, th, st);
-    case 6: return launch_solve_t<T, 4, 1024>(c, a, in3, du, out, n_dir, th, st);
     case 7: return launch_solve_t<T, 8, 1024>(c, a, in3, du, out, n_dir, th, st);
     default: return cudaErrorInvalidValue;
   }
