@@ -29,7 +29,6 @@ namespace {
 
 constexpr int kThreadsXZ = 256;
 constexpr int kThreadsYinv = 256;
-constexpr int kThreadsSolve = 128;
 constexpr int kThreadsSolveGrp = 192;  // grouped solve (4 modes per block)
 constexpr int kTileYinv = 16;   // modes per k_yinv block
 constexpr int kTileSolve = 4;   // modes per k_solve block
@@ -451,7 +450,6 @@ __global__ void __launch_bounds__(kThreadsXZ) k_xz(XzArgs<T> a) {
 // ------------------------------------------------------------ k_solve
 struct SolveArgs {
   const double* ops;
-  const double* Cfh_d;
   const float* Cfh_f;
   int n_unique, Mm, MX, MZ, Kx, NY, N, NH;
   int cv, rb0, rb1, off_v0, off_v1, off_h0, off_h1, op_stride;
@@ -771,215 +769,6 @@ __global__ void __launch_bounds__(THREADS) k_solve(const C2<T>* __restrict__ in3
 // per-mode solve, M: curl, values, plane stage, Chebyshev coefficients), so
 // J^T r' = P (1/dt + M^T) S^T P r' - P r' with r' = W r. The chain below
 // evaluates it stage by stage in reverse order.
-
-// k_solve_adj: r' = P W r, f* = S^T r' (transposed per-mode operators),
-// out = f*/dt (boundary layout) and vals = Cf^T f* (values at the
-// Gauss-Lobatto points, plane-major) for every stored mode.
-template <typename T>
-__global__ void __launch_bounds__(kThreadsSolve) k_solve_adj(const double2* __restrict__ r,
-                                                             double2* __restrict__ out,
-                                                             C2<T>* __restrict__ vals, SolveArgs a,
-                                                             int weighted) {
-  extern __shared__ __align__(16) unsigned char smem_raw[];
-  const int TM = kTileSolve;
-  const int NY = a.NY, N = a.N, NH = a.NH, Mm = a.Mm, MZ = a.MZ;
-  const int NR = N - 1;
-  double2* sg = reinterpret_cast<double2*>(smem_raw);  // [3][TM][NY] r' (u, v, w)
-  double2* sga = sg + 3 * TM * NY;                     // [TM][NY] along-k part
-  double2* sgb = sga + TM * NY;                        // [TM][NY] across-k part
-  double2* sva = sgb + TM * NY;                        // [TM][NY] v* = gv + D^T(-i ga/k)
-  double2* srv = sva + TM * NY;                        // [TM][2][cv] V_P^T v*
-  double2* sfb = srv + TM * 2 * a.cv;                  // [TM][NR] H^T gb (or H^T gu)
-  double2* sfw = sfb + TM * NR;                        // [TM][NR] H^T gw (mean mode)
-  double2* sf = sfw + TM * NR;                         // [3][TM][NR] f*
-  __shared__ int s_pos[kTileSolve], s_iz[kTileSolve], s_u[kTileSolve];
-  __shared__ double s_kx[kTileSolve], s_kz[kTileSolve], s_ik[kTileSolve];
-  const int u0 = blockIdx.x * TM;
-  const int dir = blockIdx.y;
-  if (threadIdx.x < TM) {
-    const int u = u0 + threadIdx.x;
-    int pos = 0, iz = 0;
-    if (u < a.n_unique) unique_to_mode(u, a.Kx, MZ, &pos, &iz);
-    s_pos[threadIdx.x] = pos;
-    s_iz[threadIdx.x] = iz;
-    s_u[threadIdx.x] = u;
-    const int ix = pos <= a.Kx ? pos : pos - a.MX;
-    const double kx = a.alpha * ix, kz = a.beta * iz;
-    const double k = sqrt(kx * kx + kz * kz);
-    s_kx[threadIdx.x] = kx;
-    s_kz[threadIdx.x] = kz;
-    s_ik[threadIdx.x] = k > 0 ? 1.0 / k : 0.0;
-  }
-  __syncthreads();
-  const double2* rsrc = r + (size_t)dir * 3 * Mm * NY;
-  // r' = P W r
-  for (int idx = threadIdx.x; idx < 3 * TM * NY; idx += blockDim.x) {
-    const int n = idx % NY;
-    const int t = (idx / NY) % TM;
-    const int c = idx / (NY * TM);
-    double2 v = make_double2(0.0, 0.0);
-    if (s_u[t] < a.n_unique) {
-      const int pos = s_pos[t], iz = s_iz[t];
-      v = __ldg(rsrc + ((size_t)c * Mm + pos * MZ + iz) * NY + n);
-      if (iz == 0) {
-        const int mpos = pos == 0 ? 0 : a.MX - pos;
-        const double2 w = __ldg(rsrc + ((size_t)c * Mm + mpos * MZ) * NY + n);
-        v = make_double2(0.5 * (v.x + w.x), 0.5 * (v.y - w.y));
-      } else if (weighted) {
-        v = make_double2(2.0 * v.x, 2.0 * v.y);
-      }
-    }
-    sg[(c * TM + t) * NY + n] = v;
-  }
-  __syncthreads();
-  // rotation^T: ga = (kx gu + kz gw)/k, gb = (-kz gu + kx gw)/k
-  for (int idx = threadIdx.x; idx < TM * NY; idx += blockDim.x) {
-    const int t = idx / NY, n = idx - t * NY;
-    const double2 gu = sg[(0 * TM + t) * NY + n], gw = sg[(2 * TM + t) * NY + n];
-    if (s_pos[t] == 0 && s_iz[t] == 0) {
-      sga[idx] = gu;
-      sgb[idx] = gw;
-      continue;
-    }
-    const double kx = s_kx[t], kz = s_kz[t], ik = s_ik[t];
-    sga[idx] = make_double2((kx * gu.x + kz * gw.x) * ik, (kx * gu.y + kz * gw.y) * ik);
-    sgb[idx] = make_double2((-kz * gu.x + kx * gw.x) * ik, (-kz * gu.y + kx * gw.y) * ik);
-  }
-  __syncthreads();
-  // a = (i/k) D v  =>  v* = gv + D^T (-i ga / k); (D^T x)_n = sum_{m<n, m+n odd} (2n/c_m) x_m
-  for (int idx = threadIdx.x; idx < TM * NY; idx += blockDim.x) {
-    const int t = idx / NY, n = idx - t * NY;
-    const double2 gv = sg[(1 * TM + t) * NY + n];
-    if (s_pos[t] == 0 && s_iz[t] == 0) {
-      sva[idx] = make_double2(0.0, 0.0);
-      continue;
-    }
-    double2 acc = make_double2(0.0, 0.0);
-    for (int m = (n & 1) ? 0 : 1; m < n; m += 2) {
-      const double2 x = sga[t * NY + m];
-      const double cm = m == 0 ? 0.5 : 1.0;
-      acc.x += cm * x.x;
-      acc.y += cm * x.y;
-    }
-    const double s = 2.0 * n * s_ik[t];
-    // -i ga / k: (x + i y) * (-i) = y - i x
-    sva[idx] = make_double2(gv.x + s * acc.y, gv.y - s * acc.x);
-  }
-  __syncthreads();
-  // V_P^T v* (columns of V_P: the adjoint of g) and H_Q^T gb
-  for (int idx = threadIdx.x; idx < TM * 2 * a.cv; idx += blockDim.x) {
-    const int t = idx / (2 * a.cv), rem = idx - t * 2 * a.cv;
-    const int P = rem / a.cv, col = rem - P * a.cv;
-    if (s_u[t] >= a.n_unique || (s_pos[t] == 0 && s_iz[t] == 0) || col >= (P == 0 ? a.rb0 : a.rb1)) {
-      srv[idx] = make_double2(0.0, 0.0);
-      continue;
-    }
-    const double* V = a.ops + (size_t)s_u[t] * a.op_stride + (P == 0 ? a.off_v0 : a.off_v1);
-    const int nv = P == 0 ? N / 2 + 1 : N / 2;
-    srv[idx] = dot4(V + (size_t)col * nv, 1, sva + t * NY + P, 2, nv);  // column col of V_P
-  }
-  for (int idx = threadIdx.x; idx < TM * NR; idx += blockDim.x) {
-    const int t = idx / NR, n = idx - t * NR;  // momentum row n
-    if (s_u[t] >= a.n_unique) continue;
-    const int Q = n & 1, col = n >> 1;
-    const int nrow = Q == 0 ? N / 2 + 1 : N / 2;
-    const double* H = a.ops + (size_t)s_u[t] * a.op_stride + (Q == 0 ? a.off_h0 : a.off_h1);
-    const bool mean = s_pos[t] == 0 && s_iz[t] == 0;
-    const double* Hc = H + (size_t)col * nrow;  // column col of H_Q
-    sfb[idx] = dot4(Hc, 1, sgb + t * NY + Q, 2, nrow);
-    // sga holds gu and sgb holds gw for the mean mode
-    sfw[idx] = mean ? dot4(Hc, 1, sga + t * NY + Q, 2, nrow) : make_double2(0.0, 0.0);
-  }
-  __syncthreads();
-  // g = f_v - (1/k) D f~_a  =>  f_v* = g*, f~_a*,m = -(2m/k) sum_{n < m, n + m odd} g*_n / c_n
-  // (prefix sums over the f_v rows of the other parity), kept in component 0 of sf
-  double2* sfa = sf;
-  if (threadIdx.x < 2 * TM) {
-    const int t = threadIdx.x >> 1, q = threadIdx.x & 1;  // parity of the f~_a rows
-    if (s_u[t] < a.n_unique && !(s_pos[t] == 0 && s_iz[t] == 0)) {
-      const double2* gs = srv + (t * 2 + (1 - q)) * a.cv;  // g* of parity 1 - q
-      const double ik = s_ik[t];
-      double2 S = make_double2(0.0, 0.0);
-      for (int m = q; m <= N - 2; m += 2) {
-        if (m >= 1) {
-          const int n = m - 1;
-          const double w = n == 0 ? 0.5 : 1.0;
-          const double2 x = gs[n >> 1];
-          S.x = fma(w, x.x, S.x);
-          S.y = fma(w, x.y, S.y);
-        }
-        const double f = -2.0 * m * ik;
-        sfa[t * NR + m] = make_double2(f * S.x, f * S.y);
-      }
-    }
-  }
-  __syncthreads();
-  // f* per component, rows 0..N-2 (each thread reads its f~_a* slot before overwriting it)
-  for (int idx = threadIdx.x; idx < TM * NR; idx += blockDim.x) {
-    const int t = idx / NR, n = idx - t * NR;
-    double2 fx, fy, fz;
-    if (s_pos[t] == 0 && s_iz[t] == 0) {
-      fx = make_double2(sfw[idx].x, 0.0);  // H^T gu
-      fz = make_double2(sfb[idx].x, 0.0);  // H^T gw
-      fy = make_double2(0.0, 0.0);
-    } else {
-      const int P = n & 1;
-      fy = srv[(t * 2 + P) * a.cv + (n >> 1)];
-      const double2 fta = sfa[t * NR + n];
-      const double2 fa = make_double2(-fta.y, fta.x);  // f_a* = i f~_a*
-      const double2 fb = sfb[idx];
-      const double kx = s_kx[t], kz = s_kz[t], ik = s_ik[t];
-      fx = make_double2((kx * fa.x - kz * fb.x) * ik, (kx * fa.y - kz * fb.y) * ik);
-      fz = make_double2((kz * fa.x + kx * fb.x) * ik, (kz * fa.y + kx * fb.y) * ik);
-    }
-    sf[(0 * TM + t) * NR + n] = fx;
-    sf[(1 * TM + t) * NR + n] = fy;
-    sf[(2 * TM + t) * NR + n] = fz;
-  }
-  __syncthreads();
-  // out = f*/dt (boundary layout, rows N-1, N zero), mirrored for iz = 0
-  double2* dst = out + (size_t)dir * 3 * Mm * NY;
-  for (int idx = threadIdx.x; idx < 3 * TM * NY; idx += blockDim.x) {
-    const int n = idx % NY;
-    const int t = (idx / NY) % TM;
-    const int c = idx / (NY * TM);
-    if (s_u[t] >= a.n_unique) continue;
-    const int pos = s_pos[t], iz = s_iz[t];
-    double2 v = make_double2(0.0, 0.0);
-    if (n < NR) {
-      const double2 f = sf[(c * TM + t) * NR + n];
-      v = make_double2(f.x * a.inv_dt, f.y * a.inv_dt);
-    }
-    dst[((size_t)c * Mm + pos * MZ + iz) * NY + n] = v;
-    if (iz == 0 && pos != 0) dst[((size_t)c * Mm + (a.MX - pos) * MZ) * NY + n] = make_double2(v.x, -v.y);
-  }
-  // vals = Cf^T f*: sum_n Cf[n][j] f*_n with Cf[n][N-j] = (-1)^n Cf[n][j]
-  C2<T>* vdst = vals + (size_t)dir * 3 * NY * Mm;
-  for (int idx = threadIdx.x; idx < 3 * TM * NH; idx += blockDim.x) {
-    const int t = idx % TM;
-    const int jh = (idx / TM) % NH;
-    const int c = idx / (TM * NH);
-    if (s_u[t] >= a.n_unique) continue;
-    C2<T> E = mk((T)0, (T)0), O = E;
-    const double2* f = sf + (c * TM + t) * NR;
-    for (int n = 0; n < NR; ++n) {
-      const T cf = sizeof(T) == 8 ? (T)a.Cfh_d[(size_t)n * NH + jh] : (T)a.Cfh_f[(size_t)n * NH + jh];
-      const C2<T> fv = mk((T)f[n].x, (T)f[n].y);
-      if (n & 1) O = O + scl(fv, cf);
-      else E = E + scl(fv, cf);
-    }
-    const int pos = s_pos[t], iz = s_iz[t];
-    const int m = pos * MZ + iz, mm = (a.MX - pos) * MZ;
-#pragma unroll
-    for (int side = 0; side < 2; ++side) {
-      const int j = side == 0 ? jh : N - jh;
-      if (side == 1 && j == jh) break;
-      const C2<T> v = side == 0 ? E + O : E - O;
-      vdst[((size_t)c * NY + j) * Mm + m] = v;
-      if (iz == 0 && pos != 0) vdst[((size_t)c * NY + j) * Mm + mm] = conj2(v);
-    }
-  }
-}
 
 // k_yinv_adj: the transpose of k_yinv. In value space the curl gives
 //   u* += gu - i kz gy, v* += gv + i kz gx - i kx gz, w* += gw + i kx gy,
@@ -1576,7 +1365,6 @@ static size_t solve_smem(const sp_ctx* c, int esize, int TM = kTileSolve) {
 static SolveArgs solve_args(const sp_ctx* c) {
   SolveArgs a;
   a.ops = c->ops;
-  a.Cfh_d = c->Cfh;
   a.Cfh_f = c->Cfh_f;
   a.n_unique = c->n_unique; a.Mm = c->Mm; a.MX = c->MX; a.MZ = c->MZ; a.Kx = c->Kx;
   a.NY = c->NY; a.N = c->N; a.NH = c->NH;
@@ -1659,31 +1447,6 @@ cudaError_t launch_solve(const sp_ctx* c, bool fp32, const void* in3, const doub
   const SolveArgs a = solve_args(c);
   if (fp32) return launch_solve_shape<float>(c, shape, a, in, du, out, n_dir, st);
   return launch_solve_shape<double>(c, shape, a, in, du, out, n_dir, st);
-}
-
-static size_t solve_adj_smem(const sp_ctx* c) {
-  const int TM = kTileSolve, NY = c->NY, NR = c->N - 1;
-  return (size_t)16 * (3 * TM * NY + 3 * TM * NY + TM * 2 * c->cv + 2 * TM * NR + 3 * TM * NR) + 16;
-}
-
-
-cudaError_t launch_solve_adj(const sp_ctx* c, bool fp32, const double* r, double* out, void* vals3, int n_dir,
-                             bool weighted, cudaStream_t st) {
-  SolveArgs a = solve_args(c);
-  dim3 grid((c->n_unique + kTileSolve - 1) / kTileSolve, n_dir);
-  size_t sm = solve_adj_smem(c);
-  if (fp32) {
-    cudaFuncSetAttribute(k_solve_adj<float>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
-    k_solve_adj<float><<<grid, kThreadsSolve, sm, st>>>(reinterpret_cast<const double2*>(r),
-                                                        reinterpret_cast<double2*>(out),
-                                                        reinterpret_cast<C2<float>*>(vals3), a, weighted ? 1 : 0);
-  } else {
-    cudaFuncSetAttribute(k_solve_adj<double>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
-    k_solve_adj<double><<<grid, kThreadsSolve, sm, st>>>(reinterpret_cast<const double2*>(r),
-                                                         reinterpret_cast<double2*>(out),
-                                                         reinterpret_cast<C2<double>*>(vals3), a, weighted ? 1 : 0);
-  }
-  return cudaGetLastError();
 }
 
 cudaError_t launch_yinv_adj(const sp_ctx* c, bool fp32, const void* in6, double* out, int n_dir,

@@ -654,7 +654,8 @@ sp_status sp_build_plan(sp_ctx* c) {
   for (int u = 0; u < c->n_unique; ++u) {
     int pos, iz;
     sp_unique_mode(c, u, &pos, &iz);
-    const double kx = c->alpha * (pos <= c->Kx ? pos : pos - c->MX), kz = c->beta * iz, k = std::sqrt(kx * kx + kz * kz);
+    const double kx = c->alpha * (pos <= c->Kx ? pos : pos - c->MX), kz = c->beta * iz;
+    const double k = std::sqrt(std::fma(kz, kz, kx * kx));
     wave[4 * u] = kx;
     wave[4 * u + 1] = kz;
     wave[4 * u + 2] = k > 0 ? 1.0 / k : 0.0;

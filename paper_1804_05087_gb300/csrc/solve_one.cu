@@ -11,7 +11,7 @@
 // sums are warp scans, and wavenumbers and row indices are read, not computed. Several blocks share
 // an SM, so that one block's scans overlap another's products. Measured at 48 x 65 x 48, one FP64
 // direction: 55 us with four modes per block and loads inside the products, see the rule in
-// sp_solve_shapes for the threads.
+// sp_solve_shapes for the threads. k_solve_adj is the transposed solve, in the same shape.
 #include <algorithm>
 #include <cstdint>
 
@@ -34,6 +34,45 @@ struct OneArgs {
 
 __device__ __forceinline__ uint32_t smem_of(const void* p) { return static_cast<uint32_t>(__cvta_generic_to_shared(p)); }
 
+__device__ __forceinline__ void bulk_copy(double* dst, const double* src, uint32_t bytes, uint32_t bar) {
+  asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(smem_of(dst)),
+               "l"(src), "r"(bytes), "r"(bar)
+               : "memory");
+}
+
+// one bulk copy of a mode's operators (one thread), and the wait for it (all threads): false when the
+// limit runs out
+__device__ __forceinline__ void stage_begin(double* dst, const double* op, uint32_t bytes, uint64_t* s_bar) {
+  const uint32_t bar = smem_of(s_bar);
+  asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(bar));
+  asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+  asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(bar), "r"(bytes) : "memory");
+  bulk_copy(dst, op, bytes, bar);
+}
+__device__ __forceinline__ bool stage_wait(uint64_t* s_bar) {
+  const uint32_t bar = smem_of(s_bar);
+  uint32_t done = 0;
+  for (uint32_t it = 0; it < (1u << 25) && !done; ++it)  // the second half of the limit: the copy may be in flight
+    asm volatile(
+        "{\n\t.reg .pred p;\n\tmbarrier.try_wait.parity.shared::cta.b64 p, [%1], 0;\n\tselp.u32 %0, 1, 0, p;\n\t}\n"
+        : "=r"(done)
+        : "r"(bar)
+        : "memory");
+  return done != 0;
+}
+
+__device__ __forceinline__ void mode_of(const OneArgs& a, int u, int* pos, int* iz) {
+  const int first = (a.Kx + 1) * a.MZ;
+  if (u < first) {
+    *pos = u / a.MZ;
+    *iz = u - *pos * a.MZ;
+  } else {
+    const int v = u - first;
+    *pos = a.Kx + 1 + v / (a.MZ - 1);
+    *iz = 1 + v % (a.MZ - 1);
+  }
+}
+
 // mode u of direction dir
 template <typename T>
 __device__ __forceinline__ void solve_one(const OneArgs& a, int u, int dir, unsigned char* smem, uint64_t* s_bar) {
@@ -49,30 +88,11 @@ __device__ __forceinline__ void solve_one(const OneArgs& a, int u, int dir, unsi
   double2* sb = sv + NY;        // [NY]
   double2* ss = sb + NY;        // [NY + 1] sums of p v_p over p >= n of the parity of n
   C2<T>* vals = reinterpret_cast<C2<T>*>(ss + NY + 1);  // [3][NY] (float)
-  const uint32_t bar = smem_of(s_bar);
   int pos, iz;
-  {
-    const int first = (a.Kx + 1) * MZ;
-    if (u < first) {
-      pos = u / MZ;
-      iz = u - pos * MZ;
-    } else {
-      const int v = u - first;
-      pos = a.Kx + 1 + v / (MZ - 1);
-      iz = 1 + v % (MZ - 1);
-    }
-  }
+  mode_of(a, u, &pos, &iz);
   const bool mean = u == 0;
   const double* op = a.ops + (size_t)u * a.op_stride;
-  if (a.staged && tid == 0) {
-    const uint32_t bytes = (uint32_t)a.op_stride * 8;
-    asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(bar));
-    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
-    asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(bar), "r"(bytes) : "memory");
-    asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(smem_of(sop)),
-                 "l"(op), "r"(bytes), "r"(bar)
-                 : "memory");
-  }
+  if (a.staged && tid == 0) stage_begin(sop, op, (uint32_t)a.op_stride * 8, s_bar);
   const double kx = __ldg(a.wave + 4 * u), kz = __ldg(a.wave + 4 * u + 1), ik = __ldg(a.wave + 4 * u + 2);
   // input state (Hermitian-projected)
   const double2* dsrc = a.du + ((size_t)dir * 3 * Mm + pos * MZ + iz) * NY;
@@ -162,14 +182,7 @@ __device__ __forceinline__ void solve_one(const OneArgs& a, int u, int dir, unsi
   }
   bool ok = true;
   if (a.staged) {
-    uint32_t done = 0;
-    for (uint32_t it = 0; it < (1u << 25) && !done; ++it)  // the second half of the limit: the copy may be in flight
-      asm volatile(
-          "{\n\t.reg .pred p;\n\tmbarrier.try_wait.parity.shared::cta.b64 p, [%1], 0;\n\tselp.u32 %0, 1, 0, p;\n\t}\n"
-          : "=r"(done)
-          : "r"(bar)
-          : "memory");
-    ok = done != 0;
+    ok = stage_wait(s_bar);
     op = sop;
   }
   ok = __syncthreads_and(ok) != 0;  // the limit ran out: NaN below
@@ -284,6 +297,212 @@ __global__ void __launch_bounds__(512) k_solve_one_grp(const double* __restrict_
   solve_one<T>(r.a, blockIdx.x - first[i], 0, smem, &s_bar);
 }
 
+// out[4 i] = sum of x[xs j] over j <= i, in order; the first entry halved (c_0 = 2) where asked
+__device__ __forceinline__ void prefix(const double* x, int xs, double* out, int cnt, bool half) {
+  double s = 0.0, v = cnt > 0 ? x[0] : 0.0;
+  if (half) v *= 0.5;
+  for (int i = 0; i < cnt; ++i) {
+    const double next = i + 1 < cnt ? x[(i + 1) * xs] : 0.0;  // before the store: `out` may be `x`
+    s += v;
+    out[4 * i] = s;
+    v = next;
+  }
+}
+
+// entries between columns in shared memory: a multiple of 4 puts the lanes of a warp on few banks
+__host__ __device__ inline int col_stride(int nrow) { return nrow % 4 ? nrow : nrow + 2; }
+
+// The transposed solve of the discrete adjoint, one mode of one direction per block: r' = P W r,
+// f* = S^T r' (the transposed operators), out = f*/dt, vals = Cf^T f* at the Gauss-Lobatto points
+// (float values feed the transposed plane stage in mixed precision).
+//
+// Bound by the FP64 unit, as the forward solve. With four modes per block of 128 threads the lanes of
+// a product read columns of the operator in global memory (a stride of N/2 rows), the derivative sums
+// ran on 8 threads and each multiplication of the float transform converted its factor again: 573 us
+// at 96 x 97 x 96 against 162 us of the forward solve; the gradient pass is 404 us shorter now. The
+// operators are staged as there and a thread takes one column (columns whose length is a multiple of 4
+// are copied one by one, two entries apart, so that lanes meet in a bank by twos at most); f* is
+// converted once. The prefix sums are serial, on four lanes (parity, part), and the fused products are
+// written out: all feed values that mixed precision rounds to float, where a last bit of FP64 can turn
+// into 6e-8.
+template <typename T>
+__global__ void __launch_bounds__(512) k_solve_adj(const __grid_constant__ OneArgs a, C2<T>* __restrict__ vals,
+                                                   const T* __restrict__ cf, int weighted) {
+  extern __shared__ __align__(16) unsigned char smem[];
+  __shared__ __align__(8) uint64_t s_bar;
+  const int NY = a.NY, N = NY - 1, NH = N / 2 + 1, NR = N - 1, Mm = a.Mm, MZ = a.MZ;
+  const int tid = threadIdx.x, nt = blockDim.x, warp = tid >> 5, nw = nt >> 5;
+  const int u = blockIdx.x, dir = blockIdx.y;
+  // column strides of the staged operators per parity
+  const int st0 = a.staged ? col_stride(N / 2 + 1) : N / 2 + 1, st1 = a.staged ? col_stride(N / 2) : N / 2;
+  double* sop = reinterpret_cast<double*>(smem);
+  double2* sga = reinterpret_cast<double2*>(sop + (a.staged ? 2 * (a.rb0 * st0 + a.rb1 * st1) : 0));
+  // sga: [NY] along k (mean mode: u), then its prefix sums
+  double2* sgb = sga + NY;       // [NY] across k (mean mode: w)
+  double2* sva = sgb + NY;       // [NY] v* = gv + D^T(-i ga / k)
+  double2* srv = sva + NY;       // [2][cv] V^T v*
+  double2* sfb = srv + 2 * a.cv; // [NR] H^T gb (mean mode: H^T gw)
+  double2* sfa = sfb + NR;       // [NR] sums of f~_a* (mean mode: H^T gu)
+  C2<T>* sf = reinterpret_cast<C2<T>*>(sfa + NR);  // [3][NR] f*
+  int pos, iz;
+  mode_of(a, u, &pos, &iz);
+  const bool mean = u == 0;
+  const double* op = a.ops + (size_t)u * a.op_stride;
+  const int v1 = a.staged ? a.rb0 * st0 : a.off_v1, h0 = a.staged ? v1 + a.rb1 * st1 : a.off_h0,
+            h1 = a.staged ? h0 + a.rb0 * st0 : a.off_h1;
+  if (a.staged && warp == 0) {
+    const uint32_t bar = smem_of(&s_bar);
+    if (tid == 0) {
+      const uint32_t bytes = 16u * (uint32_t)(a.rb0 * (N / 2 + 1) + a.rb1 * (N / 2));
+      asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(bar));
+      asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+      asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(bar), "r"(bytes) : "memory");
+    }
+    __syncwarp();
+    for (int o = 0; o < 4; ++o) {
+      const int Q = o & 1, nrow = Q ? N / 2 : N / 2 + 1, cols = Q ? a.rb1 : a.rb0, st = Q ? st1 : st0;
+      const double* src = op + (o == 0 ? a.off_v0 : o == 1 ? a.off_v1 : o == 2 ? a.off_h0 : a.off_h1);
+      double* to = sop + (o == 0 ? 0 : o == 1 ? v1 : o == 2 ? h0 : h1);
+      if (st == nrow) {
+        if (tid == 0 && cols > 0) bulk_copy(to, src, (uint32_t)(cols * nrow) * 8, bar);
+      } else {
+        for (int k = tid; k < cols; k += 32) bulk_copy(to + k * st, src + (size_t)k * nrow, (uint32_t)nrow * 8, bar);
+      }
+    }
+  }
+  const double kx = __ldg(a.wave + 4 * u), kz = __ldg(a.wave + 4 * u + 1), ik = __ldg(a.wave + 4 * u + 2);
+  const size_t comp = (size_t)Mm * NY;
+  const size_t at = (size_t)dir * 3 * comp + ((size_t)pos * MZ + iz) * NY;
+  const long long mir = pos == 0 ? 0 : (long long)(a.MX - 2 * pos) * MZ * NY;  // to the mirror mode
+  // r' = P W r, rotated to the components along / across the wavevector
+  for (int n = tid; n < NY; n += nt) {
+    double2 g[3];
+#pragma unroll
+    for (int c = 0; c < 3; ++c) {
+      const double2* p = a.du + at + c * comp + n;
+      double2 v = __ldg(p);
+      if (iz == 0) {
+        const double2 w = __ldg(p + mir);
+        v = make_double2(0.5 * (v.x + w.x), 0.5 * (v.y - w.y));
+      } else if (weighted) {
+        v = make_double2(2.0 * v.x, 2.0 * v.y);
+      }
+      g[c] = v;
+    }
+    sga[n] = mean ? g[0] : make_double2(fma(kx, g[0].x, kz * g[2].x) * ik, fma(kx, g[0].y, kz * g[2].y) * ik);
+    sgb[n] = mean ? g[2] : make_double2(fma(kx, g[2].x, -kz * g[0].x) * ik, fma(kx, g[2].y, -kz * g[0].y) * ik);
+    sva[n] = g[1];
+  }
+  __syncthreads();
+  // a = (i/k) D v  =>  v* = gv + D^T (-i ga / k); (D^T x)_n = sum_{m<n, m+n odd} (2n/c_m) x_m: the sums
+  // over the rows m = 2i + Q of each parity, in place
+  if (!mean) {
+    if (tid < 4) prefix(reinterpret_cast<double*>(sga + (tid >> 1)) + (tid & 1), 4,
+                        reinterpret_cast<double*>(sga + (tid >> 1)) + (tid & 1), (NY - (tid >> 1) + 1) / 2, tid < 2);
+    __syncthreads();
+    for (int n = 1 + tid; n < NY; n += nt) {
+      const double f = 2.0 * __ldg(a.row + n) * ik;
+      const double2 gv = sva[n], s = sga[n - 1];
+      // -i ga / k: (x + i y) * (-i) = y - i x
+      sva[n] = make_double2(gv.x + f * s.y, gv.y - f * s.x);
+    }
+  }
+  bool ok = true;
+  if (a.staged) {
+    ok = stage_wait(&s_bar);
+    op = sop;
+  }
+  ok = __syncthreads_and(ok) != 0;  // the limit ran out: NaN below
+  // columns of V_P (adjoint of g) and of H_Q: one per thread
+  for (int i = tid; i < 2 * NR; i += nt) {
+    const bool hel = i >= NR;
+    const int k = hel ? i - NR : i;
+    const int Q = k < a.rb0 ? 0 : 1, col = Q == 0 ? k : k - a.rb0;
+    const int nrow = Q == 0 ? N / 2 + 1 : N / 2;
+    const bool isH = hel || mean;
+    const double* M = op + (isH ? (Q == 0 ? h0 : h1) : (Q == 0 ? a.off_v0 : v1)) + (size_t)col * (Q == 0 ? st0 : st1);
+    const double2* x = (hel ? sgb : mean ? sga : sva) + Q;
+    double2 p[4] = {};
+    int c = 0;
+    for (; c + 4 <= nrow; c += 4) {
+#pragma unroll
+      for (int q = 0; q < 4; ++q) {
+        const double w = M[c + q];
+        const double2 y = x[2 * (c + q)];
+        p[q].x = fma(w, y.x, p[q].x);
+        p[q].y = fma(w, y.y, p[q].y);
+      }
+    }
+    for (; c < nrow; ++c) {
+      const double w = M[c];
+      const double2 y = x[2 * c];
+      p[0].x = fma(w, y.x, p[0].x);
+      p[0].y = fma(w, y.y, p[0].y);
+    }
+    const double2 s = make_double2((p[0].x + p[1].x) + (p[2].x + p[3].x), (p[0].y + p[1].y) + (p[2].y + p[3].y));
+    if (hel) sfb[2 * col + Q] = s;
+    else if (mean) sfa[2 * col + Q] = s;
+    else srv[Q * a.cv + col] = s;
+  }
+  __syncthreads();
+  // g = f_v - (1/k) D f~_a  =>  f_v* = g*, f~_a*,m = -(2m/k) sum_{n < m, n + m odd} g*_n / c_n: the sums
+  if (!mean) {
+    if (tid < 4) prefix(reinterpret_cast<double*>(srv + (tid >> 1) * a.cv) + (tid & 1), 2,
+                        reinterpret_cast<double*>(sfa + (tid >> 1) + 1) + (tid & 1), min(tid < 2 ? a.rb0 : a.rb1, (NR - (tid >> 1)) / 2), tid < 2);
+    if (tid == 4) sfa[0] = make_double2(0.0, 0.0);  // no rows below
+  }
+  __syncthreads();
+  // f* per component, out = f*/dt (rows N-1, N zero), mirrored for iz = 0
+  double2* dst = a.out + at;
+  for (int n = tid; n < NY; n += nt) {
+    double2 f[3] = {make_double2(0.0, 0.0), make_double2(0.0, 0.0), make_double2(0.0, 0.0)};
+    if (n < NR) {
+      if (mean) {
+        f[0].x = sfa[n].x;
+        f[2].x = sfb[n].x;
+      } else {
+        f[1] = srv[(n & 1) * a.cv + (n >> 1)];
+        const double g = -2.0 * __ldg(a.row + n) * ik;
+        const double2 S = sfa[n], t = make_double2(g * S.x, g * S.y), fb = sfb[n];
+        const double2 fa = make_double2(-t.y, t.x);  // f_a* = i f~_a*
+        f[0] = make_double2(fma(kx, fa.x, -kz * fb.x) * ik, fma(kx, fa.y, -kz * fb.y) * ik);
+        f[2] = make_double2(fma(kx, fb.x, kz * fa.x) * ik, fma(kx, fb.y, kz * fa.y) * ik);
+      }
+#pragma unroll
+      for (int c = 0; c < 3; ++c) {
+        if (!ok) f[c] = make_double2(nan(""), nan(""));
+        sf[c * NR + n] = mk((T)f[c].x, (T)f[c].y);
+      }
+    }
+#pragma unroll
+    for (int c = 0; c < 3; ++c) {
+      const double2 v = make_double2(f[c].x * a.inv_dt, f[c].y * a.inv_dt);
+      double2* o = dst + c * comp + n;
+      *o = v;
+      if (iz == 0 && pos != 0) o[mir] = make_double2(v.x, -v.y);
+    }
+  }
+  __syncthreads();
+  // vals = Cf^T f*: sum_n Cf[n][j] f*_n with Cf[n][N-j] = (-1)^n Cf[n][j]; the even rows of a point pair
+  // on one lane, the odd rows on the next
+  C2<T>* vdst = vals + (size_t)dir * 3 * NY * Mm + pos * MZ + iz;
+  const int vmir = (a.MX - 2 * pos) * MZ;
+  for (int i0 = warp * 32; i0 < 6 * NH; i0 += nw * 32) {
+    const int i = i0 + (tid & 31), q = min(i >> 1, 3 * NH - 1), par = i & 1;
+    const int c = q / NH, jh = q - c * NH;
+    C2<T> s = mk((T)0, (T)0);
+    const C2<T>* f = sf + c * NR;
+    for (int n = par; n < NR; n += 2) s = s + scl(f[n], __ldg(cf + (size_t)n * NH + jh));
+    const C2<T> o = mk(__shfl_xor_sync(0xffffffffu, s.x, 1), __shfl_xor_sync(0xffffffffu, s.y, 1));
+    const int j = par ? N - jh : jh;
+    if (i >= 6 * NH || (par && j == jh)) continue;
+    const C2<T> v = par ? o - s : s + o;
+    C2<T>* p = vdst + ((size_t)c * NY + j) * Mm;
+    *p = v;
+    if (iz == 0 && pos != 0) p[vmir] = conj2(v);
+  }
+}
+
 // operators in shared memory up to this size (N <= 104); larger ones are read in place
 constexpr size_t kStageBytes = 100 * 1024;
 
@@ -359,5 +578,23 @@ cudaError_t grp_build_solve_one(GrpKernel* k, sp_ctx* const* mem, int n, const s
 cudaError_t grp_launch_solve_one(const GrpKernel& k, bool fp32, const double* du, double* out, const int* active, cudaStream_t st) {
   auto kern = fp32 ? k_solve_one_grp<float> : k_solve_one_grp<double>;
   kern<<<k.blocks, k.threads, k.smem, st>>>(du, out, static_cast<const GOne*>(k.recs), k.inst, k.first, active);
+  return cudaGetLastError();
+}
+
+cudaError_t launch_solve_adj(const sp_ctx* c, bool fp32, const double* r, double* out, void* vals3, int n_dir,
+                             bool weighted, cudaStream_t st) {
+  const OneArgs a = one_args(c, nullptr, r, out);
+  const size_t NY = c->NY, NR = c->N - 1;
+  const size_t ops = a.staged ? 16 * ((size_t)c->rb0 * col_stride(c->N / 2 + 1) + (size_t)c->rb1 * col_stride(c->N / 2)) : 0;
+  const size_t sm = ops + 16 * (3 * NY + 2 * c->cv + 2 * NR) + (fp32 ? 8 : 16) * 3 * NR;
+  const dim3 grid(c->n_unique, n_dir);
+  const int th = solve_one_threads(c, 0);
+  const void* kern = fp32 ? (const void*)k_solve_adj<float> : (const void*)k_solve_adj<double>;
+  const cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+  if (e != cudaSuccess) return e;
+  if (fp32)
+    k_solve_adj<float><<<grid, th, sm, st>>>(a, static_cast<C2<float>*>(vals3), c->Cfh_f, weighted ? 1 : 0);
+  else
+    k_solve_adj<double><<<grid, th, sm, st>>>(a, static_cast<C2<double>*>(vals3), c->Cfh, weighted ? 1 : 0);
   return cudaGetLastError();
 }
