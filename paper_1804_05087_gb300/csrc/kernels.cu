@@ -31,6 +31,7 @@ constexpr int kThreadsXZ = 256;
 constexpr int kThreadsYinv = 256;
 constexpr int kThreadsSolveGrp = 192;  // grouped solve (4 modes per block)
 constexpr int kTileYinv = 16;   // modes per k_yinv block
+constexpr int kTileYinvAdj = 4;  // modes per k_yinv_adj block
 constexpr int kTileSolve = 4;   // modes per k_solve block
 
 // ------------------------------------------------------------------ FFT
@@ -775,71 +776,86 @@ __global__ void __launch_bounds__(THREADS) k_solve(const C2<T>* __restrict__ in3
 //   (Du)* = -gz, (Dw)* = gx;
 // then coefficients: x*_n = sum_j T_n(y_j) x*_j + sum_j T_n'(y_j) (Dx)*_j,
 // added to `out` (which already holds f*/dt).
+//
+// The float sums are a few microseconds of FMA work at 96 x 97 x 96; with 16 modes per block and a
+// thread per (mode, n) the kernel was bound by latency and by shared memory (10 loads for 10 FMAs):
+// 97 us on 126 blocks (now 41 us on 504). Here the even and odd parts of a point pair are formed once when the values
+// are read, a thread takes one n of 4 modes (its loads are broadcasts: threads take the even n first),
+// and there are four times the blocks. Every sum keeps its order.
 template <typename T>
-__global__ void __launch_bounds__(kThreadsYinv) k_yinv_adj(const C2<T>* __restrict__ in,
-                                                          double2* __restrict__ out,
-                                                          const T* __restrict__ Th,
-                                                          const T* __restrict__ TDh, YinvArgs a) {
+__global__ void __launch_bounds__(256) k_yinv_adj(const C2<T>* __restrict__ in, double2* __restrict__ out,
+                                                  const T* __restrict__ Th, const T* __restrict__ TDh,
+                                                  YinvArgs a) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  const int TM = kTileYinv;
+  constexpr int TM = kTileYinvAdj;
   const int NY = a.NY, Mm = a.Mm, N = a.N, NH = a.NH;
-  C2<T>* s5 = reinterpret_cast<C2<T>*>(smem_raw);  // [5][NY][TM]: u*, v*, w*, Du*, Dw* values
+  // [5][NY][TM]: u*, v*, w*, Du*, Dw*: x_j + x_N-j at j < N/2, x_j - x_N-j at N - j
+  C2<T>* s5 = reinterpret_cast<C2<T>*>(smem_raw);
   const int m0 = blockIdx.x * TM;
   const int dir = blockIdx.z;
   const C2<T>* src = in + (size_t)dir * 6 * NY * Mm;
-  for (int idx = threadIdx.x; idx < TM * NY; idx += blockDim.x) {
-    const int t = idx % TM, j = idx / TM;
+  for (int idx = threadIdx.x; idx < TM * NH; idx += blockDim.x) {
+    const int t = idx % TM, jh = idx / TM;
     const int m = m0 + t;
-    C2<T> g[6];
-    if (m < Mm) {
-#pragma unroll
-      for (int f = 0; f < 6; ++f) g[f] = ld_c2(src + ((size_t)f * NY + j) * Mm + m);
-    } else {
-#pragma unroll
-      for (int f = 0; f < 6; ++f) g[f] = mk((T)0, (T)0);
-    }
     const int pos = m / a.MZ, iz = m - pos * a.MZ;
     const int ix = pos <= a.Kx ? pos : pos - a.MX;
     const T kx = (T)(a.alpha * ix), kz = (T)(a.beta * iz);
-    s5[(0 * NY + j) * TM + t] = g[0] - mul_is(g[4], kz);
-    s5[(1 * NY + j) * TM + t] = g[1] + mul_is(g[3], kz) - mul_is(g[5], kx);
-    s5[(2 * NY + j) * TM + t] = g[2] + mul_is(g[4], kx);
-    s5[(3 * NY + j) * TM + t] = mk(-g[5].x, -g[5].y);
-    s5[(4 * NY + j) * TM + t] = g[3];
+    C2<T> x[2][5];
+#pragma unroll
+    for (int side = 0; side < 2; ++side) {
+      const int j = side ? N - jh : jh;
+      C2<T> g[6];
+#pragma unroll
+      for (int f = 0; f < 6; ++f) g[f] = m < Mm ? ld_c2(src + ((size_t)f * NY + j) * Mm + m) : mk((T)0, (T)0);
+      x[side][0] = g[0] - mul_is(g[4], kz);
+      x[side][1] = g[1] + mul_is(g[3], kz) - mul_is(g[5], kx);
+      x[side][2] = g[2] + mul_is(g[4], kx);
+      x[side][3] = mk(-g[5].x, -g[5].y);
+      x[side][4] = g[3];
+    }
+#pragma unroll
+    for (int f = 0; f < 5; ++f) {
+      C2<T>* p = s5 + f * NY * TM + t;
+      if (2 * jh == N) {
+        p[jh * TM] = x[0][f];
+      } else {
+        p[jh * TM] = x[0][f] + x[1][f];
+        p[(N - jh) * TM] = x[0][f] - x[1][f];
+      }
+    }
   }
   __syncthreads();
   double2* dst = out + (size_t)dir * 3 * Mm * NY;
-  for (int idx = threadIdx.x; idx < TM * NY; idx += blockDim.x) {
-    const int t = idx % TM, n = idx / TM;
-    const int m = m0 + t;
-    if (m >= Mm) continue;
-    const T sgT = (n & 1) ? (T)-1 : (T)1;  // T_n(y_{N-j}) = (-1)^n T_n(y_j)
-    const T sgD = -sgT;                    // T_n'(y_{N-j}) = (-1)^(n+1) T_n'(y_j)
-    C2<T> au = mk((T)0, (T)0), av = au, aw = au;
+  const int ne = N / 2 + 1;
+  for (int i = threadIdx.x; i < NY; i += blockDim.x) {
+    const int n = i < ne ? 2 * i : 2 * (i - ne) + 1;
+    // T_n(y_{N-j}) = (-1)^n T_n(y_j), T_n'(y_{N-j}) = (-1)^(n+1) T_n'(y_j)
+    const bool odd = n & 1;
+    C2<T> acc[3][TM];
+#pragma unroll
+    for (int c = 0; c < 3; ++c)
+#pragma unroll
+      for (int t = 0; t < TM; ++t) acc[c][t] = mk((T)0, (T)0);
     for (int jh = 0; jh < NH; ++jh) {
       const T tv = Th[(size_t)jh * NY + n], dv = TDh[(size_t)jh * NY + n];
-      const int j2 = N - jh;
-      const bool mid = (j2 == jh);
-      C2<T> xu = s5[(0 * NY + jh) * TM + t], xv = s5[(1 * NY + jh) * TM + t], xw = s5[(2 * NY + jh) * TM + t];
-      C2<T> xdu = s5[(3 * NY + jh) * TM + t], xdw = s5[(4 * NY + jh) * TM + t];
-      if (!mid) {
-        xu = xu + scl(s5[(0 * NY + j2) * TM + t], sgT);
-        xv = xv + scl(s5[(1 * NY + j2) * TM + t], sgT);
-        xw = xw + scl(s5[(2 * NY + j2) * TM + t], sgT);
-        xdu = xdu + scl(s5[(3 * NY + j2) * TM + t], sgD);
-        xdw = xdw + scl(s5[(4 * NY + j2) * TM + t], sgD);
-      }
-      au = au + scl(xu, tv) + scl(xdu, dv);
-      av = av + scl(xv, tv);
-      aw = aw + scl(xw, tv) + scl(xdw, dv);
-    }
-    const C2<T> res[3] = {au, av, aw};
+      const C2<T>* xt = s5 + (odd ? N - jh : jh) * TM;
+      const C2<T>* xd = s5 + (3 * NY + (odd ? jh : N - jh)) * TM;
 #pragma unroll
-    for (int c = 0; c < 3; ++c) {
-      double2* p = dst + ((size_t)c * Mm + m) * NY + n;
-      const double2 o = *p;
-      *p = make_double2(o.x + (double)res[c].x, o.y + (double)res[c].y);
+      for (int t = 0; t < TM; ++t) {
+        acc[0][t] = acc[0][t] + scl(xt[t], tv) + scl(xd[t], dv);
+        acc[1][t] = acc[1][t] + scl(xt[NY * TM + t], tv);
+        acc[2][t] = acc[2][t] + scl(xt[2 * NY * TM + t], tv) + scl(xd[NY * TM + t], dv);
+      }
     }
+#pragma unroll
+    for (int c = 0; c < 3; ++c)
+#pragma unroll
+      for (int t = 0; t < TM; ++t) {
+        if (m0 + t >= Mm) continue;
+        double2* p = dst + ((size_t)c * Mm + m0 + t) * NY + n;
+        const double2 o = *p;
+        *p = make_double2(o.x + (double)acc[c][t].x, o.y + (double)acc[c][t].y);
+      }
   }
 }
 
@@ -1455,18 +1471,18 @@ cudaError_t launch_yinv_adj(const sp_ctx* c, bool fp32, const void* in6, double*
   a.Mm = c->Mm; a.MZ = c->MZ; a.MX = c->MX; a.Kx = c->Kx; a.NY = c->NY; a.N = c->N; a.NH = c->NH;
   a.alpha = c->alpha; a.beta = c->beta;
   a.jchunk = c->NH;
-  const int tiles = (c->Mm + kTileYinv - 1) / kTileYinv;
-  dim3 grid(tiles, 1, n_dir);
+  const dim3 grid((c->Mm + kTileYinvAdj - 1) / kTileYinvAdj, 1, n_dir);
+  const int th = std::min((c->NY + 31) / 32 * 32, 256);
   if (fp32) {
-    size_t sm = (size_t)5 * c->NY * kTileYinv * sizeof(C2<float>);
+    size_t sm = (size_t)5 * c->NY * kTileYinvAdj * sizeof(C2<float>);
     cudaFuncSetAttribute(k_yinv_adj<float>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
-    k_yinv_adj<float><<<grid, kThreadsYinv, sm, st>>>(reinterpret_cast<const C2<float>*>(in6),
-                                                      reinterpret_cast<double2*>(out), c->Th_f, c->TDh_f, a);
+    k_yinv_adj<float><<<grid, th, sm, st>>>(reinterpret_cast<const C2<float>*>(in6), reinterpret_cast<double2*>(out),
+                                            c->Th_f, c->TDh_f, a);
   } else {
-    size_t sm = (size_t)5 * c->NY * kTileYinv * sizeof(C2<double>);
+    size_t sm = (size_t)5 * c->NY * kTileYinvAdj * sizeof(C2<double>);
     cudaFuncSetAttribute(k_yinv_adj<double>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
-    k_yinv_adj<double><<<grid, kThreadsYinv, sm, st>>>(reinterpret_cast<const C2<double>*>(in6),
-                                                       reinterpret_cast<double2*>(out), c->Th, c->TDh, a);
+    k_yinv_adj<double><<<grid, th, sm, st>>>(reinterpret_cast<const C2<double>*>(in6), reinterpret_cast<double2*>(out),
+                                             c->Th, c->TDh, a);
   }
   return cudaGetLastError();
 }

@@ -319,7 +319,7 @@ __host__ __device__ inline int col_stride(int nrow) { return nrow % 4 ? nrow : n
 // Bound by the FP64 unit, as the forward solve. With four modes per block of 128 threads the lanes of
 // a product read columns of the operator in global memory (a stride of N/2 rows), the derivative sums
 // ran on 8 threads and each multiplication of the float transform converted its factor again: 573 us
-// at 96 x 97 x 96 against 162 us of the forward solve; the gradient pass is 404 us shorter now. The
+// at 96 x 97 x 96 against 162 us of the forward solve; 177 us now. The
 // operators are staged as there and a thread takes one column (columns whose length is a multiple of 4
 // are copied one by one, two entries apart, so that lanes meet in a bank by twos at most); f* is
 // converted once. The prefix sums are serial, on four lanes (parity, part), and the fused products are
