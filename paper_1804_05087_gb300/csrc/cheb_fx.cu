@@ -225,7 +225,7 @@ struct RArgs {
   double2* W;          // (u, d, row c (N-1) + n) at u su + d sd + row sn
   const int2* tab;
   long long su, sd, sn;
-  int n_unique, Mm, MX, MZ, Kx, NY, NH, rchunk;
+  int n_dir, n_unique, Mm, MX, MZ, Kx, NY, NH, rchunk;
   double inv_dt;
 };
 
@@ -375,7 +375,7 @@ __global__ void __launch_bounds__(kThreadsC, 3) k_rhs_fx(const __grid_constant__
   __shared__ RShared<TM> s;
   // directions fastest: with one direction per 16-byte column of W, the blocks that run together
   // fill its sectors
-  rhs_fx<TM>(a, blockIdx.y, blockIdx.z, blockIdx.x, reinterpret_cast<int4*>(smem), s);
+  rhs_fx<TM>(a, blockIdx.x / a.n_dir, blockIdx.y, blockIdx.x % a.n_dir, reinterpret_cast<int4*>(smem), s);
 }
 
 // ------------------------------------------------------------------ groups
@@ -456,6 +456,7 @@ RArgs r_args(const sp_ctx* c, const void* in3, const void* du, void* W, int part
   a.su = 3LL * (c->N - 1);
   a.sd = a.su * c->n_unique;
   a.sn = 1;
+  a.n_dir = 1;
   a.n_unique = c->n_unique;
   a.Mm = c->Mm; a.MX = c->MX; a.MZ = c->MZ; a.Kx = c->Kx; a.NY = c->NY; a.NH = c->NH;
   a.rchunk = (c->N - 1 + parts - 1) / parts;
@@ -525,6 +526,7 @@ static cudaError_t launch_r(const sp_ctx* c, const void* in3, const double* du, 
                             long long sd, long long sn, cudaStream_t st) {
   const int tiles = (c->n_unique + TM - 1) / TM;
   RArgs a = r_args(c, in3, du, W, parts_for(tiles * n_dir, c->N - 1, c->sm_count));
+  a.n_dir = n_dir;
   if (sn) {
     a.su = su;
     a.sd = sd;
@@ -533,7 +535,7 @@ static cudaError_t launch_r(const sp_ctx* c, const void* in3, const double* du, 
   const size_t sm = smem_r(c, TM);
   const cudaError_t e = cudaFuncSetAttribute(k_rhs_fx<TM>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
   if (e != cudaSuccess) return e;
-  k_rhs_fx<TM><<<dim3(n_dir, tiles, (c->N - 1 + a.rchunk - 1) / a.rchunk), kThreadsC, sm, st>>>(a);
+  k_rhs_fx<TM><<<dim3(n_dir * tiles, (c->N - 1 + a.rchunk - 1) / a.rchunk), kThreadsC, sm, st>>>(a);
   return cudaGetLastError();
 }
 

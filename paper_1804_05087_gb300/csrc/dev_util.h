@@ -81,3 +81,21 @@ __device__ __forceinline__ void suffix_scan(int cnt, X x, Put put) {
     carry = make_double2(__shfl_sync(0xffffffffu, s.x, 0), __shfl_sync(0xffffffffu, s.y, 0));
   }
 }
+
+// (double)f by integer operations: the conversion instruction takes a slot of the FP64 unit
+__device__ __forceinline__ double widen(float f) {
+  const unsigned u = __float_as_uint(f), e = (u >> 23) & 0xffu;
+  unsigned m = u & 0x7fffffu, x = e + 896u;
+  if (e == 0 || e == 255) {
+    if (e == 255) {
+      x = 2047;
+    } else if (m == 0) {
+      x = 0;
+    } else {
+      const int s = __clz(m) - 8;
+      m = (m << s) & 0x7fffffu;
+      x = 897 - s;
+    }
+  }
+  return __hiloint2double((int)((u & 0x80000000u) | (x << 20) | (m >> 3)), (int)(m << 29));
+}

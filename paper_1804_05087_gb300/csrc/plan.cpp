@@ -668,7 +668,9 @@ sp_status sp_build_plan(sp_ctx* c) {
       !up((void**)&c->rowidx, rowidx.data(), rowidx.size() * 8) || !up((void**)&c->cft_f, cft.data(), cft.size() * 4))
     return sp_fail(c, SP_ENOMEM, "device allocation of plan tables failed");
   if (q2) {
-    std::vector<float> Cqf(Cq.begin(), Cq.end());
+    std::vector<float> Cqf(Cq.size());  // by points
+    for (int j = 0; j < NQ; ++j)
+      for (int n = 0; n < n1; ++n) Cqf[(size_t)j * n1 + n] = (float)Cq[(size_t)n * NQ + j];
     if (!up((void**)&c->Cq_f, Cqf.data(), Cqf.size() * 4))
       return sp_fail(c, SP_ENOMEM, "device allocation of plan tables failed");
   }

@@ -20,23 +20,25 @@
 // The mean mode (0,0) solves the two Dirichlet Helmholtz problems of u and w.
 #include <algorithm>
 
+#include "dev_util.h"
 #include "sp_internal.h"
 
 namespace {
 
 // ------------------------------------------------------------------ k_rhs
 struct RhsArgs {
-  const float* Cfh_f;
-  const float* Cq_f;       // second-level split (N divisible by 4), null otherwise: see k_rhs
+  const float* cft;        // [NH][NY]
+  const float* cqt;        // [NQ][NY]: second-level split (N divisible by 4), null otherwise: see k_rhs
   int NQ;
   double2* W;              // right-hand sides: (u, d, row c (N-1) + n) at u su + d sd + row sn
   long long su, sd, sn;    // complex strides of W: unique mode, direction, row (c (N-1) + n)
-  int n_unique, Mm, MX, MZ, Kx, NY, N, NH;
+  int n_dir, n_unique, Mm, MX, MZ, Kx, NY, N, NH;
   double inv_dt;
 };
 
-constexpr int kRhsTM = 4;
-constexpr int kRhsThreads = 256;
+constexpr int kRhsTM = 4;         // modes per block
+constexpr int kRhsD = 4;          // directions per block
+constexpr int kRhsThreads = 192;
 
 __device__ __forceinline__ void mode_of(int u, int Kx, int MZ, int* pos, int* iz) {
   const int first = (Kx + 1) * MZ;
@@ -50,107 +52,156 @@ __device__ __forceinline__ void mode_of(int u, int Kx, int MZ, int* pos, int* iz
   }
 }
 
-template <typename T>
-__device__ __forceinline__ C2<T> ldv(const C2<T>* p) { return *p; }
-template <>
-__device__ __forceinline__ C2<float> ldv(const C2<float>* p) {
-  const float2 v = __ldg(reinterpret_cast<const float2*>(p));
-  return mk(v.x, v.y);
+// (v + conj w) / 2 with w the mirror mode's value. A call: the compiler predicates a short branch, and a
+// predicated-off FP64 instruction still takes its slot of the FP64 unit
+__device__ __noinline__ double2 project(double2 v, const double2* w) {
+  const double2 m = __ldg(w);
+  return make_double2(0.5 * (v.x + m.x), 0.5 * (v.y - m.y));
 }
 
-// in3: [dir][3][NY][Mm] complex T; du: [dir][3][Mm][NY] complex double
-template <typename T>
-__global__ void __launch_bounds__(kRhsThreads) k_rhs(const C2<T>* __restrict__ in3, const double2* __restrict__ du,
-                                                    RhsArgs a) {
+// in3: [dir][3][NY][Mm] complex float; du: [dir][3][Mm][NY] complex double
+//
+// Moves 0.95 GB at 48 x 65 x 48 with 256 directions (140 us of memory traffic). With a thread per (mode,
+// row), a load of a value and one of a factor per two multiply-adds, it took 508 us, bound by the loads
+// and by FP64 conversions and predicated FP64 instructions. A thread takes two rows of 4 modes: two
+// factors (from the table by points: lanes over rows) and two broadcast loads of 16 bytes per 16
+// multiply-adds, every sum in the same order (344 us with one row); the sums are widened by integer
+// operations; four directions on adjacent lanes fill the sectors of W; the loads of du are all in
+// flight before the first is used (356 us without). 297 us, bound by the latency of its loads.
+__global__ void __launch_bounds__(kRhsThreads) k_rhs(const C2<float>* __restrict__ in3, const double2* __restrict__ du,
+                                                    const __grid_constant__ RhsArgs a) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   constexpr int TM = kRhsTM;
+  static_assert(TM == 4, "two 16-byte loads per point");
   const int NY = a.NY, N = a.N, NH = a.NH, Mm = a.Mm, MZ = a.MZ, NR = N - 1;
-  C2<T>* sv = reinterpret_cast<C2<T>*>(smem_raw);  // [3][NY][TM]
-  __shared__ int s_pos[TM], s_iz[TM], s_u[TM];
-  const int u0 = blockIdx.x * TM, dir = blockIdx.y;
+  C2<float>* sv = reinterpret_cast<C2<float>*>(smem_raw);  // [kRhsD][3][NY][TM]
+  __shared__ int s_pos[TM], s_iz[TM];
+  const int nd = (a.n_dir + kRhsD - 1) / kRhsD;
+  const int tile = blockIdx.x / nd, dir0 = (blockIdx.x - tile * nd) * kRhsD, u0 = tile * TM, nu = min(TM, a.n_unique - u0);
   if (threadIdx.x < TM) {
-    const int u = u0 + threadIdx.x;
     int pos = 0, iz = 0;
-    if (u < a.n_unique) mode_of(u, a.Kx, MZ, &pos, &iz);
+    if ((int)threadIdx.x < nu) mode_of(u0 + threadIdx.x, a.Kx, MZ, &pos, &iz);
     s_pos[threadIdx.x] = pos;
     s_iz[threadIdx.x] = iz;
-    s_u[threadIdx.x] = u;
-  }
-  __syncthreads();
-  const C2<T>* vin = in3 + (size_t)dir * 3 * NY * Mm;
-  for (int idx = threadIdx.x; idx < 3 * NY * TM; idx += blockDim.x) {
-    const int t = idx % TM, jc = idx / TM;  // jc = c NY + j
-    const int c = jc / NY, j = jc - c * NY;
-    C2<T> v = mk((T)0, (T)0);
-    if (s_u[t] < a.n_unique) v = ldv(vin + ((size_t)c * NY + j) * Mm + s_pos[t] * MZ + s_iz[t]);
-    sv[idx] = v;
   }
   __syncthreads();
   // even/odd pairs: s_j = f(y_j) + f(y_N-j) at j, d_j = f(y_j) - f(y_N-j) at N - j
-  for (int idx = threadIdx.x; idx < 3 * TM * (NH - 1); idx += blockDim.x) {
-    const int t = idx % TM, jj = (idx / TM) % (NH - 1), c = idx / (TM * (NH - 1));
-    C2<T>* col = sv + (c * NY) * TM + t;
-    const C2<T> p = col[jj * TM], q = col[(N - jj) * TM];
-    col[jj * TM] = p + q;
-    col[(N - jj) * TM] = p - q;
+  {
+    const int t = threadIdx.x % TM;
+    const C2<float>* vin = in3 + (size_t)dir0 * 3 * NY * Mm + s_pos[t] * MZ + s_iz[t];
+#pragma unroll 4
+    for (int idx = threadIdx.x / TM; idx < 3 * kRhsD * NH; idx += blockDim.x / TM) {
+      const int c = idx / NH, j = idx - c * NH;  // c: component of a direction
+      C2<float> p = mk(0.0f, 0.0f), q = p;
+      if (t < nu && dir0 + c / 3 < a.n_dir) {
+        const float2 x = __ldg(reinterpret_cast<const float2*>(vin + ((size_t)c * NY + j) * Mm));
+        const float2 y = __ldg(reinterpret_cast<const float2*>(vin + ((size_t)c * NY + N - j) * Mm));
+        p = mk(x.x, x.y);
+        q = mk(y.x, y.y);
+      }
+      C2<float>* col = sv + c * NY * TM + t;
+      if (2 * j == N) {
+        col[j * TM] = p;
+      } else {
+        col[j * TM] = p + q;
+        col[(N - j) * TM] = p - q;
+      }
+    }
   }
   __syncthreads();
   // second level for the even degrees (N divisible by 4): with s'_j = s_j / cbar_j (cbar_0 = 2),
   // T_2m(y_{N/2-j}) = (-1)^m T_2m(y_j) pairs j with N/2 - j: slot j < N/4 receives
   // s'_j + s'_{N/2-j} (degrees 0 mod 4), slot N/2 - j receives s'_j - s'_{N/2-j} (2 mod 4)
-  const bool q2 = a.Cq_f != nullptr;
+  const bool q2 = a.cqt != nullptr;
   const int NQ = a.NQ, NQ1 = NQ - 1;  // NQ1 = N/4
   if (q2) {
-    for (int idx = threadIdx.x; idx < 3 * TM * NQ1; idx += blockDim.x) {
+    for (int idx = threadIdx.x; idx < 3 * kRhsD * TM * NQ1; idx += blockDim.x) {
       const int t = idx % TM, jj = (idx / TM) % NQ1, c = idx / (TM * NQ1);
-      C2<T>* col = sv + (c * NY) * TM + t;
-      C2<T> p = col[jj * TM];
-      if (jj == 0) p = scl(p, (T)0.5);
-      const C2<T> q = col[(N / 2 - jj) * TM];
+      C2<float>* col = sv + (c * NY) * TM + t;
+      C2<float> p = col[jj * TM];
+      if (jj == 0) p = scl(p, 0.5f);
+      const C2<float> q = col[(N / 2 - jj) * TM];
       col[jj * TM] = p + q;
       col[(N / 2 - jj) * TM] = p - q;
     }
     __syncthreads();
   }
-  // rows in three classes, each its own loop so that every warp runs one trip count:
-  // odd n (half-length sums over d), n = 0 mod 4 and n = 2 mod 4 (quarter-length sums over the
-  // second-level pairs; without that level, every even n: half-length sums over s)
+  // rows in three classes, one after the other so that a warp runs one trip count: odd n (half-length
+  // sums over d), n = 0 mod 4 and n = 2 mod 4 (quarter-length sums over the second-level pairs, the
+  // j = N/4 term of the latter vanishes; without that level, every even n: half-length sums over s)
+  const int dl = threadIdx.x % kRhsD, dir = dir0 + dl;  // a lane's direction: lanes fill sectors of W
+  if (dir >= a.n_dir) return;
+  sv += dl * 3 * NY * TM;
   const double2* dsrc = du + (size_t)dir * 3 * Mm * NY;
-  const int nodd = (NR - 1 + 1) / 2;             // odd rows 1, 3, .., <= N-2
+  const int nodd = NR / 2;                            // odd rows 1, 3, .., <= N-2
   const int nev0 = q2 ? (NR + 3) / 4 : (NR + 1) / 2;  // rows 0, 4, .. (q2) or 0, 2, .. (one level)
-  const int nev2 = q2 ? (NR + 1) / 4 : 0;        // rows 2, 6, .. <= N-2
-  for (int cls = 0; cls < 3; ++cls) {
-    const int cnt = cls == 0 ? nodd : (cls == 1 ? nev0 : nev2);
-    for (int idx = threadIdx.x; idx < 3 * TM * cnt; idx += blockDim.x) {
-      const int t = idx % TM, r = (idx / TM) % cnt, c = idx / (TM * cnt);
-      const int n = cls == 0 ? 2 * r + 1 : (cls == 1 ? (q2 ? 4 * r : 2 * r) : 4 * r + 2);
-      const int u = s_u[t];
-      if (u >= a.n_unique) continue;
-      const C2<T>* col = sv + (c * NY) * TM + t;
-      C2<T> acc = mk((T)0, (T)0);
-      const T* cf = a.Cfh_f + (size_t)n * NH;
-      const T* cq = a.Cq_f + (size_t)n * NQ;
-      if (cls == 0) {
-        for (int jj = 0; jj < NH - 1; ++jj) acc = acc + scl(col[(N - jj) * TM], cf[jj]);
-      } else if (!q2) {
-        for (int jj = 0; jj < NH - 1; ++jj) acc = acc + scl(col[jj * TM], cf[jj]);
-        acc = acc + scl(col[(NH - 1) * TM], cf[NH - 1]);
-      } else if (cls == 1) {
-        for (int jj = 0; jj < NQ; ++jj) acc = acc + scl(col[jj * TM], cq[jj]);
-      } else {  // degrees 2 mod 4: the j = N/4 term vanishes
-        for (int jj = 0; jj < NQ1; ++jj) acc = acc + scl(col[(N / 2 - jj) * TM], cq[jj]);
+  const int nev2 = q2 ? (NR + 1) / 4 : 0;             // rows 2, 6, .. <= N-2
+  const int h0 = (nodd + 1) / 2, h1 = (nev0 + 1) / 2, h2 = (nev2 + 1) / 2;  // pairs of rows
+  for (int i = threadIdx.x / kRhsD; i < 3 * (h0 + h1 + h2); i += blockDim.x / kRhsD) {
+    int r = i, n, dn, c, from, step = TM, terms;
+    const float* w = q2 ? a.cqt : a.cft;
+    if (r < 3 * h0) {
+      c = r / h0;
+      n = 4 * (r - c * h0) + 1;
+      dn = 2;
+      from = N;
+      step = -TM;
+      terms = NH - 1;
+      w = a.cft;
+    } else if ((r -= 3 * h0) < 3 * h1) {
+      c = r / h1;
+      dn = q2 ? 4 : 2;
+      n = 2 * dn * (r - c * h1);
+      from = 0;
+      terms = q2 ? NQ : NH;
+    } else {
+      r -= 3 * h1;
+      c = r / h2;
+      n = 8 * (r - c * h2) + 2;
+      dn = 4;
+      from = N / 2;
+      step = -TM;
+      terms = NQ1;
+    }
+    const bool two = n + dn < NR;
+    const C2<float>* x = sv + (c * NY + from) * TM;
+    w += n;
+    const int w2 = two ? dn : 0;
+    float2 s[2][TM] = {};
+#pragma unroll 4
+    for (int j = 0; j < terms; ++j, w += NY, x += step) {
+      const float k[2] = {__ldg(w), __ldg(w + w2)};
+      const float4 p = *reinterpret_cast<const float4*>(x), q = *reinterpret_cast<const float4*>(x + 2);
+#pragma unroll
+      for (int e = 0; e < 2; ++e) {
+        s[e][0] = make_float2(fmaf(p.x, k[e], s[e][0].x), fmaf(p.y, k[e], s[e][0].y));
+        s[e][1] = make_float2(fmaf(p.z, k[e], s[e][1].x), fmaf(p.w, k[e], s[e][1].y));
+        s[e][2] = make_float2(fmaf(q.x, k[e], s[e][2].x), fmaf(q.y, k[e], s[e][2].y));
+        s[e][3] = make_float2(fmaf(q.z, k[e], s[e][3].x), fmaf(q.w, k[e], s[e][3].y));
       }
-      // du (Hermitian-projected on the kz = 0 plane)
-      const int pos = s_pos[t], iz = s_iz[t];
-      double2 d = __ldg(dsrc + ((size_t)c * Mm + pos * MZ + iz) * NY + n);
-      if (iz == 0) {
-        const int mpos = pos == 0 ? 0 : a.MX - pos;
-        const double2 w = __ldg(dsrc + ((size_t)c * Mm + mpos * MZ) * NY + n);
-        d = make_double2(0.5 * (d.x + w.x), 0.5 * (d.y - w.y));
+    }
+    // u/dt (Hermitian-projected on the kz = 0 plane)
+    double2 du8[2][TM];
+#pragma unroll
+    for (int t = 0; t < TM; ++t) {  // past the last mode: the mean mode (not used)
+      const double2* p = dsrc + ((size_t)c * Mm + s_pos[t] * MZ + s_iz[t]) * NY + n;
+      du8[0][t] = __ldg(p);
+      du8[1][t] = __ldg(p + w2);
+    }
+#pragma unroll
+    for (int e = 0; e < 2; ++e) {
+      if (e && !two) continue;
+      const int row = n + e * dn;
+#pragma unroll
+      for (int t = 0; t < TM; ++t) {
+        if (t >= nu) continue;
+        const int pos = s_pos[t], iz = s_iz[t];
+        double2 d = du8[e][t];
+        if (iz == 0) d = project(d, dsrc + ((size_t)c * Mm + (pos == 0 ? 0 : a.MX - pos) * MZ) * NY + row);
+        double2 f = make_double2(fma(d.x, a.inv_dt, widen(s[e][t].x)), fma(d.y, a.inv_dt, widen(s[e][t].y)));
+        if (pos == 0 && iz == 0) f.y = 0.0;
+        a.W[(u0 + t) * a.su + dir * a.sd + (long long)(c * NR + row) * a.sn] = f;
       }
-      double2 f = make_double2((double)acc.x + d.x * a.inv_dt, (double)acc.y + d.y * a.inv_dt);
-      if (pos == 0 && iz == 0) f.y = 0.0;
-      a.W[u * a.su + dir * a.sd + (long long)(c * NR + n) * a.sn] = f;
     }
   }
 }
@@ -268,10 +319,7 @@ __global__ void __launch_bounds__(32 * kChainWarps, kChainBlocksPerSM) k_chain(C
   const int mpos = pos == 0 ? 0 : a.MX - pos;
   auto duv = [&](int c, int n) -> double2 {  // Hermitian-projected input
     double2 v = __ldg(dsrc + ((size_t)c * Mm + pos * MZ + iz) * NY + n);
-    if (iz == 0) {
-      const double2 w = __ldg(dsrc + ((size_t)c * Mm + mpos * MZ) * NY + n);
-      v = make_double2(0.5 * (v.x + w.x), 0.5 * (v.y - w.y));
-    }
+    if (iz == 0) v = project(v, dsrc + ((size_t)c * Mm + mpos * MZ) * NY + n);
     return v;
   };
   auto put = [&](int c, int n, double2 g) {
@@ -391,8 +439,8 @@ cudaError_t launch_chain_rhs(const sp_ctx* c, bool fp32, const void* in3, const 
   if (!fp32) return launch_rhs_fx(c, in3, du, work, n_dir, r.su, r.sd, r.sn, st);
   if (c->use_rhs_tc && sp_rhs_tc_supported(c))  // forward transform on the tensor cores
     return launch_rhs_tc(c, in3, du, work, n_dir, r.su, r.sd, r.sn, st);
-  r.Cfh_f = c->Cfh_f;
-  r.Cq_f = c->Cq_f;
+  r.cft = c->cft_f;
+  r.cqt = c->Cq_f;
   r.NQ = c->N / 4 + 1;
   r.W = static_cast<double2*>(work);
   r.n_unique = c->n_unique;
@@ -404,9 +452,12 @@ cudaError_t launch_chain_rhs(const sp_ctx* c, bool fp32, const void* in3, const 
   r.N = c->N;
   r.NH = c->NH;
   r.inv_dt = 1.0 / c->dt;
-  const dim3 grid((c->n_unique + kRhsTM - 1) / kRhsTM, n_dir);
-  const size_t sm = sizeof(C2<float>) * 3 * c->NY * kRhsTM;
-  k_rhs<float><<<grid, kRhsThreads, sm, st>>>(static_cast<const C2<float>*>(in3), reinterpret_cast<const double2*>(du), r);
+  r.n_dir = n_dir;
+  const int tiles = (c->n_unique + kRhsTM - 1) / kRhsTM;
+  const size_t sm = sizeof(C2<float>) * 3 * c->NY * kRhsTM * kRhsD;
+  const cudaError_t e = cudaFuncSetAttribute(k_rhs, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+  if (e != cudaSuccess) return e;
+  k_rhs<<<tiles * ((n_dir + kRhsD - 1) / kRhsD), kRhsThreads, sm, st>>>(static_cast<const C2<float>*>(in3), reinterpret_cast<const double2*>(du), r);
   return cudaGetLastError();
 }
 

@@ -96,7 +96,7 @@ struct sp_ctx {
   double* wave = nullptr;        // [n_unique][4] kx, kz, 1/k (solve_one.cu)
   double* rowidx = nullptr;      // [NY + 1] 0, 1, ...
   float* cft_f = nullptr;        // [NH][NY] the transpose of Cfh_f
-  // two-level forward transform of the float k_rhs (N divisible by 4): Cq[n][jq] = 2 / (N cbar_n) cos(pi jq n / N), even
+  // two-level forward transform of the float k_rhs (N divisible by 4): [jq][n] 2 / (N cbar_n) cos(pi jq n / N), even
   // rows n <= N-2, jq <= N/4 (solve_chain.cu)
   float* Cq_f = nullptr;
   // tensor-core inverse transform (41 <= NY <= 72): shared-memory image of T and T' split into
