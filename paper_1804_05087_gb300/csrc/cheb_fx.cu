@@ -18,6 +18,7 @@
 #include <cmath>
 #include <vector>
 
+#include "dev_util.h"
 #include "fx_arith.h"
 #include "sp_internal.h"
 
@@ -168,8 +169,16 @@ __device__ __forceinline__ void yinv_fx(const YArgs& a, int bx, int by, int bz, 
   const int j_lo = by * a.jchunk, j_hi = min(a.NH, j_lo + a.jchunk), items = 2 * TM * (j_hi - j_lo);
   const size_t NYMm = (size_t)NY * Mm;
   double2* o = a.out + (size_t)bz * 6 * NYMm;
+  const int t = lane % TM, m = m0 + t;  // a lane keeps its mode
+  double kx = 0.0, kz = 0.0;
+  auto wave = [&] {
+    const int pos = m / a.MZ, iz = m - pos * a.MZ;
+    kx = a.alpha * (pos <= a.Kx ? pos : pos - a.MX);
+    kz = a.beta * iz;
+  };
+  if (TM == kModes) wave();  // many items per lane: once; else it would delay the only sum
   for (int i0 = warp * 32; i0 < items; i0 += kThreadsC) {
-    const int it = i0 + lane, t = it % TM, odd = it / TM & 1, jh = min(j_lo + it / (2 * TM), j_hi - 1), m = m0 + t;
+    const int it = i0 + lane, odd = it / TM & 1, jh = min(j_lo + it / (2 * TM), j_hi - 1);
     Sum2 S[5];
     const int4* tr = reinterpret_cast<const int4*>(a.tab + (size_t)(2 * jh + odd) * PH);
     const int4* td = tr + (size_t)a.NH * PH;  // 2 NH rows of PH / 2 loads
@@ -195,8 +204,7 @@ __device__ __forceinline__ void yinv_fx(const YArgs& a, int bx, int by, int bz, 
     }
     const int j = odd ? N - jh : jh;
     if (it >= items || m >= Mm || (odd && j == jh)) continue;
-    const int pos = m / a.MZ, iz = m - pos * a.MZ;
-    const double kx = a.alpha * (pos <= a.Kx ? pos : pos - a.MX), kz = a.beta * iz;
+    if (TM != kModes) wave();
     double2 v[5];
 #pragma unroll
     for (int f = 0; f < 5; ++f) v[f] = unscale(vx[f], vy[f], sh[f][t]);
@@ -226,7 +234,7 @@ struct RArgs {
   const int2* tab;
   long long su, sd, sn;
   int n_dir, n_unique, Mm, MX, MZ, Kx, NY, NH, rchunk;
-  double inv_dt;
+  double inv_dt, c0, cn;  // 1 / N, 2 / N
 };
 
 __device__ __forceinline__ void unique_mode_of(int u, int Kx, int MZ, int* pos, int* iz) {
@@ -353,14 +361,17 @@ __device__ __forceinline__ void rhs_fx(const RArgs& a, int bx, int by, int bz, i
       }
       x += 2 * ST;
     }
-    const double cn = (n == 0 ? 1.0 : 2.0) / N;  // 2 / (N cbar_n)
+    const double cn = n == 0 ? a.c0 : a.cn;  // 2 / (N cbar_n)
+    double2 du[3], dm[3];
 #pragma unroll
     for (int f = 0; f < 3; ++f) {
-      double2 d = __ldg(dsrc + ((size_t)f * Mm + pos * a.MZ + iz) * NY + n);
-      if (iz == 0) {  // Hermitian projection
-        const double2 w = __ldg(dsrc + ((size_t)f * Mm + mpos * a.MZ) * NY + n);
-        d = make_double2(0.5 * (d.x + w.x), 0.5 * (d.y - w.y));
-      }
+      du[f] = __ldg(dsrc + ((size_t)f * Mm + pos * a.MZ + iz) * NY + n);
+      if (iz == 0) dm[f] = __ldg(dsrc + ((size_t)f * Mm + mpos * a.MZ) * NY + n);
+    }
+#pragma unroll
+    for (int f = 0; f < 3; ++f) {
+      double2 d = du[f];
+      if (iz == 0) d = project(d, dm[f]);
       const double2 v = unscale(S[f].x.value(), S[f].y.value(), s.sh[f * TM + t]);
       double2 g = make_double2(fma(cn, v.x, d.x * a.inv_dt), fma(cn, v.y, d.y * a.inv_dt));
       if (pos == 0 && iz == 0) g.y = 0.0;
@@ -461,6 +472,8 @@ RArgs r_args(const sp_ctx* c, const void* in3, const void* du, void* W, int part
   a.Mm = c->Mm; a.MX = c->MX; a.MZ = c->MZ; a.Kx = c->Kx; a.NY = c->NY; a.NH = c->NH;
   a.rchunk = (c->N - 1 + parts - 1) / parts;
   a.inv_dt = 1.0 / c->dt;
+  a.c0 = 1.0 / c->N;
+  a.cn = 2.0 / c->N;
   return a;
 }
 

@@ -99,3 +99,9 @@ __device__ __forceinline__ double widen(float f) {
   }
   return __hiloint2double((int)((u & 0x80000000u) | (x << 20) | (m >> 3)), (int)(m << 29));
 }
+
+// (v + conj w) / 2 with w the mirror mode's value. A call: the compiler predicates a short branch, and a
+// predicated-off FP64 instruction still takes its slot of the FP64 unit
+static __device__ __noinline__ double2 project(double2 v, double2 w) {
+  return make_double2(0.5 * (v.x + w.x), 0.5 * (v.y - w.y));
+}

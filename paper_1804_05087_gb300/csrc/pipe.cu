@@ -106,11 +106,7 @@ __device__ __forceinline__ void unique_mode_d(int u, int Kx, int MZ, int* pos, i
 // Hermitian projection of entry (c, pos, iz, j) of a state
 __device__ __forceinline__ double2 sym_load(const double2* s, int c, int pos, int iz, int j, const PArgs& a) {
   double2 v = __ldg(s + ((size_t)c * a.Mm + pos * a.MZ + iz) * a.NR + j);
-  if (iz == 0) {
-    const int mpos = pos == 0 ? 0 : a.MX - pos;
-    const double2 w = __ldg(s + ((size_t)c * a.Mm + mpos * a.MZ) * a.NR + j);
-    v = make_double2(0.5 * (v.x + w.x), 0.5 * (v.y - w.y));
-  }
+  if (iz == 0) v = project(v, __ldg(s + ((size_t)c * a.Mm + (pos == 0 ? 0 : a.MX - pos) * a.MZ) * a.NR + j));
   return v;
 }
 

@@ -18,6 +18,11 @@
 //            parity P and G_u, G_w on the rows of parity 1-P. Every row it writes
 //            depends only on its own sweeps, so threads never wait on each other.
 // The mean mode (0,0) solves the two Dirichlet Helmholtz problems of u and w.
+//
+// k_chain is bound by the FP64 unit (87 % busy in its active cycles, 2 operations per SM and clock), so
+// what counts is FP64 instructions per row, predicated ones included: the projection of the kz = 0 plane
+// is a call (1277 -> 1170 us at 48 x 65 x 48, 256 directions), and the factors -k^2, i / k and the
+// difference with the input are folded into the last multiply-adds (1170 -> 1057 us).
 #include <algorithm>
 
 #include "dev_util.h"
@@ -50,13 +55,6 @@ __device__ __forceinline__ void mode_of(int u, int Kx, int MZ, int* pos, int* iz
     *pos = Kx + 1 + v / (MZ - 1);
     *iz = 1 + v % (MZ - 1);
   }
-}
-
-// (v + conj w) / 2 with w the mirror mode's value. A call: the compiler predicates a short branch, and a
-// predicated-off FP64 instruction still takes its slot of the FP64 unit
-__device__ __noinline__ double2 project(double2 v, const double2* w) {
-  const double2 m = __ldg(w);
-  return make_double2(0.5 * (v.x + m.x), 0.5 * (v.y - m.y));
 }
 
 // in3: [dir][3][NY][Mm] complex float; du: [dir][3][Mm][NY] complex double
@@ -197,7 +195,7 @@ __global__ void __launch_bounds__(kRhsThreads) k_rhs(const C2<float>* __restrict
         if (t >= nu) continue;
         const int pos = s_pos[t], iz = s_iz[t];
         double2 d = du8[e][t];
-        if (iz == 0) d = project(d, dsrc + ((size_t)c * Mm + (pos == 0 ? 0 : a.MX - pos) * MZ) * NY + row);
+        if (iz == 0) d = project(d, __ldg(dsrc + ((size_t)c * Mm + (pos == 0 ? 0 : a.MX - pos) * MZ) * NY + row));
         double2 f = make_double2(fma(d.x, a.inv_dt, widen(s[e][t].x)), fma(d.y, a.inv_dt, widen(s[e][t].y)));
         if (pos == 0 && iz == 0) f.y = 0.0;
         a.W[(u0 + t) * a.su + dir * a.sd + (long long)(c * NR + row) * a.sn] = f;
@@ -319,7 +317,7 @@ __global__ void __launch_bounds__(32 * kChainWarps, kChainBlocksPerSM) k_chain(C
   const int mpos = pos == 0 ? 0 : a.MX - pos;
   auto duv = [&](int c, int n) -> double2 {  // Hermitian-projected input
     double2 v = __ldg(dsrc + ((size_t)c * Mm + pos * MZ + iz) * NY + n);
-    if (iz == 0) v = project(v, dsrc + ((size_t)c * Mm + mpos * MZ) * NY + n);
+    if (iz == 0) v = project(v, __ldg(dsrc + ((size_t)c * Mm + mpos * MZ) * NY + n));
     return v;
   };
   auto put = [&](int c, int n, double2 g) {
@@ -355,12 +353,13 @@ __global__ void __launch_bounds__(32 * kChainWarps, kChainBlocksPerSM) k_chain(C
   const double* rQ = rec + Q * a.par;
   const int m = (N - P) / 2;
 
-  // (1) w_A: (lam - nu D^2) w = -k^2 g on the rows of parity P, w(+-1) = 0, with the
+  // All of (1) to (4) is divided by -k^2: the factor goes into the last products.
+  // (1) w_A: (lam - nu D^2) w = g on the rows of parity P, w(+-1) = 0, with the
   // reduced right-hand side g_n = f_v,n - (2 / (c_n k)) S_n, S_n = sum over rows
   // m' > n of parity Q of m' f~_a,m' (f~_a = -i f_a), built while the sweep descends
   double2 S = zero;
   int next_add = 2 * m + P - 1;  // the next row m' of parity Q to add to S
-  auto gneg = [&](int n) -> double2 {  // -k^2 g_n, called for n = top, then descending
+  auto gred = [&](int n) -> double2 {  // g_n, called for n = top, then descending
     if (n > N - 2) return zero;
     while (next_add > n) {
       if (next_add <= N - 2) {
@@ -371,10 +370,9 @@ __global__ void __launch_bounds__(32 * kChainWarps, kChainBlocksPerSM) k_chain(C
       next_add -= 2;
     }
     const double2 fv = fval(1, n);
-    const double2 g = caxpy(fv, S, n == 0 ? -ik : -ik2);
-    return cscl(g, -k2);
+    return caxpy(fv, S, n == 0 ? -ik : -ik2);
   };
-  const double2 wtop = tri_sweep(rP, rP[14 * NH], N, P, gneg, zero, S1, st);
+  const double2 wtop = tri_sweep(rP, rP[14 * NH], N, P, gred, zero, S1, st);
   // (2) v_A: (D^2 - k^2) v = w_A on the rows <= N-2 of parity P, v(+-1) = 0
   const double2 vtop = tri_sweep(rP + 6 * NH, rP[14 * NH + 1], N, P,
                                  [&](int n) { return n <= N - 2 ? S1[((n - P) >> 1) * st] : zero; }, zero, S2, st2);
@@ -386,7 +384,7 @@ __global__ void __launch_bounds__(32 * kChainWarps, kChainBlocksPerSM) k_chain(C
   const double2 sig = cmix(e1, -sc[2], e2, -sc[3]);
   const double2 tau = cmix(e1, -sc[4], e2, -sc[5]);
   // (4) v = v_A + sigma v_psi + tau v_h, G_v on the rows of parity P; a = (i/k) D v on the
-  // rows of parity Q by a suffix sum, stored in S2 (slot i holds a_{2i+P-1})
+  // rows of parity Q by a suffix sum, kept in S2 (slot i holds the sum of a_{2i+P-1})
   const double* v2 = rP + 12 * NH;
   double2 Sa = zero;
   for (int i = m; i >= 0; --i) {
@@ -394,25 +392,26 @@ __global__ void __launch_bounds__(32 * kChainWarps, kChainBlocksPerSM) k_chain(C
     double2 v = S2[i * st2];
     v = caxpy(v, sig, v2[2 * i]);
     v = caxpy(v, tau, v2[2 * i + 1]);
-    put(1, n, csub(v, duv(1, n)));
+    const double2 d = duv(1, n);
+    put(1, n, make_double2(fma(v.x, -k2, -d.x), fma(v.y, -k2, -d.y)));
     Sa = caxpy(Sa, v, kRow.n[n]);
-    if (n >= 1) {
-      const double f = n - 1 == 0 ? ik : ik2;  // (i/k)(2/c_{n-1}) Sa
-      S2[i * st2] = make_double2(-Sa.y * f, Sa.x * f);
-    }
+    if (n >= 1) S2[i * st2] = Sa;
   }
+  if (P == 1) S2[0] = cscl(S2[0], 0.5);  // 1 / c_0
   // (5) b of parity Q: (lam - nu D^2) b = f_b, b(+-1) = 0; then u = cx a - cz b,
   // w = cz a + cx b and G_u, G_w on the rows of parity Q
   tri_sweep(rQ, rQ[14 * NH], N, Q,
             [&](int n) { return cmix(fval(0, n), -cz, fval(2, n), cx); }, zero, S1, st);
   const int mq = (N - Q) / 2;
+  const double ax = -k2 * ik2 * cx, az = -k2 * ik2 * cz;  // a_n = (i/k)(2/c_n)(-k^2) S_n along x, z
   for (int i = 0; i <= mq; ++i) {
     const int n = 2 * i + Q;
     const int ia = P == 0 ? i + 1 : i;  // slot of a_n in S2
     const double2 an = (ia <= m) ? S2[ia * st2] : zero;
     const double2 bn = S1[i * st];
-    put(0, n, csub(cmix(an, cx, bn, -cz), duv(0, n)));
-    put(2, n, csub(cmix(an, cz, bn, cx), duv(2, n)));
+    const double2 du0 = duv(0, n), du2 = duv(2, n);
+    put(0, n, make_double2(fma(-an.y, ax, fma(bn.x, -cz, -du0.x)), fma(an.x, ax, fma(bn.y, -cz, -du0.y))));
+    put(2, n, make_double2(fma(-an.y, az, fma(bn.x, cx, -du2.x)), fma(an.x, az, fma(bn.y, cx, -du2.y))));
   }
 }
 

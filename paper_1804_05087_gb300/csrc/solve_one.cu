@@ -101,10 +101,7 @@ __device__ __forceinline__ void solve_one(const OneArgs& a, int u, int dir, unsi
     const int c = i / NY;
     const double2* p = dsrc + (size_t)c * Mm * NY + (i - c * NY);
     double2 v = __ldg(p);
-    if (iz == 0) {
-      const double2 w = __ldg(p + mir);
-      v = make_double2(0.5 * (v.x + w.x), 0.5 * (v.y - w.y));
-    }
+    if (iz == 0) v = project(v, __ldg(p + mir));
     sdu[i] = v;
   }
   if constexpr (sizeof(T) == 8) {
