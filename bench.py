@@ -197,11 +197,11 @@ def kernel_flops(stage, n_dir, prec="mixed"):
         return n_dir * n_unique() * per
     if stage == "k_solve" and chain(n_dir):
         # O(N) chains, FP64, per (mode, parity) thread and coefficient: the w_A sweep with the
-        # reduced right-hand side (38 flops), the v_A sweep (22), the influence correction,
+        # reduced right-hand side (36 flops), the v_A sweep (22), the influence correction,
         # G_v and the continuity suffix sum (20), the b sweep with the back-rotation and
-        # G_u, G_w (44): 124 flops per coefficient, NH coefficients per parity. A sweep step
+        # G_u, G_w (44): 122 flops per coefficient, NH coefficients per parity. A sweep step
         # is 18 flops (the row weights folded into the records) and a substitution step 4.
-        return n_dir * n_unique() * 2 * nh * 124
+        return n_dir * n_unique() * 2 * nh * 122
     if stage == "k_solve":
         # FP64 work: the per-mode operators (real matrices on complex right-hand sides,
         # 4 flops per entry), the reduced right-hand side g (one complex FMA and one complex
@@ -230,16 +230,7 @@ def kernel_traffic(stage, n_dir, prec, lam_adv):
     """DRAM bytes of one launch from an ncu capture of the current kernel, or None."""
     if stage == "k_solve" and prec == "mixed" and not lam_adv and not chain(n_dir):
         return solve_traffic(n_dir)
-    if stage == "k_xz" and prec == "fp64" and not lam_adv and (NX, NY, NZ) == (48, 65, 48):
-        rd, wr = K_XZ64_DRAM_64  # every byte scales with the directions (one plane per block)
-        return (rd + wr) * n_dir / 64
     return None
-
-
-# DRAM bytes of one FP64 tangent launch of the register plane stage k_xz_reg64<48, 48> at
-# 48x65x48 with 64 directions (dram__bytes_read.sum, dram__bytes_write.sum of that launch;
-# the kernel with the packed row pairs of phase 1 and the quarter-turn twiddles)
-K_XZ64_DRAM_64 = (205629696, 68856832)
 
 
 # DRAM bytes of one mixed-precision k_solve tangent launch at 48x65x48 with 64 directions, from
@@ -1358,14 +1349,18 @@ def throughput(args, prec_name, rank, world, local, keep_out=False, e2e=True):
     tfs = flops_l / avg_s / 1e12
     hbm = peaks["hbm_gbs"]
     fp32_peak = 152 * 128 * 2 * 2.07e9 / 1e12  # SMs x FP32 lanes x FMA x max clock
-    fp64_bound = prec_name == "fp64" or dom == "k_solve"  # the solve is FP64 in both modes
-    alu_peak = FP64_NOMINAL if fp64_bound else fp32_peak
+    fp64_bound = dom == "k_solve"  # the solve is FP64 in both modes
+    # FP64 transforms run in 64-bit fixed point: three 32-bit multiply-adds with a 64-bit sum per real
+    # multiply-add, 32 of them per SM and clock
+    int_peak = 152 * 32 * 2.07e9 * 2 / 3 / 1e12
+    alu_peak = FP64_NOMINAL if fp64_bound else int_peak if prec_name == "fp64" else fp32_peak
     if gbs / hbm >= tfs / alu_peak:
         roof = {"bound": "hbm", "achieved": gbs, "peak": hbm, "unit": "GB/s", "frac": gbs / hbm,
                 "peak_source": "measured (MEASURED_PEAKS.json hbm_gbs)"}
     else:
         roof = {"bound": "alu", "achieved": tfs, "peak": alu_peak, "unit": "TFLOP/s", "frac": tfs / alu_peak,
                 "peak_source": f"nominal FP64 {FP64_NOMINAL} TFLOP/s" if fp64_bound
+                else "152 SMs x 32 wide integer multiply-adds / 3 x 2 flop x 2.07 GHz" if prec_name == "fp64"
                 else "152 SMs x 128 FP32 lanes x 2 flop x 2.07 GHz", "fp64": fp64_bound}
     roof.update({"kernel": dom, "traffic": kernel_traffic(dom, nd, prec_name, bool(args.lam_adv)),
                  "avg_launch_ms": dom_ms / dom_n,

@@ -1,5 +1,4 @@
-// Compile-time register FFTs shared by the plane-stage kernels (xz_reg.cu: float,
-// xz_reg64.cu: double).
+// Compile-time register FFTs of the float plane-stage kernels (xz_reg.cu).
 //
 // The FFT is a decimation-in-frequency Cooley-Tukey recursion with radices
 // 4, 3 and 2 fully unrolled at compile time: inputs in natural order, outputs

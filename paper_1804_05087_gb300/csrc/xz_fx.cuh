@@ -4,8 +4,9 @@
 // forward FFT along x truncated to the retained modes. Values in and out are doubles; in between
 // they are integers with one power-of-two scale per stage (fx_arith.h).
 //
-// Why integers: the FP64 pipe issues 2 operations per SM and clock, the integer pipes 64
-// multiply-adds or additions, and a plane's transforms need no range, only precision.
+// Why integers: the FP64 pipe issues 2 operations per SM and clock, the integer pipes about 28 multiply-
+// adds of 32-bit halves or 52 additions of 64 bits (measured), and a plane's transforms need no range,
+// only precision. 48 x 65 x 48, 256 tangents: 12.57 ms in FP64 registers, 3.11 ms here.
 //
 // Scales (every transformed value stays below 2^61). The x transforms of a group of fields
 // (velocity, vorticity) are scaled by the largest sum of moduli of a column, the z transforms by
