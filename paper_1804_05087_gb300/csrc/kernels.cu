@@ -533,11 +533,7 @@ __device__ __forceinline__ void solve_body(const C2<T>* __restrict__ in3, const 
     if (s_u[t] < a.n_unique) {
       const int pos = s_pos[t], iz = s_iz[t];
       v = __ldg(dsrc + ((size_t)c * Mm + pos * MZ + iz) * NY + n);
-      if (iz == 0) {
-        const int mpos = pos == 0 ? 0 : a.MX - pos;
-        const double2 w = __ldg(dsrc + ((size_t)c * Mm + mpos * MZ) * NY + n);
-        v = make_double2(0.5 * (v.x + w.x), 0.5 * (v.y - w.y));
-      }
+      if (iz == 0) v = project(v, __ldg(dsrc + ((size_t)c * Mm + (pos == 0 ? 0 : a.MX - pos) * MZ) * NY + n));
     }
     sdu[(c * TM + t) * NY + n] = v;
   }
@@ -603,7 +599,7 @@ __device__ __forceinline__ void solve_body(const C2<T>* __restrict__ in3, const 
       for (int jj = 0; jj < NH - 1; ++jj) acc = acc + scl(col[(N - jj) * TM], (T)cf[jj]);
     }
     const double2 d = sdu[(c * TM + t) * NY + n];
-    double2 f = make_double2((double)acc.x + d.x * a.inv_dt, (double)acc.y + d.y * a.inv_dt);
+    double2 f = make_double2(fma(d.x, a.inv_dt, widen(acc.x)), fma(d.y, a.inv_dt, widen(acc.y)));
     add_lam(f, c, t, n);
     if (s_pos[t] == 0 && s_iz[t] == 0) f.y = 0.0;
     sf[(c * TM + t) * NR + n] = f;
@@ -1396,7 +1392,9 @@ static SolveArgs solve_args(const sp_ctx* c) {
 // tile shapes of k_solve: (modes per block, threads per block); the autotuner picks one. Shape 0, the
 // default, has a thread per solved row (threads = 0: TM * NY rounded up to a whole warp, at most
 // 1024): with 128 threads for 4 modes of 35 rows the second round held 12 of 140 rows, and an FP64
-// instruction costs a scheduler 64 cycles whatever the lanes.
+// instruction costs a scheduler 64 cycles whatever the lanes. us, a thread per row | 128 threads, 16
+// directions and one: 48 x 35 x 48 224 | 230, 33 | 43; 48 x 65 x 48 607 | 650, 60 | 91; 24 x 25 x 24
+// the same.
 struct SolveShape {
   int tm, threads;
 };
