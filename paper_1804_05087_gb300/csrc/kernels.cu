@@ -525,17 +525,31 @@ __device__ __forceinline__ void solve_body(const C2<T>* __restrict__ in3, const 
       svals[idx] = v;
     }
   }
-  for (int idx = threadIdx.x; idx < 3 * TM * NY; idx += blockDim.x) {
-    const int n = idx % NY;
-    const int t = (idx / NY) % TM;
-    const int c = idx / (NY * TM);
-    double2 v = make_double2(0.0, 0.0);
-    if (s_u[t] < a.n_unique) {
+  // (the loads of kLoads rounds are in flight together: the projection is a call)
+  constexpr int kLoads = 3;
+  for (int i0 = threadIdx.x; i0 < 3 * TM * NY; i0 += kLoads * blockDim.x) {
+    double2 v[kLoads], w[kLoads];
+    int herm = 0;
+#pragma unroll
+    for (int q = 0; q < kLoads; ++q) {
+      const int idx = i0 + q * blockDim.x;
+      v[q] = make_double2(0.0, 0.0);
+      if (idx >= 3 * TM * NY) continue;
+      const int ct = idx / NY, n = idx - ct * NY, t = ct % TM, c = ct / TM;
+      if (s_u[t] >= a.n_unique) continue;
       const int pos = s_pos[t], iz = s_iz[t];
-      v = __ldg(dsrc + ((size_t)c * Mm + pos * MZ + iz) * NY + n);
-      if (iz == 0) v = project(v, __ldg(dsrc + ((size_t)c * Mm + (pos == 0 ? 0 : a.MX - pos) * MZ) * NY + n));
+      v[q] = __ldg(dsrc + ((size_t)c * Mm + pos * MZ + iz) * NY + n);
+      if (iz == 0) {
+        w[q] = __ldg(dsrc + ((size_t)c * Mm + (pos == 0 ? 0 : a.MX - pos) * MZ) * NY + n);
+        herm |= 1 << q;
+      }
     }
-    sdu[(c * TM + t) * NY + n] = v;
+#pragma unroll
+    for (int q = 0; q < kLoads; ++q) {
+      const int idx = i0 + q * blockDim.x;
+      if (idx >= 3 * TM * NY) continue;
+      sdu[idx] = herm >> q & 1 ? project(v[q], w[q]) : v[q];
+    }
   }
   __syncthreads();
   // + M du on the momentum rows of the laminar-advection step: i kx (Y du)_n, and dv_n in the
@@ -1391,20 +1405,22 @@ static SolveArgs solve_args(const sp_ctx* c) {
 
 // tile shapes of k_solve: (modes per block, threads per block); the autotuner picks one. Shape 0, the
 // default, has a thread per solved row (threads = 0: TM * NY rounded up to a whole warp, at most
-// 1024): with 128 threads for 4 modes of 35 rows the second round held 12 of 140 rows, and an FP64
+// 1024) and at least 128 (threads = -128: the suffix sums take 8 warps' turns, and 96 threads made
+// 32 x 21 x 32 with 4 directions 40 -> 44 us): with 128 threads for 4 modes of 35 rows the second round held 12 of 140 rows, and an FP64
 // instruction costs a scheduler 64 cycles whatever the lanes. us, a thread per row | 128 threads, 16
 // directions and one: 48 x 35 x 48 224 | 230, 33 | 43; 48 x 65 x 48 607 | 650, 60 | 91; 24 x 25 x 24
 // the same.
 struct SolveShape {
   int tm, threads;
 };
-constexpr SolveShape kSolveShapes[SP_TUNE_MAX] = {{4, 0}, {2, 64}, {8, 256}, {4, 192},
+constexpr SolveShape kSolveShapes[SP_TUNE_MAX] = {{4, -128}, {2, 64}, {8, 256}, {4, 192},
                                                   {16, 512}, {2, 0}, {4, 128}, {8, 0}};
 constexpr int kNumSolveShapes = 8;
 
 static int shape_threads(const sp_ctx* c, int shape) {
   const SolveShape sh = kSolveShapes[shape];
-  return sh.threads > 0 ? sh.threads : std::min((sh.tm * c->NY + 31) / 32 * 32, 1024);
+  const int rows = std::min((sh.tm * c->NY + 31) / 32 * 32, 1024);
+  return sh.threads > 0 ? sh.threads : std::max(rows, -sh.threads);
 }
 
 template <typename T, int TM, int MAXT>
