@@ -33,28 +33,13 @@ constexpr int kModes = 8, kModesFew = 4;
 // columns of a block's rows: u, v, w, Du, Dw (values: the three components) of every mode, padded
 __host__ __device__ constexpr int stride_y(int tm) { return 5 * tm + 1; }
 __host__ __device__ constexpr int stride_r(int tm) { return 3 * tm + 1; }
-constexpr int kSumBits = 62, kMaxBits = 59;     // bits of a column's sum of moduli and of its values
 constexpr int kNotFinite = 1 << 28;             // exponent of a column with a non-finite input
 
-// x = hi 2^28 + lo, both signed
-__device__ __forceinline__ int2 halves(i64 x) {
-  const i64 hi = (x + (1 << 27)) >> 28;
-  return make_int2((int)hi, (int)(x - (hi << 28)));
-}
 __device__ __forceinline__ int4 halves2(i64 x, i64 y) {
-  const int2 a = halves(x), b = halves(y);
+  const int2 a = halves28(x), b = halves28(y);
   return make_int4(a.x, a.y, b.x, b.y);
 }
 
-// sum of x c: c in units of 2^-56 as halves
-struct Sum {
-  i64 m = 0, h = 0;
-  __device__ __forceinline__ void add(int xh, int xl, int2 c) {
-    m = wide(xh, c.x, m);
-    h = wide(xh, c.y, wide(xl, c.x, h));
-  }
-  __device__ __forceinline__ i64 value() const { return m + ((h + (1 << 27)) >> 28); }
-};
 struct Sum2 {  // complex columns
   Sum x, y;
   __device__ __forceinline__ void add(int4 v, int2 c) {
@@ -65,16 +50,6 @@ struct Sum2 {  // complex columns
 
 __device__ __forceinline__ unsigned top_of(double2 v) {
   return max((unsigned)__double2hiint(v.x) & 0x7fffffffu, (unsigned)__double2hiint(v.y) & 0x7fffffffu);
-}
-// |v| rounded up, in units of 2^(e - 1037), 15 bits
-__device__ __forceinline__ int part_of(double v, int e) {
-  const unsigned h = (unsigned)__double2hiint(v) & 0x7fffffffu;
-  return (int)(((h & 0xfffffu) | 0x100000u) >> min(31, e - (int)(h >> 20) + 6)) + 1;
-}
-// exponent that scales values of at most top 2^(e - 1037), whose moduli sum to s 2^(e - 1037)
-__device__ __forceinline__ int exponent_of(u64 s, u64 top, int e) {
-  const int bs = 64 - __clzll((i64)(s | 1)), bt = 64 - __clzll((i64)(top | 1));
-  return min(kSumBits - bs, kMaxBits - bt) - (e - 1037);
 }
 // round(v f 2^sh), f a small integer
 __device__ __forceinline__ i64 from_double_times(double v, int sh, double f) {
@@ -314,8 +289,7 @@ __device__ __forceinline__ void rhs_fx(const RArgs& a, int bx, int by, int bz, i
   __syncthreads();
   if (tid < 3 * TM) {
     const int e = (int)(s.em[tid] >> 20);
-    // values below 2^(e - 1022); the parts of a pair below twice that
-    s.sh[tid] = e == 0x7ff ? kNotFinite : exponent_of((u64)s.sum[tid], 0xffff, e);
+    s.sh[tid] = e == 0x7ff ? kNotFinite : exponent_of((u64)s.sum[tid], pair_top(s.em[tid]), e);
   }
   __syncthreads();
   // even and odd parts of the point pairs (j, N - j), in place; the end points enter with half weight

@@ -9,6 +9,9 @@
 
 #include <cuda_runtime.h>
 
+#include <cmath>
+#include <cstring>
+
 namespace fx {
 
 using i64 = long long;
@@ -175,14 +178,43 @@ __host__ __device__ __forceinline__ void dft(cx (&v)[R]) {
 }
 
 // ------------------------------------------------------------ conversions
+// words of a double, on either side
+__host__ __device__ __forceinline__ unsigned high_word(double v) {
+#ifdef __CUDA_ARCH__
+  return (unsigned)__double2hiint(v);
+#else
+  u64 b;
+  std::memcpy(&b, &v, 8);
+  return (unsigned)(b >> 32);
+#endif
+}
+// v 2^sh by an addition to the exponent field
+__host__ __device__ __forceinline__ double add_exponent(double v, int sh) {
+#ifdef __CUDA_ARCH__
+  return __hiloint2double(__double2hiint(v) + sh * (1 << 20), __double2loint(v));
+#else
+  u64 b;
+  std::memcpy(&b, &v, 8);
+  b += (u64)(i64)sh << 52;
+  std::memcpy(&v, &b, 8);
+  return v;
+#endif
+}
+__host__ __device__ __forceinline__ i64 round_double(double v) {
+#ifdef __CUDA_ARCH__
+  return __double2ll_rn(v);
+#else
+  return llrint(v);
+#endif
+}
+
 // round(v 2^sh), |v| 2^sh < 2^61. One operation of the FP64 pipe, which the rest leaves idle; the
 // scaling is an addition to the exponent field (values that it would take below 1 round to 0, as
 // do subnormal v).
-__device__ __forceinline__ i64 from_double(double v, int sh) {
-  const int hi = __double2hiint(v), e = (hi >> 20) & 0x7ff;
+__host__ __device__ __forceinline__ i64 from_double(double v, int sh) {
+  const int e = (int)(high_word(v) >> 20) & 0x7ff;
   const bool in = e != 0 && e + sh > 1000;
-  const double d = __hiloint2double(hi + sh * (1 << 20), __double2loint(v));
-  return in ? __double2ll_rn(d) : 0;
+  return in ? round_double(add_exponent(v, sh)) : 0;
 }
 
 // X 2^-sh, integer operations only in the normal range (rounded to nearest)
@@ -227,6 +259,44 @@ __device__ __forceinline__ i64 shift(i64 v, int l) {
 }
 // v / 2^k rounded, 0 <= k <= 62
 __device__ __forceinline__ i64 shift_down(i64 v, int k) { return (v + ((1ll << k) >> 1)) >> k; }
+
+// ------------------------------------------------------------ columns of the Chebyshev transforms
+// x = hi 2^28 + lo, both signed; |x| < 2^59 - 2^27, so that hi, which is rounded, stays below 2^31
+__host__ __device__ __forceinline__ int2 halves28(i64 x) {
+  const i64 hi = (x + (1 << 27)) >> 28;
+  return int2{(int)hi, (int)(x - hi * (1 << 28))};
+}
+// sum of x c: c in units of 2^-56 as halves
+struct Sum {
+  i64 m = 0, h = 0;
+  __host__ __device__ __forceinline__ void add(int xh, int xl, int2 c) {
+    m = wide(xh, c.x, m);
+    h = wide(xh, c.y, wide(xl, c.x, h));
+  }
+  __host__ __device__ __forceinline__ i64 value() const { return m + ((h + (1 << 27)) >> 28); }
+};
+constexpr int kSumBits = 62, kMaxBits = 59;  // bits of a column's sum of moduli and of its values
+// |v| rounded up, in units of 2^(e - 1037), 15 bits or 2^15
+__host__ __device__ __forceinline__ int part_of(double v, int e) {
+  const unsigned h = high_word(v) & 0x7fffffffu;
+  const int d = e - (int)(h >> 20) + 6;
+  return (int)(((h & 0xfffffu) | 0x100000u) >> (d < 31 ? d : 31)) + 1;
+}
+// a bound of p + q of two values whose high words are at most em, in units of 2^(e - 1037): twice the
+// part of the largest (2^16 where that is rounded up to a power of two, which takes a bit more)
+__host__ __device__ __forceinline__ u64 pair_top(unsigned em) {
+  return 2 * (u64)((((em & 0xfffffu) | 0x100000u) >> 6) + 1);
+}
+// exponent that scales values of at most top 2^(e - 1037), whose moduli sum to s 2^(e - 1037)
+__host__ __device__ __forceinline__ int exponent_of(u64 s, u64 top, int e) {
+#ifdef __CUDA_ARCH__
+  const int bs = 64 - __clzll((i64)(s | 1)), bt = 64 - __clzll((i64)(top | 1));
+#else
+  const int bs = 64 - __builtin_clzll(s | 1), bt = 64 - __builtin_clzll(top | 1);
+#endif
+  const int a = kSumBits - bs, b = kMaxBits - bt;
+  return (a < b ? a : b) - (e - 1037);
+}
 
 // n / d for n < 2^16 by a precomputed reciprocal
 struct Div {
