@@ -232,8 +232,14 @@ sp_status sp_jvp_n(sp_ctx* ctx, const double* du, double* Jdu, int n_dir, void* 
  * The first call on each device looks up the array's device address; make
  * that first call before any stream capture. All calls share the one array:
  * calls whose work overlaps on the GPU (other streams, other host threads)
- * race on it and must be serialised by the caller. Every intermediate value
- * is written before it is read, so nothing has to be cleared between calls. */
+ * race on it and must be serialised by the caller. The context's other calls
+ * may run beside it (the base must not change meanwhile), except on grids
+ * whose planes fit neither into the shared memory of a multiprocessor
+ * (96 nx MZ bytes in FP64, 48 nx (MZ + 1) in mixed precision, above about
+ * 190 KB) nor, in FP64, twice with the values above into the 8 MiB: there the
+ * plane stage goes through a buffer of the context, and the call must be
+ * ordered with them too. Every intermediate value is written before it is
+ * read, so nothing has to be cleared between calls. */
 sp_status sp_jvp_static(sp_ctx* ctx, const double* du, double* Jdu, void* stream);
 
 /* ---- vector operations in the inner product above ---------------------- */

@@ -9,7 +9,10 @@
 // committed to its own pool allocator (a further cudaMalloc may fail or
 // fragment that reservation), or code on a latency-critical path where
 // cudaMalloc/cudaFree would stall other streams with an implicit device
-// synchronisation.
+// synchronisation. It reads the context's plan and base but writes none of its
+// buffers, so that it can run beside the context's other calls; the exceptions are
+// grids whose planes fit neither on chip nor (FP64) into the static array, where the
+// plane stage uses the context's plane buffer.
 #include <mutex>
 
 #include "sp_internal.h"
@@ -70,7 +73,13 @@ extern "C" sp_status sp_jvp_static(sp_ctx* c, const double* du, double* Jdu, voi
   // every entry of both intermediates is written before it is read, so the
   // contents left by an earlier call need no clearing
   if ((s = sp_cuda(c, launch_yinv(c, f32, du, ws6, 1, st), "yinv")) != SP_OK) return s;
-  if ((s = sp_cuda(c, launch_xz(c, f32, XZ_TANGENT, ws6, ws3, 1, st), "xz tangent")) != SP_OK) return s;
+  // FP64 planes stay out of the context's buffers: on chip (48 x 65 x 48: 60 us against 42 with several
+  // blocks per plane through the context's buffer, where an sp_step on another stream could write) or
+  // behind ws3, which the solve's scratch takes over afterwards
+  const cudaError_t e = !f32 && c->use_fx ? launch_xz_fx_apart(c, XZ_TANGENT, ws6, ws3, p + b6 + b3,
+                                                               kStaticScratchBytes - b6 - b3, st)
+                                          : launch_xz(c, f32, XZ_TANGENT, ws6, ws3, 1, st);
+  if ((s = sp_cuda(c, e, "xz tangent")) != SP_OK) return s;
   // the second part runs to the end of the array: the chains' scratch may use all of it
   return sp_tangent_solve(c, f32, ws3, kStaticScratchBytes - b6, du, Jdu, ws6, 1, st);
 }

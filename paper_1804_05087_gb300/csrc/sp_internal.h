@@ -291,6 +291,10 @@ size_t yinv_tc_smem(int NY);
 // fixed-point plane stage (xz_fx.cu): every FP64 mode; setup sets use_fx when the grid is covered
 sp_status sp_fx_setup(sp_ctx* c);
 cudaError_t launch_xz_fx(const sp_ctx* c, int mode, const void* in, void* out, int n_dir, cudaStream_t st);
+// one direction without the context's plane buffers: in one launch where a plane fits on chip, else through
+// scratch where that holds the planes (else, and only then, through the context's)
+cudaError_t launch_xz_fx_apart(const sp_ctx* c, int mode, const void* in, void* out, void* scratch, size_t bytes,
+                               cudaStream_t st);
 // batched tangent solve by O(N) chains (solve_chain.cu), two launches: k_rhs (values ->
 // right-hand sides in work, n_unique x 3 x (N-1) complex per direction), then k_chain
 // (one thread per mode, parity and direction); together the same inputs and outputs as

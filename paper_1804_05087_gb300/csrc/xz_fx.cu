@@ -118,7 +118,7 @@ sp_status sp_fx_setup(sp_ctx* c) {
   for (int d = c->cfg.max_batch; d >= 1 && !split_dirs; --d)
     if (use_split(c, XZ_TANGENT, d) || use_split(c, XZ_ADJOINT, d)) split_dirs = d;
   const size_t nplanes = std::max<size_t>((size_t)c->NY * split_dirs, 1);
-  const size_t meta = 5 + 4 * (size_t)chunks;  // the adjoint has the most chunks
+  const size_t meta = meta_ints(chunks);  // the adjoint has the most chunks
   bool ok = cudaMalloc((void**)&c->fx_tw, tw.size() * 16) == cudaSuccess &&
             cudaMemcpy(c->fx_tw, tw.data(), tw.size() * 16, cudaMemcpyHostToDevice) == cudaSuccess &&
             cudaMalloc(&c->fx_G, nplanes * plane_bytes(c)) == cudaSuccess &&
@@ -148,6 +148,18 @@ static cudaError_t launch_args(const sp_ctx* c, const Args& a, int mode, int n_d
 
 cudaError_t launch_xz_fx(const sp_ctx* c, int mode, const void* in, void* out, int n_dir, cudaStream_t st) {
   return launch_args(c, make_args(c, mode, in, out), mode, n_dir, use_split(c, mode, n_dir), st);
+}
+
+cudaError_t launch_xz_fx_apart(const sp_ctx* c, int mode, const void* in, void* out, void* scratch, size_t bytes,
+                               cudaStream_t st) {
+  Args a = make_args(c, mode, in, out);
+  const bool split = fused_smem(c, mode) > kSmemMax;
+  const size_t planes = (size_t)c->NY * plane_bytes(c);
+  if (split && planes + c->NY * meta_ints(a.nchunk) * 4 <= bytes) {
+    a.G = static_cast<cx*>(scratch);
+    a.gmeta = reinterpret_cast<int*>(static_cast<unsigned char*>(scratch) + planes);
+  }
+  return launch_args(c, a, mode, 1, split, st);
 }
 
 // ------------------------------------------------------------------ groups

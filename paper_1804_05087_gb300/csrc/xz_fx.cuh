@@ -50,7 +50,7 @@ struct Args {
   const double* lam;   // [NY][6] laminar U and Omega
   const int4* tw;      // [nx] then [nz]: cos, sin of 2 pi k / n as halves of 62-bit constants
   cx* G;               // split launches: [dir][NY][nx][6 MZ] between the phases
-  int* gmeta;          // split launches: [dir][NY][5 + 4 chunks]
+  int* gmeta;          // split launches: [dir][NY][meta_ints]
   int nx, nz, NY, Mm, MX, MZ, Kx, Kz;
   int n1x, n2x, n1z, n2z;
   Div dMZ, dnz, dn1z, dn2z, dn2x;
@@ -58,6 +58,9 @@ struct Args {
   int pin, pout;       // split launches: blocks per plane of the x transforms
   const int* active;   // split launches of a group member: device flag, 0 = do nothing (null: run)
 };
+
+// integers that a split call keeps per plane between its launches
+__host__ __device__ constexpr size_t meta_ints(int nchunk) { return 5 + 4 * (size_t)nchunk; }
 
 template <class F>
 __device__ __forceinline__ void with_radix(int r, F f) {
@@ -613,7 +616,7 @@ __device__ __forceinline__ void plane(const Args& a, int phase, int part, int j,
     x_forward<KIND>(a, s, twx, X, RS, 0, nout * a.MZ, X, RS, out, planeMm, j);
   } else {
     cx* G = a.G + ((size_t)dir * a.NY + j) * a.nx * RS;
-    int* meta = a.gmeta + ((size_t)dir * a.NY + j) * (5 + 4 * a.nchunk);
+    int* meta = a.gmeta + ((size_t)dir * a.NY + j) * meta_ints(a.nchunk);
     if (phase == kPhaseIn) {
       begin();
       if (part == 0 && threadIdx.x == 0) {
