@@ -589,7 +589,7 @@ extern "C" sp_status sp_step_n(sp_ctx* c, const double* U, double* G, int n, voi
 static size_t base_slot_bytes(const sp_ctx* c) {
   const size_t grid = (size_t)6 * c->NY * c->nx * c->nz;
   if (c->cfg.prec == SP_MIXED) return 2 * grid * 4;
-  return c->use_fx ? grid * 8 + (size_t)c->NY * 16 : grid * 8;
+  return c->use_fx ? grid * 8 + (size_t)c->NY * 48 : grid * 8;
 }
 
 // copy the base fields of the tangent's precision to (save = true) or from trajectory slot k

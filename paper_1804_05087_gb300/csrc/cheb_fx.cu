@@ -58,14 +58,7 @@ __device__ __forceinline__ i64 from_double_times(double v, int sh, double f) {
   return e != 0 && e + sh > 1000 ? __double2ll_rn(d * f) : 0;
 }
 
-// X 2^-sh: one operation of the FP64 pipe, the scaling on the exponent field
-__device__ __forceinline__ double unscale(i64 X, int sh) {
-  const double d = (double)X;
-  if (sh > -900 && sh < 900) {
-    return X == 0 ? 0.0 : __hiloint2double(__double2hiint(d) - sh * (1 << 20), __double2loint(d));
-  }
-  return sh == kNotFinite ? nan("") : to_double(X, sh);
-}
+__device__ __forceinline__ double unscale(i64 X, int sh) { return sh == kNotFinite ? nan("") : from_fixed(X, sh); }
 __device__ __forceinline__ double2 unscale(i64 x, i64 y, int sh) { return make_double2(unscale(x, sh), unscale(y, sh)); }
 
 // Tables of constants, 56-bit halves, each row padded to PH entries (even, zeros) so that two come

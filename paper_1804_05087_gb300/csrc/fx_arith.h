@@ -233,6 +233,12 @@ __device__ __forceinline__ double to_double(i64 X, int sh) {
   return __longlong_as_double((i64)(sign | (((u64)(ex - 1) << 52) + m)));
 }
 
+// X 2^-sh: one operation of the FP64 pipe, the scaling on the exponent field
+__device__ __forceinline__ double from_fixed(i64 X, int sh) {
+  if (sh <= -900 || sh >= 900) return to_double(X, sh);
+  return X == 0 ? 0.0 : add_exponent((double)X, -sh);
+}
+
 // X f 2^-sh by the FP64 pipe (scale = f 2^-sh where that is a normal number, see scale_of)
 struct Scale {
   double s;

@@ -155,7 +155,7 @@ struct sp_ctx {
   void* fx_G = nullptr;          // planes between the launches of a split call
   int* fx_gmeta = nullptr;       // their exponents
   long long* base_fx = nullptr;  // FP64 contexts: base fields as integers, then base_meta
-  int* base_meta = nullptr;      // [NY][4] exponents and bit lengths
+  int* base_meta = nullptr;      // [NY][12] exponents and bit lengths
   std::string err;
   // tracing: event pairs per stage, recorded while `trace` is on
   bool trace = false;

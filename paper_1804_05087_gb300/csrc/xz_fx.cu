@@ -124,7 +124,7 @@ sp_status sp_fx_setup(sp_ctx* c) {
             cudaMalloc(&c->fx_G, nplanes * plane_bytes(c)) == cudaSuccess &&
             cudaMalloc((void**)&c->fx_gmeta, nplanes * meta * 4) == cudaSuccess;
   if (ok && c->cfg.prec == SP_FP64)
-    ok = cudaMalloc((void**)&c->base_fx, (size_t)6 * c->NY * nxz * 8 + (size_t)c->NY * 16) == cudaSuccess;
+    ok = cudaMalloc((void**)&c->base_fx, (size_t)6 * c->NY * nxz * 8 + (size_t)c->NY * 48) == cudaSuccess;
   if (!ok) {
     cudaGetLastError();
     return SP_ENOMEM;

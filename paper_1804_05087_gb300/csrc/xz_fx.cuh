@@ -8,13 +8,15 @@
 // adds of 32-bit halves or 52 additions of 64 bits (measured), and a plane's transforms need no range,
 // only precision. 48 x 65 x 48, 256 tangents: 12.57 ms in FP64 registers, 3.11 ms here.
 //
-// Scales (every transformed value stays below 2^61). The x transforms of a group of fields
-// (velocity, vorticity) are scaled by the largest sum of moduli of a column, the z transforms by
-// that of the plane: bounds of every value they form, so that a rounding is 2^-60 of them. At the
-// product the values of one chunk of x-rows are shifted up to their largest magnitude; the products
-// keep 32 fraction bits until their own largest magnitude is known, and the rows that the r2c
-// transforms leave carry an exponent per chunk, which the forward x transform brings to a common
-// one. Each pass loses only what its sums can grow by. A plane with a non-finite input gives NaN.
+// Scales (every transformed value stays below 2^61). The x transforms of a field are scaled by the
+// largest sum of moduli of its columns, the z transforms by that of its plane: bounds of every value
+// they form, so that a rounding is 2^-60 of them. Every field has its own scale: v beside u near a
+// wall, or v and w of a nearly streamwise-constant flow, keep their bits. At the product the values
+// of one chunk of x-rows are shifted up to their field's largest magnitude there, and each term of an
+// output component is shifted down to the component's coarsest exponent: a rounding is 2^-60 of the
+// largest term. The products keep 32 fraction bits until their component's largest magnitude is known,
+// and the rows that the r2c transforms leave carry an exponent per component and chunk, which the
+// forward x transform brings to a common one. A plane with a non-finite input gives NaN.
 //
 // Transforms. Length N = N1 N2 with N1, N2 in {2, 3, 4, 6, 8, 9, 12}: N2 transforms of length N1
 // in registers, a twiddle, N1 transforms of length N2, in place in shared memory. The inverse
@@ -44,7 +46,7 @@ struct Args {
   double2* out;        // [dir][NOUT][NY][Mm]; null: no product (base fields only)
   int4* bfx;           // [NY][nx][nz][6] base fields (U_tot, Omega_tot), slot order, as halves (high,
                        // low): read by the tangent and the adjoint, written by the step (null: not)
-  int* bmeta;          // [NY][4]: exponents and bit lengths of the two groups of the base fields
+  int* bmeta;          // [NY][12]: exponents, then bit lengths, of the base fields
   float* b32;          // [6][NY][nx][nz] and [6][NY][nz][nx] float base fields, written by the step
   float* b32t;         // (null: not)
   const double* lam;   // [NY][6] laminar U and Omega
@@ -60,7 +62,7 @@ struct Args {
 };
 
 // integers that a split call keeps per plane between its launches
-__host__ __device__ constexpr size_t meta_ints(int nchunk) { return 5 + 4 * (size_t)nchunk; }
+__host__ __device__ constexpr size_t meta_ints(int nchunk) { return 13 + 12 * (size_t)nchunk; }
 
 template <class F>
 __device__ __forceinline__ void with_radix(int r, F f) {
@@ -76,18 +78,24 @@ __device__ __forceinline__ void with_radix(int r, F f) {
 }
 
 struct Shared {
-  unsigned emax[2];      // per group: largest high word of the inputs
-  int col[6 * kMaxKz];   // sums of moduli of every column in units of 2^(emax exponent - 14)
-  int sh[2];             // exponents of the z transforms per group: X = v 2^sh
-  int up[2];             // bits that the x transforms are scaled finer
+  unsigned emax[6];      // per field: largest high word of the inputs
+  int sh[6];             // exponents of the z transforms: X = v 2^sh
+  int up[6];             // bits that the x transforms are scaled finer
   int bad;               // a non-finite value in the plane
-  unsigned orv[2];       // high words in use by the physical values of a chunk, per group
-  unsigned orr[2];       // by the products, per output group
-  unsigned ors[2];       // by the rows after r2c
+  unsigned orv[6];       // high words in use by the physical values of a chunk, per field
+  unsigned orr[6];       // by the products, per output component
+  unsigned ors[6];       // by the rows after r2c
+  int ex[6];             // exponents of a chunk's products
+  int ecom[6];           // exponents of the forward x transforms
   i64 lam[6];
-  int cexp[2][kMaxChunks];   // exponent and bit length of each chunk's rows after r2c
-  int cbits[2][kMaxChunks];
-  int lsh[2][kMaxPairs];     // shift of each row pair to the common exponent
+  union {
+    int col[6 * kMaxKz];  // sums of moduli of every column in units of 2^(emax exponent - 14)
+    struct {
+      short cexp[6][kMaxChunks];        // exponent and bit length of each chunk's rows after r2c
+      signed char cbits[6][kMaxChunks];
+      signed char lsh[6][kMaxPairs];    // shift of each row pair to the common exponent
+    };
+  };
 };
 
 // ceil(log2 n), n >= 2: bits that a sum of n terms can grow by
@@ -104,25 +112,39 @@ __device__ __forceinline__ unsigned mag(i64 v) {
 }
 __device__ __forceinline__ unsigned mag(cx v) { return mag(v.x) | mag(v.y); }
 
-// *dst |= v over the block's threads (converged warps)
-__device__ __forceinline__ void block_or(unsigned* dst, unsigned v) {
-  v = __reduce_or_sync(0xffffffffu, v);
-  if ((threadIdx.x & 31) == 0) atomicOr(dst, v);
+// dst[i] |= v[i] over the block's threads (converged warps)
+template <int N>
+__device__ __forceinline__ void block_or(unsigned* dst, const unsigned (&v)[N]) {
+  const int lane = threadIdx.x & 31;
+  unsigned mine = 0;
+#pragma unroll
+  for (int i = 0; i < N; ++i) {
+    const unsigned t = __reduce_or_sync(0xffffffffu, v[i]);
+    if (lane == i) mine = t;
+  }
+  if (lane < N) atomicOr(dst + lane, mine);
+}
+// v[f] |= o, f known at run time only
+template <int N>
+__device__ __forceinline__ void or_at(unsigned (&v)[N], int f, unsigned o) {
+#pragma unroll
+  for (int i = 0; i < N; ++i)
+    if (i == f) v[i] |= o;
 }
 
-// exponents of the plane's inputs. A few threads walk each column twice (the second time from the
+// exponents of the plane's fields. A few threads walk each column twice (the second time from the
 // caches): the largest exponent, then the sums of moduli with 15-bit terms (integers, so that the
-// result does not depend on the order).
+// result does not depend on the order). The laminar profile counts in the field it is added to.
 __device__ __forceinline__ void plane_scale(const Args& a, Shared& s, const double2* in, size_t planeMm, int j,
                                             int nin, bool lam) {
   const int tid = threadIdx.x, ncol = nin * a.MZ;
-  if (tid < 2) s.emax[tid] = 0;
+  if (tid < 6) s.emax[tid] = 0;
+  if (tid == 0) s.bad = 0;
   for (int i = tid; i < 6 * kMaxKz; i += kThreads) s.col[i] = 0;
   __syncthreads();
   auto top = [](double v) { return (unsigned)__double2hiint(v) & 0x7fffffffu; };
   const int per = max(1, kThreads / ncol), h0 = ncol >= kThreads ? 0 : tid / ncol;
   const int c0 = tid - h0 * ncol;
-  unsigned em[2] = {0, 0};
   if (h0 < per)
     for (int c = c0; c < ncol; c += kThreads) {
       const int f = quot(c, a.dMZ);
@@ -132,29 +154,17 @@ __device__ __forceinline__ void plane_scale(const Args& a, Shared& s, const doub
         const double2 v = __ldg(p + q * a.MZ);
         t = max(t, max(top(v.x), top(v.y)));
       }
-      if (f < 3) em[0] = max(em[0], t);
-      else em[1] = max(em[1], t);
+      atomicMax(&s.emax[f], t);
     }
-  if (lam && tid < 6) {
-    const unsigned t = top(a.lam[j * 6 + tid]);
-    if (tid < 3) em[0] = max(em[0], t);
-    else em[1] = max(em[1], t);
-  }
-  __syncwarp();
-#pragma unroll
-  for (int g = 0; g < 2; ++g) {
-    const unsigned t = __reduce_max_sync(0xffffffffu, em[g]);
-    if ((tid & 31) == 0) atomicMax(&s.emax[g], t);
-  }
+  if (lam && tid < 6) atomicMax(&s.emax[tid], top(a.lam[j * 6 + tid]));
   __syncthreads();
-  const int e0[2] = {(int)(s.emax[0] >> 20), (int)(s.emax[1] >> 20)};
   auto part = [&](double v, int e) -> int {
     const unsigned h = top(v);
     return (int)(((h & 0xfffffu) | 0x100000u) >> min(31, e - (int)(h >> 20) + 6)) + 1;
   };
   if (h0 < per)
     for (int c = c0; c < ncol; c += kThreads) {
-      const int f = quot(c, a.dMZ), iz = c - f * a.MZ, e = f < 3 ? e0[0] : e0[1];
+      const int f = quot(c, a.dMZ), iz = c - f * a.MZ, e = (int)(s.emax[f] >> 20);
       const double2* p = in + f * planeMm + iz;
       int acc = 0;
       for (int q = h0; q < a.MX; q += per) {
@@ -164,32 +174,27 @@ __device__ __forceinline__ void plane_scale(const Args& a, Shared& s, const doub
       atomicAdd(&s.col[f * kMaxKz + iz], acc);
     }
   __syncthreads();
-  if (tid < 32) {
-    int big[2] = {1, 1}, bigc[2] = {1, 1};
-    for (int f = 0; f < nin; ++f) {
-      int tot = 0, most = 0;
-      for (int iz = tid; iz < a.MZ; iz += 32) {
-        const int v = s.col[f * kMaxKz + iz];
-        tot += iz == 0 ? v : 2 * v;
-        most = max(most, v);
-      }
-      tot = __reduce_add_sync(0xffffffffu, tot);
-      most = __reduce_max_sync(0xffffffffu, most);
-      const int g = f < 3 ? 0 : 1;
-      if (lam) tot += part(a.lam[j * 6 + f], g ? e0[1] : e0[0]);
-      big[g] = max(big[g], tot);
-      bigc[g] = max(bigc[g], most);
+  static_assert(kThreads >= 6 * 32, "a warp per field");
+  const int f = tid >> 5;
+  if (f < nin) {
+    const int e = (int)(s.emax[f] >> 20);
+    int tot = 0, most = 0;
+    for (int iz = tid & 31; iz < a.MZ; iz += 32) {
+      const int v = s.col[f * kMaxKz + iz];
+      tot += iz == 0 ? v : 2 * v;
+      most = max(most, v);
     }
-    if (tid == 0) {
-      // sums of moduli <= big 2^(e0 - 1023 - 14): 60 bits
-      for (int g = 0; g < 2; ++g) {
-        s.sh[g] = 60 - (32 - __clz(big[g]) + e0[g] - 1037);
-        s.up[g] = __clz(bigc[g]) - __clz(big[g]);
-      }
-      s.bad = e0[0] == 0x7ff || e0[1] == 0x7ff;
+    tot = __reduce_add_sync(0xffffffffu, tot);
+    most = __reduce_max_sync(0xffffffffu, most);
+    if ((tid & 31) == 0) {
+      if (lam) tot += part(a.lam[j * 6 + f], e);
+      // sums of moduli <= tot 2^(e - 1023 - 14): 60 bits
+      const int sh = 60 - (32 - __clz(tot) + e - 1037);
+      s.sh[f] = sh;
+      s.up[f] = __clz(most) - __clz(tot);
+      if (e == 0x7ff) s.bad = 1;
+      if (lam) s.lam[f] = from_double(a.lam[j * 6 + f], sh);
     }
-    __syncwarp();
-    if (lam && tid < 6) s.lam[tid] = from_double(a.lam[j * 6 + tid], s.sh[tid / 3]);
   }
   __syncthreads();
 }
@@ -207,7 +212,7 @@ __device__ __forceinline__ void x_inverse(const Args& a, const Shared& s, const 
       const int n2 = quot(idx, dnc), col = idx - n2 * nc;
       const int f = quot(c0 + col, a.dMZ), iz = c0 + col - f * a.MZ;
       // the adjoint's transposed forward transform halves the iz > 0 terms
-      const int g = f < 3 ? 0 : 1, sh = s.sh[g] + s.up[g] - (KIND == kAdjoint && iz > 0 ? 1 : 0);
+      const int sh = s.sh[f] + s.up[f] - (KIND == kAdjoint && iz > 0 ? 1 : 0);
       const double2* p = in + f * planeMm + iz;
       cx v[R];
 #pragma unroll
@@ -249,27 +254,23 @@ __device__ __forceinline__ void x_forward(const Args& a, Shared& s, const int4* 
                                           int nc, cx* X, int ldx, double2* out, size_t planeMm, int j) {
   const int N1 = a.n1x, N2 = a.n2x, nx = a.nx;
   const Div dnc = div_of(nc);
-  // common exponent per group: the sums of the first pass stay below 2^61, the second pass
-  // shifts its inputs by its own growth
+  // common exponent per component (a warp each): the sums of the first pass stay below 2^61, the
+  // second pass shifts its inputs by its own growth
   const int lg = 32 - __clz(N2 - 1);
-  int ecom[2];
-#pragma unroll
-  for (int g = 0; g < 2; ++g) {
+  constexpr int nout = KIND == kAdjoint ? 6 : 3;
+  if (const int f = threadIdx.x >> 5, lane = threadIdx.x & 31; f < nout) {
     int top = -(1 << 28);
-    for (int q = 0; q < a.nchunk; ++q) top = max(top, s.cbits[g][q] - s.cexp[g][q]);
-    ecom[g] = 60 - lg - top;
-  }
-  for (int i = threadIdx.x; i < nx / 2; i += kThreads) {
-    const int q = i / a.rp;
-    s.lsh[0][i] = ecom[0] - s.cexp[0][q];
-    s.lsh[1][i] = ecom[1] - s.cexp[1][q];
+    for (int q = lane; q < a.nchunk; q += 32) top = max(top, s.cbits[f][q] - s.cexp[f][q]);
+    const int e = 60 - lg - __reduce_max_sync(0xffffffffu, top);
+    if (lane == 0) s.ecom[f] = e;
+    for (int i = lane; i < nx / 2; i += 32) s.lsh[f][i] = (signed char)max(-62, min(e - s.cexp[f][i / a.rp], 63));
   }
   __syncthreads();
   with_radix(N2, [&](auto rc) {
     constexpr int R = decltype(rc)::value;
     for (int idx = threadIdx.x; idx < N1 * nc; idx += kThreads) {
       const int p = quot(idx, dnc), col = idx - p * nc;
-      const int* ls = s.lsh[KIND == kAdjoint && c0 + col >= 3 * a.MZ ? 1 : 0];
+      const signed char* ls = s.lsh[quot(c0 + col, a.dMZ)];
       const cx* g = src + (size_t)(p * R) * lds + c0 + col;
       cx* x = X + p * R * ldx + col;
       cx v[R];
@@ -278,7 +279,7 @@ __device__ __forceinline__ void x_forward(const Args& a, Shared& s, const int4* 
         const int l = ls[(p * R + k) >> 1];
         v[k] = g[k * lds];
         if (l >= 0) v[k] = {shift(v[k].x, l), shift(v[k].y, l)};
-        else v[k] = {shift_down(v[k].x, min(-l, 62)), shift_down(v[k].y, min(-l, 62))};
+        else v[k] = {shift_down(v[k].x, -l), shift_down(v[k].y, -l)};
       }
       dft<R, -1>(v);
 #pragma unroll
@@ -287,7 +288,7 @@ __device__ __forceinline__ void x_forward(const Args& a, Shared& s, const int4* 
   });
   __syncthreads();
   const double inv = 1.0 / ((double)a.nx * (double)a.nz);
-  const bool bad = s.bad || (KIND != kStep && a.bmeta[4 * j] == kBadExp);
+  const bool bad = s.bad || (KIND != kStep && a.bmeta[12 * j] == kBadExp);
   with_radix(N1, [&](auto rc) {
     constexpr int R = decltype(rc)::value;
     for (int idx = threadIdx.x; idx < N2 * nc; idx += kThreads) {
@@ -302,9 +303,7 @@ __device__ __forceinline__ void x_forward(const Args& a, Shared& s, const int4* 
       }
       dft<R, -1>(v);
       // the adjoint's transposed inverse transform doubles the iz > 0 terms
-      const Scale sc = scale_of(bad ? nan("") : inv,
-                                (KIND == kAdjoint && f >= 3 ? ecom[1] : ecom[0]) - growth(R) -
-                                    (KIND == kAdjoint && iz > 0 ? 1 : 0));
+      const Scale sc = scale_of(bad ? nan("") : inv, s.ecom[f] - growth(R) - (KIND == kAdjoint && iz > 0 ? 1 : 0));
       double2* o = out + f * planeMm + iz;
 #pragma unroll
       for (int k = 0; k < R; ++k) {
@@ -315,6 +314,42 @@ __device__ __forceinline__ void x_forward(const Args& a, Shared& s, const int4* 
     }
   });
 }
+
+// The products: term t of output component t / per is an input field times another field (the step: a
+// vorticity; else a base field); the first half of a component's terms is added, the second subtracted.
+// i = c + 1, k = c + 2 (mod 3).
+template <Kind KIND>
+struct Terms;
+template <>
+struct Terms<kStep> {  // U_i Omega_k - U_k Omega_i
+  static constexpr int per = 2, count = 6;
+  static __device__ __forceinline__ constexpr int input(int t) { return (t / 2 + 1 + t % 2) % 3; }
+  static __device__ __forceinline__ constexpr int other(int t) { return 3 + (t / 2 + 2 - t % 2) % 3; }
+};
+template <>
+struct Terms<kTangent> {  // omega_k U_i + u_i Omega_k - omega_i U_k - u_k Omega_i
+  static constexpr int per = 4, count = 12;
+  static __device__ __forceinline__ constexpr int input(int t) {
+    const int c = t / 4, i = (c + 1) % 3, k = (c + 2) % 3, q = t % 4;
+    return q == 0 ? 3 + k : q == 1 ? i : q == 2 ? 3 + i : k;
+  }
+  static __device__ __forceinline__ constexpr int other(int t) {
+    const int c = t / 4, i = (c + 1) % 3, k = (c + 2) % 3, q = t % 4;
+    return q == 0 ? i : q == 1 ? 3 + k : q == 2 ? k : 3 + i;
+  }
+};
+template <>
+struct Terms<kAdjoint> {  // u* = Omega x a: a_k Omega_i - a_i Omega_k; omega* = a x U: a_i U_k - a_k U_i
+  static constexpr int per = 2, count = 12;
+  static __device__ __forceinline__ constexpr int input(int t) {
+    const int c = t / 2 % 3;
+    return (c + (t < 6 ? 2 - t % 2 : 1 + t % 2)) % 3;
+  }
+  static __device__ __forceinline__ constexpr int other(int t) {
+    const int c = t / 2 % 3;
+    return t < 6 ? 3 + (c + 1 + t % 2) % 3 : (c + 2 - t % 2) % 3;
+  }
+};
 
 // products of two fixed-point values by halves: the sum's high part and its 32 fraction bits
 struct Acc {
@@ -337,7 +372,7 @@ __device__ __forceinline__ void z_chunk(const Args& a, Shared& s, const int4* tw
   constexpr int nin = KIND == kAdjoint ? 3 : 6, nout = KIND == kAdjoint ? 6 : 3, NF = kZf<KIND>;
   const int N1 = a.n1z, N2 = a.n2z, nz = a.nz, MZ = a.MZ, P = N2 + 1, ZF = N1 * P;
   const int q0 = q * a.rp, nq = min(a.rp, a.nx / 2 - q0);
-  if (threadIdx.x == 0) s.orv[0] = s.orv[1] = s.orr[0] = s.orr[1] = s.ors[0] = s.ors[1] = 0;
+  if (threadIdx.x < 6) s.orv[threadIdx.x] = s.orr[threadIdx.x] = s.ors[threadIdx.x] = 0;
   // c2r of the packed pair A + iB: spectrum A + iB at kz, conj(A) + i conj(B) at nz - kz
   with_radix(N1, [&](auto rc) {
     constexpr int R = decltype(rc)::value;
@@ -345,7 +380,7 @@ __device__ __forceinline__ void z_chunk(const Args& a, Shared& s, const int4* tw
       const int r = quot(idx, a.dn2z), n2 = idx - r * N2, qq = r / nin, f = r - qq * nin;
       const cx* A = src + (size_t)(2 * (q0 + qq)) * lds + f * MZ;
       const cx* B = A + lds;
-      const int dn = s.up[f < 3 ? 0 : 1];
+      const int dn = s.up[f];
       cx v[R];
 #pragma unroll
       for (int k = 0; k < R; ++k) {
@@ -365,7 +400,7 @@ __device__ __forceinline__ void z_chunk(const Args& a, Shared& s, const int4* tw
     }
   });
   __syncthreads();
-  unsigned o0 = 0, o1 = 0;
+  unsigned ov[nin] = {};
   with_radix(N2, [&](auto rc) {
     constexpr int R = decltype(rc)::value;
     for (int idx = threadIdx.x; idx < nq * nin * N1; idx += kThreads) {
@@ -383,45 +418,46 @@ __device__ __forceinline__ void z_chunk(const Args& a, Shared& s, const int4* tw
         o |= mag(v[k]);
         z[k] = v[k];
       }
-      if (f < 3) o0 |= o;
-      else o1 |= o;
+      or_at(ov, f, o);
     }
   });
   __syncwarp();
-  block_or(&s.orv[0], o0);
-  if (nin == 6) block_or(&s.orv[1], o1);
+  block_or(s.orv, ov);
   __syncthreads();
-  // products: shifts that use the bits left above the chunk's largest values, so that the results
-  // stay below 2^(60 - lgz) and the first pass's sums of a packed pair below 2^61; the second
-  // pass shifts its inputs by its own growth
+  // Products: shifts that use the bits left above the chunk's largest values, so that the results
+  // stay below 2^(60 - lgz) and the first pass's sums of a packed pair below 2^61; the second pass
+  // shifts its inputs by its own growth. Lane t of every warp takes term t: its factor of the inputs
+  // at as many bits as its other factor (and their number per component) leaves, less what brings it to the
+  // component's coarsest exponent.
   const int lgz = 32 - __clz(N2 - 1), lgb = 32 - __clz(N1 - 1);
-  const int n0 = bits(s.orv[0]), n1 = bits(s.orv[1]);
-  int l0 = 0, l1 = 0, ex0 = 0, ex1 = 0;
-  if (KIND == kTangent) {
-    const int4 bm = __ldg(reinterpret_cast<const int4*>(a.bmeta) + j);  // exponents, bits of (U, Omega)
-    l1 = min(60, 122 - lgz - bm.z) - n1;
-    l0 = min(60, 122 - lgz - bm.w) - n0;
-    // omega x U and u x Omega at the smaller of their exponents
-    const int e1 = s.sh[1] + l1 + bm.x, e0 = s.sh[0] + l0 + bm.y, e = min(e0, e1);
-    l1 -= e1 - e;
-    l0 -= e0 - e;
-    ex0 = e - 63;
-  } else if (KIND == kAdjoint) {
-    const int4 bm = __ldg(reinterpret_cast<const int4*>(a.bmeta) + j);
-    l0 = min(60, 123 - lgz - max(bm.z, bm.w)) - n0;
-    ex0 = s.sh[0] + l0 + bm.y - 63;
-    ex1 = s.sh[0] + l0 + bm.x - 63;
-  } else {
-    const int m = 123 - lgz, x0 = min(60, m / 2), x1 = min(60, m - x0);
-    l0 = x0 - n0;
-    l1 = x1 - n1;
-    ex0 = s.sh[0] + l0 + s.sh[1] + l1 - 63;
-    if (threadIdx.x == 0 && a.bmeta) {
-      atomicMax(a.bmeta + 4 * j + 2, n0);
-      atomicMax(a.bmeta + 4 * j + 3, n1);
+  const int xa = KIND == kTangent ? 122 - lgz : 123 - lgz;  // bits of both factors
+  const int x0 = min(60, xa / 2), x1 = min(60, xa - x0);    // the step's velocity and vorticity
+  int down[Terms<KIND>::count];  // of a value of 60 bits
+  {
+    using TT = Terms<KIND>;
+    const int lane = threadIdx.x & 31, t = min(lane, TT::count - 1), fx = TT::input(t), fb = TT::other(t);
+    const int n = bits(s.orv[fx]);
+    int most, eb;
+    if (KIND == kStep) {
+      most = x0;
+      eb = s.sh[fb] + x1 - bits(s.orv[fb]);
+    } else {
+      eb = __ldg(a.bmeta + 12 * j + fb);
+      most = min(60, xa - __ldg(a.bmeta + 12 * j + 6 + fb));
     }
+    const int e = s.sh[fx] + most - n + eb;
+    int least = min(e, __shfl_xor_sync(0xffffffffu, e, 1));
+    if (TT::per == 4) least = min(least, __shfl_xor_sync(0xffffffffu, least, 2));
+    const int d = min(60 - most + (e - least), 63);
+#pragma unroll
+    for (int i = 0; i < TT::count; ++i) down[i] = __shfl_sync(0xffffffffu, d, i);
+    if (threadIdx.x < TT::count && lane % TT::per == 0) s.ex[lane / TT::per] = least - 63;
+    if (KIND == kStep && a.bmeta && threadIdx.x < 6) atomicMax(a.bmeta + 12 * j + 6 + threadIdx.x, bits(s.orv[threadIdx.x]));
   }
-  unsigned p0 = 0, p1 = 0;
+  int full[nin];  // shifts of the inputs to 60 bits (the step's vorticity: to x1)
+#pragma unroll
+  for (int f = 0; f < nin; ++f) full[f] = (KIND == kStep && f >= 3 ? x1 : 60) - bits(s.orv[f]);
+  unsigned pv[nout] = {};
   for (int idx = threadIdx.x; idx < nq * nz; idx += kThreads) {
     const int qq = quot(idx, a.dnz), zi = idx - qq * nz, z1 = quot(zi, a.dn2z);
     cx* z = Z + qq * NF * ZF + zi + z1;  // slot z1 (N2 + 1) + zi - z1 N2
@@ -444,12 +480,11 @@ __device__ __forceinline__ void z_chunk(const Args& a, Shared& s, const int4* tw
         const int zn = z1 + N1 * (zi - z1 * N2);
         const int sa = quot(slot0, a.dn2x), sb = quot(slot0 + 1, a.dn2x);
         const int xa = sa + a.n1x * (slot0 - sa * a.n2x), xb = sb + a.n1x * (slot0 + 1 - sb * a.n2x);
-        const double one = s.bad ? nan("") : 1.0;
-        const Scale sc[2] = {scale_of(one, s.sh[0]), scale_of(one, s.sh[1])};
 #pragma unroll
         for (int f = 0; f < 6; ++f) {
           const size_t o = ((size_t)f * a.NY + j) * a.nx * nz;
-          const float va = (float)scaled(F[f].x, sc[f / 3]), vb = (float)scaled(F[f].y, sc[f / 3]);
+          const float va = s.bad ? nanf("") : (float)from_fixed(F[f].x, s.sh[f]);
+          const float vb = s.bad ? nanf("") : (float)from_fixed(F[f].y, s.sh[f]);
           a.b32[o + xa * nz + zn] = va;
           a.b32[o + xb * nz + zn] = vb;
           a.b32t[o + zn * a.nx + xa] = va;
@@ -460,14 +495,15 @@ __device__ __forceinline__ void z_chunk(const Args& a, Shared& s, const int4* tw
     }
 #pragma unroll
     for (int r = 0; r < 2; ++r) {
-      // halves of the shifted values and of the base fields
-      int2 x[6], b[6];
+      // the shifted values and the halves of the base fields (the step: of the vorticity)
+      i64 x[nin];
+      int2 b[6];
 #pragma unroll
-      for (int f = 0; f < nin; ++f) {
-        const i64 v = shift(r ? F[f].y : F[f].x, f < 3 ? l0 : l1);
-        x[f] = make_int2(half_hi(v), half_lo(v));
-      }
-      if (KIND != kStep) {
+      for (int f = 0; f < nin; ++f) x[f] = shift(r ? F[f].y : F[f].x, full[f]);
+      if constexpr (KIND == kStep) {
+#pragma unroll
+        for (int f = 3; f < 6; ++f) b[f] = make_int2(half_hi(x[f]), half_lo(x[f]));
+      } else {
 #pragma unroll
         for (int f = 0; f < 3; ++f) {
           const int4 t = __ldg(a.bfx + (pt + r * nz) * 3 + f);
@@ -480,32 +516,19 @@ __device__ __forceinline__ void z_chunk(const Args& a, Shared& s, const int4* tw
         reinterpret_cast<int*>(z + (nout + c) * ZF)[r] = (int)h;  // fraction
         if (r) z[c * ZF].y = v;
         else z[c * ZF].x = v;
-        if (c < 3) p0 |= mag(v);
-        else p1 |= mag(v);
+        pv[c] |= mag(v);
       };
+      using TT = Terms<KIND>;
 #pragma unroll
-      for (int c = 0; c < 3; ++c) {
-        const int i = (c + 1) % 3, k = (c + 2) % 3;
+      for (int c = 0; c < nout; ++c) {
         Acc p, n;
-        if (KIND == kTangent) {  // U_tot x omega + u x Omega_tot
-          p.add(x[3 + k], b[i]);
-          p.add(x[i], b[3 + k]);
-          n.add(x[3 + i], b[k]);
-          n.add(x[k], b[3 + i]);
-          put(c, p, n);
-        } else if (KIND == kAdjoint) {  // u* = Omega_tot x a, omega* = a x U_tot
-          p.add(x[k], b[3 + i]);
-          n.add(x[i], b[3 + k]);
-          put(c, p, n);
-          Acc p2, n2;
-          p2.add(x[i], b[k]);
-          n2.add(x[k], b[i]);
-          put(3 + c, p2, n2);
-        } else {  // U_tot x Omega_tot
-          p.add(x[i], x[3 + k]);
-          n.add(x[k], x[3 + i]);
-          put(c, p, n);
+#pragma unroll
+        for (int q = 0; q < TT::per; ++q) {
+          const int t = c * TT::per + q;
+          const i64 v = x[TT::input(t)] >> down[t];
+          (2 * q < TT::per ? p : n).add(make_int2(half_hi(v), half_lo(v)), b[TT::other(t)]);
         }
+        put(c, p, n);
       }
     }
   }
@@ -514,18 +537,17 @@ __device__ __forceinline__ void z_chunk(const Args& a, Shared& s, const int4* tw
     return;
   }
   __syncwarp();
-  block_or(&s.orr[0], p0);
-  if (nout == 6) block_or(&s.orr[1], p1);
+  block_or(s.orr, pv);
   __syncthreads();
   // r2c: input slot order, factors the other way round, natural order out; the products' fraction
   // bits fill what their largest magnitude leaves
-  const int f0 = max(0, min(60 - lgz - bits(s.orr[0]), 31)), f1 = max(0, min(60 - lgz - bits(s.orr[1]), 31));
+  auto fraction = [&](int f) { return max(0, min(60 - lgz - bits(s.orr[f]), 31)); };
   with_radix(N2, [&](auto rc) {
     constexpr int R = decltype(rc)::value;
     for (int idx = threadIdx.x; idx < nq * nout * N1; idx += kThreads) {
       const int r = quot(idx, a.dn1z), p = idx - r * N1, qq = r / nout, f = r - qq * nout;
       cx* z = Z + (qq * NF + f) * ZF + p * P;
-      const int fb = f < 3 ? f0 : f1;
+      const int fb = fraction(f);
       const u64 rnd = 1ull << (31 - fb);
       cx v[R];
 #pragma unroll
@@ -555,7 +577,7 @@ __device__ __forceinline__ void z_chunk(const Args& a, Shared& s, const int4* tw
     }
   });
   __syncthreads();
-  p0 = p1 = 0;
+  unsigned sv[nout] = {};
   // twice the two real rows' spectra: X(k) + conj X(-k) and (X(k) - conj X(-k)) / i
   for (int idx = threadIdx.x; idx < nq * nout * MZ; idx += kThreads) {
     const int r = quot(idx, a.dMZ), k = idx - r * MZ, qq = r / nout, f = r - qq * nout;
@@ -566,18 +588,14 @@ __device__ __forceinline__ void z_chunk(const Args& a, Shared& s, const int4* tw
     const cx ra = {u.x + v.x, u.y - v.y}, rb = {u.y + v.y, v.x - u.x};
     A[0] = ra;
     A[lds] = rb;
-    if (f < 3) p0 |= mag(ra) | mag(rb);
-    else p1 |= mag(ra) | mag(rb);
+    or_at(sv, f, mag(ra) | mag(rb));
   }
   __syncwarp();
-  block_or(&s.ors[0], p0);
-  if (nout == 6) block_or(&s.ors[1], p1);
+  block_or(s.ors, sv);
   __syncthreads();
-  if (threadIdx.x == 0) {
-    s.cexp[0][q] = ex0 + f0 - lgb;
-    s.cexp[1][q] = ex1 + f1 - lgb;
-    s.cbits[0][q] = bits(s.ors[0]);
-    s.cbits[1][q] = bits(s.ors[1]);
+  if (const int f = threadIdx.x; f < nout) {
+    s.cexp[f][q] = (short)max(-30000, min(s.ex[f] + fraction(f) - lgb, 30000));
+    s.cbits[f][q] = (signed char)bits(s.ors[f]);
   }
 }
 
@@ -599,10 +617,10 @@ __device__ __forceinline__ void plane(const Args& a, int phase, int part, int j,
   auto begin = [&]() {
     plane_scale(a, s, in, planeMm, j, nin, KIND == kStep);
     if (KIND == kStep && threadIdx.x == 0 && part == 0 && a.bmeta) {
-      a.bmeta[4 * j] = s.bad ? kBadExp : s.sh[0];
-      a.bmeta[4 * j + 1] = s.sh[1];
-      a.bmeta[4 * j + 2] = 0;
-      a.bmeta[4 * j + 3] = 0;
+      for (int f = 0; f < 6; ++f) {
+        a.bmeta[12 * j + f] = f == 0 && s.bad ? kBadExp : s.sh[f];
+        a.bmeta[12 * j + 6 + f] = 0;
+      }
     }
   };
   if constexpr (!SPLIT) {
@@ -619,37 +637,33 @@ __device__ __forceinline__ void plane(const Args& a, int phase, int part, int j,
     int* meta = a.gmeta + ((size_t)dir * a.NY + j) * meta_ints(a.nchunk);
     if (phase == kPhaseIn) {
       begin();
-      if (part == 0 && threadIdx.x == 0) {
-        meta[0] = s.sh[0];
-        meta[1] = s.sh[1];
-        meta[2] = s.bad;
-        meta[3] = s.up[0];
-        meta[4] = s.up[1];
+      if (part == 0 && threadIdx.x < nin) {
+        meta[threadIdx.x] = s.sh[threadIdx.x];
+        meta[6 + threadIdx.x] = s.up[threadIdx.x];
+        if (threadIdx.x == 0) meta[12] = s.bad;
       }
       const int ncol = nin * a.MZ, c0 = part * ncol / a.pin, nc = (part + 1) * ncol / a.pin - c0;
       x_inverse<KIND>(a, s, twx, in, planeMm, c0, nc, X, nc, G, RS);
     } else if (phase == kPhaseZ) {
-      if (threadIdx.x < 2) {
-        s.sh[threadIdx.x] = meta[threadIdx.x];
-        s.up[threadIdx.x] = meta[3 + threadIdx.x];
+      if (const int f = threadIdx.x; f < nin) {
+        s.sh[f] = meta[f];
+        s.up[f] = meta[6 + f];
+        if (f == 0) s.bad = meta[12];
+        if (KIND == kStep) s.lam[f] = from_double(a.lam[j * 6 + f], meta[f]);
       }
-      if (threadIdx.x == 0) s.bad = meta[2];
-      if (KIND == kStep && threadIdx.x < 6) s.lam[threadIdx.x] = from_double(a.lam[j * 6 + threadIdx.x], meta[threadIdx.x / 3]);
       __syncthreads();
       z_chunk<KIND>(a, s, twz, G, G, RS, X, part, j);
-      if (threadIdx.x == 0) {
-        for (int g = 0; g < 2; ++g) {
-          meta[5 + g * a.nchunk + part] = s.cexp[g][part];
-          meta[5 + (2 + g) * a.nchunk + part] = s.cbits[g][part];
-        }
+      if (const int f = threadIdx.x; f < nout) {  // the thread that wrote them
+        meta[13 + f * a.nchunk + part] = s.cexp[f][part];
+        meta[13 + (6 + f) * a.nchunk + part] = s.cbits[f][part];
       }
     } else {
-      for (int i = threadIdx.x; i < 2 * a.nchunk; i += kThreads) {
-        const int g = i >= a.nchunk, q = i - g * a.nchunk;
-        s.cexp[g][q] = meta[5 + i];
-        s.cbits[g][q] = meta[5 + 2 * a.nchunk + i];
+      for (int i = threadIdx.x; i < nout * a.nchunk; i += kThreads) {
+        const int f = i / a.nchunk, q = i - f * a.nchunk;
+        s.cexp[f][q] = (short)meta[13 + i];
+        s.cbits[f][q] = (signed char)meta[13 + 6 * a.nchunk + i];
       }
-      if (threadIdx.x == 0) s.bad = meta[2];
+      if (threadIdx.x == 0) s.bad = meta[12];
       __syncthreads();
       const int ncol = nout * a.MZ, c0 = part * ncol / a.pout, nc = (part + 1) * ncol / a.pout - c0;
       x_forward<KIND>(a, s, twx, G, RS, c0, nc, X, nc, out, planeMm, j);
