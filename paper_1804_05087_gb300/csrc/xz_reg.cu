@@ -312,6 +312,8 @@ cudaError_t grp_launch_xz_reg(const GrpKernel* ks, const int* active, cudaStream
 
 bool sp_xz_reg_supported(const sp_ctx* c) {
   if (c->nx != c->nz) return false;
+  // the kernel's strides are those of all modes of the 2/3 rule; a pipe may keep fewer
+  if (c->Kx != (c->nx - 1) / 3 || c->Kz != (c->nz - 1) / 3) return false;
   return c->nx == 16 || c->nx == 24 || c->nx == 32 || c->nx == 48 || c->nx == 64;
 }
 
