@@ -1,5 +1,5 @@
-// Per-mode Stokes solve by the precomputed dense operators, one Fourier mode of one direction per
-// block: the step, single tangents and small batches (batches from kChainMinBatch directions take the
+// Per-mode Stokes solve by the precomputed dense operators, one Fourier mode of one or a few directions
+// per block: the step, single tangents and small batches (batches from kChainMinBatch directions take the
 // O(N) chains, solve_chain.cu; laminar advection in L takes k_solve, kernels.cu). Same problem as
 // k_solve: right-hand side u/dt + N, rotation along / across the wavevector, reduced right-hand side,
 // v = V g and b = H f_b per parity, back-rotation, G = u_new - u (Sec. 2, Eq. befe; Sec. 3.2).
@@ -10,8 +10,10 @@
 // operators come into shared memory by one bulk copy that runs during the earlier phases, the suffix
 // sums are warp scans, and wavenumbers and row indices are read, not computed. Several blocks share
 // an SM, so that one block's scans overlap another's products. Measured at 48 x 65 x 48, one FP64
-// direction: 55 us with four modes per block and loads inside the products, 28 us here; see the rule in
-// sp_solve_shapes for the threads. k_solve_adj is the transposed solve, in the same shape.
+// direction: 55 us with four modes per block and loads inside the products, 28 us here. A batch is bound by
+// FP64 instructions, whose idle lanes cost as much as busy ones, so there a block takes two or four
+// directions of its mode (directions_of; threads: threads_of). k_solve_adj is the transposed solve, one
+// direction per block.
 #include <algorithm>
 #include <cstdint>
 
@@ -28,7 +30,7 @@ struct OneArgs {
   const double* wave;  // [mode][4]: kx, kz, 1/k, 0
   const float* cft;    // [NH][NY] forward transform (float), points fastest last
   const double* row;   // row indices 0, 1, ... as doubles
-  int n_unique, Mm, MX, MZ, Kx, NY, cv, rb0, rb1, off_v0, off_v1, off_h0, off_h1, op_stride, staged;
+  int n_dir, n_unique, Mm, MX, MZ, Kx, NY, cv, rb0, rb1, off_v0, off_v1, off_h0, off_h1, op_stride, staged;
   double inv_dt;
 };
 
@@ -73,21 +75,35 @@ __device__ __forceinline__ void mode_of(const OneArgs& a, int u, int* pos, int* 
   }
 }
 
-// mode u of direction dir
-template <typename T>
-__device__ __forceinline__ void solve_one(const OneArgs& a, int u, int dir, unsigned char* smem, uint64_t* s_bar) {
+// mode u of the directions dir0 to dir0 + D - 1 (as far as there are). Work items take the directions
+// slowest, so that the last warp of a phase is filled by the next direction.
+template <typename T, int D>
+__device__ __forceinline__ void solve_one(const OneArgs& a, int u, int dir0, unsigned char* smem, uint64_t* s_bar) {
   const int NY = a.NY, N = NY - 1, NH = N / 2 + 1, NR = N - 1, Mm = a.Mm, MZ = a.MZ;
   const int tid = threadIdx.x, nt = blockDim.x, warp = tid >> 5, nw = nt >> 5;
+  const int nd = D == 1 ? 1 : min(D, a.n_dir - dir0);
   double* sop = reinterpret_cast<double*>(smem);
-  double2* sdu = reinterpret_cast<double2*>(sop + (a.staged ? a.op_stride : 0));  // [3][NY]
-  double2* sfa = sdu + 3 * NY;  // [NR] -i f_a
-  double2* sfb = sfa + NR;      // [NR] (mean mode: f_u)
-  double2* srv = sfb + NR;      // [2][cv] reduced right-hand sides per parity
-  double2* sfw = srv + 2 * a.cv;  // [NR] mean mode: f_w; float: staged right-hand sides
-  double2* sv = sfw + 3 * NR;   // [NY]
-  double2* sb = sv + NY;        // [NY]
-  double2* ss = sb + NY;        // [NY + 1] sums of p v_p over p >= n of the parity of n
-  C2<T>* vals = reinterpret_cast<C2<T>*>(ss + NY + 1);  // [3][NY] (float)
+  double2* sdu = reinterpret_cast<double2*>(sop + (a.staged ? a.op_stride : 0));  // [D][3][NY]
+  double2* sfa = sdu + D * 3 * NY;  // [D][NR] -i f_a
+  double2* sfb = sfa + D * NR;      // [D][NR] (mean mode: f_u)
+  double2* srv = sfb + D * NR;      // [D][2][cv] reduced right-hand sides per parity
+  double2* sfw = srv + D * 2 * a.cv;  // [D][3][NR] staged right-hand sides
+  double2* sv = sfw + D * 3 * NR;   // [D][NY]
+  double2* sb = sv + D * NY;        // [D][NY]
+  double2* ss = sb + D * NY;        // [D][NY + 1] sums of p v_p over p >= n of the parity of n
+  C2<T>* vals = reinterpret_cast<C2<T>*>(ss + D * (NY + 1));  // [D][3][NY] (float)
+  // direction of item i, per items each; i becomes the item in it
+  auto split = [&](int& i, int per) -> int {
+    if constexpr (D == 1) return 0;
+    int d = 0;
+#pragma unroll
+    for (int q = 1; q < D; ++q)
+      if (i >= per) {
+        i -= per;
+        ++d;
+      }
+    return d;
+  };
   int pos, iz;
   mode_of(a, u, &pos, &iz);
   const bool mean = u == 0;
@@ -95,24 +111,26 @@ __device__ __forceinline__ void solve_one(const OneArgs& a, int u, int dir, unsi
   if (a.staged && tid == 0) stage_begin(sop, op, (uint32_t)a.op_stride * 8, s_bar);
   const double kx = __ldg(a.wave + 4 * u), kz = __ldg(a.wave + 4 * u + 1), ik = __ldg(a.wave + 4 * u + 2);
   // input state (Hermitian-projected)
-  const double2* dsrc = a.du + ((size_t)dir * 3 * Mm + pos * MZ + iz) * NY;
+  const double2* dsrc = a.du + ((size_t)dir0 * 3 * Mm + pos * MZ + iz) * NY;
   const long long mir = pos == 0 ? 0 : (long long)(a.MX - 2 * pos) * MZ * NY;  // to the mirror mode
-  for (int i = tid; i < 3 * NY; i += nt) {
-    const int c = i / NY;
+  for (int i = tid; i < nd * 3 * NY; i += nt) {
+    const int c = i / NY;  // component of a direction: the directions follow one another
     const double2* p = dsrc + (size_t)c * Mm * NY + (i - c * NY);
     double2 v = __ldg(p);
     if (iz == 0) v = project(v, __ldg(p + mir));
     sdu[i] = v;
   }
   if constexpr (sizeof(T) == 8) {
-    const double2* W = static_cast<const double2*>(a.in) + ((size_t)dir * a.n_unique + u) * 3 * NR;
-    for (int i = tid; i < 3 * NR; i += nt) sfw[i] = __ldg(W + i);
+    for (int d = 0; d < nd; ++d) {
+      const double2* W = static_cast<const double2*>(a.in) + ((size_t)(dir0 + d) * a.n_unique + u) * 3 * NR;
+      for (int i = tid; i < 3 * NR; i += nt) sfw[d * 3 * NR + i] = __ldg(W + i);
+    }
     __syncthreads();
   } else {
     // forward transform of the values: even and odd parts of the point pairs, then one thread per row
     // (even rows first; the order of k_solve's sums)
-    const C2<T>* vin = static_cast<const C2<T>*>(a.in) + (size_t)dir * 3 * NY * Mm + pos * MZ + iz;
-    for (int i = tid; i < 3 * NH; i += nt) {
+    const C2<T>* vin = static_cast<const C2<T>*>(a.in) + (size_t)dir0 * 3 * NY * Mm + pos * MZ + iz;
+    for (int i = tid; i < nd * 3 * NH; i += nt) {
       const int c = i / NH, j = i - c * NH;
       const C2<T> p = vin[((size_t)c * NY + j) * Mm], q = vin[((size_t)c * NY + N - j) * Mm];
       C2<T>* col = vals + c * NY;
@@ -124,52 +142,57 @@ __device__ __forceinline__ void solve_one(const OneArgs& a, int u, int dir, unsi
       }
     }
     __syncthreads();
-    const int ne = (NR + 1) / 2;
-    for (int i = tid; i < 3 * NR; i += nt) {
-      const bool odd = i >= 3 * ne;
-      const int k = odd ? i - 3 * ne : i, per = odd ? NR - ne : ne;
+    const int ne = (NR + 1) / 2, even = nd * 3 * ne;
+    for (int i = tid; i < nd * 3 * NR; i += nt) {
+      const bool odd = i >= even;
+      const int k = odd ? i - even : i, per = odd ? NR - ne : ne;
       const int c = k / per, n = 2 * (k - c * per) + (odd ? 1 : 0);
       const C2<T>* col = vals + c * NY;
       const float* cf = a.cft + n;
       C2<T> acc = mk((T)0, (T)0);
       if (!odd) {
-        for (int j = 0; j < NH - 1; ++j) acc = acc + scl(col[j], (T)__ldg(cf + j * NY));
-        acc = acc + scl(col[NH - 1], (T)__ldg(cf + (NH - 1) * NY));
+        for (int j = 0; j < NH - 1; ++j) acc = acc + scl(col[j], __ldg(cf + j * NY));
+        acc = acc + scl(col[NH - 1], __ldg(cf + (NH - 1) * NY));
       } else {
-        for (int j = 0; j < NH - 1; ++j) acc = acc + scl(col[N - j], (T)__ldg(cf + j * NY));
+        for (int j = 0; j < NH - 1; ++j) acc = acc + scl(col[N - j], __ldg(cf + j * NY));
       }
       const double2 d = sdu[c * NY + n];
-      double2 f = make_double2((double)acc.x + d.x * a.inv_dt, (double)acc.y + d.y * a.inv_dt);
+      double2 f = make_double2(fma(d.x, a.inv_dt, widen(acc.x)), fma(d.y, a.inv_dt, widen(acc.y)));
       if (mean) f.y = 0.0;
       sfw[c * NR + n] = f;
     }
     __syncthreads();
   }
   // rotation to the components along / across the wavevector
-  for (int n = tid; n < NR; n += nt) {
-    const double2 fx = sfw[n], fy = sfw[NR + n], fz = sfw[2 * NR + n];
+  for (int i = tid; i < nd * NR; i += nt) {
+    int n = i;
+    const int d = split(n, NR);
+    const double2* fw = sfw + d * 3 * NR;
+    const double2 fx = fw[n], fy = fw[NR + n], fz = fw[2 * NR + n];
     if (mean) {
-      sfb[n] = fx;
-      sfa[n] = fz;
+      sfb[i] = fx;
+      sfa[i] = fz;
       continue;
     }
     const double2 fa = make_double2((kx * fx.x + kz * fz.x) * ik, (kx * fx.y + kz * fz.y) * ik);
-    sfb[n] = make_double2((-kz * fx.x + kx * fz.x) * ik, (-kz * fx.y + kx * fz.y) * ik);
-    srv[(n & 1) * a.cv + n / 2] = fy;
-    sfa[n] = make_double2(fa.y, -fa.x);  // -i f_a
+    sfb[i] = make_double2((-kz * fx.x + kx * fz.x) * ik, (-kz * fx.y + kx * fz.y) * ik);
+    srv[d * 2 * a.cv + (n & 1) * a.cv + n / 2] = fy;
+    sfa[i] = make_double2(fa.y, -fa.x);  // -i f_a
   }
   __syncthreads();
   // reduced right-hand side g_n = f_v,n - (2 / (c_n k)) sum over m > n, m + n odd, of m (-i f_a,m)
   if (!mean) {
-    for (int P = warp; P < 2; P += nw) {
-      double2* g = srv + P * a.cv;
+    for (int q = warp; q < 2 * nd; q += nw) {
+      const int P = q & 1;
+      double2* g = srv + q * a.cv;
+      const double2* fa = sfa + (q >> 1) * NR;
       suffix_scan(
           P == 0 ? a.rb0 : a.rb1,
           [&](int i) -> double2 {
             const int m = 2 * i + P + 1;
             if (m > N - 2) return make_double2(0.0, 0.0);
             const double w = __ldg(a.row + m);
-            return make_double2(w * sfa[m].x, w * sfa[m].y);
+            return make_double2(w * fa[m].x, w * fa[m].y);
           },
           [&](int i, double2 s) {
             const double f = (2 * i + P == 0 ? 1.0 : 2.0) * ik;
@@ -185,15 +208,17 @@ __device__ __forceinline__ void solve_one(const OneArgs& a, int u, int dir, unsi
   ok = __syncthreads_and(ok) != 0;  // the limit ran out: NaN below
   // v = V g and b = H f_b: one row of one operator per thread
   const int nv0 = N / 2 + 1;
-  for (int i = tid; i < 2 * NY; i += nt) {
-    const bool hel = i < NY;
-    const int k = hel ? i : i - NY;
+  for (int i = tid; i < nd * 2 * NY; i += nt) {
+    int r = i;
+    const int d = split(r, 2 * NY);
+    const bool hel = r < NY;
+    const int k = hel ? r : r - NY;
     const int Q = k < nv0 ? 0 : 1, row = Q == 0 ? k : k - nv0, n = 2 * row + Q;
     const int nrow = Q == 0 ? nv0 : NY - nv0, rb = Q == 0 ? a.rb0 : a.rb1;
     const double* H = op + (Q == 0 ? a.off_h0 : a.off_h1) + row;
     const double* V = op + (Q == 0 ? a.off_v0 : a.off_v1) + row;
     // mean flow: u and w from the Helmholtz operator, v = 0
-    const double2* x = hel ? sfb + Q : mean ? sfa + Q : srv + Q * a.cv;
+    const double2* x = hel ? sfb + d * NR + Q : mean ? sfa + d * NR + Q : srv + (2 * d + Q) * a.cv;
     const double* M = hel || mean ? H : V;
     const int xs = hel || mean ? 2 : 1;
     double2 s[4] = {};
@@ -213,62 +238,68 @@ __device__ __forceinline__ void solve_one(const OneArgs& a, int u, int dir, unsi
       s[0].x = fma(w, y.x, s[0].x);
       s[0].y = fma(w, y.y, s[0].y);
     }
-    (hel ? sb : sv)[n] = make_double2((s[0].x + s[1].x) + (s[2].x + s[3].x), (s[0].y + s[1].y) + (s[2].y + s[3].y));
+    (hel ? sb : sv)[d * NY + n] = make_double2((s[0].x + s[1].x) + (s[2].x + s[3].x), (s[0].y + s[1].y) + (s[2].y + s[3].y));
   }
   __syncthreads();
   // (D v)_n = (2 / c_n) sum over p > n, p + n odd, of p v_p
   if (!mean) {
-    for (int P = warp; P < 2; P += nw)
+    for (int q = warp; q < 2 * nd; q += nw) {
+      const int P = q & 1;
+      const double2* v = sv + (q >> 1) * NY;
+      double2* to = ss + (q >> 1) * (NY + 1);
       suffix_scan(
           P == 0 ? nv0 : NY - nv0,
           [&](int i) -> double2 {
             const int p = 2 * i + P;
             const double w = __ldg(a.row + p);
-            return make_double2(w * sv[p].x, w * sv[p].y);
+            return make_double2(w * v[p].x, w * v[p].y);
           },
-          [&](int i, double2 s) { ss[2 * i + P] = s; });
+          [&](int i, double2 s) { to[2 * i + P] = s; });
+    }
   }
   __syncthreads();
   // a = (i/k) D v, back-rotation, G = u_new - u, Hermitian output
-  double2* dst = a.out + ((size_t)dir * 3 * Mm + pos * MZ + iz) * NY;
-  for (int n = tid; n < NY; n += nt) {
+  double2* dst = a.out + ((size_t)dir0 * 3 * Mm + pos * MZ + iz) * NY;
+  for (int i = tid; i < nd * NY; i += nt) {
+    int n = i;
+    const int d = split(n, NY);
     double2 un, vn, wn;
     if (mean) {
-      un = make_double2(sb[n].x, 0.0);
-      wn = make_double2(sv[n].x, 0.0);
+      un = make_double2(sb[i].x, 0.0);
+      wn = make_double2(sv[i].x, 0.0);
       vn = make_double2(0.0, 0.0);
     } else {
       double2 dv = make_double2(0.0, 0.0);
       if (n + 1 < NY) {
-        const double2 sp = ss[n + 1];
+        const double2 sp = ss[d * (NY + 1) + n + 1];
         const double f = n == 0 ? 1.0 : 2.0;
         dv = make_double2(f * sp.x, f * sp.y);
       }
       const double2 an = make_double2(-dv.y * ik, dv.x * ik);  // (i/k) Dv
-      const double2 bn = sb[n];
+      const double2 bn = sb[i];
       un = make_double2((kx * an.x - kz * bn.x) * ik, (kx * an.y - kz * bn.y) * ik);
       wn = make_double2((kz * an.x + kx * bn.x) * ik, (kz * an.y + kx * bn.y) * ik);
-      vn = sv[n];
+      vn = sv[i];
     }
     const double2 res[3] = {un, vn, wn};
 #pragma unroll
     for (int c = 0; c < 3; ++c) {
-      const double2 d = sdu[c * NY + n];
-      double2 g = make_double2(res[c].x - d.x, res[c].y - d.y);
+      const double2 e = sdu[(3 * d + c) * NY + n];
+      double2 g = make_double2(res[c].x - e.x, res[c].y - e.y);
       if (mean) g.y = 0.0;
       if (!ok) g = make_double2(nan(""), nan(""));
-      double2* o = dst + (size_t)c * Mm * NY + n;
+      double2* o = dst + (size_t)(3 * d + c) * Mm * NY + n;
       *o = g;
       if (iz == 0 && pos != 0) o[mir] = make_double2(g.x, -g.y);
     }
   }
 }
 
-template <typename T>
+template <typename T, int D>
 __global__ void __launch_bounds__(512) k_solve_one(const __grid_constant__ OneArgs a) {
   extern __shared__ __align__(16) unsigned char smem[];
   __shared__ __align__(8) uint64_t s_bar;
-  solve_one<T>(a, blockIdx.x, blockIdx.y, smem, &s_bar);
+  solve_one<T, D>(a, blockIdx.x, blockIdx.y * D, smem, &s_bar);
 }
 
 struct GOne {
@@ -291,7 +322,7 @@ __global__ void __launch_bounds__(512) k_solve_one_grp(const double* __restrict_
     r.a.out = reinterpret_cast<double2*>(out + r.off);
   }
   __syncthreads();
-  solve_one<T>(r.a, blockIdx.x - first[i], 0, smem, &s_bar);
+  solve_one<T, 1>(r.a, blockIdx.x - first[i], 0, smem, &s_bar);
 }
 
 // out[4 i] = sum of x[xs j] over j <= i, in order; the first entry halved (c_0 = 2) where asked
@@ -503,10 +534,10 @@ __global__ void __launch_bounds__(512) k_solve_adj(const __grid_constant__ OneAr
 // operators in shared memory up to this size (N <= 104); larger ones are read in place
 constexpr size_t kStageBytes = 100 * 1024;
 
-size_t one_smem(const sp_ctx* c, int esize) {
+size_t one_smem(const sp_ctx* c, int esize, int D = 1) {
   const size_t ops = (size_t)c->op_stride * 8 <= kStageBytes ? (size_t)c->op_stride * 8 : 0;
   const size_t NY = c->NY, NR = c->N - 1;
-  return ops + 16 * (3 * NY + 2 * NR + 2 * c->cv + 3 * NR + 3 * NY + 1) + (esize == 4 ? 3 * NY * 8 + 8 : 0);
+  return ops + D * (16 * (3 * NY + 2 * NR + 2 * c->cv + 3 * NR + 3 * NY + 1) + (esize == 4 ? 3 * NY * 8 + 8 : 0));
 }
 
 OneArgs one_args(const sp_ctx* c, const void* in, const double* du, double* out) {
@@ -518,6 +549,7 @@ OneArgs one_args(const sp_ctx* c, const void* in, const double* du, double* out)
   a.wave = c->wave;
   a.cft = c->cft_f;
   a.row = c->rowidx;
+  a.n_dir = 1;
   a.n_unique = c->n_unique;
   a.Mm = c->Mm; a.MX = c->MX; a.MZ = c->MZ; a.Kx = c->Kx; a.NY = c->NY;
   a.cv = c->cv; a.rb0 = c->rb0; a.rb1 = c->rb1;
@@ -530,22 +562,45 @@ OneArgs one_args(const sp_ctx* c, const void* in, const double* du, double* out)
 
 }  // namespace
 
-// threads of a block: one per row of the two operators (shape 0), or a fixed number
-int solve_one_threads(const sp_ctx* c, int shape) {
-  const int rows = std::min((2 * c->NY + 31) / 32 * 32, 512);
+// Threads of a block: one per row of the two operators of every direction (shape 0; in equal rounds past
+// 512), or a fixed number. us with 224, 288 and 352 threads, two directions of 48 x 81 x 48, 31 mixed ones:
+// 823, 770, 676.
+static int threads_of(const sp_ctx* c, int shape, int D) {
+  const int all = 2 * c->NY * D, rounds = (all + 511) / 512;
+  const int rows = D == 1 ? std::min((all + 31) / 32 * 32, 512) : ((all + rounds - 1) / rounds + 31) / 32 * 32;
   const int fixed[SP_TUNE_MAX] = {rows, 64, 96, 128, 192, 256, 384, 512};
   return fixed[shape];
+}
+int solve_one_threads(const sp_ctx* c, int shape) { return threads_of(c, shape, 1); }
+
+// Directions of a block. With one, a phase's last warp is partly filled (70 rows on 96 lanes at 35 points) and
+// the operators are staged for every direction; with several, a call of few blocks leaves SMs idle. us per
+// solve with 1, 2 and 4 directions, mixed: 48 x 35 x 48, 4 directions 41, 37, 37; 8: 68, 60, 60; 31: 238, 207,
+// 195; 48 x 65 x 48, 3: 70, 64, 72; 31: 612, 518, 535; 24 x 25 x 24 (113 modes), 8: 16.5, 16.4, 19.4; 12: 20.6,
+// 22.6, 24.7; 31: 45.5, 45.1, 49.6. So two from nine blocks per SM, four for short columns from 36; and both
+// only where two blocks share an SM.
+static int directions_of(const sp_ctx* c, int n_dir, int esize) {
+  const long long blocks = (long long)c->n_unique * n_dir, sms = c->sm_count;
+  if (blocks >= 36 * sms && 8 * c->NY <= 288 && one_smem(c, esize, 4) <= 112 * 1024) return 4;
+  return blocks >= 9 * sms && one_smem(c, esize, 2) <= 112 * 1024 ? 2 : 1;
+}
+
+template <typename T>
+static cudaError_t launch_one(const sp_ctx* c, const OneArgs& a, int shape, int D, cudaStream_t st) {
+  const size_t sm = one_smem(c, sizeof(T), D);
+  auto kern = D == 1 ? k_solve_one<T, 1> : D == 2 ? k_solve_one<T, 2> : k_solve_one<T, 4>;
+  const cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+  if (e != cudaSuccess) return e;
+  kern<<<dim3(c->n_unique, (a.n_dir + D - 1) / D), threads_of(c, shape, D), sm, st>>>(a);
+  return cudaGetLastError();
 }
 
 cudaError_t launch_solve_one(const sp_ctx* c, bool fp32, const void* in, const double* du, double* out, int n_dir,
                              int shape, cudaStream_t st) {
-  const OneArgs a = one_args(c, in, du, out);
-  const size_t sm = one_smem(c, fp32 ? 4 : 8);
-  auto kern = fp32 ? k_solve_one<float> : k_solve_one<double>;
-  const cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
-  if (e != cudaSuccess) return e;
-  kern<<<dim3(c->n_unique, n_dir), solve_one_threads(c, shape), sm, st>>>(a);
-  return cudaGetLastError();
+  OneArgs a = one_args(c, in, du, out);
+  a.n_dir = n_dir;
+  const int D = directions_of(c, n_dir, fp32 ? 4 : 8);
+  return fp32 ? launch_one<float>(c, a, shape, D, st) : launch_one<double>(c, a, shape, D, st);
 }
 
 cudaError_t grp_build_solve_one(GrpKernel* k, sp_ctx* const* mem, int n, const size_t* offs, const int* order, int esize) {
