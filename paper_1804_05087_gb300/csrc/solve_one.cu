@@ -581,8 +581,8 @@ int solve_one_threads(const sp_ctx* c, int shape) { return threads_of(c, shape, 
 // only where two blocks share an SM.
 static int directions_of(const sp_ctx* c, int n_dir, int esize) {
   const long long blocks = (long long)c->n_unique * n_dir, sms = c->sm_count;
-  if (blocks >= 36 * sms && 8 * c->NY <= 288 && one_smem(c, esize, 4) <= 112 * 1024) return 4;
-  return blocks >= 9 * sms && one_smem(c, esize, 2) <= 112 * 1024 ? 2 : 1;
+  if (n_dir >= 4 && blocks >= 36 * sms && 8 * c->NY <= 288 && one_smem(c, esize, 4) <= 112 * 1024) return 4;
+  return n_dir >= 2 && blocks >= 9 * sms && one_smem(c, esize, 2) <= 112 * 1024 ? 2 : 1;
 }
 
 template <typename T>
