@@ -73,7 +73,7 @@ extern "C" sp_status sp_jvp_static(sp_ctx* c, const double* du, double* Jdu, voi
   // every entry of both intermediates is written before it is read, so the
   // contents left by an earlier call need no clearing
   if ((s = sp_cuda(c, launch_yinv(c, f32, du, ws6, 1, st), "yinv")) != SP_OK) return s;
-  // FP64 planes stay out of the context's buffers: on chip (48 x 65 x 48: 60 us against 42 with several
+  // FP64 planes stay out of the context's buffers: on chip (48 x 65 x 48: 51 us against 35 with several
   // blocks per plane through the context's buffer, where an sp_step on another stream could write) or
   // behind ws3, which the solve's scratch takes over afterwards
   const cudaError_t e = !f32 && c->use_fx ? launch_xz_fx_apart(c, XZ_TANGENT, ws6, ws3, p + b6 + b3,

@@ -32,7 +32,9 @@ size_t chunk_bytes(const sp_ctx* c, int rp, int fields) {
   return (size_t)rp * fields * c->fx_n1z * (c->fx_n2z + 1) * 16;
 }
 size_t plane_bytes(const sp_ctx* c) { return (size_t)c->nx * 6 * c->MZ * 16; }
-// row pairs per chunk: z buffers of about 34 KB
+// row pairs per chunk: z buffers of about 34 KB, which leave two blocks of 48 x 48 planes on an SM (us with 24,
+// 34 and 48 KB: 256 tangents of 48 x 65 x 48 3460, 3157, 4670; 32 of 64 x 65 x 64 1377, 1160, 1125; one of
+// 36 x 45 x 24 26.8, 26.8, 24.6)
 int chunk_rows(const sp_ctx* c, int mode) {
   return std::max(1, std::min(c->nx / 2, (int)(34 * 1024 / chunk_bytes(c, 1, z_fields(mode)))));
 }
@@ -40,7 +42,9 @@ size_t fused_smem(const sp_ctx* c, int mode) {
   return tw_bytes(c) + plane_bytes(c) + chunk_bytes(c, chunk_rows(c, mode), z_fields(mode));
 }
 
-// blocks per plane of a split x transform: about 24 KB of staging each
+// blocks per plane of a split x transform: about 24 KB of staging each (every block scans the plane for its
+// scales; us of the three launches with 12, 24 and 48 KB, one tangent: 48 x 65 x 48 41, 35, 39; 64 x 65 x 64
+// 82, 66, 58; 96 x 97 x 96 282, 196, 156: large planes would take larger parts)
 int split_parts(const sp_ctx* c, int ncol) {
   const int most = std::max(8, (int)(24576 / (16 * c->nx)));
   return (ncol + most - 1) / most;
@@ -77,12 +81,13 @@ Args make_args(const sp_ctx* c, int mode, const void* in, void* out) {
 }
 
 // Three launches with several blocks per plane instead of one block per plane: planes that do not
-// fit on chip, and large planes that are too few to give every SM one. Measured (us, one block |
-// several): 48 x 48, 65 planes 60 | 42; 64 x 64, 65 planes 95 | 76; 48 x 48, 260 planes 72 | 103;
-// 32 x 32, 49 planes 31 | 36; 36 x 24, 45 planes 31 | 35; 16 x 16, 33 planes 14 | 25.
+// fit on chip, and large planes that fill less than two thirds of the SMs. Measured (us of a tangent, one
+// block | several): 48 x 48, 65 planes 51 | 35; 97: 51 | 45; 113: 51 | 55; 260: 60 | 89; 64 x 64, 65 planes
+// 84 | 66; 97: 83 | 74; 113: 84 | 92; 32 x 32, 49 planes 27 | 31; 36 x 24, 45 planes 27 | 31; 16 x 16, 33 planes
+// 12.5 | 23.
 bool use_split(const sp_ctx* c, int mode, int n_dir) {
   if (fused_smem(c, mode) > kSmemMax) return true;
-  return c->nx * c->nz > 1600 && (long long)c->NY * n_dir < c->sm_count;
+  return c->nx * c->nz > 1600 && 3LL * c->NY * n_dir < 2LL * c->sm_count;
 }
 
 }  // namespace
