@@ -627,8 +627,11 @@ static cudaError_t psolve_t(const sp_ctx* c, const PArgs& a, const void* in3, co
   return cudaGetLastError();
 }
 
-// directions per block: sixteen (full warps of chains) where two such blocks share an SM, else eight where
-// they fit, else one
+// Directions per block: eight from two directions on, where their factors and vectors fit; sixteen (full warps
+// of chains) where two such blocks share an SM and there are at least eight per SM. us with 1, 8 and 16, FP64:
+// 613 modes of Nr = 64, 2 directions 273, 254, 362; 4: 445, 281, 389; 16: 1627, 566, 600; 24: 2467, 902, 874;
+// 64: 6627, 2037, 1882; 163 modes of Nr = 32, 4: 86, 78, 78; 16: 281, 109, 123; 64: 962, 300, 294; 145 modes
+// of Nr = 96, 2: 210, 207, 206; 16: 844, 262, 305; 64: 3359, 1037, 1174.
 template <typename T, bool TG>
 static cudaError_t psolve_nd(const sp_ctx* c, const PArgs& a, const void* in3, const double2* uu, const double2* U0,
                              double2* o, int n_dir, cudaStream_t st) {
@@ -636,9 +639,10 @@ static cudaError_t psolve_nd(const sp_ctx* c, const PArgs& a, const void* in3, c
   // the grids that a block with one mode's four matrices holds (radial counts up to 235)
   if (4 * c->pb_chunk + (size_t)4 * psolve_nrp(c->NY) * 16 + (size_t)2 * c->NY * 9 * 12 > kMax) return cudaErrorInvalidValue;
   const bool r64 = c->NY == 64;
-  if (n_dir >= 12 && psolve_smem(16, c->NY, c->pb_chunk) <= kMax / 2)
+  const long long blocks16 = (long long)c->n_unique * ((n_dir + 15) / 16);
+  if (n_dir > 16 && blocks16 >= 8LL * c->sm_count && psolve_smem(16, c->NY, c->pb_chunk) <= kMax / 2)
     return r64 ? psolve_t<T, TG, 16, 64>(c, a, in3, uu, U0, o, n_dir, st) : psolve_t<T, TG, 16, 0>(c, a, in3, uu, U0, o, n_dir, st);
-  if (n_dir >= 4 && psolve_smem(8, c->NY, c->pb_chunk) <= kMax)
+  if (n_dir >= 2 && psolve_smem(8, c->NY, c->pb_chunk) <= kMax)
     return r64 ? psolve_t<T, TG, 8, 64>(c, a, in3, uu, U0, o, n_dir, st) : psolve_t<T, TG, 8, 0>(c, a, in3, uu, U0, o, n_dir, st);
   return r64 ? psolve_t<T, TG, 1, 64>(c, a, in3, uu, U0, o, n_dir, st) : psolve_t<T, TG, 1, 0>(c, a, in3, uu, U0, o, n_dir, st);
 }
