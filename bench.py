@@ -223,6 +223,43 @@ def kernel_flops(stage, n_dir, prec="mixed"):
     return 0
 
 
+# 32-bit integer multiply-adds with a 64-bit sum per SM and clock (measured: lanes of mad.wide.s32 in a loop of
+# nothing else), the unit of the fixed-point transforms
+WIDE_MADS_PER_CLOCK = 25.1
+
+
+def fx_factors(n):
+    """n = a b with both factors among the radices of the fixed-point plane stage, or None (xz_fx.cu)."""
+    radices = (12, 9, 8, 6, 4, 3, 2)
+    for a in radices:
+        if a * a <= n and n % a == 0 and n // a in radices:
+            return a, n // a
+    return None
+
+
+def wide_mads(stage, n_dir):
+    """Integer multiply-adds of one FP64 launch (three per real product; additions not counted), or None
+    where the stage does not run in fixed point."""
+    kx, kz, mx, mz, ny = dims()
+    nh = (ny - 1) // 2 + 1
+    ph = (nh + 1) & ~1
+    if stage == "k_yinv":  # five complex columns, values and derivatives
+        return n_dir * mx * mz * nh * 2 * ph * 5 * 6
+    if stage == "k_rhs":
+        return n_dir * n_unique() * (ny - 2) * ph * 3 * 6
+    if stage != "k_xz" or mz > 48 or not fx_factors(NX) or not fx_factors(NZ):
+        return None
+    radix = {2: 0, 3: 6, 4: 0, 6: 12, 8: 12, 9: 84, 12: 24}  # constant products of one transform
+
+    def length(n, forward):
+        a, b = fx_factors(n)
+        a, b = (b, a) if forward else (a, b)
+        return b * (radix[a] + 12 * (a - 1)) + a * radix[b]  # twiddles: 12 each
+    plane = (6 * mz * length(NX, False) + 3 * NX * length(NZ, False) + NX * NZ * 12 * 3 +
+             3 * NX // 2 * length(NZ, True) + 3 * mz * length(NX, True))
+    return n_dir * ny * plane
+
+
 FP64_NOMINAL = 1.25  # TFLOP/s, the recipe's nominal GB300 FP64 rate (replaced by the measured probe)
 
 
@@ -230,7 +267,16 @@ def kernel_traffic(stage, n_dir, prec, lam_adv):
     """DRAM bytes of one launch from an ncu capture of the current kernel, or None."""
     if stage == "k_solve" and prec == "mixed" and not lam_adv and not chain(n_dir):
         return solve_traffic(n_dir)
+    if prec == "fp64" and not lam_adv and chain(n_dir) and (NX, NY, NZ) == (48, 65, 48):
+        if stage in FP64_DRAM_64:
+            return sum(FP64_DRAM_64[stage]) * n_dir / 64
     return None
+
+
+# DRAM bytes (read, written) of one FP64 launch at 48x65x48 with 64 directions, from an ncu capture of
+# the four launches (dram__bytes_read.sum, dram__bytes_write.sum); they scale with the directions
+FP64_DRAM_64 = {"k_yinv": (99151872, 143092992), "k_xz": (205447168, 72466688), "k_rhs": (198198272, 64971520),
+                "k_solve": (339796992, 193709824)}
 
 
 # DRAM bytes of one mixed-precision k_solve tangent launch at 48x65x48 with 64 directions, from
@@ -1350,18 +1396,21 @@ def throughput(args, prec_name, rank, world, local, keep_out=False, e2e=True):
     hbm = peaks["hbm_gbs"]
     fp32_peak = 152 * 128 * 2 * 2.07e9 / 1e12  # SMs x FP32 lanes x FMA x max clock
     fp64_bound = dom == "k_solve"  # the solve is FP64 in both modes
-    # FP64 transforms run in 64-bit fixed point: three 32-bit multiply-adds with a 64-bit sum per real
-    # multiply-add, 32 of them per SM and clock
-    int_peak = 152 * 32 * 2.07e9 * 2 / 3 / 1e12
-    alu_peak = FP64_NOMINAL if fp64_bound else int_peak if prec_name == "fp64" else fp32_peak
-    if gbs / hbm >= tfs / alu_peak:
+    mads = wide_mads(dom, nd) if prec_name == "fp64" and not fp64_bound else None
+    if mads:  # fixed point
+        alu, alu_peak, unit = mads / avg_s / 1e12, 152 * WIDE_MADS_PER_CLOCK * 2.07e9 / 1e12, "T multiply-adds/s"
+        source = f"152 SMs x {WIDE_MADS_PER_CLOCK} wide integer multiply-adds per clock (measured) x 2.07 GHz"
+    else:
+        fp64_pipe = fp64_bound or prec_name == "fp64"
+        alu, alu_peak, unit = tfs, FP64_NOMINAL if fp64_pipe else fp32_peak, "TFLOP/s"
+        source = (f"nominal FP64 {FP64_NOMINAL} TFLOP/s" if fp64_pipe
+                  else "152 SMs x 128 FP32 lanes x 2 flop x 2.07 GHz")
+    if gbs / hbm >= alu / alu_peak:
         roof = {"bound": "hbm", "achieved": gbs, "peak": hbm, "unit": "GB/s", "frac": gbs / hbm,
                 "peak_source": "measured (MEASURED_PEAKS.json hbm_gbs)"}
     else:
-        roof = {"bound": "alu", "achieved": tfs, "peak": alu_peak, "unit": "TFLOP/s", "frac": tfs / alu_peak,
-                "peak_source": f"nominal FP64 {FP64_NOMINAL} TFLOP/s" if fp64_bound
-                else "152 SMs x 32 wide integer multiply-adds / 3 x 2 flop x 2.07 GHz" if prec_name == "fp64"
-                else "152 SMs x 128 FP32 lanes x 2 flop x 2.07 GHz", "fp64": fp64_bound}
+        roof = {"bound": "alu", "achieved": alu, "peak": alu_peak, "unit": unit, "frac": alu / alu_peak,
+                "peak_source": source, "fp64": fp64_bound}
     roof.update({"kernel": dom, "traffic": kernel_traffic(dom, nd, prec_name, bool(args.lam_adv)),
                  "avg_launch_ms": dom_ms / dom_n,
                  "algorithmic_bytes_per_launch": bytes_l, "algorithmic_flops_per_launch": flops_l,

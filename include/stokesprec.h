@@ -35,6 +35,12 @@
  *   No call traps or aborts the process. Invalid arguments return SP_EINVAL
  *   before any work is enqueued.
  * Threads: a context may be used by one host thread at a time.
+ * Values: SP_FP64 transforms run in 64-bit fixed point, scaled per field and
+ *   plane or column, with errors at or below those of transforms in double;
+ *   planes whose sides are not products of two of 2, 3, 4, 6, 8, 9, 12, or
+ *   with more than 48 kept kz, stay in double. There a subnormal input counts
+ *   as zero, and a NaN or an infinity makes every value of its plane NaN
+ *   (hence, through the solves, of its state's result).
  */
 #ifndef STOKESPREC_H
 #define STOKESPREC_H
@@ -59,7 +65,7 @@ typedef enum {
 } sp_status;
 
 typedef enum {
-  SP_FP64 = 0,      /* every stage in double precision                       */
+  SP_FP64 = 0,      /* every stage in double precision (see Values above)    */
   SP_MIXED = 1      /* transforms and products in float, solve/residual in double */
 } sp_prec;
 
@@ -271,7 +277,7 @@ sp_status sp_trace_read(sp_ctx* ctx, double* ms, long long* launches, int n);
 
 /* The paper has no counterpart: a measurement of the device's FP64 fused
  * multiply-add rate, the denominator of the roofline of the FP64-bound kernels
- * (the per-mode solve, the FP64 transforms). Launches blocks x 256 threads on
+ * (the per-mode solve). Launches blocks x 256 threads on
  * `stream`, each running 8 independent chains of `iters` FMAs: 4096 x blocks x
  * iters flops per launch. The caller times it with events on the same stream.
  * out: device buffer of blocks x 256 doubles (written, so the chains are not

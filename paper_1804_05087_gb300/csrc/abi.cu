@@ -362,11 +362,12 @@ static sp_status pipe_phase(sp_ctx* c, const double* du, double* out, int n_dir,
   return SP_OK;
 }
 
-// The tangent's per-mode solve of one pass: the O(N) chains (k_rhs, then k_chain) on
-// contexts built for large batches, else the dense per-mode operators (k_solve).
 // bytes of the context's ws3 (max_batch planes of three complex fields)
 static size_t ws3_bytes(const sp_ctx* c) { return (size_t)c->cfg.max_batch * 3 * c->NY * c->Mm * 16; }
 
+// The tangent's per-mode solve of one pass: the O(N) chains (k_rhs or k_rhs_fx, then k_chain) on
+// contexts built for large batches, else the dense per-mode operators (k_solve_one; with laminar
+// advection in L k_solve).
 sp_status sp_tangent_solve(sp_ctx* c, bool f32, void* vals, size_t vals_bytes, const double* du, double* out,
                            void* work, int nb, cudaStream_t st) {
   // the O(N) chains use vals (consumed by their right-hand-side launch) as their scratch

@@ -6,12 +6,12 @@
 //   k_rhs_fx : values of the product -> coefficients of the rows 0..N-2, plus u/dt: the right-hand
 //              sides of the per-mode solves (k_chain, k_solve).
 //
-// Both are sums over the constants T_n(y_j) = cos(pi j n / N). The FP64 pipe issues 2 operations per
-// SM and clock, the integer pipes about 28 multiply-adds of 32-bit halves (measured), three of which
-// make one term of a sum whose inputs share a scale. 48 x 65 x 48, 256 directions: k_yinv_fx 1.69 ms
-// (FP64 4.05), k_rhs_fx 1.01 ms (FP64 2.39). A column (one component of one mode) is scaled by its largest
-// value (59 bits) and its sum of moduli (62 bits, a bound of every result) and split as
-// x = hi 2^28 + lo; the constants are 56-bit, split the same way. hi hi and hi lo + lo hi are summed
+// Both are sums over the constants T_n(y_j) = cos(pi j n / N). An SM does 25 multiply-adds of 32-bit halves per
+// clock but 1.7 in FP64 (fx_arith.h), and three of them make one term of a sum whose inputs share a scale.
+// 48 x 65 x 48, 256 directions: k_yinv_fx 1.72 ms (FP64 4.05; its multiply-adds alone 1.09), k_rhs_fx 1.03 ms
+// (FP64 2.39; 0.61). A column (one component of one mode) is scaled by its largest value, a point pair's sum
+// by twice that (59 bits, after rounding up), and by its sum of moduli (62 bits, a bound of every result), and
+// split as x = hi 2^28 + lo; the constants are 56-bit, split the same way. hi hi and hi lo + lo hi are summed
 // in two 64-bit accumulators (both stay below 2^63 up to 129 terms, N <= 256); lo lo, below a quarter
 // of a unit, is dropped. Derivatives: n^2 a_n, scaled as a column of its own, times T_n'(y_j) / n^2.
 // Points y and -y share a table row: T_n(-y) = (-1)^n T_n(y), T_n'(-y) = -(-1)^n T_n'(y).

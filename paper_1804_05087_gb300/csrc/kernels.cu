@@ -1,6 +1,8 @@
 // CUDA kernels of the BEFE step, its tangent and the vector operations.
 //
-// One step (Sec. 2, Eq. befe) in Fourier x,z / Chebyshev y is three kernels:
+// One step (Sec. 2, Eq. befe) in Fourier x,z / Chebyshev y is three stages. Here are the float ones, the
+// generic FP64 plane stage and the solve with laminar advection; the others are in cheb_fx.cu, xz_fx.cuh
+// (FP64 in fixed point), xz_reg.cu, yinv_tc.cu (float), solve_one.cu and solve_chain.cu.
 //   k_yinv : per Fourier mode, Chebyshev coefficients -> values at the
 //            Gauss-Lobatto points of u, v, w and of the vorticity (curl taken
 //            in spectral space: i kx, i kz and the coefficient derivative),
@@ -12,10 +14,10 @@
 //            Sec. 3.2).
 //   k_solve: per Fourier mode, values -> Chebyshev coefficients, the
 //            right-hand side u/dt + N, the Chebyshev-tau Stokes solve through
-//            the precomputed per-mode operators, and G = u_new - u.
-//            With laminar advection in L (Sec. 3.6) the right-hand side gains
+//            the precomputed per-mode operators, and G = u_new - u, with laminar
+//            advection in L (Sec. 3.6): the right-hand side gains
 //            M u = y du/dx + v e_x and the operators are the complex ones of
-//            that system (template flag LA).
+//            that system (the plain step: k_solve_one).
 // T is the real type of the transforms and the product (double or float);
 // the solve and everything after it are double.
 #include <algorithm>
@@ -35,14 +37,6 @@ constexpr int kTileYinvAdj = 4;  // modes per k_yinv_adj block
 constexpr int kTileSolve = 4;   // modes per k_solve block
 
 // ------------------------------------------------------------------ FFT
-// Batched complex FFT of length pl.n in shared memory, Stockham
-// decimation-in-time with radices 2, 3 and 4. Stage s combines p = radix[s]
-// sub-transforms of length L (product of the earlier radices):
-//   out[(t0 + L d) R' + b'] = sum_c (w_n^{c t0 R'} in[t0 R + b' + R' c]) w_p^{c d}
-// with R = n/L, R' = R/p, w_m = exp(sgn 2 pi i / m). The first stage reads its
-// input through `load(b, e)` (element e of transform b), the last stage hands
-// its outputs to `store(b, e, v)`; the stages in between ping-pong between s0
-// and s1 (layout [element][batch]). Ends with __syncthreads().
 // One stage of radix P on nb transforms: butterfly bf = t0 Rp + bp of transform b.
 template <typename T, int P, class LoadF, class StoreF>
 __device__ __forceinline__ void fft_stage(int n, int L, int Rp, fx::Div dRp, int nb, fx::Div dnb, bool first, bool last,
@@ -95,6 +89,14 @@ __device__ __forceinline__ void fft_stage(int n, int L, int Rp, fx::Div dRp, int
   }
 }
 
+// Batched complex FFT of length pl.n in shared memory, Stockham
+// decimation-in-time with radices 2, 3 and 4. Stage s combines p = radix[s]
+// sub-transforms of length L (product of the earlier radices):
+//   out[(t0 + L d) R' + b'] = sum_c (w_n^{c t0 R'} in[t0 R + b' + R' c]) w_p^{c d}
+// with R = n/L, R' = R/p, w_m = exp(sgn 2 pi i / m). The first stage reads its
+// input through `load(b, e)` (element e of transform b), the last stage hands
+// its outputs to `store(b, e, v)`; the stages in between ping-pong between s0
+// and s1 (layout [element][batch]). Ends with __syncthreads().
 template <typename T, class LoadF, class StoreF>
 __device__ __forceinline__ void fft_batch(const FftPlan& pl, int nb, const C2<T>* __restrict__ tw, T sgn, C2<T>* s0,
                                           C2<T>* s1, LoadF load, StoreF store) {
@@ -476,7 +478,7 @@ __device__ __forceinline__ void unique_to_mode(int u, int Kx, int MZ, int* pos, 
 // du : [dir][3][Mm][NY] complex double; out: same layout (G = u_new - u)
 // (bx, by): tile of solved modes, direction
 // TM: solved modes per block (any block size works; every mode's arithmetic is the same)
-// LA: laminar advection in L (right-hand side + M du, complex operators)
+// The step with laminar advection in L: right-hand side + M du, complex operators (without it: k_solve_one)
 template <typename T, int TM>
 __device__ __forceinline__ void solve_body(const C2<T>* __restrict__ in3, const double2* __restrict__ du,
                                            double2* __restrict__ out, const SolveArgs& a, int bx, int by) {
@@ -583,42 +585,42 @@ __device__ __forceinline__ void solve_body(const C2<T>* __restrict__ in3, const 
     }
     __syncthreads();
   } else {
-  // phase A2: even/odd pairs of the values, once per (component, mode, point pair):
-  // s_j = f(y_j) + f(y_N-j) replaces f(y_j), d_j = f(y_j) - f(y_N-j) replaces f(y_N-j)
-  // (T_n(y_N-j) = (-1)^n T_n(y_j), so even rows read s and odd rows read d)
-  for (int idx = threadIdx.x; idx < 3 * TM * (NH - 1); idx += blockDim.x) {
-    const int t = idx % TM;
-    const int jj = (idx / TM) % (NH - 1);
-    const int c = idx / (TM * (NH - 1));
-    C2<T>* col = svals + (c * NY) * TM + t;
-    const C2<T> p = col[jj * TM], q = col[(N - jj) * TM];
-    col[jj * TM] = p + q;
-    col[(N - jj) * TM] = p - q;
-  }
-  __syncthreads();
-  // phase B: forward Chebyshev transform of N (rows 0..N-2) and the RHS u/dt + N; the even and
-  // the odd rows in separate loops, so that no warp mixes the two trip counts
-  for (int par = 0; par < 2; ++par)
-  for (int idx = threadIdx.x, cnt = par ? NR / 2 : (NR + 1) / 2; idx < 3 * TM * cnt; idx += blockDim.x) {
-    const int t = idx % TM;
-    const int n = 2 * ((idx / TM) % cnt) + par;
-    const int c = idx / (TM * cnt);
-    C2<T> acc = mk((T)0, (T)0);
-    const C2<T>* col = svals + (c * NY) * TM + t;
-    const float* cf = a.Cfh_f + (size_t)n * NH;
-    if ((n & 1) == 0) {
-      for (int jj = 0; jj < NH - 1; ++jj) acc = acc + scl(col[jj * TM], (T)cf[jj]);
-      acc = acc + scl(col[(NH - 1) * TM], (T)cf[NH - 1]);
-    } else {
-      for (int jj = 0; jj < NH - 1; ++jj) acc = acc + scl(col[(N - jj) * TM], (T)cf[jj]);
+    // phase A2: even/odd pairs of the values, once per (component, mode, point pair):
+    // s_j = f(y_j) + f(y_N-j) replaces f(y_j), d_j = f(y_j) - f(y_N-j) replaces f(y_N-j)
+    // (T_n(y_N-j) = (-1)^n T_n(y_j), so even rows read s and odd rows read d)
+    for (int idx = threadIdx.x; idx < 3 * TM * (NH - 1); idx += blockDim.x) {
+      const int t = idx % TM;
+      const int jj = (idx / TM) % (NH - 1);
+      const int c = idx / (TM * (NH - 1));
+      C2<T>* col = svals + (c * NY) * TM + t;
+      const C2<T> p = col[jj * TM], q = col[(N - jj) * TM];
+      col[jj * TM] = p + q;
+      col[(N - jj) * TM] = p - q;
     }
-    const double2 d = sdu[(c * TM + t) * NY + n];
-    double2 f = make_double2(fma(d.x, a.inv_dt, widen(acc.x)), fma(d.y, a.inv_dt, widen(acc.y)));
-    add_lam(f, c, t, n);
-    if (s_pos[t] == 0 && s_iz[t] == 0) f.y = 0.0;
-    sf[(c * TM + t) * NR + n] = f;
-  }
-  __syncthreads();
+    __syncthreads();
+    // phase B: forward Chebyshev transform of N (rows 0..N-2) and the RHS u/dt + N; the even and
+    // the odd rows in separate loops, so that no warp mixes the two trip counts
+    for (int par = 0; par < 2; ++par)
+    for (int idx = threadIdx.x, cnt = par ? NR / 2 : (NR + 1) / 2; idx < 3 * TM * cnt; idx += blockDim.x) {
+      const int t = idx % TM;
+      const int n = 2 * ((idx / TM) % cnt) + par;
+      const int c = idx / (TM * cnt);
+      C2<T> acc = mk((T)0, (T)0);
+      const C2<T>* col = svals + (c * NY) * TM + t;
+      const float* cf = a.Cfh_f + (size_t)n * NH;
+      if ((n & 1) == 0) {
+        for (int jj = 0; jj < NH - 1; ++jj) acc = acc + scl(col[jj * TM], (T)cf[jj]);
+        acc = acc + scl(col[(NH - 1) * TM], (T)cf[NH - 1]);
+      } else {
+        for (int jj = 0; jj < NH - 1; ++jj) acc = acc + scl(col[(N - jj) * TM], (T)cf[jj]);
+      }
+      const double2 d = sdu[(c * TM + t) * NY + n];
+      double2 f = make_double2(fma(d.x, a.inv_dt, widen(acc.x)), fma(d.y, a.inv_dt, widen(acc.y)));
+      add_lam(f, c, t, n);
+      if (s_pos[t] == 0 && s_iz[t] == 0) f.y = 0.0;
+      sf[(c * TM + t) * NR + n] = f;
+    }
+    __syncthreads();
   }
   // phase C: rotate to the components along / across the wavevector; f_v goes to
   // srv (per parity), f~_a = -i f_a replaces f_x in sf (same thread, same slot)

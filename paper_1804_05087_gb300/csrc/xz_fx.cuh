@@ -4,9 +4,10 @@
 // forward FFT along x truncated to the retained modes. Values in and out are doubles; in between
 // they are integers with one power-of-two scale per stage (fx_arith.h).
 //
-// Why integers: the FP64 pipe issues 2 operations per SM and clock, the integer pipes about 28 multiply-
-// adds of 32-bit halves or 52 additions of 64 bits (measured), and a plane's transforms need no range,
-// only precision. 48 x 65 x 48, 256 tangents: 12.57 ms in FP64 registers, 3.11 ms here.
+// Why integers: an SM does 25 multiply-adds of 32-bit halves and 56 additions of 64 bits per clock but 1.7 in
+// FP64 (fx_arith.h), and a plane's transforms need no range, only precision. 48 x 65 x 48, 256 tangents:
+// 12.57 ms in FP64 registers, 3.16 ms here, of which the multiply-adds alone are 0.68 (three per real product;
+// the rest is shifts, carries, barriers and instruction fetch).
 //
 // Scales (every transformed value stays below 2^61). The x transforms of a field are scaled by the
 // largest sum of moduli of its columns, the z transforms by that of its plane: bounds of every value
