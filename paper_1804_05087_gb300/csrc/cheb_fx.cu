@@ -206,18 +206,6 @@ struct RArgs {
   double inv_dt, c0, cn;  // 1 / N, 2 / N
 };
 
-__device__ __forceinline__ void unique_mode_of(int u, int Kx, int MZ, int* pos, int* iz) {
-  const int first = (Kx + 1) * MZ;
-  if (u < first) {
-    *pos = u / MZ;
-    *iz = u - *pos * MZ;
-  } else {
-    const int v = u - first;
-    *pos = Kx + 1 + v / (MZ - 1);
-    *iz = 1 + v % (MZ - 1);
-  }
-}
-
 template <int TM>
 struct RShared {
   unsigned em[3 * TM];
@@ -235,7 +223,7 @@ __device__ __forceinline__ void rhs_fx(const RArgs& a, int bx, int by, int bz, i
   const int tid = threadIdx.x;
   if (tid < TM) {
     int pos = 0, iz = 0;
-    if (u0 + tid < a.n_unique) unique_mode_of(u0 + tid, a.Kx, a.MZ, &pos, &iz);
+    if (u0 + tid < a.n_unique) unique_mode(u0 + tid, a.Kx, a.MZ, &pos, &iz);
     s.pos[tid] = pos;
     s.iz[tid] = iz;
   }

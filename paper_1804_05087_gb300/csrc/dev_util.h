@@ -3,6 +3,20 @@
 
 #include <cuda_runtime.h>
 
+// stored position (x index in FFT order) and kz index of solved mode u: all kz of ix >= 0, then kz >= 1 of
+// ix < 0 (the others follow by Hermitian symmetry)
+__device__ __forceinline__ void unique_mode(int u, int Kx, int MZ, int* pos, int* iz) {
+  const int first = (Kx + 1) * MZ;
+  if (u < first) {
+    *pos = u / MZ;
+    *iz = u - *pos * MZ;
+  } else {
+    const int v = u - first;
+    *pos = Kx + 1 + v / (MZ - 1);
+    *iz = 1 + v % (MZ - 1);
+  }
+}
+
 // sum_c w[c * ws] x[c * xs] with four independent partial sums (real w, complex x):
 // eight independent FMA chains per thread hide the FP64 latency
 __device__ __forceinline__ double2 dot4(const double* __restrict__ w, int ws, const double2* x, int xs, int n) {

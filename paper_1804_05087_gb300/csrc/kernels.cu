@@ -461,18 +461,6 @@ struct SolveArgs {
   double alpha, beta, inv_dt;
 };
 
-__device__ __forceinline__ void unique_to_mode(int u, int Kx, int MZ, int* pos, int* iz) {
-  const int first = (Kx + 1) * MZ;
-  if (u < first) {
-    *pos = u / MZ;
-    *iz = u - *pos * MZ;
-  } else {
-    const int v = u - first;
-    *pos = Kx + 1 + v / (MZ - 1);
-    *iz = 1 + v % (MZ - 1);
-  }
-}
-
 // in3: float: [dir][3][NY][Mm] complex values of N at the Gauss-Lobatto points; double: the
 //      right-hand sides u/dt + N of k_rhs_fx, [dir][mode][3][N - 1]
 // du : [dir][3][Mm][NY] complex double; out: same layout (G = u_new - u)
@@ -501,7 +489,7 @@ __device__ __forceinline__ void solve_body(const C2<T>* __restrict__ in3, const 
   if (threadIdx.x < TM) {
     const int u = u0 + threadIdx.x;
     int pos = 0, iz = 0;
-    if (u < a.n_unique) unique_to_mode(u, a.Kx, MZ, &pos, &iz);
+    if (u < a.n_unique) unique_mode(u, a.Kx, MZ, &pos, &iz);
     s_pos[threadIdx.x] = pos;
     s_iz[threadIdx.x] = iz;
     s_u[threadIdx.x] = u;

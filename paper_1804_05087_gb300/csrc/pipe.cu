@@ -91,18 +91,6 @@ __global__ void __launch_bounds__(kThreadsP) k_pvals(const double2* __restrict__
   }
 }
 
-__device__ __forceinline__ void unique_mode_d(int u, int Kx, int MZ, int* pos, int* iz) {
-  const int first = (Kx + 1) * MZ;
-  if (u < first) {
-    *pos = u / MZ;
-    *iz = u - *pos * MZ;
-  } else {
-    const int v = u - first;
-    *pos = Kx + 1 + v / (MZ - 1);
-    *iz = 1 + v % (MZ - 1);
-  }
-}
-
 // Hermitian projection of entry (c, pos, iz, j) of a state
 __device__ __forceinline__ double2 sym_load(const double2* s, int c, int pos, int iz, int j, const PArgs& a) {
   double2 v = __ldg(s + ((size_t)c * a.Mm + pos * a.MZ + iz) * a.NR + j);
@@ -271,7 +259,7 @@ __global__ void __launch_bounds__(psolve_threads(ND)) k_psolve(const C2<T>* __re
   const int tid = threadIdx.x, nt = blockDim.x;
   const uint32_t bar = smem_addr(&s_bar);
   int pos, iz;
-  unique_mode_d(mode, a.Kx, a.MZ, &pos, &iz);
+  unique_mode(mode, a.Kx, a.MZ, &pos, &iz);
   const bool mean = pos == 0 && iz == 0;
   const int kzi = pos <= a.Kx ? pos : pos - a.MX;
   const double k = a.alpha * kzi, mm = a.sym * iz;

@@ -45,18 +45,6 @@ constexpr int kRhsTM = 4;         // modes per block
 constexpr int kRhsD = 4;          // directions per block
 constexpr int kRhsThreads = 192;
 
-__device__ __forceinline__ void mode_of(int u, int Kx, int MZ, int* pos, int* iz) {
-  const int first = (Kx + 1) * MZ;
-  if (u < first) {
-    *pos = u / MZ;
-    *iz = u - *pos * MZ;
-  } else {
-    const int v = u - first;
-    *pos = Kx + 1 + v / (MZ - 1);
-    *iz = 1 + v % (MZ - 1);
-  }
-}
-
 // in3: [dir][3][NY][Mm] complex float; du: [dir][3][Mm][NY] complex double
 //
 // Moves 0.95 GB at 48 x 65 x 48 with 256 directions (140 us of memory traffic). With a thread per (mode,
@@ -78,7 +66,7 @@ __global__ void __launch_bounds__(kRhsThreads) k_rhs(const C2<float>* __restrict
   const int tile = blockIdx.x / nd, dir0 = (blockIdx.x - tile * nd) * kRhsD, u0 = tile * TM, nu = min(TM, a.n_unique - u0);
   if (threadIdx.x < TM) {
     int pos = 0, iz = 0;
-    if ((int)threadIdx.x < nu) mode_of(u0 + threadIdx.x, a.Kx, MZ, &pos, &iz);
+    if ((int)threadIdx.x < nu) unique_mode(u0 + threadIdx.x, a.Kx, MZ, &pos, &iz);
     s_pos[threadIdx.x] = pos;
     s_iz[threadIdx.x] = iz;
   }
@@ -306,7 +294,7 @@ __global__ void __launch_bounds__(32 * kChainWarps, kChainBlocksPerSM) k_chain(C
     u = item - d * a.n_unique;
   }
   int pos, iz;
-  mode_of(u, a.Kx, a.MZ, &pos, &iz);
+  unique_mode(u, a.Kx, a.MZ, &pos, &iz);
   const int N = a.N, NY = a.NY, Mm = a.Mm, MZ = a.MZ, NR = N - 1;
   const double2* Wb = a.W + u * a.su + d * a.sd;
   auto fval = [&](int c, int n) -> double2 {  // right-hand side row n of component c (0 above N-2)

@@ -63,18 +63,6 @@ __device__ __forceinline__ bool stage_wait(uint64_t* s_bar) {
   return done != 0;
 }
 
-__device__ __forceinline__ void mode_of(const OneArgs& a, int u, int* pos, int* iz) {
-  const int first = (a.Kx + 1) * a.MZ;
-  if (u < first) {
-    *pos = u / a.MZ;
-    *iz = u - *pos * a.MZ;
-  } else {
-    const int v = u - first;
-    *pos = a.Kx + 1 + v / (a.MZ - 1);
-    *iz = 1 + v % (a.MZ - 1);
-  }
-}
-
 // mode u of the directions dir0 to dir0 + D - 1 (as far as there are). Work items take the directions
 // slowest, so that the last warp of a phase is filled by the next direction.
 template <typename T, int D>
@@ -105,7 +93,7 @@ __device__ __forceinline__ void solve_one(const OneArgs& a, int u, int dir0, uns
     return d;
   };
   int pos, iz;
-  mode_of(a, u, &pos, &iz);
+  unique_mode(u, a.Kx, a.MZ, &pos, &iz);
   const bool mean = u == 0;
   const double* op = a.ops + (size_t)u * a.op_stride;
   if (a.staged && tid == 0) stage_begin(sop, op, (uint32_t)a.op_stride * 8, s_bar);
@@ -373,7 +361,7 @@ __global__ void __launch_bounds__(512) k_solve_adj(const __grid_constant__ OneAr
   double2* sfa = sfb + NR;       // [NR] sums of f~_a* (mean mode: H^T gu)
   C2<T>* sf = reinterpret_cast<C2<T>*>(sfa + NR);  // [3][NR] f*
   int pos, iz;
-  mode_of(a, u, &pos, &iz);
+  unique_mode(u, a.Kx, a.MZ, &pos, &iz);
   const bool mean = u == 0;
   const double* op = a.ops + (size_t)u * a.op_stride;
   const int v1 = a.staged ? a.rb0 * st0 : a.off_v1, h0 = a.staged ? v1 + a.rb1 * st1 : a.off_h0,

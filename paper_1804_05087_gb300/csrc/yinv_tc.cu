@@ -23,6 +23,7 @@
 #include <cstring>
 #include <vector>
 
+#include "dev_util.h"
 #include "sp_internal.h"
 
 namespace {
@@ -338,18 +339,6 @@ struct RhsTcArgs {
   double inv_dt;
 };
 
-__device__ __forceinline__ void unique_mode_tc(int u, int Kx, int MZ, int* pos, int* iz) {
-  const int first = (Kx + 1) * MZ;
-  if (u < first) {
-    *pos = u / MZ;
-    *iz = u - *pos * MZ;
-  } else {
-    const int v = u - first;
-    *pos = Kx + 1 + v / (MZ - 1);
-    *iz = 1 + v % (MZ - 1);
-  }
-}
-
 template <int KP>
 __global__ void __launch_bounds__(kTcThreads, 1) k_rhs_tc(RhsTcArgs a) {
   extern __shared__ __align__(128) unsigned char smem[];
@@ -410,7 +399,7 @@ __global__ void __launch_bounds__(kTcThreads, 1) k_rhs_tc(RhsTcArgs a) {
       const int u = u0 + ml, dir = dg * 4 + dl;
       if (c < 3 && k < NY && u < a.n_unique && dir < a.n_dir) {
         int pos, iz;
-        unique_mode_tc(u, a.Kx, a.MZ, &pos, &iz);
+        unique_mode(u, a.Kx, a.MZ, &pos, &iz);
         pre[r] = __ldg(a.in + (size_t)dir * 3 * NY * a.Mm + ((size_t)c * NY + k) * a.Mm + pos * a.MZ + iz);
       }
     }
@@ -422,7 +411,7 @@ __global__ void __launch_bounds__(kTcThreads, 1) k_rhs_tc(RhsTcArgs a) {
     if (threadIdx.x < 4) {
       const int u = u0 + threadIdx.x;
       int pos = 0, iz = 0;
-      if (u < a.n_unique) unique_mode_tc(u, a.Kx, a.MZ, &pos, &iz);
+      if (u < a.n_unique) unique_mode(u, a.Kx, a.MZ, &pos, &iz);
       s_m[threadIdx.x] = u;
       s_pos[threadIdx.x] = pos;
       s_iz[threadIdx.x] = iz;
